@@ -262,9 +262,8 @@ swf_status swf_set_dedupe(swf_ctx* ctx, int on);
  * call that sit on different grids but share the time grid (t_out, t_in, step count) and the
  * non-trivial axes, and that run on the pass kernels at fixed steps (Schwinger, and
  * Breit-Wheeler with the integrand of Eq. 17), can be marched together, up to eight groups at a
- * time: one launch per pass serves all of them, persistent blocks taking (group, block) work
- * items from a device counter, largest grids first, and one CUDA graph replays their step
- * pairs.  Each group's results are bitwise those of marching it alone.
+ * time: side by side on one stream per group, one CUDA graph per group and pair of steps, so that
+ * small grids fill the GPU together.  Each group's results are bitwise those of marching it alone.
  * mode = 1 (default): together when the groups hold fewer than 4 Mi fields x grid points (above
  * that each group fills the GPU alone); 2: always together; 0: one group after another. */
 swf_status swf_set_multi_grid(swf_ctx* ctx, int mode);
@@ -280,8 +279,8 @@ swf_status swf_fields_fused(swf_ctx* ctx, long long* count);
  * a NULL pointer. */
 swf_status swf_plan_split(int n_fields, int clusters, int sms, int* pass_fields);
 
-/* Launch shapes of the pass kernels (rows per block of the x passes, tile width of the y and z
- * passes, 256 or 128 threads per block).  on = 1 (default): the first march of each grid
+/* Launch shapes of the pass kernels (rows per block of the x passes, columns per block of the y and
+ * z passes).  on = 1 (default): the first march of each grid
  * shape in this context times the candidate shapes (a few launches each, before the march
  * starts) and keeps the fastest;
  * on = 0: a fixed rule from the grid size.  A shape only decides which lines a block

@@ -17,6 +17,10 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libswf.so")
 SOURCES = ["swf_api.cu", "swf_march.cu", "swf_project.cu", "swf_fused.cu", "swf_noalloc.cu", "swf_bw.cu", "swf_mlp.cu",
            "swf_pairs.cu"]
+# the register line kernels: one unit per list of lengths (swf_line_list.h)
+LINE_LISTS = 5
+UNITS = [(src, [], os.path.splitext(src)[0]) for src in SOURCES] + [
+    ("swf_line.cu", [f"-DSWF_LINE_LIST={i}", "-DSWF_LINE_REAL=float"], f"swf_line{i}") for i in range(LINE_LISTS)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
@@ -28,9 +32,10 @@ def nvcc() -> str:
     return path
 
 
-def _compile(src: str, verbose: bool) -> str:
-    obj = os.path.join(OUT_DIR, os.path.splitext(src)[0] + ".o")
-    cmd = [nvcc(), *ARCH, *FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+def _compile(unit, verbose: bool) -> str:
+    src, defines, name = unit
+    obj = os.path.join(OUT_DIR, name + ".o")
+    cmd = [nvcc(), *ARCH, *FLAGS, *defines, "-c", os.path.join(CSRC, src), "-o", obj]
     if verbose:
         cmd.insert(1, "-Xptxas=-v")
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -50,8 +55,8 @@ def build(verbose: bool = False, force: bool = False) -> str:
         lib_t = os.path.getmtime(LIB)
         if all(os.path.getmtime(d) <= lib_t for d in deps):
             return LIB
-    with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(lambda s: _compile(s, verbose), SOURCES))
+    with ThreadPoolExecutor(max_workers=max(4, os.cpu_count() or 4)) as ex:
+        objs = list(ex.map(lambda u: _compile(u, verbose), UNITS))
     tmp = LIB + ".tmp"
     cmd = [nvcc(), *ARCH, "-shared", "-o", tmp, *objs, "-lcudart"]
     res = subprocess.run(cmd, capture_output=True, text=True)

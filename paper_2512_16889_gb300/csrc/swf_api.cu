@@ -50,36 +50,33 @@ swf_status ws_get(swf_ctx* ctx, const std::string& name, size_t bytes, void** pt
   return SWF_OK;
 }
 
-swf_status twiddles(swf_ctx* ctx, int n, int is_double, const void** ptr) {
-  auto key = std::make_pair(n, is_double);
+// Twiddles of length n in double or single precision, rounded once from long double: natural order
+// exp(-2 pi i m/n), m < n (r2 = 0), or the table of the register line kernels, entry k1 r2 + i =
+// exp(-2 pi i i k1/n).
+swf_status twiddles(swf_ctx* ctx, int n, int is_double, const void** ptr, int r2) {
+  auto key = std::make_pair(n, (is_double ? 1 : 0) + 2 * r2);
   auto it = ctx->tw.tables.find(key);
   if (it != ctx->tw.tables.end()) {
     *ptr = it->second;
     return SWF_OK;
   }
-  std::vector<double> re(n), im(n);
-  for (int m = 0; m < n; ++m) {
-    // exp(-2 pi i m/n) evaluated in long double and rounded once
-    long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)m / (long double)n;
-    re[m] = (double)cosl(a);
-    im[m] = (double)sinl(a);
+  const size_t esz = is_double ? 16 : 8;
+  std::vector<unsigned char> host(esz * n);
+  for (int e = 0; e < n; ++e) {
+    const int m = r2 ? ((e / r2) * (e % r2)) % n : e;
+    const long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)m / (long double)n;
+    const double v[2] = {(double)cosl(a), (double)sinl(a)};
+    const float w[2] = {(float)v[0], (float)v[1]};
+    std::memcpy(&host[esz * e], is_double ? (const void*)v : (const void*)w, esz);
   }
   void* p = nullptr;
-  size_t bytes = (size_t)n * (is_double ? 16 : 8);
-  cudaError_t e = cudaMalloc(&p, bytes);
+  cudaError_t e = cudaMalloc(&p, host.size());
   if (e != cudaSuccess) return cuda_status(e, "cudaMalloc(twiddles)");
-  std::vector<unsigned char> host(bytes);
-  for (int m = 0; m < n; ++m) {
-    if (is_double) {
-      double v[2] = {re[m], im[m]};
-      std::memcpy(&host[16 * m], v, 16);
-    } else {
-      float v[2] = {(float)re[m], (float)im[m]};
-      std::memcpy(&host[8 * m], v, 8);
-    }
+  e = cudaMemcpy(p, host.data(), host.size(), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(p);
+    return cuda_status(e, "upload twiddles");
   }
-  e = cudaMemcpy(p, host.data(), bytes, cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return cuda_status(e, "upload twiddles");
   ctx->tw.tables[key] = p;
   *ptr = p;
   return SWF_OK;
@@ -97,9 +94,10 @@ int prof_begin(swf_ctx* ctx, const char* family, cudaStream_t st) {
     }
   }
   int fam = -1;
+  const std::string name = ctx->in_multi ? std::string(family) + "_multi" : std::string(family);
   for (size_t i = 0; i < P.families.size(); ++i)
-    if (P.families[i] == family) fam = (int)i;
-  if (fam < 0) { P.families.push_back(family); fam = (int)P.families.size() - 1; }
+    if (P.families[i] == name) fam = (int)i;
+  if (fam < 0) { P.families.push_back(name); fam = (int)P.families.size() - 1; }
   const size_t first = P.used;
   P.used += 2;
   cudaEventRecord(P.pool[first], st);
@@ -822,6 +820,11 @@ swf_status swf_destroy(swf_ctx* ctx) {
   for (auto& kv : ctx->ws.bufs) cudaFree(kv.second.first);
   for (auto& kv : ctx->tw.tables) cudaFree(kv.second);
   for (auto ev : ctx->prof.pool) cudaEventDestroy(ev);
+  for (auto ms : ctx->multi_st) {
+    cudaStreamSynchronize(ms);
+    cudaStreamDestroy(ms);
+  }
+  for (auto ev : ctx->multi_ev) cudaEventDestroy(ev);
   if (ctx->aux) {
     cudaStreamSynchronize(ctx->aux);
     for (auto ev : ctx->aux_ev)

@@ -142,6 +142,9 @@ struct swf_ctx {
   bool sm_split = true;   // automatic path: pass kernels on the SMs the fused clusters leave free
   cudaStream_t aux = nullptr;            // stream of that concurrent pass-kernel march (lazy)
   cudaEvent_t aux_ev[2] = {nullptr, nullptr};
+  std::vector<cudaStream_t> multi_st;    // one stream and event per group of a multi-grid march (lazy)
+  std::vector<cudaEvent_t> multi_ev;
+  bool in_multi = false;                 // a multi-grid march is being queued (kernel timing names)
 };
 
 namespace swf {
@@ -165,8 +168,9 @@ swf_status cuda_status(cudaError_t e, const char* what);
 
 // Returns a device buffer of at least `bytes` under `name` (grows, never shrinks).
 swf_status ws_get(swf_ctx* ctx, const std::string& name, size_t bytes, void** ptr);
-// Device table exp(-2 pi i m/n), m < n, in float2 (is_double = 0) or double2.
-swf_status twiddles(swf_ctx* ctx, int n, int is_double, const void** ptr);
+// Device table exp(-2 pi i m/n), m < n, in float2 (is_double = 0) or double2; with r2 > 0 in the order
+// of the register line kernels.
+swf_status twiddles(swf_ctx* ctx, int n, int is_double, const void** ptr, int r2 = 0);
 
 // ---- march (swf_march.cu)
 // March n_f fields (all on grid g) from psi(t_out) = 0 to t_in; psi_out receives psi(t_in)
@@ -209,9 +213,9 @@ swf_status bw_packet(swf_ctx* ctx, int n, const swf_result* results, const doubl
 swf_status bw_finalize_partial(swf_ctx* ctx, const GridDesc& g, int n_inst, const void* bw_host,
                                const double2* macc, const double* norms, swf_result* results, cudaStream_t st);
 
-// Multi-grid march: groups of fields on different grids sharing one time grid, marched by one
-// launch per pass for all groups (persistent blocks on a device work queue) and one CUDA graph
-// per step pair.  Each group's result is bitwise that of marching it alone.
+// Multi-grid march: groups of fields on different grids sharing one time grid, marched side by side
+// on one stream per group (one CUDA graph per group and step pair).  Each group's result is bitwise
+// that of marching it alone.
 struct MultiGroup {
   GridDesc g;
   int F;                  // fields (Breit-Wheeler: 2 per instance, U then V)

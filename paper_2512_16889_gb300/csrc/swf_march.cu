@@ -4,14 +4,16 @@
 //     k = -i [ H0 Y + V(t, x) (Y + psi_b(t, x)) ]
 // with H0 applied per Fourier mode (Eq. 10).  One evaluation is a chain of line passes over
 // the planar state [f][4][z][y][x]:
-//   first pass (x lines):  Y = y + h sum_j a_ij k_j (stage combine, Dormand-Prince), the local
-//                          term Z = -i V (Y + psi_b) stashed in the output slot, forward x-FFT;
-//   middle passes (y, z):  forward FFT along the axis; on the last axis -i H0(kappa)/N and the
-//                          inverse FFT;
-//   last pass (x lines):   inverse x-FFT and k = (that) + Z.
+//   x pass:             Y = y + h sum_j a_ij k_j (stage combine, Dormand-Prince), the local term
+//                       Z = -i V (Y + psi_b) stashed in the output slot, forward x-FFT;
+//   y and z passes:     forward FFT along the axis; on the last axis -i H0(kappa)/N and the
+//                       inverse FFT;
+//   the next x pass:    inverse x-FFT and k = (that) + Z, before its own evaluation's work.
+// Complex64 lengths with line kernels (swf_line.cuh) transform in registers; complex128 and the other
+// lengths run on the small-radix passes (k_xpass, k_mid).
 // Gauge field and background are analytic and evaluated on the fly from per-field 1D tables
 // (every field kind is a product of a time factor and one factor per axis).
-#include <array>
+#include <type_traits>
 #include <atomic>
 #include <algorithm>
 #include <cmath>
@@ -20,7 +22,7 @@
 #include <cstdio>
 #include <cstring>
 
-#include "swf_internal.h"
+#include "swf_line.cuh"
 
 namespace swf {
 
@@ -36,78 +38,6 @@ static const double DP_A[7][6] = {
     {9017.0 / 3168, -355.0 / 33, 46732.0 / 5247, 49.0 / 176, -5103.0 / 18656, 0},
     {35.0 / 384, 0, 500.0 / 1113, 125.0 / 192, -2187.0 / 6784, 11.0 / 84}};
 
-template <typename R>
-struct StageArgs {
-  cpx<R>* y;
-  const cpx<R>* kin[6];
-  double coef[6];
-  int nterm;
-  int write_y;
-  cpx<R>* kout;
-  cpx<R>* T;
-  const FieldDesc* fd;
-  const R* greal;       // per field: gx[nx] gy[ny] gz[nz]
-  const cpx<R>* gcplx;  // per field: ex[nx] ey[ny] ez[nz] w[4]
-  const cpx<R>* tw[3];
-  const R* kap;         // mode momenta kappa_j = 2 pi j'/L_a of the axes with n_a > 1, rounded once
-                        // from FP64, at offsets 0, nx, nx + ny (FP64 is scarce on this GPU)
-  R inv_n;              // 1/N rounded once
-  RadixPlan plan[3];
-  GridDesc g;
-  int nrows;            // ny * nz
-  double t;             // stage time when clk is null
-  cpx<R>* ystage;       // optional: receives the stage value Y (Breit-Wheeler integrand)
-  const struct MarchClock* clk;  // march clock (graph replays), or null
-  int ls;               // step within the replayed pair of steps (0 or 1)
-  double c;             // Dormand-Prince node c_i of the stage
-  const struct StepControl* ctl;  // step-size-controlled march, or null (see march_adaptive)
-  cpx<R>* ynew;         // with ctl: the last stage writes the step's result here, not into y
-  cpx<R>* yspec;        // optional: receives the grid transform of the stage value (written by the
-                        // y or z pass that applies H0, before it does)
-  cpx<R>* ylo;          // optional (complex64 fixed-step marches): the rounding error of y, so that
-                        // y + ylo carries the state in float-float (Knuth's two-sum per step)
-};
-
-// (hi, lo) += s in float-float arithmetic (Knuth's two-sum, then a fast renormalisation): on
-// return s holds the new rounded state and lo its rounding error.
-__device__ __forceinline__ void ff_accumulate(float hi, float& lo, float& s) {
-  const float t = __fadd_rn(hi, s);
-  const float bp = __fsub_rn(t, hi);
-  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bp)), __fsub_rn(s, bp));
-  const float l = __fadd_rn(lo, e);
-  const float nh = __fadd_rn(t, l);
-  lo = __fsub_rn(l, __fsub_rn(nh, t));
-  s = nh;
-}
-
-// State of a step-size-controlled march, in device memory: the accepted time t and the step h
-// of the current attempt (the stage times are t + c_i h and the stage coefficients h a_ij), the
-// tolerances, counters and flags.  One thread of k_step_control updates it after every attempt.
-struct StepControl {
-  double t, h, t_in, span, rtol, atol;
-  int done;        // t_in reached, or the march failed: later attempts do nothing
-  int ok;          // the last attempt was accepted (its result and k_7 are copied in)
-  int failed;      // too many attempts or a non-finite error
-  int accepted, rejected, max_attempts;
-};
-
-// Device clock of a march whose steps are replayed from a CUDA graph: the stage time is
-// (t_out + (step + ls) h) + c_i h, the host loop's arithmetic, with `step` advanced on the device
-// after each replay.
-struct MarchClock {
-  double t_out, h;
-  int step;
-  int pad;
-};
-
-template <typename R>
-__device__ __forceinline__ double stage_time(const StageArgs<R>& A) {
-  if (A.ctl) return A.ctl->t + A.c * A.ctl->h;
-  if (!A.clk) return A.t;
-  const double tn = A.clk->t_out + (A.clk->step + A.ls) * A.clk->h;
-  return tn + A.c * A.clk->h;
-}
-
 __global__ void k_clock_set(MarchClock* c, double t_out, double h) {
   c->t_out = t_out;
   c->h = h;
@@ -116,56 +46,6 @@ __global__ void k_clock_set(MarchClock* c, double t_out, double h) {
 }
 
 __global__ void k_clock_advance(MarchClock* c, int by) { c->step += by; }
-
-// ---------------------------------------------------------------- field and background
-__device__ __forceinline__ double field_time_factor(const FieldDesc& F, double t, double y) {
-  switch (F.kind) {
-    case SWF_FIELD_SAUTER_GAUSS: {
-      const double c = cosh(F.prm[1] * t);
-      return (F.prm[0] / F.prm[1]) / (c * c);
-    }
-    case SWF_FIELD_PULSE_GAUSS: {
-      const double u = t - y;
-      return F.prm[0] * sin(F.prm[1] * u) * exp(-u * u / (F.prm[2] * F.prm[2]));
-    }
-    case SWF_FIELD_SINGLE_E:
-    case SWF_FIELD_DOUBLE_E: {
-      const double a = F.prm[1] * t;
-      return exp(-a * a);
-    }
-    default:
-      return 0.0;
-  }
-}
-
-__device__ __forceinline__ double single_e_x(const FieldDesc& F, double x) {
-  const double kx = F.prm[2];
-  return -(F.prm[0] / kx) * sin(kx * x) * exp(-(kx * x) * (kx * x));
-}
-
-__device__ double axis_factor(const FieldDesc& F, int axis, double xc) {
-  switch (F.kind) {
-    case SWF_FIELD_SAUTER_GAUSS: {
-      const double lam = F.prm[2];
-      return lam > 0.0 ? exp(-xc * xc / (lam * lam)) : 1.0;
-    }
-    case SWF_FIELD_PULSE_GAUSS:
-      if (axis == 0) return exp(-xc * xc / (F.prm[3] * F.prm[3]));
-      if (axis == 1) return F.prm[4] > 0.0 ? exp(-xc * xc / (F.prm[4] * F.prm[4])) : 1.0;
-      return 1.0;
-    case SWF_FIELD_SINGLE_E:
-    case SWF_FIELD_DOUBLE_E: {
-      if (axis == 0) {
-        if (F.kind == SWF_FIELD_SINGLE_E) return single_e_x(F, xc);
-        return single_e_x(F, xc + F.prm[5]) + single_e_x(F, xc - F.prm[5]);
-      }
-      const double k = F.prm[2 + axis];
-      return exp(-(k * xc) * (k * xc));
-    }
-    default:
-      return 0.0;
-  }
-}
 
 // Per-field tables, computed in FP64 and rounded once to the march precision.
 template <typename R>
@@ -201,175 +81,13 @@ __global__ void k_kappa_table(GridDesc g, R* kap) {
   }
 }
 
-// V phi for the one non-zero covariant component A_mu = a (V = A_0 + alpha^k A_k).
-template <typename R>
-__device__ __forceinline__ void apply_v(int acomp, R a, const cpx<R>* p, cpx<R>* o) {
-  switch (acomp) {
-    case 0:
-      o[0] = a * p[0]; o[1] = a * p[1]; o[2] = a * p[2]; o[3] = a * p[3];
-      break;
-    case 1:  // alpha^x
-      o[0] = a * p[3]; o[1] = a * p[2]; o[2] = a * p[1]; o[3] = a * p[0];
-      break;
-    case 2:  // alpha^y
-      o[0] = a * mul_mi(p[3]); o[1] = a * mul_i(p[2]); o[2] = a * mul_mi(p[1]); o[3] = a * mul_i(p[0]);
-      break;
-    case 3:  // alpha^z
-      o[0] = a * p[2]; o[1] = (R)(-1) * (a * p[3]); o[2] = a * p[0]; o[3] = (R)(-1) * (a * p[1]);
-      break;
-    default:
-      o[0] = o[1] = o[2] = o[3] = mk<R>(0, 0);
-  }
-}
-
-// v <- -i s (alpha.kappa + beta) v  (Dirac representation, sigma.kappa blocks).
-template <typename R>
-__device__ __forceinline__ void h0_mi(cpx<R>* v, R kx, R ky, R kz, R s) {
-  const cpx<R> a = v[0], b = v[1], c = v[2], d = v[3];
-  // sigma.k (u0, u1) = (kz u0 + (kx - i ky) u1, (kx + i ky) u0 - kz u1)
-  const cpx<R> sl0 = kz * c + kx * d + ky * mul_mi(d);
-  const cpx<R> sl1 = kx * c + ky * mul_i(c) - kz * d;
-  const cpx<R> su0 = kz * a + kx * b + ky * mul_mi(b);
-  const cpx<R> su1 = kx * a + ky * mul_i(a) - kz * b;
-  v[0] = s * mul_mi(a + sl0);
-  v[1] = s * mul_mi(b + sl1);
-  v[2] = s * mul_mi(su0 - c);
-  v[3] = s * mul_mi(su1 - d);
-}
-
-__device__ __forceinline__ double kappa_of(int j, int n, double L, double K) {
-  return n > 1 ? mode_kappa(j, n, L) : K;
-}
-
-
-// ---------------------------------------------------------------- composite DFTs in registers
-// cos and sin of 2 pi e / N for the composite radices (written out to 25 digits).
-__host__ __device__ constexpr double tw_const(int N, int e, bool want_cos) {
-  if (N == 8) {
-    switch (e) {
-      case 0: return want_cos ? 1.0000000000000000000000000 : 0.0000000000000000000000000;
-      case 1: return want_cos ? 0.7071067811865475244008444 : 0.7071067811865475244008444;
-      case 2: return want_cos ? -0.0000000000000000000000000 : 1.0000000000000000000000000;
-      case 3: return want_cos ? -0.7071067811865475244008444 : 0.7071067811865475244008444;
-      case 4: return want_cos ? -1.0000000000000000000000000 : 0.0000000000000000000000000;
-      case 5: return want_cos ? -0.7071067811865475244008444 : -0.7071067811865475244008444;
-      case 6: return want_cos ? -0.0000000000000000000000000 : -1.0000000000000000000000000;
-      case 7: return want_cos ? 0.7071067811865475244008444 : -0.7071067811865475244008444;
-    }
-  }
-  if (N == 12) {
-    switch (e) {
-      case 0: return want_cos ? 1.0000000000000000000000000 : 0.0000000000000000000000000;
-      case 1: return want_cos ? 0.8660254037844386467637232 : 0.5000000000000000000000000;
-      case 2: return want_cos ? 0.5000000000000000000000000 : 0.8660254037844386467637232;
-      case 3: return want_cos ? -0.0000000000000000000000000 : 1.0000000000000000000000000;
-      case 4: return want_cos ? -0.5000000000000000000000000 : 0.8660254037844386467637232;
-      case 5: return want_cos ? -0.8660254037844386467637232 : 0.5000000000000000000000000;
-      case 6: return want_cos ? -1.0000000000000000000000000 : 0.0000000000000000000000000;
-      case 7: return want_cos ? -0.8660254037844386467637232 : -0.5000000000000000000000000;
-      case 8: return want_cos ? -0.5000000000000000000000000 : -0.8660254037844386467637232;
-      case 9: return want_cos ? -0.0000000000000000000000000 : -1.0000000000000000000000000;
-      case 10: return want_cos ? 0.5000000000000000000000000 : -0.8660254037844386467637232;
-      case 11: return want_cos ? 0.8660254037844386467637232 : -0.5000000000000000000000000;
-    }
-  }
-  if (N == 16) {
-    switch (e) {
-      case 0: return want_cos ? 1.0000000000000000000000000 : 0.0000000000000000000000000;
-      case 1: return want_cos ? 0.9238795325112867561281832 : 0.3826834323650897717284600;
-      case 2: return want_cos ? 0.7071067811865475244008444 : 0.7071067811865475244008444;
-      case 3: return want_cos ? 0.3826834323650897717284600 : 0.9238795325112867561281832;
-      case 4: return want_cos ? -0.0000000000000000000000000 : 1.0000000000000000000000000;
-      case 5: return want_cos ? -0.3826834323650897717284600 : 0.9238795325112867561281832;
-      case 6: return want_cos ? -0.7071067811865475244008444 : 0.7071067811865475244008444;
-      case 7: return want_cos ? -0.9238795325112867561281832 : 0.3826834323650897717284600;
-      case 8: return want_cos ? -1.0000000000000000000000000 : 0.0000000000000000000000000;
-      case 9: return want_cos ? -0.9238795325112867561281832 : -0.3826834323650897717284600;
-      case 10: return want_cos ? -0.7071067811865475244008444 : -0.7071067811865475244008444;
-      case 11: return want_cos ? -0.3826834323650897717284600 : -0.9238795325112867561281832;
-      case 12: return want_cos ? -0.0000000000000000000000000 : -1.0000000000000000000000000;
-      case 13: return want_cos ? 0.3826834323650897717284600 : -0.9238795325112867561281832;
-      case 14: return want_cos ? 0.7071067811865475244008444 : -0.7071067811865475244008444;
-      case 15: return want_cos ? 0.9238795325112867561281832 : -0.3826834323650897717284600;
-    }
-  }
-  if (N == 20) {
-    switch (e) {
-      case 0: return want_cos ? 1.0000000000000000000000000 : 0.0000000000000000000000000;
-      case 1: return want_cos ? 0.9510565162951535721164393 : 0.3090169943749474241022934;
-      case 2: return want_cos ? 0.8090169943749474241022934 : 0.5877852522924731291687060;
-      case 3: return want_cos ? 0.5877852522924731291687060 : 0.8090169943749474241022934;
-      case 4: return want_cos ? 0.3090169943749474241022934 : 0.9510565162951535721164393;
-      case 5: return want_cos ? -0.0000000000000000000000000 : 1.0000000000000000000000000;
-      case 6: return want_cos ? -0.3090169943749474241022934 : 0.9510565162951535721164393;
-      case 7: return want_cos ? -0.5877852522924731291687060 : 0.8090169943749474241022934;
-      case 8: return want_cos ? -0.8090169943749474241022934 : 0.5877852522924731291687060;
-      case 9: return want_cos ? -0.9510565162951535721164393 : 0.3090169943749474241022934;
-      case 10: return want_cos ? -1.0000000000000000000000000 : 0.0000000000000000000000000;
-      case 11: return want_cos ? -0.9510565162951535721164393 : -0.3090169943749474241022934;
-      case 12: return want_cos ? -0.8090169943749474241022934 : -0.5877852522924731291687060;
-      case 13: return want_cos ? -0.5877852522924731291687060 : -0.8090169943749474241022934;
-      case 14: return want_cos ? -0.3090169943749474241022934 : -0.9510565162951535721164393;
-      case 15: return want_cos ? -0.0000000000000000000000000 : -1.0000000000000000000000000;
-      case 16: return want_cos ? 0.3090169943749474241022934 : -0.9510565162951535721164393;
-      case 17: return want_cos ? 0.5877852522924731291687060 : -0.8090169943749474241022934;
-      case 18: return want_cos ? 0.8090169943749474241022934 : -0.5877852522924731291687060;
-      case 19: return want_cos ? 0.9510565162951535721164393 : -0.3090169943749474241022934;
-    }
-  }
-  return 0.0;
-}
-
-// v * W_N^e (forward, W = exp(-2 pi i / N)) or v * conj(W_N^e) (inverse); quarter turns exact.
-template <typename R>
-__device__ __forceinline__ cpx<R> twiddle_const(cpx<R> v, int N, int e, bool inv) {
-  if (e == 0) return v;
-  if ((4 * e) % N == 0) {
-    const int q = (4 * e / N) & 3;
-    if (q == 2) return mk<R>(-v.x, -v.y);
-    if ((q == 1) != inv) return mul_mi(v);
-    return mul_i(v);
-  }
-  const R c = (R)tw_const(N, e, true), s = (R)tw_const(N, e, false);
-  return v * mk<R>(c, inv ? s : -s);
-}
-
-// DFT of length A*B in registers (Cooley-Tukey): index n = B n1 + n2 in, k = k1 + A k2 out.
-template <typename R, int A, int B>
-struct DftCT {
-  __device__ __forceinline__ static void run(cpx<R>* a, bool inv) {
-    constexpr int N = A * B;
-    cpx<R> y[N];
-#pragma unroll
-    for (int n2 = 0; n2 < B; ++n2) {
-      cpx<R> t[A];
-#pragma unroll
-      for (int n1 = 0; n1 < A; ++n1) t[n1] = a[B * n1 + n2];
-      Dft<R, A>::run(t, inv);
-#pragma unroll
-      for (int k1 = 0; k1 < A; ++k1) y[n2 * A + k1] = twiddle_const<R>(t[k1], N, n2 * k1, inv);
-    }
-#pragma unroll
-    for (int k1 = 0; k1 < A; ++k1) {
-      cpx<R> t[B];
-#pragma unroll
-      for (int n2 = 0; n2 < B; ++n2) t[n2] = y[n2 * A + k1];
-      Dft<R, B>::run(t, inv);
-#pragma unroll
-      for (int k2 = 0; k2 < B; ++k2) a[k1 + A * k2] = t[k2];
-    }
-  }
-};
-template <typename R> struct Dft<R, 8> : DftCT<R, 4, 2> {};
-template <typename R> struct Dft<R, 12> : DftCT<R, 4, 3> {};
-template <typename R> struct Dft<R, 16> : DftCT<R, 4, 4> {};
-template <typename R> struct Dft<R, 20> : DftCT<R, 4, 5> {};
-
 // ---------------------------------------------------------------- out-of-place line FFT
-// Element e of a line sits at e + e/32 (a gap every 32 elements spreads the strided stores of
-// the early passes over the shared-memory banks).
-__host__ __device__ __forceinline__ int pad32(int e) { return e + (e >> 5); }
-static inline int padded_len(int n) { return pad32(n - 1) + 1; }
+// Element e of a line sits at e + e/16 (complex64) or e + e/8 (complex128): a gap every 128 bytes
+// spreads the strided stores of the early passes over the shared-memory banks.
+template <typename R>
+__host__ __device__ __forceinline__ int pad(int e) { return e + (e >> (sizeof(R) == 4 ? 4 : 3)); }
+template <typename R>
+static inline int padded_len(int n) { return pad<R>(n - 1) + 1; }
 
 // One self-sorting (Stockham) radix-RAD pass from `src` to `dst` over `nlines` lines of length
 // n (stride ld, padded positions): butterfly (line, i < n/RAD) reads elements i + q n/RAD,
@@ -391,7 +109,7 @@ __device__ __forceinline__ void pp_pass(const cpx<R>* __restrict__ src, cpx<R>* 
     cpx<R>* d = dst + line * ld;
     cpx<R> v[RAD];
 #pragma unroll
-    for (int q = 0; q < RAD; ++q) v[q] = s[pad32(i + q * m)];
+    for (int q = 0; q < RAD; ++q) v[q] = s[pad<R>(i + q * m)];
     if (k != 0) {
       const int ks = k * twstep;
       if (RAD <= 5) {
@@ -421,7 +139,7 @@ __device__ __forceinline__ void pp_pass(const cpx<R>* __restrict__ src, cpx<R>* 
     Dft<R, RAD>::run(v, inv);
     const int o = (i - k) * RAD + k;
 #pragma unroll
-    for (int q = 0; q < RAD; ++q) d[pad32(o + q * p)] = v[q];
+    for (int q = 0; q < RAD; ++q) d[pad<R>(o + q * p)] = v[q];
   }
   __syncthreads();
 }
@@ -453,300 +171,323 @@ __device__ cpx<R>* fft_pp(cpx<R>* a, cpx<R>* b, int ld, int nlines, const RadixP
 }
 
 // ---------------------------------------------------------------- pass kernels
-// Shared memory of every pass kernel: two line buffers (the FFT works out of place) within
-// kPassSmem, so that three blocks of 256 threads fit an SM.
+// Shared memory of a whole-line transform (two line buffers, the FFT works out of place) by the fixed
+// rule, so that three blocks of 256 threads fit an SM; and the most that any pass may take.
 static const size_t kPassSmem = 72 * 1024;
-// The tuner may also try wider shapes (more rows per x block, wider y/z tiles) up to this much
-// shared memory per block (one or two blocks per SM): wider y/z tiles read longer contiguous
-// runs of each line and give every FFT pass more butterflies per barrier.
-static const size_t kPassSmemTune = 200 * 1024;
+static const size_t kPassSmemMax = 200 * 1024;
 
-// x lines of `rows` grid rows (4 components each): stage combine, local term, forward x-FFT
-// (and the whole derivative when x is the only non-trivial axis).
-// Block (bx, f) of the pass: rows bx*rows .. of field f.
+// Grids with x as the only non-trivial axis: `rows` rows (4 components each) per block, the whole
+// right-hand side in one launch.  Block (bx, f): rows bx*rows .. of field f.
 template <typename R>
-__device__ __forceinline__ void first_body(const StageArgs<R>& A, int bx, int f, int rows, int ld, int only_x) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_first(StageArgs<R> A, int rows, int ld) {
   if (A.ctl && A.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* buf = reinterpret_cast<cpx<R>*>(smem_raw);
   cpx<R>* buf2 = buf + 4 * rows * ld;
-  const double hscale = A.ctl ? A.ctl->h : 1.0;  // stage coefficients are a_ij (times h here) under control
-  cpx<R>* const yout = A.ynew ? A.ynew : A.y;
-  __shared__ R s_ft[64];  // field time factor per row, computed in FP64 and rounded once
+  __shared__ R s_ft[64];
   __shared__ cpx<R> s_tf;
-  const int row0 = bx * rows;
-  const int nx = A.g.n[0], ny = A.g.n[1], nz = A.g.n[2];
-  const int N = A.g.N;
-  const size_t fo = (size_t)f * 4 * N;
-  const FieldDesc* F = A.fd + f;
-  const double tst = stage_time(A);
-  for (int j = threadIdx.x; j < rows; j += blockDim.x) {
-    const int iy = (row0 + j) % ny;
-    const double yc = ny > 1 ? A.g.x0[1] + iy * A.g.dx[1] : 0.0;
-    s_ft[j] = (R)field_time_factor(*F, tst, yc);
-  }
-  if (threadIdx.x == 0) {
-    double sn, cs;
-    sincos(F->tsign * F->e0 * tst, &sn, &cs);
-    s_tf = mk<R>((R)cs, (R)sn);
-  }
+  const int f = blockIdx.y, row0 = blockIdx.x * rows;
+  const int nx = A.g.n[0];
+  const size_t N = A.g.N;
+  row_factors(A, false, f, row0, rows, s_ft, &s_tf);
   __syncthreads();
-  const int nt = nx + ny + nz;
-  const R* gx = A.greal + (size_t)f * nt;
-  const R* gy = gx + nx;
-  const R* gz = gy + ny;
-  const cpx<R>* ex = A.gcplx + (size_t)f * (nt + 4);
-  const cpx<R>* ey = ex + nx;
-  const cpx<R>* ez = ey + ny;
-  const cpx<R>* wsp = ez + nz;
-  const int acomp = F->acomp;
-  const int per = rows * nx;
-  const size_t cs = (size_t)N;
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int j = e / nx;
-    const int x = e - j * nx;
-    const int row = row0 + j;
-    cpx<R> v[4];
+  const bool ff = sizeof(R) == 4 && A.ylo && A.write_y;
+  for (int e = threadIdx.x; e < 4 * rows * nx; e += blockDim.x) {
+    const int l = e / nx, x = e - l * nx;  // line l: row l / 4, component l % 4
+    const int row = row0 + (l >> 2), c = l & 3;
+    cpx<R> v = mk<R>(0, 0);
     if (row < A.nrows) {
-      const size_t gi = fo + (size_t)row * nx + x;
-      if (sizeof(R) == 4 && A.ylo && A.write_y) {
-        // the new state: the step's increment h sum_j b_j k_j apart, then (y, ylo) += it in
-        // float-float, so that the single-precision rounding of y does not accumulate over steps
-#pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = mk<R>(0, 0);
-#pragma unroll
-        for (int q = 0; q < 6; ++q)
-          if (q < A.nterm) {
-            const R co = (R)(A.coef[q] * hscale);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) v[c] = v[c] + co * A.kin[q][gi + c * cs];
-          }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const cpx<R> yh = A.y[gi + c * cs];
-          cpx<R> lo = A.ylo[gi + c * cs];
-          float sx = (float)v[c].x, sy = (float)v[c].y, lx = (float)lo.x, ly = (float)lo.y;
-          ff_accumulate((float)yh.x, lx, sx);
-          ff_accumulate((float)yh.y, ly, sy);
-          v[c] = mk<R>((R)sx, (R)sy);
-          A.ylo[gi + c * cs] = mk<R>((R)lx, (R)ly);
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = A.y[gi + c * cs];
-#pragma unroll
-        for (int q = 0; q < 6; ++q)
-          if (q < A.nterm) {
-            const R co = (R)(A.coef[q] * hscale);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) v[c] = v[c] + co * A.kin[q][gi + c * cs];
-          }
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        if (A.write_y) yout[gi + c * cs] = v[c];
-        if (A.ystage) A.ystage[gi + c * cs] = v[c];
-      }
-      // local term Z = -i V (Y + psi_b), kept in the output slot until the last pass
-      const int iy = row % ny, iz = row / ny;
-      const R a = s_ft[j] * gx[x] * gy[iy] * gz[iz];
-      const cpx<R> ph = s_tf * ex[x] * ey[iy] * ez[iz];
-      cpx<R> phi[4], vz[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) phi[c] = v[c] + wsp[c] * ph;
-      apply_v<R>(acomp, a, phi, vz);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) A.kout[gi + c * cs] = mul_mi(vz[c]);
-    } else {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) v[c] = mk<R>(0, 0);
+      const size_t gi = ((size_t)f * 4 + c) * N + (size_t)row * nx + x;
+      combine_sites<R, 1>(A, A.nterm, ff, gi, 0, &v);
+      open_sites<R, 1>(A, ff, gi, x, 0, f, c, row, s_ft[l >> 2], s_tf, &v);
     }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) buf[(c * rows + j) * ld + pad32(x)] = v[c];
+    buf[l * ld + pad<R>(x)] = v;
   }
   __syncthreads();
   cpx<R>* res = fft_pp<R>(buf, buf2, ld, 4 * rows, A.plan[0], false, A.tw[0]);
-  if (!only_x) {
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / nx;
-      const int x = e - j * nx;
-      const int row = row0 + j;
-      if (row < A.nrows) {
-        const size_t gi = fo + (size_t)row * nx + x;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) A.T[gi + c * cs] = res[(c * rows + j) * ld + pad32(x)];
-      }
-    }
-    return;
-  }
-  // one non-trivial axis: the whole derivative in this block
-  const R sc = A.inv_n;
+  const FieldDesc* F = A.fd + f;
   const R kx0 = (R)F->K[0], ky = (R)F->K[1], kz = (R)F->K[2];
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
+  for (int e = threadIdx.x; e < rows * nx; e += blockDim.x) {
     const int j = e / nx, x = e - j * nx;
-    cpx<R> v[4];
+    cpx<R>* l = res + 4 * j * ld + pad<R>(x);
+    cpx<R> v[4] = {l[0], l[ld], l[2 * ld], l[3 * ld]};
+    h0_mi<R>(v, nx > 1 ? A.kap[x] : kx0, ky, kz, A.inv_n);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) v[c] = res[(c * rows + j) * ld + pad32(x)];
-    h0_mi<R>(v, nx > 1 ? A.kap[x] : kx0, ky, kz, sc);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) res[(c * rows + j) * ld + pad32(x)] = v[c];
+    for (int c = 0; c < 4; ++c) l[c * ld] = v[c];
   }
   __syncthreads();
   res = fft_pp<R>(res, res == buf ? buf2 : buf, ld, 4 * rows, A.plan[0], true, A.tw[0]);
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int j = e / nx;
-    const int x = e - j * nx;
-    const int row = row0 + j;
-    if (row < A.nrows) {
-      const size_t gi = fo + (size_t)row * nx + x;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) A.kout[gi + c * cs] = A.kout[gi + c * cs] + res[(c * rows + j) * ld + pad32(x)];
-    }
+  for (int e = threadIdx.x; e < 4 * rows * nx; e += blockDim.x) {
+    const int l = e / nx, x = e - l * nx;
+    const int row = row0 + (l >> 2);
+    if (row >= A.nrows) continue;
+    const size_t gi = ((size_t)f * 4 + (l & 3)) * N + (size_t)row * nx + x;
+    A.kout[gi] = A.kout[gi] + res[l * ld + pad<R>(x)];
   }
 }
 
-// The x-pass kernels are held to 64 registers in complex64 (no spills), so that four 256-thread
-// blocks fit an SM when the tuner picks a shape of at most 56 KB of shared memory.
-template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_first(StageArgs<R> A, int rows, int ld, int only_x) {
-  first_body<R>(A, blockIdx.x, blockIdx.y, rows, ld, only_x);
+// ---- passes of small radices (2, 3, 4, 5), for every length and both precisions
+// The same two kinds of passes as the register line kernels (swf_line.cuh), for complex128 and for
+// lengths that have no line kernel: the first and the last butterfly of a transform work in the
+// registers of the thread that loads, stores or uses the values, those between run in shared memory.
+// FP64 decides the shape: the unit of an SM quarter takes 64 cycles per warp instruction, so a thread
+// holds few values (one radix-4 butterfly) and a line is spread over n/4 threads, which loads all
+// quarters of all SMs evenly even for a single 128 x 128 field.  The operations are those of 16 x 8
+// butterflies within a few percent (22 per point).  One 128 x 128 complex128 field, per evaluation: 56
+// us with 16 x 8 in shared memory, 50 us with 8 x 16 in registers (8 to 16 values a thread), 33 us here.
+constexpr int kPassThreads = 512;  // at most, per block
+
+// The march's plan for these passes: fours at both ends where the length has two, else the largest
+// radices outside; sites side first.
+__host__ __device__ inline int end_radix(const RadixPlan& pl, bool site) {
+  return pl.npass == 0 ? 1 : pl.rad[site ? 0 : pl.npass - 1];
+}
+// Threads per line: one butterfly of the site side each, or several where `per` lines of that many
+// threads would not fit a block.
+static inline int pass_threads(const RadixPlan& pl, int per) {
+  const int nb = pl.n / end_radix(pl, true);
+  const int rounds = (nb * per + kPassThreads - 1) / kPassThreads;
+  return (nb + rounds - 1) / rounds;
 }
 
-// Lines along axis 1 (y) or 2 (z) of a tile of TX = 2^lgtx consecutive x columns: forward FFT,
-// -i H0(kappa)/N, inverse FFT, as selected.  The tile sits in shared memory as 4 TX lines of
-// stride ld (chosen so that the transposing loads and stores of a warp spread over the banks).
-// Block (bx, f): tile bx of field f.
+// The passes between the first and the last of a forward or inverse transform; a holds the first
+// one's results (synchronised).  Returns the buffer with the last one's operands.
 template <typename R>
-__device__ __forceinline__ void mid_body(const StageArgs<R>& A, int bx, int f, int axis, int lgtx, int ld, int do_fwd,
-                                         int do_h0, int do_inv) {
+__device__ __forceinline__ cpx<R>* middle_passes(cpx<R>* a, cpx<R>* b, int ld, int nlines, const RadixPlan& pl, bool inv,
+                                                 const cpx<R>* __restrict__ tw) {
+  int p = end_radix(pl, !inv);
+  for (int s = 1; s < pl.npass - 1; ++s) {
+    const int r = pl.rad[inv ? pl.npass - 1 - s : s];
+    switch (r) {
+      case 4: pp_pass<R, 4>(a, b, ld, nlines, pl.n, p, inv, tw); break;
+      case 2: pp_pass<R, 2>(a, b, ld, nlines, pl.n, p, inv, tw); break;
+      case 3: pp_pass<R, 3>(a, b, ld, nlines, pl.n, p, inv, tw); break;
+      default: pp_pass<R, 5>(a, b, ld, nlines, pl.n, p, inv, tw); break;
+    }
+    cpx<R>* t = a;
+    a = b;
+    b = t;
+    p *= r;
+  }
+  return a;
+}
+
+template <typename R> struct Dft<R, 1> {
+  __device__ __forceinline__ static void run(cpx<R>*, bool) {}
+};
+
+// First butterfly b of a transform: DFT of v to positions b RAD .. of a line.
+template <typename R, int RAD>
+__device__ __forceinline__ void first_butterfly(cpx<R>* v, int b, bool inv, cpx<R>* line) {
+  Dft<R, RAD>::run(v, inv);
+#pragma unroll
+  for (int q = 0; q < RAD; ++q) line[pad<R>(b * RAD + q)] = v[q];
+}
+// Last butterfly b of a transform of n points: the values b + q n/RAD (a transform of one pass has
+// left them ready).
+template <typename R, int RAD>
+__device__ __forceinline__ void last_butterfly(const cpx<R>* line, int b, int n, bool one_pass, bool inv,
+                                               const cpx<R>* __restrict__ tw, cpx<R>* v) {
+  const int m = n / RAD;
+#pragma unroll
+  for (int q = 0; q < RAD; ++q) v[q] = line[pad<R>(b + q * m)];
+  if (one_pass) return;
+#pragma unroll
+  for (int q = 1; q < RAD; ++q) {
+    cpx<R> w = tw[q * b];
+    if (inv) w.y = -w.y;
+    v[q] = v[q] * w;
+  }
+  Dft<R, RAD>::run(v, inv);
+}
+
+// body(std::integral_constant<int, radix>) for the runtime radix of a plan's end.
+template <typename Body>
+__device__ __forceinline__ void with_radix(int r, Body&& body) {
+  switch (r) {
+    case 4: body(std::integral_constant<int, 4>()); break;
+    case 2: body(std::integral_constant<int, 2>()); break;
+    case 3: body(std::integral_constant<int, 3>()); break;
+    case 5: body(std::integral_constant<int, 5>()); break;
+    default: body(std::integral_constant<int, 1>()); break;
+  }
+}
+
+// x pass (k_xline's work; R0: the site side's radix), tpl threads per line.
+template <typename R, int R0>
+__global__ void __launch_bounds__(kPassThreads, 1)
+k_xpass(const __grid_constant__ StageArgs<R> P, const __grid_constant__ StageArgs<R> A, int rows, int ld, int tpl,
+        int flags) {
   if (A.ctl && A.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<R>* buf = reinterpret_cast<cpx<R>*>(smem_raw);
-  const int nx = A.g.n[0], ny = A.g.n[1], nz = A.g.n[2];
-  const int N = A.g.N;
-  const int na = A.g.n[axis];
-  const int TX = 1 << lgtx;
-  cpx<R>* buf2 = buf + 4 * TX * ld;
-  const int ntx = (nx + TX - 1) >> lgtx;
-  const int xt = bx % ntx;
-  const int o = bx / ntx;  // z index (axis 1) or y index (axis 2)
-  const size_t base = axis == 1 ? (size_t)o * nx * ny : (size_t)o * nx;
-  const size_t stride = axis == 1 ? (size_t)nx : (size_t)nx * ny;
-  const size_t fo = (size_t)f * 4 * N;
-  const size_t cs = (size_t)N;
-  const int per = TX * na;
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int m = e >> lgtx;
-    const int t = e & (TX - 1);
-    const int x = xt * TX + t;
-    const size_t gi = fo + base + m * stride + x;
+  __shared__ R s_ft[64];
+  __shared__ cpx<R> s_tf;
+  const RadixPlan& pl = A.plan[0];
+  const int nx = pl.n, nb = nx / R0, rl = end_radix(pl, false);
+  const size_t N = A.g.N;
+  const int f = blockIdx.y, row0 = blockIdx.x * rows;
+  const int line = threadIdx.x / tpl, g = threadIdx.x - line * tpl;
+  const int c = line & 3, j = line >> 2, row = row0 + j;
+  const bool ok = line < 4 * rows && row < A.nrows;
+  const size_t gl = ((size_t)f * 4 + c) * N + (size_t)row * nx;  // the line
+  cpx<R>* a = reinterpret_cast<cpx<R>*>(smem_raw);
+  cpx<R>* b2 = a + 4 * rows * ld;
+  const cpx<R>* __restrict__ tw = A.tw[0];
+  const bool last = flags & XL_LAST, first = flags & XL_FIRST, one = pl.npass < 2;
+  if (first) row_factors(A, flags & XL_FACTORS, f, row0, rows, s_ft, &s_tf);
+  const bool ff = sizeof(R) == 4 && A.ylo && A.write_y;
+  const int nold = A.nterm - ((flags & XL_REGK) ? 1 : 0);
+  cpx<R> v[R0];
+  if (first && ok && g < nb) combine_sites<R, R0>(A, nold, ff, gl + g, nb, v);  // overlaps the loads of T
+  if (last) {
+    if (ok)
+      with_radix(rl, [&](auto rc) {
+        constexpr int RL = decltype(rc)::value;
+        const int nm = nx / RL;
+        for (int b = g; b < nm; b += tpl) {
+          cpx<R> m[RL];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) buf[(c * TX + t) * ld + pad32(m)] = x < nx ? A.T[gi + c * cs] : mk<R>(0, 0);
+          for (int q = 0; q < RL; ++q) m[q] = P.T[gl + b + q * nm];
+          first_butterfly<R, RL>(m, b, true, a + line * ld);
+        }
+      });
+    __syncthreads();
+    cpx<R>* cur = middle_passes<R>(a, b2, ld, 4 * rows, pl, true, tw);
+    if (cur != a) {
+      b2 = a;
+      a = cur;
+    }
+  } else {
+    __syncthreads();  // the time factors
   }
-  __syncthreads();
-  cpx<R>* res = buf;
-  if (do_fwd) res = fft_pp<R>(res, buf2, ld, 4 * TX, A.plan[axis], false, A.tw[axis]);
-  if (do_h0 && A.yspec) {
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int m = e >> lgtx;
-      const int t = e & (TX - 1);
-      const int x = xt * TX + t;
-      if (x < nx) {
-        const size_t gi = fo + base + m * stride + x;
+  if (ok)
+    for (int b = g; b < nb; b += tpl) {
+      if (first && b != g) combine_sites<R, R0>(A, nold, ff, gl + b, nb, v);
+      if (last) {
+        cpx<R> r[R0];
+        last_butterfly<R, R0>(a + line * ld, b, nx, one, true, tw, r);
+        close_sites<R, R0>(P, gl + b, nb, r);
+        if (first && (flags & XL_REGK)) {
+          const R co = A.ctl ? (R)(A.coef[nold] * A.ctl->h) : A.coef_r[nold];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) A.yspec[gi + c * cs] = res[(c * TX + t) * ld + pad32(m)];
+          for (int q = 0; q < R0; ++q) v[q] = v[q] + co * r[q];
+        }
+      }
+      if (first) {
+        open_sites<R, R0>(A, ff, gl + b, b, nb, f, c, row, s_ft[j], s_tf, v);
+        first_butterfly<R, R0>(v, b, false, b2 + line * ld);
       }
     }
-    __syncthreads();
-  }
-  if (do_h0) {
-    const FieldDesc* F = A.fd + f;
-    const R sc = A.inv_n;
-    const R K0 = (R)F->K[0], K1 = (R)F->K[1], K2 = (R)F->K[2];  // momenta along trivial axes
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int t = e / na, m = e - t * na;
-      const int x = xt * TX + t;
-      if (x >= nx) continue;
-      const int iy = axis == 1 ? m : o;
-      const int iz = axis == 2 ? m : o;
-      cpx<R> v[4];
+  if (!first) return;
+  __syncthreads();
+  const cpx<R>* cur = middle_passes<R>(b2, a, ld, 4 * rows, pl, false, tw);
+  if (ok)
+    with_radix(rl, [&](auto rc) {
+      constexpr int RL = decltype(rc)::value;
+      const int nm = nx / RL;
+      for (int b = g; b < nm; b += tpl) {
+        cpx<R> m[RL];
+        last_butterfly<R, RL>(cur + line * ld, b, nx, one, false, tw, m);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) v[c] = res[(c * TX + t) * ld + pad32(m)];
-      h0_mi<R>(v, nx > 1 ? A.kap[x] : K0, ny > 1 ? A.kap[nx + iy] : K1, nz > 1 ? A.kap[nx + ny + iz] : K2, sc);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) res[(c * TX + t) * ld + pad32(m)] = v[c];
-    }
-    __syncthreads();
-  }
-  if (do_inv) res = fft_pp<R>(res, res == buf ? buf2 : buf, ld, 4 * TX, A.plan[axis], true, A.tw[axis]);
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int m = e >> lgtx;
-    const int t = e & (TX - 1);
-    const int x = xt * TX + t;
-    if (x < nx) {
-      const size_t gi = fo + base + m * stride + x;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) A.T[gi + c * cs] = res[(c * TX + t) * ld + pad32(m)];
-    }
-  }
+        for (int q = 0; q < RL; ++q) A.T[gl + b + q * nm] = m[q];
+      }
+    });
 }
 
+// y or z pass (k_line's work): lines along `axis` of TX = 2^lgtx x columns, tpl threads per line, the
+// four components of a mode in one warp.
 template <typename R>
-__global__ void __launch_bounds__(256) k_mid(StageArgs<R> A, int axis, int lgtx, int ld, int do_fwd, int do_h0,
-                                             int do_inv) {
-  mid_body<R>(A, blockIdx.x, blockIdx.y, axis, lgtx, ld, do_fwd, do_h0, do_inv);
-}
-
-// x lines: inverse x-FFT, k = (that) + Z.  Block (bx, f): rows bx*rows .. of field f.
-template <typename R>
-__device__ __forceinline__ void last_body(const StageArgs<R>& A, int bx, int f, int rows, int ld) {
+__global__ void __launch_bounds__(kPassThreads, 1)
+k_mid(const __grid_constant__ StageArgs<R> A, int axis, int lgtx, int ld, int tpl, int flags) {
   if (A.ctl && A.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<R>* buf = reinterpret_cast<cpx<R>*>(smem_raw);
-  cpx<R>* buf2 = buf + 4 * rows * ld;
-  const int row0 = bx * rows;
-  const int nx = A.g.n[0];
-  const int N = A.g.N;
-  const size_t fo = (size_t)f * 4 * N;
-  const size_t cs = (size_t)N;
-  const int per = rows * nx;
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int j = e / nx;
-    const int x = e - j * nx;
-    const int row = row0 + j;
-    const size_t gi = fo + (size_t)row * nx + x;
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-      buf[(c * rows + j) * ld + pad32(x)] = row < A.nrows ? A.T[gi + c * cs] : mk<R>(0, 0);
+  const int nx = A.g.n[0], ny = A.g.n[1], nz = A.g.n[2];
+  const int f = blockIdx.y;
+  const int TX = 1 << lgtx, ntx = (nx + TX - 1) >> lgtx;
+  const int other = axis == 1 ? nz : ny;
+  if (blockIdx.x >= ntx * other) {
+    coming_factors(A, f);
+    return;
   }
-  __syncthreads();
-  cpx<R>* res = fft_pp<R>(buf, buf2, ld, 4 * rows, A.plan[0], true, A.tw[0]);
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int j = e / nx;
-    const int x = e - j * nx;
-    const int row = row0 + j;
-    if (row < A.nrows) {
-      const size_t gi = fo + (size_t)row * nx + x;
+  const RadixPlan& pl = A.plan[axis];
+  const int na = pl.n, r0 = end_radix(pl, true), rl = end_radix(pl, false);
+  const int xt = blockIdx.x % ntx, o = blockIdx.x / ntx;  // o: z index (axis 1) or y index (axis 2)
+  const int t = threadIdx.x & (TX - 1), c = (threadIdx.x >> lgtx) & 3, g = threadIdx.x >> (lgtx + 2);
+  const int x = xt * TX + t;
+  const bool ok = x < nx && g < tpl;
+  const size_t base = (axis == 1 ? (size_t)o * nx * ny : (size_t)o * nx) + ((size_t)f * 4 + c) * A.g.N + x;
+  const size_t stride = axis == 1 ? (size_t)nx : (size_t)nx * ny;
+  cpx<R>* a = reinterpret_cast<cpx<R>*>(smem_raw);
+  cpx<R>* b2 = a + 4 * TX * ld;
+  const int lo = (c * TX + t) * ld;
+  const cpx<R>* __restrict__ tw = A.tw[axis];
+  const bool one = pl.npass < 2;
+  const bool fwd = flags & LN_FWD, h0 = flags & LN_H0, inv = flags & LN_INV;
+  if (fwd) {
+    if (ok)
+      with_radix(r0, [&](auto rc) {
+        constexpr int R0 = decltype(rc)::value;
+        const int nb = na / R0;
+        for (int b = g; b < nb; b += tpl) {
+          cpx<R> v[R0];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) A.kout[gi + c * cs] = A.kout[gi + c * cs] + res[(c * rows + j) * ld + pad32(x)];
+          for (int q = 0; q < R0; ++q) v[q] = A.T[base + (size_t)(b + q * nb) * stride];
+          first_butterfly<R, R0>(v, b, false, a + lo);
+        }
+      });
+    __syncthreads();
+    cpx<R>* cur = middle_passes<R>(a, b2, ld, 4 * TX, pl, false, tw);
+    if (cur != a) {
+      b2 = a;
+      a = cur;
     }
   }
-}
-
-template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_last(StageArgs<R> A, int rows, int ld) {
-  last_body<R>(A, blockIdx.x, blockIdx.y, rows, ld);
-}
-
-// The x lines of one evaluation's end and the next one's start in one launch: k_i = inverse
-// x-FFT of T + Z for stage P, then the stage combine, local term and forward x-FFT of stage Nx on
-// the same rows.  Each thread reads back the k_i entries it has just written (the two bodies map
-// the rows' entries to threads alike), so the arithmetic is that of k_last then k_first.
-template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_last_first(StageArgs<R> P, StageArgs<R> Nx, int rows, int ld) {
-  last_body<R>(P, blockIdx.x, blockIdx.y, rows, ld);
+  with_radix(rl, [&](auto rc) {
+    constexpr int RL = decltype(rc)::value;
+    const int nm = na / RL, rounds = (nm + tpl - 1) / tpl;
+    for (int k = 0; k < rounds; ++k) {
+      const int b = g + k * tpl;
+      const bool mode = ok && b < nm;
+      cpx<R> m[RL];
+#pragma unroll
+      for (int q = 0; q < RL; ++q) m[q] = mk<R>(0, 0);
+      if (mode) {
+        if (fwd) {
+          last_butterfly<R, RL>(a + lo, b, na, one, false, tw, m);
+        } else {
+#pragma unroll
+          for (int q = 0; q < RL; ++q) m[q] = A.T[base + (size_t)(b + q * nm) * stride];
+        }
+        if (h0 && A.yspec) {
+#pragma unroll
+          for (int q = 0; q < RL; ++q) A.yspec[base + (size_t)(b + q * nm) * stride] = m[q];
+        }
+      }
+      if (h0) h0_modes<R, RL>(A, axis, lgtx, f, c, x, o, b, nm, mode, m);
+      if (mode) {
+        if (inv) {
+          first_butterfly<R, RL>(m, b, true, b2 + lo);
+        } else {
+#pragma unroll
+          for (int q = 0; q < RL; ++q) A.T[base + (size_t)(b + q * nm) * stride] = m[q];
+        }
+      }
+    }
+  });
+  if (!inv) return;
   __syncthreads();
-  first_body<R>(Nx, blockIdx.x, blockIdx.y, rows, ld, 0);
+  const cpx<R>* cur = middle_passes<R>(b2, a, ld, 4 * TX, pl, true, tw);
+  if (ok)
+    with_radix(r0, [&](auto rc) {
+      constexpr int R0 = decltype(rc)::value;
+      const int nb = na / R0;
+      for (int b = g; b < nb; b += tpl) {
+        cpx<R> v[R0];
+        last_butterfly<R, R0>(cur + lo, b, na, one, true, tw, v);
+#pragma unroll
+        for (int q = 0; q < R0; ++q) A.T[base + (size_t)(b + q * nb) * stride] = v[q];
+      }
+    });
 }
 
 // ---------------------------------------------------------------- host side
@@ -756,8 +497,9 @@ template <> struct Prec<double> { static constexpr int is_double = 1; };
 
 static const int kThreads = 256;
 
-// Radix plan of the march's line FFTs: radix 16 first, then the composite radices 20 and 12,
-// then 8, 4, 2, 3, 5 (every length of the form 2^a 3^b 5^c).
+// Radix plan of the line FFTs that run as a whole in shared memory (fft_pp: one-axis grids, the
+// partial-integration integrand): radix 16 first, then the composite radices 20 and 12, then 8, 4,
+// 2, 3, 5 (every length of the form 2^a 3^b 5^c).
 static bool make_march_plan(int n, RadixPlan* pl) {
   pl->n = n;
   pl->npass = 0;
@@ -769,6 +511,30 @@ static bool make_march_plan(int n, RadixPlan* pl) {
       m /= r;
     }
   return m == 1;
+}
+
+// Radix plan of the small-radix passes (k_xpass, k_mid): fours, then fives, threes and a two; the two
+// largest go to the ends.
+static bool make_pass_plan(int n, RadixPlan* pl) {
+  pl->n = n;
+  pl->npass = 0;
+  int m = n;
+  const int order[4] = {4, 5, 3, 2};
+  for (int r : order)
+    while (m % r == 0 && pl->npass < 12) {
+      pl->rad[pl->npass++] = r;
+      m /= r;
+    }
+  if (pl->npass > 2) std::rotate(pl->rad + 1, pl->rad + 2, pl->rad + pl->npass);  // the second largest to the end
+  return m == 1;
+}
+
+// The plan of an axis: whole-line transforms where x is the only axis in complex64, small-radix
+// passes otherwise.
+template <typename R>
+static bool make_line_plan(const GridDesc& g, int axis, RadixPlan* pl) {
+  const bool only_x = g.n[1] == 1 && g.n[2] == 1;
+  return sizeof(R) == 4 && only_x ? make_march_plan(g.n[axis], pl) : make_pass_plan(g.n[axis], pl);
 }
 
 // Streaming multiprocessors of the current device (cached per device).
@@ -788,60 +554,12 @@ static int sm_count() {
 // (up to two blocks per SM).  0 if one row does not fit.
 template <typename R>
 static int x_rows(int nx, int nrows, int F) {
-  const size_t line = (size_t)2 * 4 * padded_len(nx) * sizeof(cpx<R>);
+  const size_t line = (size_t)2 * 4 * padded_len<R>(nx) * sizeof(cpx<R>);
   int rows = (int)(kPassSmem / line);
   if (rows > 64) rows = 64;
   if (rows > nrows) rows = nrows;
   while (rows > 1 && (long)F * ((nrows + rows - 1) / rows) < 2L * sm_count()) rows = (rows + 1) / 2;
   return rows;
-}
-
-// Tile of a y or z pass: the widest power-of-two column count TX <= 16 whose two buffers fit
-// kPassSmem, narrowed on small grids (down to 32 bytes of contiguous x per line) for up to two
-// blocks per SM; line stride ld >= the padded length with ld = 32/TX modulo the elements of one
-// 128-byte shared-memory wavefront, so that the transposing accesses of a warp (TX columns x
-// 32/TX lines) fall on distinct banks.  `tiles` = (field, other-axis index) pairs of the pass.
-struct MidShape {
-  int lgtx, ld;
-  size_t smem;
-};
-
-template <typename R>
-static int mid_stride(int n_a, int lg) {
-  const int unit = 128 / (int)sizeof(cpx<R>);
-  const int base = padded_len(n_a);
-  const int pad = (((32 >> lg) % unit - base % unit) % unit + unit) % unit;
-  return base + pad;
-}
-
-template <typename R>
-static size_t mid_smem(int n_a, int lg) {
-  return (size_t)2 * 4 * (1 << lg) * mid_stride<R>(n_a, lg) * sizeof(cpx<R>);
-}
-
-// widest tile that fits `cap` bytes of shared memory (TX <= nx as well)
-template <typename R>
-static int mid_max_lg(int n_a, int nx, size_t cap = kPassSmem) {
-  int lg = 4;
-  while (lg > 0 && ((1 << lg) > nx || mid_smem<R>(n_a, lg) > cap)) --lg;
-  return lg;
-}
-
-template <typename R>
-static MidShape mid_shape_lg(int n_a, int lg) {
-  MidShape m{};
-  m.lgtx = lg;
-  m.ld = mid_stride<R>(n_a, lg);
-  m.smem = mid_smem<R>(n_a, lg);
-  return m;
-}
-
-template <typename R>
-static MidShape mid_shape(int n_a, int nx, long tiles) {
-  const int min_lg = sizeof(cpx<R>) == 8 ? 2 : 1;
-  int lg = mid_max_lg<R>(n_a, nx);
-  while (lg > min_lg && tiles * ((nx + (1 << lg) - 1) >> lg) < 2L * sm_count()) --lg;
-  return mid_shape_lg<R>(n_a, lg);
 }
 
 // Keys of the tuned shapes: pass kind, element size and the sizes that decide the launch.
@@ -857,131 +575,279 @@ static int tune_lookup(swf_ctx* ctx, const std::string& key, int fallback) {
   return it == ctx->tune.best.end() ? fallback : it->second;
 }
 
+template <typename R, int... R0>
+static cudaError_t xpass_attrs(std::integer_sequence<int, R0...>) {
+  cudaError_t e = cudaSuccess;
+  ((e = e != cudaSuccess ? e : cudaFuncSetAttribute(k_xpass<R, R0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemMax)), ...);
+  return e;
+}
 template <typename R>
 static swf_status set_smem_attrs() {
   // per device; several host threads may arrive at once, and setting the attributes twice is harmless
   static std::atomic<bool> done[64];
   const int dv = dev_slot();
   if (done[dv].load(std::memory_order_acquire)) return SWF_OK;
-  cudaError_t e;
-  e = cudaFuncSetAttribute(k_first<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemTune);
-  if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_first)");
-  e = cudaFuncSetAttribute(k_mid<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemTune);
-  if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_mid)");
-  e = cudaFuncSetAttribute(k_last<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemTune);
-  if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_last)");
-  e = cudaFuncSetAttribute(k_last_first<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemTune);
-  if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_last_first)");
+  cudaError_t e = cudaFuncSetAttribute(k_first<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemMax);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mid<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemMax);
+  if (e == cudaSuccess) e = xpass_attrs<R>(std::integer_sequence<int, 1, 2, 3, 4, 5>());
+  if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(pass kernels)");
   done[dv].store(true, std::memory_order_release);
   return SWF_OK;
 }
 
-// Launch shape of the x passes (k_first, k_last, k_last_first): rows per block, threads, padded
-// line length, shared memory, grid.
-struct XLaunch {
-  int rows, thr, ld;
-  size_t smem;
-  dim3 grid;
-};
+// ---- register line kernels (swf_line.cuh): host side.  Complex64 only: a thread of theirs holds 8 to
+// 32 values, which FP64's rate turns into long serial chains on few SM quarters (one 128 x 128 field in
+// complex128: 50 us per evaluation, 33 us with the small-radix passes).
+const LineEntry<float>* find_line0_float(int n);
+const LineEntry<float>* find_line1_float(int n);
+const LineEntry<float>* find_line2_float(int n);
+const LineEntry<float>* find_line3_float(int n);
+const LineEntry<float>* find_line4_float(int n);
 
+// The line kernels of length n (null: the small-radix passes take it).
 template <typename R>
-static XLaunch x_launch(swf_ctx* ctx, const StageArgs<R>& A, int F) {
+static const LineEntry<R>* line_entry(int n) {
+  if constexpr (sizeof(R) == 8) {
+    return nullptr;
+  } else {
+    for (auto* find : {find_line0_float, find_line1_float, find_line2_float, find_line3_float, find_line4_float})
+      if (const LineEntry<float>* e = find(n)) return e;
+    return nullptr;
+  }
+}
+
+// The line kernels of an axis of a grid: null on a trivial axis and where x is the only axis (one
+// launch does the whole evaluation).
+template <typename R>
+static const LineEntry<R>* line_of(const GridDesc& g, int axis) {
+  if (g.n[1] == 1 && g.n[2] == 1) return nullptr;
+  return g.n[axis] > 1 ? line_entry<R>(g.n[axis]) : nullptr;
+}
+
+// Rows per block of k_xline and log2 columns of k_line: at most this many fit a block.
+template <typename R>
+static int xline_max_rows(const LineEntry<R>* e) {
+  return std::max(1, kXLineThreads / (4 * line_threads(e->r1, e->r2)));
+}
+template <typename R>
+static int line_max_lg(const LineEntry<R>* e, int nx) {
+  int lg = 3;
+  while (lg > 0 && ((1 << lg) > nx || line_block(e->r1, e->r2, lg) > line_max_threads((int)sizeof(cpx<R>))))
+    --lg;
+  return lg;
+}
+template <typename R>
+static size_t xline_smem(const LineEntry<R>* e, int rows) {
+  return (size_t)4 * rows * xline_stride(e->r1, e->r2) * sizeof(cpx<R>);
+}
+template <typename R>
+static size_t line_smem(const LineEntry<R>* e, int lg) {
+  return ((size_t)4 << lg) * line_stride(e->r1, e->r2) * sizeof(cpx<R>);
+}
+
+// Sets the shared-memory limits of an entry's kernels (once per device) before their first launch.
+template <typename R>
+static swf_status line_ready(const LineEntry<R>* e) {
+  static std::atomic<bool> done[64][513];
+  const int dv = dev_slot();
+  if (done[dv][e->n].load(std::memory_order_acquire)) return SWF_OK;
+  cudaError_t r = cudaFuncSetAttribute(e->x, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)xline_smem<R>(e, xline_max_rows<R>(e)));
+  if (r == cudaSuccess)
+    r = cudaFuncSetAttribute(e->line, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)line_smem<R>(e, line_max_lg<R>(e, 8)));
+  if (r != cudaSuccess) return cuda_status(r, "cudaFuncSetAttribute(line kernels)");
+  done[dv][e->n].store(true, std::memory_order_release);
+  return SWF_OK;
+}
+
+// Launch shape of an x pass (v rows per block) or of a y or z pass (2^v columns per block) of either
+// kind, and the largest v that fits a block.
+struct PassShape {
+  int thr = 0, ld = 0, tpl = 0;
+  size_t smem = 0;
+  bool fits = false;
+};
+template <typename R>
+static PassShape x_shape(const StageArgs<R>& A, int rows) {
+  PassShape S;
+  if (A.ltw[0]) {
+    const LineEntry<R>* e = line_entry<R>(A.g.n[0]);
+    S.thr = 4 * rows * line_threads(e->r1, e->r2);
+    S.smem = xline_smem<R>(e, rows);
+    S.fits = rows <= xline_max_rows<R>(e);
+  } else {
+    S.ld = padded_len<R>(A.g.n[0]);
+    S.tpl = pass_threads(A.plan[0], 4);
+    S.thr = 4 * rows * S.tpl;
+    S.smem = (size_t)8 * rows * S.ld * sizeof(cpx<R>);
+    S.fits = rows <= 64 && S.thr <= kPassThreads && S.smem <= kPassSmemMax;
+  }
+  return S;
+}
+template <typename R>
+static PassShape mid_shape(const StageArgs<R>& A, int axis, int lg) {
+  PassShape S;
+  const int nx = A.g.n[0];
+  if (A.ltw[axis]) {
+    const LineEntry<R>* e = line_entry<R>(A.g.n[axis]);
+    S.thr = line_block(e->r1, e->r2, lg);
+    S.smem = line_smem<R>(e, lg);
+    S.fits = lg <= line_max_lg<R>(e, nx);
+  } else {
+    S.ld = padded_len<R>(A.g.n[axis]) | 1;  // neighbouring threads hold neighbouring lines
+    S.tpl = pass_threads(A.plan[axis], 4);
+    S.thr = ((4 << lg) * S.tpl + 31) & ~31;  // whole warps: the shuffles of H0 name all 32 lanes
+    S.smem = ((size_t)8 << lg) * S.ld * sizeof(cpx<R>);
+    S.fits = lg <= 3 && (lg == 0 || (1 << lg) <= nx) && S.thr <= kPassThreads && S.smem <= kPassSmemMax;
+  }
+  return S;
+}
+
+// The fixed rule: as many rows (columns) as a block takes, fewer on small grids (about two blocks per
+// SM; at least 32 bytes of contiguous x per line in the y and z passes).
+template <typename R>
+static int x_rule(const StageArgs<R>& A, int F) {
+  int rows = 1;
+  while (2 * rows <= A.nrows && x_shape<R>(A, 2 * rows).fits &&
+         (long)F * ((A.nrows + 2 * rows - 1) / (2 * rows)) >= 2L * sm_count())
+    rows *= 2;
+  return rows;
+}
+template <typename R>
+static int mid_rule(const StageArgs<R>& A, int axis, long tiles) {
+  const int nx = A.g.n[0], min_lg = sizeof(cpx<R>) == 8 ? 2 : 1;
+  int lg = 3;
+  while (lg > 0 && !mid_shape<R>(A, axis, lg).fits) --lg;
+  while (lg > min_lg && tiles * ((nx + (1 << lg) - 1) >> lg) < 2L * sm_count()) --lg;
+  return lg;
+}
+
+// Launches the x pass `rows` rows per block (flags as k_xline's).
+template <typename R>
+static void run_x(const StageArgs<R>& P, const StageArgs<R>& A, int rows, int flags, int F, cudaStream_t st) {
+  const PassShape S = x_shape<R>(A, rows);
+  const dim3 grid((A.nrows + rows - 1) / rows, F);
+  if (A.ltw[0]) {
+    line_entry<R>(A.g.n[0])->x<<<grid, S.thr, S.smem, st>>>(P, A, rows, flags);
+    return;
+  }
+  auto* kernel = k_xpass<R, 1>;
+  switch (end_radix(A.plan[0], true)) {
+    case 4: kernel = k_xpass<R, 4>; break;
+    case 2: kernel = k_xpass<R, 2>; break;
+    case 3: kernel = k_xpass<R, 3>; break;
+    case 5: kernel = k_xpass<R, 5>; break;
+    default: break;
+  }
+  kernel<<<grid, S.thr, S.smem, st>>>(P, A, rows, S.ld, S.tpl, flags);
+}
+
+// Launches the y or z pass, 2^lg columns per block; factors: with the blocks that compute the coming
+// evaluation's time factors.
+template <typename R>
+static void run_mid(const StageArgs<R>& A, int axis, int lg, int flags, bool factors, int F, cudaStream_t st) {
+  const PassShape S = mid_shape<R>(A, axis, lg);
+  const int tiles = ((A.g.n[0] + (1 << lg) - 1) >> lg) * (axis == 1 ? A.g.n[2] : A.g.n[1]);
+  const dim3 grid(tiles + (factors ? 1 : 0), F);
+  if (A.ltw[axis]) line_entry<R>(A.g.n[axis])->line<<<grid, S.thr, S.smem, st>>>(A, axis, lg, flags);
+  else k_mid<R><<<grid, S.thr, S.smem, st>>>(A, axis, lg, S.ld, S.tpl, flags);
+}
+
+// Grids with x as the only axis: `rows` rows per block of k_first, `thr` threads.
+template <typename R>
+static void run_only_x(const StageArgs<R>& A, int rows, int thr, int F, cudaStream_t st) {
+  const int ld = padded_len<R>(A.g.n[0]);
+  k_first<R><<<dim3((A.nrows + rows - 1) / rows, F), thr, (size_t)8 * rows * ld * sizeof(cpx<R>), st>>>(A, rows, ld);
+}
+
+// One x pass: closes evaluation P (close) and/or opens evaluation A (open) on the same rows; factors:
+// the pass before this one computed A's time factors.  Where x is the only axis the launch is the
+// whole evaluation.
+template <typename R>
+static swf_status launch_x(swf_ctx* ctx, const StageArgs<R>& P, const StageArgs<R>& A, bool close, bool open,
+                           bool factors, int F, cudaStream_t st) {
   constexpr int esz = (int)sizeof(cpx<R>);
   const int nx = A.g.n[0];
-  // tuned values: rows (x passes) or log2 TX (y, z passes) times 4, plus 1 for 128-thread blocks
-  const int xv = tune_lookup(ctx, tune_key('x', esz, nx, A.nrows, 0, F), 4 * x_rows<R>(nx, A.nrows, F));
-  XLaunch L;
-  L.rows = xv >> 2;
-  L.thr = (xv & 3) ? kThreads / 2 : kThreads;
-  L.ld = padded_len(nx);
-  L.smem = (size_t)2 * 4 * (L.rows > 0 ? L.rows : 1) * L.ld * sizeof(cpx<R>);
-  L.grid = dim3(L.rows > 0 ? (A.nrows + L.rows - 1) / L.rows : 1, F);
-  return L;
+  ProfScope ps(ctx, close ? (open ? "k_last_first" : "k_last") : "k_first", st);
+  if (A.g.n[1] == 1 && A.g.n[2] == 1) {
+    // tuned values: rows times 4, plus 1 for 128-thread blocks
+    const int xv = tune_lookup(ctx, tune_key('x', esz, nx, A.nrows, 0, F), 4 * x_rows<R>(nx, A.nrows, F));
+    if (xv < 4) return SWF_EUNSUPPORTED;
+    run_only_x<R>(A, xv >> 2, (xv & 3) ? kThreads / 2 : kThreads, F, st);
+    return SWF_OK;
+  }
+  const int rows = tune_lookup(ctx, tune_key('X', esz, nx, A.nrows, 0, F), x_rule<R>(A, F));
+  const bool regk = close && open && A.nterm > 0 && A.kin[A.nterm - 1] == P.kout;
+  run_x<R>(P, A, rows,
+           (close ? XL_LAST : 0) | (open ? XL_FIRST : 0) | (regk ? XL_REGK : 0) | (factors ? XL_FACTORS : 0), F, st);
+  return SWF_OK;
+}
+
+// One y or z pass; last: the last one of its evaluation (it computes the coming time factors).
+template <typename R>
+static void launch_mid(swf_ctx* ctx, const StageArgs<R>& A, int axis, int fwd, int h0, int inv, bool last, int F,
+                       cudaStream_t st) {
+  constexpr int esz = (int)sizeof(cpx<R>);
+  const long tiles = (long)(axis == 1 ? A.g.n[2] : A.g.n[1]) * F;
+  ProfScope ps(ctx, "k_mid", st);
+  const int lg = tune_lookup(ctx, tune_key('M', esz, axis * 8 + fwd * 4 + h0 * 2 + inv, A.g.n[axis], A.g.n[0], tiles),
+                             mid_rule<R>(A, axis, tiles));
+  run_mid<R>(A, axis, lg, (fwd ? LN_FWD : 0) | (h0 ? LN_H0 : 0) | (inv ? LN_INV : 0), last && A.ft, F, st);
 }
 
 // The y and z passes of one evaluation.
 template <typename R>
 static void launch_mids(swf_ctx* ctx, const StageArgs<R>& A, int F, cudaStream_t st) {
-  const int nx = A.g.n[0], ny = A.g.n[1], nz = A.g.n[2];
-  constexpr int esz = (int)sizeof(cpx<R>);
-  int axes[2], na = 0;
-  if (ny > 1) axes[na++] = 1;
-  if (nz > 1) axes[na++] = 2;
-  auto mid = [&](int axis, int fwd, int h0, int inv) {
-    const int other = axis == 1 ? nz : ny;
-    const int lg_h = mid_shape<R>(A.g.n[axis], nx, (long)other * F).lgtx;
-    const int mv = tune_lookup(ctx, tune_key('m', esz, axis * 8 + fwd * 4 + h0 * 2 + inv, A.g.n[axis], nx, (long)other * F),
-                               4 * lg_h);
-    const MidShape ms = mid_shape_lg<R>(A.g.n[axis], mv >> 2);
-    const int ntx = (nx + (1 << ms.lgtx) - 1) >> ms.lgtx;
-    dim3 grid(ntx * other, F);
-    ProfScope ps(ctx, "k_mid", st);
-    k_mid<R><<<grid, (mv & 3) ? kThreads / 2 : kThreads, ms.smem, st>>>(A, axis, ms.lgtx, ms.ld, fwd, h0, inv);
-  };
-  if (na == 1) {
-    mid(axes[0], 1, 1, 1);
-  } else if (na == 2) {
-    mid(1, 1, 0, 0);
-    mid(2, 1, 1, 1);
-    mid(1, 0, 0, 1);
+  const bool y = A.g.n[1] > 1, z = A.g.n[2] > 1;
+  if (y && z) {
+    launch_mid<R>(ctx, A, 1, 1, 0, 0, false, F, st);
+    launch_mid<R>(ctx, A, 2, 1, 1, 1, false, F, st);
+    launch_mid<R>(ctx, A, 1, 0, 0, 1, true, F, st);
+  } else if (y || z) {
+    launch_mid<R>(ctx, A, y ? 1 : 2, 1, 1, 1, true, F, st);
   }
 }
 
 // Launches one right-hand-side evaluation for F fields (ctx may be null: no profiling).
 template <typename R>
 static swf_status launch_eval(swf_ctx* ctx, const StageArgs<R>& A, int F, cudaStream_t st) {
-  const bool only_x = (A.g.n[1] == 1 && A.g.n[2] == 1);
-  const XLaunch L = x_launch<R>(ctx, A, F);
-  if (L.rows < 1) return SWF_EUNSUPPORTED;
-  {
-    ProfScope ps(ctx, "k_first", st);
-    k_first<R><<<L.grid, L.thr, L.smem, st>>>(A, L.rows, L.ld, only_x ? 1 : 0);
-  }
-  if (only_x) return SWF_OK;
+  swf_status s = launch_x<R>(ctx, A, A, false, true, false, F, st);
+  if (s != SWF_OK || (A.g.n[1] == 1 && A.g.n[2] == 1)) return s;
   launch_mids<R>(ctx, A, F, st);
-  {
-    ProfScope ps(ctx, "k_last", st);
-    k_last<R><<<L.grid, L.thr, L.smem, st>>>(A, L.rows, L.ld);
-  }
-  return SWF_OK;
+  return launch_x<R>(ctx, A, A, true, false, false, F, st);
 }
 
 // An evaluation whose inverse x pass is left for the next launch (march chains with at least one
-// non-trivial axis besides x): k_first and the y/z passes of A.
+// non-trivial axis besides x): the forward x pass and the y/z passes of A.
 template <typename R>
 static swf_status launch_eval_open(swf_ctx* ctx, const StageArgs<R>& A, int F, cudaStream_t st) {
-  const XLaunch L = x_launch<R>(ctx, A, F);
-  if (L.rows < 1) return SWF_EUNSUPPORTED;
-  {
-    ProfScope ps(ctx, "k_first", st);
-    k_first<R><<<L.grid, L.thr, L.smem, st>>>(A, L.rows, L.ld, 0);
-  }
-  launch_mids<R>(ctx, A, F, st);
-  return SWF_OK;
+  const swf_status s = launch_x<R>(ctx, A, A, false, true, false, F, st);
+  if (s == SWF_OK) launch_mids<R>(ctx, A, F, st);
+  return s;
 }
 
-// Closes the open evaluation P and runs evaluation Nx with it: k_last_first, then Nx's y/z passes.
+// Closes the open evaluation P and runs evaluation Nx with it in one x pass, then Nx's y/z passes.
 template <typename R>
 static swf_status launch_eval_chain(swf_ctx* ctx, const StageArgs<R>& P, const StageArgs<R>& Nx, int F,
                                     cudaStream_t st) {
-  const XLaunch L = x_launch<R>(ctx, Nx, F);
-  if (L.rows < 1) return SWF_EUNSUPPORTED;
-  {
-    ProfScope ps(ctx, "k_last_first", st);
-    k_last_first<R><<<L.grid, L.thr, L.smem, st>>>(P, Nx, L.rows, L.ld);
-  }
-  launch_mids<R>(ctx, Nx, F, st);
-  return SWF_OK;
+  const swf_status s = launch_x<R>(ctx, P, Nx, true, true, Nx.ft != nullptr, F, st);
+  if (s == SWF_OK) launch_mids<R>(ctx, Nx, F, st);
+  return s;
 }
 
 // Closes the open evaluation P (its inverse x pass).
 template <typename R>
 static swf_status launch_eval_close(swf_ctx* ctx, const StageArgs<R>& P, int F, cudaStream_t st) {
-  const XLaunch L = x_launch<R>(ctx, P, F);
-  if (L.rows < 1) return SWF_EUNSUPPORTED;
-  ProfScope ps(ctx, "k_last", st);
-  k_last<R><<<L.grid, L.thr, L.smem, st>>>(P, L.rows, L.ld);
-  return SWF_OK;
+  return launch_x<R>(ctx, P, P, true, false, false, F, st);
+}
+
+// The node that follows stage i (1..6, or 0 for the march's first evaluation) of step ls: the time
+// factors its last y/z pass computes.
+template <typename R>
+static void set_next_node(StageArgs<R>* A, int ls, int i) {
+  A->nls = i == 6 ? ls + 1 : ls;
+  A->nc = DP_C[i == 6 ? 1 : i + 1];
 }
 
 // Times the candidate launch shapes of one evaluation's pass kernels (rows per block or tile
@@ -1002,11 +868,11 @@ static swf_status autotune_eval(swf_ctx* ctx, const StageArgs<R>& B, int F, cuda
     return cuda_status(cudaGetLastError(), "tuning events");
   }
   swf_status status = SWF_OK;
-  // time `launch` (one warm-up, then three back to back); +inf on a launch error
+  // time `launch` (one warm-up, then four back to back); +inf on a launch error
   auto timed = [&](auto&& launch) -> float {
     launch();
     cudaEventRecord(ev[0], st);
-    for (int r = 0; r < 3; ++r) launch();
+    for (int r = 0; r < 4; ++r) launch();
     cudaEventRecord(ev[1], st);
     cudaError_t e = cudaEventSynchronize(ev[1]);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -1018,56 +884,50 @@ static swf_status autotune_eval(swf_ctx* ctx, const StageArgs<R>& B, int F, cuda
     cudaEventElapsedTime(&ms, ev[0], ev[1]);
     return ms;
   };
-  const std::string xkey = tune_key('x', esz, nx, B.nrows, 0, F);
-  if (!ctx->tune.best.count(xkey)) {
-    const size_t line = (size_t)2 * 4 * padded_len(nx) * esz;
-    int rmax = (int)(kPassSmemTune / line);
-    rmax = std::min(std::min(rmax, 64), B.nrows);
-    int best = 4 * x_rows<R>(nx, B.nrows, F);
-    float tbest = 3.4e38f;
-    const int ld = padded_len(nx);
-    for (int rows = 1; rows <= rmax && status == SWF_OK; rows *= 2) {
-      for (int half = 0; half < 2 && status == SWF_OK; ++half) {
-        const int thr = half ? kThreads / 2 : kThreads;
-        const size_t smem = (size_t)2 * 4 * rows * ld * esz;
-        const dim3 grid((B.nrows + rows - 1) / rows, F);
-        const float t = timed([&] {
-          k_first<R><<<grid, thr, smem, st>>>(B, rows, ld, only_x ? 1 : 0);
-          if (!only_x) k_last<R><<<grid, thr, smem, st>>>(B, rows, ld);
-        });
-        if (t < tbest) { tbest = t; best = 4 * rows + half; }
-      }
-    }
-    if (status == SWF_OK) ctx->tune.best[xkey] = best;
-  }
-  if (!only_x) {
-    int axes[2], na = 0;
-    if (ny > 1) axes[na++] = 1;
-    if (nz > 1) axes[na++] = 2;
-    const int combos1[1][4] = {{0, 1, 1, 1}};
-    const int combos2[3][4] = {{1, 1, 0, 0}, {2, 1, 1, 1}, {1, 0, 0, 1}};
-    const int nc = na == 1 ? 1 : 3;
-    for (int ci = 0; ci < nc && status == SWF_OK; ++ci) {
-      const int* cb = na == 1 ? combos1[ci] : combos2[ci];
-      const int axis = na == 1 ? axes[0] : cb[0];
-      const int other = axis == 1 ? nz : ny;
-      const int n_a = B.g.n[axis];
-      const std::string key = tune_key('m', esz, axis * 8 + cb[1] * 4 + cb[2] * 2 + cb[3], n_a, nx, (long)other * F);
-      if (ctx->tune.best.count(key)) continue;
-      int best = 4 * mid_shape<R>(n_a, nx, (long)other * F).lgtx;
+  if (only_x) {
+    const std::string key = tune_key('x', esz, nx, B.nrows, 0, F);
+    if (!ctx->tune.best.count(key)) {
+      int rmax = (int)(kPassSmemMax / ((size_t)8 * padded_len<R>(nx) * esz));
+      rmax = std::min(std::min(rmax, 64), B.nrows);
+      int best = 4 * x_rows<R>(nx, B.nrows, F);
       float tbest = 3.4e38f;
-      for (int lg = mid_max_lg<R>(n_a, nx, kPassSmemTune); lg >= 0 && status == SWF_OK; --lg) {
+      for (int rows = 1; rows <= rmax && status == SWF_OK; rows *= 2)
         for (int half = 0; half < 2 && status == SWF_OK; ++half) {
-          const MidShape ms = mid_shape_lg<R>(n_a, lg);
-          const int ntx = (nx + (1 << lg) - 1) >> lg;
-          const dim3 grid(ntx * other, F);
-          const float t = timed([&] {
-            k_mid<R><<<grid, half ? kThreads / 2 : kThreads, ms.smem, st>>>(B, axis, lg, ms.ld, cb[1], cb[2], cb[3]);
-          });
-          if (t < tbest) { tbest = t; best = 4 * lg + half; }
+          const float t = timed([&] { run_only_x<R>(B, rows, half ? kThreads / 2 : kThreads, F, st); });
+          if (t < tbest) { tbest = t; best = 4 * rows + half; }
         }
+      if (status == SWF_OK) ctx->tune.best[key] = best;
+    }
+  } else {
+    const std::string key = tune_key('X', esz, nx, B.nrows, 0, F);
+    if (!ctx->tune.best.count(key)) {
+      int best = 1;
+      float tbest = 3.4e38f;
+      for (int rows = 1; (rows == 1 || (rows <= B.nrows && x_shape<R>(B, rows).fits)) && status == SWF_OK; rows *= 2) {
+        const float t = timed([&] { run_x<R>(B, B, rows, XL_LAST | XL_FIRST | (B.ft ? XL_FACTORS : 0), F, st); });
+        if (t < tbest) { tbest = t; best = rows; }
       }
       if (status == SWF_OK) ctx->tune.best[key] = best;
+    }
+    const int one[1][4] = {{ny > 1 ? 1 : 2, 1, 1, 1}};
+    const int three[3][4] = {{1, 1, 0, 0}, {2, 1, 1, 1}, {1, 0, 0, 1}};
+    const bool both = ny > 1 && nz > 1;
+    for (int ci = 0; ci < (both ? 3 : 1) && status == SWF_OK; ++ci) {
+      const int* cb = both ? three[ci] : one[0];
+      const int axis = cb[0];
+      const std::string mkey = tune_key('M', esz, axis * 8 + cb[1] * 4 + cb[2] * 2 + cb[3], B.g.n[axis], nx,
+                                        (long)(axis == 1 ? nz : ny) * F);
+      if (ctx->tune.best.count(mkey)) continue;
+      int best = 0;
+      float tbest = 3.4e38f;
+      for (int lg = 3; lg >= 0 && status == SWF_OK; --lg) {
+        if (!mid_shape<R>(B, axis, lg).fits) continue;
+        const float t = timed([&] {
+          run_mid<R>(B, axis, lg, (cb[1] ? LN_FWD : 0) | (cb[2] ? LN_H0 : 0) | (cb[3] ? LN_INV : 0), false, F, st);
+        });
+        if (t < tbest) { tbest = t; best = lg; }
+      }
+      if (status == SWF_OK) ctx->tune.best[mkey] = best;
     }
   }
   cudaEventDestroy(ev[0]);
@@ -1084,7 +944,7 @@ static swf_status prepare_args(swf_ctx* ctx, const GridDesc& g, int F, const Fie
   A->g = g;
   A->nrows = g.n[1] * g.n[2];
   for (int a = 0; a < 3; ++a) {
-    if (!make_march_plan(g.n[a], &A->plan[a])) {
+    if (!make_line_plan<R>(g, a, &A->plan[a])) {
       set_error("grid size must factor into 2, 3 and 5");
       return SWF_EINVAL;
     }
@@ -1092,8 +952,20 @@ static swf_status prepare_args(swf_ctx* ctx, const GridDesc& g, int F, const Fie
     s = twiddles(ctx, g.n[a], Prec<R>::is_double, &tw);
     if (s != SWF_OK) return s;
     A->tw[a] = reinterpret_cast<const cpx<R>*>(tw);
+    if (const LineEntry<R>* le = line_of<R>(g, a)) {
+      if ((s = line_ready<R>(le)) != SWF_OK) return s;
+      if ((s = twiddles(ctx, g.n[a], Prec<R>::is_double, &tw, le->r2)) != SWF_OK) return s;
+      A->ltw[a] = reinterpret_cast<const cpx<R>*>(tw);
+    }
   }
   const int nt = g.n[0] + g.n[1] + g.n[2];
+  if (g.n[1] > 1 || g.n[2] > 1) {  // the last y/z pass computes the x pass's time factors
+    void *pft = nullptr, *ptf = nullptr;
+    if ((s = ws_get(ctx, std::string(tag) + ".ft", sizeof(R) * F * g.n[1], &pft)) != SWF_OK) return s;
+    if ((s = ws_get(ctx, std::string(tag) + ".tf", sizeof(cpx<R>) * F, &ptf)) != SWF_OK) return s;
+    A->ft = (R*)pft;
+    A->tf = (cpx<R>*)ptf;
+  }
   void *pfd = nullptr, *pgr = nullptr, *pgc = nullptr;
   std::string t(tag);
   if ((s = ws_get(ctx, t + ".fd", sizeof(FieldDesc) * F, &pfd)) != SWF_OK) return s;
@@ -1118,60 +990,63 @@ static swf_status prepare_args(swf_ctx* ctx, const GridDesc& g, int F, const Fie
   return SWF_OK;
 }
 
-// Runs `pairs` repetitions of two Dormand-Prince steps recorded by `record` (launches only, on
-// st), each followed by advancing the march clock by two steps.  Unless kernel timing is on or
-// st is the legacy default stream, the pair is captured once into a CUDA graph and replayed:
-// one launch per two steps instead of one per kernel.  The slots rotate with period two, so
-// the recorded pointers repeat; the stage times come from the device clock.
-template <typename Rec>
-static swf_status run_step_pairs(swf_ctx* ctx, cudaStream_t st, int pairs, MarchClock* clk, Rec&& record) {
-  if (pairs <= 0) return SWF_OK;
-  swf_status s = SWF_OK;
-  bool graph = !ctx->prof.on && st != 0 && ctx->use_graphs;
+// `pairs` repetitions of two Dormand-Prince steps recorded by record(st) (launches only), each followed
+// by advancing the march clock by two steps.  Unless kernel timing is on or st is the legacy default
+// stream, the pair is captured once into a CUDA graph and replayed: one launch per two steps instead
+// of one per kernel.  The slots rotate with period two, so the recorded pointers repeat; the stage
+// times come from the device clock.  prepare() captures, launch() queues one repetition, finish()
+// waits for the replays and releases the graph.
+struct StepPairs {
+  cudaStream_t st = nullptr;
   cudaGraphExec_t exec = nullptr;
   long long per_pair = 0;
-  if (graph) {
+
+  template <typename Rec>
+  swf_status prepare(swf_ctx* ctx, cudaStream_t stream, MarchClock* clk, Rec&& record) {
+    st = stream;
+    if (ctx->prof.on || st == 0 || !ctx->use_graphs) return SWF_OK;
     const long long l0 = ctx->prof.launches;
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       cudaGetLastError();
-      graph = false;
-    } else {
-      s = record();
-      k_clock_advance<<<1, 1, 0, st>>>(clk, 2);
-      cudaGraph_t gr = nullptr;
-      cudaError_t e = cudaStreamEndCapture(st, &gr);
-      per_pair = ctx->prof.launches - l0 + 1;
-      ctx->prof.launches = l0;
-      if (s != SWF_OK) {
-        if (gr) cudaGraphDestroy(gr);
-        return s;
-      }
-      if (e != cudaSuccess) return cuda_status(e, "capture of the march steps");
-      e = cudaGraphInstantiate(&exec, gr, 0);
-      cudaGraphDestroy(gr);
-      if (e != cudaSuccess) return cuda_status(e, "instantiate the march graph");
+      return SWF_OK;
     }
+    const swf_status s = record();
+    k_clock_advance<<<1, 1, 0, st>>>(clk, 2);
+    cudaGraph_t gr = nullptr;
+    cudaError_t e = cudaStreamEndCapture(st, &gr);
+    per_pair = ctx->prof.launches - l0 + 1;
+    ctx->prof.launches = l0;
+    if (s != SWF_OK) {
+      if (gr) cudaGraphDestroy(gr);
+      return s;
+    }
+    if (e != cudaSuccess) return cuda_status(e, "capture of the march steps");
+    e = cudaGraphInstantiate(&exec, gr, 0);
+    cudaGraphDestroy(gr);
+    if (e != cudaSuccess) return cuda_status(e, "instantiate the march graph");
+    return SWF_OK;
   }
-  if (!graph) {
-    for (int p = 0; p < pairs && s == SWF_OK; ++p) {
-      s = record();
-      k_clock_advance<<<1, 1, 0, st>>>(clk, 2);
-      ++ctx->prof.launches;
+  template <typename Rec>
+  swf_status launch(swf_ctx* ctx, MarchClock* clk, Rec&& record) {
+    if (exec) {
+      const cudaError_t e = cudaGraphLaunch(exec, st);
+      ctx->prof.launches += per_pair;
+      return e == cudaSuccess ? SWF_OK : cuda_status(e, "launch the march graph");
     }
+    const swf_status s = record();
+    k_clock_advance<<<1, 1, 0, st>>>(clk, 2);
+    ++ctx->prof.launches;
     return s;
   }
-  cudaError_t e = cudaSuccess;
-  for (int p = 0; p < pairs && e == cudaSuccess; ++p) {
-    e = cudaGraphLaunch(exec, st);
-    ctx->prof.launches += per_pair;
-  }
   // the executable graph is released once its launches have run
-  cudaError_t e2 = cudaStreamSynchronize(st);
-  cudaGraphExecDestroy(exec);
-  if (e != cudaSuccess) return cuda_status(e, "launch the march graph");
-  if (e2 != cudaSuccess) return cuda_status(e2, "march graph");
-  return SWF_OK;
-}
+  swf_status finish() {
+    if (!exec) return SWF_OK;
+    const cudaError_t e = cudaStreamSynchronize(st);
+    cudaGraphExecDestroy(exec);
+    exec = nullptr;
+    return e == cudaSuccess ? SWF_OK : cuda_status(e, "march graph");
+  }
+};
 
 // complex64 fixed-step marches carry the state in float-float: a zeroed low part beside y.
 template <typename R>
@@ -1189,96 +1064,8 @@ static swf_status state_low_part(swf_ctx* ctx, const std::string& name, size_t b
 }
 
 template <typename R>
-static swf_status march_impl(swf_ctx* ctx, const GridDesc& g, double t_in, double t_out, int n_steps,
-                             int F, const FieldDesc* fd_host, void* psi_out, cudaStream_t st) {
-  StageArgs<R> A;
-  swf_status s = prepare_args<R>(ctx, g, F, fd_host, &A, "march", st);
-  if (s != SWF_OK) return s;
-  const size_t state = (size_t)F * 4 * g.N * sizeof(cpx<R>);
-  void *py = nullptr, *pT = nullptr, *pk[7];
-  if ((s = ws_get(ctx, "march.y", state, &py)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "march.T", state, &pT)) != SWF_OK) return s;
-  for (int i = 0; i < 7; ++i) {
-    char nm[32];
-    std::snprintf(nm, sizeof nm, "march.k%d", i);
-    if ((s = ws_get(ctx, nm, state, &pk[i])) != SWF_OK) return s;
-  }
-  cudaError_t e = cudaMemsetAsync(py, 0, state, st);
-  if (e != cudaSuccess) return cuda_status(e, "memset state");
-  A.y = (cpx<R>*)py;
-  A.T = (cpx<R>*)pT;
-  if ((s = state_low_part<R>(ctx, "march.ylo", state, &A, st)) != SWF_OK) return s;
-  {
-    // shapes by timing, on the slots before they hold anything (the heaviest stage: six inputs)
-    StageArgs<R> B = A;
-    B.nterm = 6;
-    for (int q = 0; q < 6; ++q) {
-      B.kin[q] = (const cpx<R>*)pk[q + 1];
-      B.coef[q] = 0.0;
-    }
-    B.write_y = 0;
-    B.ystage = nullptr;
-    B.kout = (cpx<R>*)pk[0];
-    B.t = t_out;
-    if ((s = autotune_eval<R>(ctx, B, F, st)) != SWF_OK) return s;
-  }
-  int slot[7] = {0, 1, 2, 3, 4, 5, 6};
-  const double h = (t_in - t_out) / n_steps;
-  void* pclk = nullptr;
-  if ((s = ws_get(ctx, "march.clock", sizeof(MarchClock), &pclk)) != SWF_OK) return s;
-  MarchClock* clk = (MarchClock*)pclk;
-  k_clock_set<<<1, 1, 0, st>>>(clk, t_out, h);
-  A.clk = clk;
-  // Evaluations chain: each one's inverse x pass runs in one launch with the next one's forward x
-  // pass (k_last_first), except on grids with x as the only non-trivial axis (one pass per
-  // evaluation).  The open evaluation after every second step writes slot 0, as the first
-  // evaluation does, so a recorded pair of steps replays unchanged.
-  const bool chain = !(g.n[1] == 1 && g.n[2] == 1);
-  StageArgs<R> open = A;
-  // k_1 = f(t_out, 0)
-  A.nterm = 0;
-  A.write_y = 0;
-  A.kout = (cpx<R>*)pk[slot[0]];
-  A.ls = 0;
-  A.c = 0.0;
-  if ((s = chain ? launch_eval_open<R>(ctx, A, F, st) : launch_eval<R>(ctx, A, F, st)) != SWF_OK) return s;
-  open = A;
-  // one step at clock offset ls (stage times from the clock: the same arithmetic as
-  // tn = t_out + n h, t = tn + c_i h)
-  auto step = [&](int ls) -> swf_status {
-    for (int i = 1; i < 7; ++i) {
-      int nt = 0;
-      for (int j = 0; j < i; ++j) {
-        if (DP_A[i][j] == 0.0) continue;
-        A.kin[nt] = (const cpx<R>*)pk[slot[j]];
-        A.coef[nt] = h * DP_A[i][j];
-        ++nt;
-      }
-      A.nterm = nt;
-      A.write_y = (i == 6);
-      A.kout = (cpx<R>*)pk[slot[i]];
-      A.ls = ls;
-      A.c = DP_C[i];
-      swf_status r = chain ? launch_eval_chain<R>(ctx, open, A, F, st) : launch_eval<R>(ctx, A, F, st);
-      if (r != SWF_OK) return r;
-      open = A;
-    }
-    std::swap(slot[0], slot[6]);
-    return SWF_OK;
-  };
-  s = run_step_pairs(ctx, st, n_steps / 2, clk, [&]() -> swf_status {
-    swf_status r = step(0);
-    return r == SWF_OK ? step(1) : r;
-  });
-  if (s != SWF_OK) return s;
-  if (n_steps % 2 && (s = step(0)) != SWF_OK) return s;
-  if (chain && (s = launch_eval_close<R>(ctx, open, F, st)) != SWF_OK) return s;
-  e = cudaMemcpyAsync(psi_out, py, state, cudaMemcpyDeviceToDevice, st);
-  if (e != cudaSuccess) return cuda_status(e, "copy psi(t_in)");
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_status(e, "march kernels");
-  return SWF_OK;
-}
+static swf_status march_impl(swf_ctx* ctx, const GridDesc& g, double t_in, double t_out, int n_steps, int F,
+                             const FieldDesc* fd_host, void* psi_out, cudaStream_t st);
 
 // ---------------------------------------------------------------- step-size control
 // Fifth- minus fourth-order weights b_i - b*_i of the Dormand-Prince pair (1980).
@@ -1568,6 +1355,7 @@ static swf_status march_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double t_
     for (int q = 0; q < 6; ++q) {
       B.kin[q] = (const cpx<R>*)pk[q + 1];
       B.coef[q] = 0.0;
+      B.coef_r[q] = (R)0;
     }
     B.write_y = 0;
     B.ystage = nullptr;
@@ -1602,6 +1390,7 @@ static swf_status march_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double t_
       A.write_y = (i == 6);
       A.kout = (cpx<R>*)pk[i];
       A.c = DP_C[i];
+      set_next_node<R>(&A, 0, i);
       swf_status r = !chain ? launch_eval<R>(ctx, A, F, st)
                             : (i == 1 ? launch_eval_open<R>(ctx, A, F, st) : launch_eval_chain<R>(ctx, open, A, F, st));
       if (r != SWF_OK) return r;
@@ -1732,9 +1521,15 @@ static swf_status reserve_march(swf_ctx* ctx, const GridDesc& g, int F) {
     if ((s = ws_get(ctx, nm, state, &p)) != SWF_OK) return s;
   }
   if ((s = ws_get(ctx, "march.clock", sizeof(MarchClock), &p)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, "march.kap", sizeof(R) * nt, &p)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, "march.ft", sizeof(R) * F * g.n[1], &p)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, "march.tf", sizeof(cpx<R>) * F, &p)) != SWF_OK) return s;
   for (int a = 0; a < 3; ++a) {
     const void* tw = nullptr;
     if ((s = twiddles(ctx, g.n[a], Prec<R>::is_double, &tw)) != SWF_OK) return s;
+    const LineEntry<R>* le = line_of<R>(g, a);
+    if (le && (s = line_ready<R>(le)) != SWF_OK) return s;
+    if (le && (s = twiddles(ctx, g.n[a], Prec<R>::is_double, &tw, le->r2)) != SWF_OK) return s;
   }
   return SWF_OK;
 }
@@ -1881,11 +1676,12 @@ swf_status rhs_eval(swf_ctx* ctx, const GridDesc& g, const FieldDesc& fd, swf_pr
 namespace swf {
 
 template <typename R>
-__global__ void k_twiddles_into(cpx<R>* tw, int n) {
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n; m += gridDim.x * blockDim.x) {
+__global__ void k_twiddles_into(cpx<R>* tw, int n, int r2) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const int m = r2 ? ((e / r2) * (e % r2)) % n : e;
     double s, c;
     sincospi(-2.0 * m / (double)n, &s, &c);
-    tw[m] = mk<R>((R)c, (R)s);
+    tw[e] = mk<R>((R)c, (R)s);
   }
 }
 
@@ -1927,14 +1723,16 @@ static swf_status rhs_scratch_impl(const GridDesc& g, const FieldDesc& fd, doubl
   A.g = g;
   A.nrows = g.n[1] * g.n[2];
   for (int a = 0; a < 3; ++a) {
-    if (!make_march_plan(g.n[a], &A.plan[a])) {
+    if (!make_line_plan<R>(g, a, &A.plan[a])) {
       set_error("grid size must factor into 2, 3 and 5");
       return SWF_EINVAL;
     }
+    const LineEntry<R>* le = line_of<R>(g, a);
     cpx<R>* tw = (cpx<R>*)p;
     p += align256(512 * sizeof(cpx<R>));
-    k_twiddles_into<R><<<(g.n[a] + 127) / 128, 128, 0, st>>>(tw, g.n[a]);
-    A.tw[a] = tw;
+    k_twiddles_into<R><<<(g.n[a] + 127) / 128, 128, 0, st>>>(tw, g.n[a], le ? le->r2 : 0);
+    (le ? A.ltw : A.tw)[a] = tw;
+    if (le && (s = line_ready<R>(le)) != SWF_OK) return s;
   }
   k_store_field_desc<<<1, 1, 0, st>>>(fd, dfd);
   k_tables<R><<<dim3((nt + 4 + 127) / 128, 1), 128, 0, st>>>(dfd, g, greal, gcplx);
@@ -2311,7 +2109,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_f2_x(StageArgs<
         for (int c = 0; c < 4; ++c) v[c] = mk<R>(0, 0);
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) buf[(c * rows + j) * ld + pad32(x)] = v[c];
+      for (int c = 0; c < 4; ++c) buf[(c * rows + j) * ld + pad<R>(x)] = v[c];
     }
     __syncthreads();
     cpx<R>* res = fft_pp<R>(buf, buf2, ld, 4 * rows, A.plan[0], false, A.tw[0]);
@@ -2323,7 +2121,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_f2_x(StageArgs<
       if (row < A.nrows) {
         const size_t gi = (size_t)row * nx + x;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) dst[gi + c * cs] = res[(c * rows + j) * ld + pad32(x)];
+        for (int c = 0; c < 4; ++c) dst[gi + c * cs] = res[(c * rows + j) * ld + pad<R>(x)];
       }
     }
     __syncthreads();
@@ -2528,7 +2326,7 @@ static swf_status f2_prepare(swf_ctx* ctx, const GridDesc& g, int n_inst, const 
     set_error("partial-integration integrand: an x line does not fit shared memory");
     return SWF_EUNSUPPORTED;
   }
-  p->ld = padded_len(nx);
+  p->ld = padded_len<R>(nx);
   p->smem_x = (size_t)2 * 4 * p->rows * p->ld * sizeof(cpx<R>);
   p->nbx = (nrows + p->rows - 1) / p->rows;
   // one mode per thread where the grid allows (the gathers of the V modes are latency-bound)
@@ -2619,6 +2417,7 @@ static swf_status f2_integrand(swf_ctx* ctx, const StageArgs<R>& A, const F2Plan
   StageArgs<R> B = A;
   B.ls = ls;
   B.c = DP_C[stage];
+  if (sizeof(R) == 4) make_march_plan(g.n[0], &B.plan[0]);  // a whole-line transform (lengths were checked)
   {
     ProfScope ps(ctx, "k_f2_x", st);
     k_f2_x<R><<<dim3(p.nbx, 2 * G), p.xthr, p.smem_x, st>>>(B, ys, p.Yspec, p.Zspec, p.has_mid ? 0 : 1, p.dph,
@@ -2627,15 +2426,8 @@ static swf_status f2_integrand(swf_ctx* ctx, const StageArgs<R>& A, const F2Plan
   StageArgs<R> C = A;
   C.T = p.Zspec;
   C.yspec = nullptr;
-  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-  for (int axis = 1; axis <= 2; ++axis) {
-    if (g.n[axis] <= 1) continue;
-    const int other = axis == 1 ? nz : ny;
-    const MidShape ms = mid_shape<R>(g.n[axis], nx, (long)other * 2 * G);
-    const int ntx = (nx + (1 << ms.lgtx) - 1) >> ms.lgtx;
-    ProfScope ps(ctx, "k_mid", st);
-    k_mid<R><<<dim3(ntx * other, 2 * G), kThreads, ms.smem, st>>>(C, axis, ms.lgtx, ms.ld, 1, 0, 0);
-  }
+  for (int axis = 1; axis <= 2; ++axis)
+    if (g.n[axis] > 1) launch_mid<R>(ctx, C, axis, 1, 0, 0, false, 2 * G, st);
   {
     ProfScope ps(ctx, "k_f2_ss", st);
     k_f2_ss<R><<<dim3(p.nbs, G), kThreads, 0, st>>>(p.Yspec, p.Zspec, g, A.fd, photon_dev, p.f2i, p.omt, ptab, A.clk,
@@ -2644,164 +2436,237 @@ static swf_status f2_integrand(swf_ctx* ctx, const StageArgs<R>& A, const F2Plan
   return SWF_OK;
 }
 
+// One fixed-step march of F fields on one grid: plain (form 0), or U and V of F/2 Breit-Wheeler
+// instances with the integrand of Eq. 17 (form 1; n_ph photons per instance) or of Eqs. 30-33 (form
+// 2) integrated along.  setup() sizes the workspace and queues the tables, first() the evaluation
+// k_1 = f(t_out, 0), step(ls) one step at clock offset ls (of a pair of steps), finish() what follows
+// the last step.  All launches of one march go to one stream; several marches with workspaces of
+// their own (tag) may run at once (march_multi).
 template <typename R>
-static swf_status march_bw_impl(swf_ctx* ctx, const GridDesc& g, double t_in, double t_out, int n_steps, int n_inst,
-                                const FieldDesc* fd_host, const double* photon_host, void* psi_out, double2* macc,
-                                cudaStream_t st, int form, const double* wave_k_host, int n_ph) {
-  const int F = 2 * n_inst;
-  const int NP = n_inst * n_ph;  // photon-instances: photon j of instance i is i n_ph + j
-  StageArgs<R> A;
-  swf_status s = prepare_args<R>(ctx, g, F, fd_host, &A, "bw", st);
-  if (s != SWF_OK) return s;
-  const size_t state = (size_t)F * 4 * g.N * sizeof(cpx<R>);
-  const int nt = g.n[0] + g.n[1] + g.n[2];
-  void *py, *pT, *pys, *pk[7], *pph, *pkph;
-  if ((s = ws_get(ctx, "march.y", state, &py)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "march.T", state, &pT)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "bw.ystage", state, &pys)) != SWF_OK) return s;
-  for (int i = 0; i < 7; ++i) {
-    char nm[32];
-    std::snprintf(nm, sizeof nm, "march.k%d", i);
-    if ((s = ws_get(ctx, nm, state, &pk[i])) != SWF_OK) return s;
-  }
-  if ((s = ws_get(ctx, "bw.photon", sizeof(double) * 6 * NP, &pph)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "bw.kph", sizeof(cpx<R>) * NP * nt, &pkph)) != SWF_OK) return s;
-  // blocks per instance of the M-dot reduction: about four waves of the GPU in total, at least
-  // 1024 sites per block (the same split for every photon count, so a photon of a scan sums
-  // exactly as a solve of that photon alone); photons per block: 1, or 4 (8 in complex64) for
-  // scans, which then read U and V once per site for the block's photons
-  const int nph_blk = n_ph == 1 ? 1 : (sizeof(R) == 4 && n_ph > 4 ? 8 : 4);
-  const int nchunk = (n_ph + nph_blk - 1) / nph_blk;
-  const int nb = std::max(1, std::min((g.N + 1023) / 1024, (4 * sm_count() + n_inst - 1) / n_inst));
-  void* ptab;
-  if ((s = ws_get(ctx, "bw.phase_table", sizeof(cpx<double>) * 3 * 7 * (size_t)n_steps * NP, &ptab)) != SWF_OK)
-    return s;
-  void* ppart;
-  if ((s = ws_get(ctx, "bw.mpart", sizeof(cpx<double>) * 3 * (size_t)nb * NP, &ppart)) != SWF_OK) return s;
-  cudaError_t e = cudaMemcpyAsync(pph, photon_host, sizeof(double) * 6 * NP, cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return cuda_status(e, "upload photon table");
-  {
-    ProfScope ps(ctx, "k_photon_tables", st);
-    k_photon_tables<R><<<(NP * nt + 127) / 128, 128, 0, st>>>((const double*)pph, g, NP, (cpx<R>*)pkph);
-  }
-  {
-    const long total = (long)NP * n_steps * 7;
-    ProfScope ps(ctx, "k_bw_phase_table", st);
-    k_bw_phase_table<<<(int)std::min((total + 127) / 128, 4096L), 128, 0, st>>>(
-        A.fd, (const double*)pph, NP, n_ph, n_steps, t_out, (t_in - t_out) / n_steps, g.dx[0] * g.dx[1] * g.dx[2],
-        form, (cpx<double>*)ptab);
-  }
-  if ((e = cudaMemsetAsync(py, 0, state, st)) != cudaSuccess) return cuda_status(e, "memset state");
-  if ((e = cudaMemsetAsync(ppart, 0, sizeof(cpx<double>) * 3 * (size_t)nb * NP, st)) != cudaSuccess)
-    return cuda_status(e, "memset M accumulators");
-  A.y = (cpx<R>*)py;
-  A.T = (cpx<R>*)pT;
-  if ((s = state_low_part<R>(ctx, "march.ylo", state, &A, st)) != SWF_OK) return s;
-  {
-    StageArgs<R> B = A;  // shapes by timing, as in the plain march
-    B.nterm = 6;
-    for (int q = 0; q < 6; ++q) {
-      B.kin[q] = (const cpx<R>*)pk[q + 1];
-      B.coef[q] = 0.0;
-    }
-    B.write_y = 0;
-    B.ystage = nullptr;
-    B.kout = (cpx<R>*)pk[0];
-    B.t = t_out;
-    if ((s = autotune_eval<R>(ctx, B, F, st)) != SWF_OK) return s;
-  }
-  F2Plan<R> p2;
-  if (form == 2 && (s = f2_prepare<R>(ctx, g, n_inst, fd_host, photon_host, wave_k_host, &p2, st)) != SWF_OK)
-    return s;
+struct MarchPlan {
+  swf_ctx* ctx = nullptr;
+  cudaStream_t st = nullptr;
+  GridDesc g;
+  int n_steps = 0, F = 0, form = 0, n_inst = 0, n_ph = 1, NP = 0;
+  int nph_blk = 1, nchunk = 1, nb = 1;
+  double h = 0.0;
+  StageArgs<R> A, open;
+  bool chain = true;
+  size_t state = 0;
+  void *py = nullptr, *pk[7], *pys = nullptr, *pph = nullptr, *pkph = nullptr, *ptab = nullptr, *ppart = nullptr;
   int slot[7] = {0, 1, 2, 3, 4, 5, 6};
-  const double h = (t_in - t_out) / n_steps;
-  void* pclk = nullptr;
-  if ((s = ws_get(ctx, "march.clock", sizeof(MarchClock), &pclk)) != SWF_OK) return s;
-  MarchClock* clk = (MarchClock*)pclk;
-  k_clock_set<<<1, 1, 0, st>>>(clk, t_out, h);
-  A.clk = clk;
-  A.nterm = 0;
-  A.write_y = 0;
-  A.kout = (cpx<R>*)pk[slot[0]];
-  A.ls = 0;
-  A.c = 0.0;
-  A.ystage = nullptr;  // the integrand of Eq. 17 vanishes at psi_s(t_out) = 0
-  // evaluations chain through k_last_first as in march_impl (the integrands read only the stage
-  // value and the transforms written by the forward passes, never T or the k slots)
-  const bool chain = !(g.n[1] == 1 && g.n[2] == 1);
-  if ((s = chain ? launch_eval_open<R>(ctx, A, F, st) : launch_eval<R>(ctx, A, F, st)) != SWF_OK) return s;
-  StageArgs<R> open = A;
-  // the partial-integration integrand does not (its source term is V psi_b): stage value y = 0
-  if (form == 2 && (s = f2_integrand<R>(ctx, A, p2, (const cpx<R>*)py, (const double*)pph, (const cpx<double>*)ptab,
-                                        7 * n_steps, 0, 0, st)) != SWF_OK)
+  MarchClock* clk = nullptr;
+  F2Plan<R> p2;
+  StepPairs pairs;
+
+  swf_status buf(const std::string& name, size_t bytes, void** p) { return ws_get(ctx, name, bytes, p); }
+
+  // tag: prefix of the workspace ("march" for a march that runs alone)
+  swf_status setup(swf_ctx* c, const std::string& tag, const GridDesc& grid, double t_in, double t_out, int steps,
+                   int n_f, const FieldDesc* fd_host, int form_, const double* photon_host, const double* wave_k_host,
+                   int photons, cudaStream_t stream) {
+    ctx = c;
+    st = stream;
+    g = grid;
+    n_steps = steps;
+    F = n_f;
+    form = form_;
+    n_ph = photons;
+    n_inst = F / 2;
+    NP = n_inst * n_ph;  // photon-instances: photon j of instance i is i n_ph + j
+    h = (t_in - t_out) / n_steps;
+    const bool alone = tag == "march";
+    const std::string bt = alone ? "bw" : tag;  // prefix of the integrand's buffers
+    // evaluations chain: each one's inverse x pass runs in one launch with the next one's forward x
+    // pass, except on grids with x as the only non-trivial axis (one pass per evaluation).  The open
+    // evaluation after every second step writes slot 0, as the first evaluation does, so a recorded
+    // pair of steps replays unchanged.  (The integrands read only the stage value and the transforms
+    // written by the forward passes, never T or the k slots.)
+    chain = !(g.n[1] == 1 && g.n[2] == 1);
+    swf_status s = prepare_args<R>(ctx, g, F, fd_host, &A, (form ? bt : tag).c_str(), st);
+    if (s != SWF_OK) return s;
+    state = (size_t)F * 4 * g.N * sizeof(cpx<R>);
+    void *pT = nullptr, *pclk = nullptr;
+    if ((s = buf(tag + ".y", state, &py)) != SWF_OK) return s;
+    if ((s = buf(tag + ".T", state, &pT)) != SWF_OK) return s;
+    for (int i = 0; i < 7; ++i)
+      if ((s = buf(tag + ".k" + std::to_string(i), state, &pk[i])) != SWF_OK) return s;
+    if ((s = buf(tag + ".clock", sizeof(MarchClock), &pclk)) != SWF_OK) return s;
+    clk = (MarchClock*)pclk;
+    cudaError_t e;
+    if (form) {
+      const int nt = g.n[0] + g.n[1] + g.n[2];
+      if ((s = buf(bt + ".ystage", state, &pys)) != SWF_OK) return s;
+      if ((s = buf(bt + ".photon", sizeof(double) * 6 * NP, &pph)) != SWF_OK) return s;
+      if ((s = buf(bt + ".kph", sizeof(cpx<R>) * NP * nt, &pkph)) != SWF_OK) return s;
+      // blocks per instance of the M-dot reduction: about four waves of the GPU in total, at least
+      // 1024 sites per block (the same split for every photon count, so a photon of a scan sums
+      // exactly as a solve of that photon alone); photons per block: 1, or 4 (8 in complex64) for
+      // scans, which then read U and V once per site for the block's photons
+      nph_blk = n_ph == 1 ? 1 : (sizeof(R) == 4 && n_ph > 4 ? 8 : 4);
+      nchunk = (n_ph + nph_blk - 1) / nph_blk;
+      nb = std::max(1, std::min((g.N + 1023) / 1024, (4 * sm_count() + n_inst - 1) / n_inst));
+      if ((s = buf(bt + ".phase_table", sizeof(cpx<double>) * 3 * 7 * (size_t)n_steps * NP, &ptab)) != SWF_OK) return s;
+      if ((s = buf(bt + ".mpart", sizeof(cpx<double>) * 3 * (size_t)nb * NP, &ppart)) != SWF_OK) return s;
+      if ((e = cudaMemcpyAsync(pph, photon_host, sizeof(double) * 6 * NP, cudaMemcpyHostToDevice, st)) != cudaSuccess)
+        return cuda_status(e, "upload photon table");
+      {
+        ProfScope ps(ctx, "k_photon_tables", st);
+        k_photon_tables<R><<<(NP * nt + 127) / 128, 128, 0, st>>>((const double*)pph, g, NP, (cpx<R>*)pkph);
+      }
+      {
+        const long total = (long)NP * n_steps * 7;
+        ProfScope ps(ctx, "k_bw_phase_table", st);
+        k_bw_phase_table<<<(int)std::min((total + 127) / 128, 4096L), 128, 0, st>>>(
+            A.fd, (const double*)pph, NP, n_ph, n_steps, t_out, h, g.dx[0] * g.dx[1] * g.dx[2], form,
+            (cpx<double>*)ptab);
+      }
+      if ((e = cudaMemsetAsync(ppart, 0, sizeof(cpx<double>) * 3 * (size_t)nb * NP, st)) != cudaSuccess)
+        return cuda_status(e, "memset M accumulators");
+    }
+    if ((e = cudaMemsetAsync(py, 0, state, st)) != cudaSuccess) return cuda_status(e, "memset state");
+    A.y = (cpx<R>*)py;
+    A.T = (cpx<R>*)pT;
+    if ((s = state_low_part<R>(ctx, tag + ".ylo", state, &A, st)) != SWF_OK) return s;
+    {
+      // shapes by timing, on the slots before they hold anything (the heaviest stage: six inputs)
+      StageArgs<R> B = A;
+      B.nterm = 6;
+      for (int q = 0; q < 6; ++q) {
+        B.kin[q] = (const cpx<R>*)pk[q + 1];
+        B.coef[q] = 0.0;
+        B.coef_r[q] = (R)0;
+      }
+      B.kout = (cpx<R>*)pk[0];
+      B.t = t_out;
+      if ((s = autotune_eval<R>(ctx, B, F, st)) != SWF_OK) return s;
+    }
+    if (form == 2 && (s = f2_prepare<R>(ctx, g, n_inst, fd_host, photon_host, wave_k_host, &p2, st)) != SWF_OK)
+      return s;
+    k_clock_set<<<1, 1, 0, st>>>(clk, t_out, h);
+    A.clk = clk;
+    return SWF_OK;
+  }
+
+  // k_1 = f(t_out, 0); the integrand of Eq. 17 vanishes at psi_s(t_out) = 0, the partial-integration
+  // integrand does not (its source term is V psi_b): stage value y = 0
+  swf_status first() {
+    A.nterm = 0;
+    A.write_y = 0;
+    A.kout = (cpx<R>*)pk[slot[0]];
+    A.ls = 0;
+    A.c = 0.0;
+    A.ystage = nullptr;
+    set_next_node<R>(&A, 0, 0);
+    swf_status s = chain ? launch_eval_open<R>(ctx, A, F, st) : launch_eval<R>(ctx, A, F, st);
+    open = A;
+    if (s == SWF_OK && form == 2)
+      s = f2_integrand<R>(ctx, A, p2, (const cpx<R>*)py, (const double*)pph, (const cpx<double>*)ptab, 7 * n_steps, 0,
+                          0, st);
     return s;
-  auto step = [&](int ls) -> swf_status {
+  }
+
+  // One step at clock offset ls (stage times from the clock: tn = t_out + n h, t = tn + c_i h).  Stage
+  // values with a quadrature weight: b_{i+1} for i = 2..5 and, for the new state (i = 6), b_1 of the
+  // next step (the phase table holds 0 there on the last step, so every step launches the same kernels).
+  swf_status step(int ls) {
     for (int i = 1; i < 7; ++i) {
-      int ntm = 0;
+      int nt = 0;
       for (int j = 0; j < i; ++j) {
         if (DP_A[i][j] == 0.0) continue;
-        A.kin[ntm] = (const cpx<R>*)pk[slot[j]];
-        A.coef[ntm] = h * DP_A[i][j];
-        ++ntm;
+        A.kin[nt] = (const cpx<R>*)pk[slot[j]];
+        A.coef[nt] = h * DP_A[i][j];
+        A.coef_r[nt] = (R)A.coef[nt];
+        ++nt;
       }
-      A.nterm = ntm;
+      A.nterm = nt;
       A.write_y = (i == 6);
       A.kout = (cpx<R>*)pk[slot[i]];
       A.ls = ls;
       A.c = DP_C[i];
-      // stage values with a quadrature weight: b_{i+1} for i = 2..5 and, for the new state
-      // (i = 6), b_1 of the next step (the phase table holds 0 there on the last step, so every
-      // step launches the same kernels)
-      const bool weighted = i >= 2;
+      set_next_node<R>(&A, ls, i);
+      const bool weighted = form && i >= 2;
       A.ystage = weighted ? (cpx<R>*)pys : nullptr;
       A.yspec = (weighted && form == 2) ? p2.Yspec : nullptr;  // the y or z pass writes F[Y] (if there is one)
       swf_status r = chain ? launch_eval_chain<R>(ctx, open, A, F, st) : launch_eval<R>(ctx, A, F, st);
       if (r != SWF_OK) return r;
       open = A;
-      if (weighted && form == 2) {
+      if (!weighted) continue;
+      if (form == 2) {
         if ((r = f2_integrand<R>(ctx, A, p2, (const cpx<R>*)pys, (const double*)pph, (const cpx<double>*)ptab,
                                  7 * n_steps, ls, i, st)) != SWF_OK)
           return r;
-      } else if (weighted) {
-        ProfScope ps(ctx, "k_mdot", st);
-        const cpx<R>* ysc = (const cpx<R>*)pys;
-        const cpx<R>* kpc = (const cpx<R>*)pkph;
-        const cpx<double>* tb = (const cpx<double>*)ptab;
-        cpx<double>* pa = (cpx<double>*)ppart;
-        const dim3 grid(nb, n_inst * nchunk);
-        if (nph_blk == 1)
-          k_mdot<R, 1><<<grid, 256, 0, st>>>(ysc, A.gcplx, kpc, (const double*)pph, g, tb, clk, ls, i, 7 * n_steps,
-                                             n_ph, pa);
-        else if (nph_blk == 4)
-          k_mdot<R, 4><<<grid, 256, 0, st>>>(ysc, A.gcplx, kpc, (const double*)pph, g, tb, clk, ls, i, 7 * n_steps,
-                                             n_ph, pa);
-        else
-          k_mdot<R, 8><<<grid, 256, 0, st>>>(ysc, A.gcplx, kpc, (const double*)pph, g, tb, clk, ls, i, 7 * n_steps,
-                                             n_ph, pa);
+        continue;
       }
+      ProfScope ps(ctx, "k_mdot", st);
+      auto* kernel = nph_blk == 1 ? k_mdot<R, 1> : nph_blk == 4 ? k_mdot<R, 4> : k_mdot<R, 8>;
+      kernel<<<dim3(nb, n_inst * nchunk), 256, 0, st>>>((const cpx<R>*)pys, A.gcplx, (const cpx<R>*)pkph,
+                                                        (const double*)pph, g, (const cpx<double>*)ptab, clk, ls, i,
+                                                        7 * n_steps, n_ph, (cpx<double>*)ppart);
     }
     std::swap(slot[0], slot[6]);
     return SWF_OK;
-  };
-  s = run_step_pairs(ctx, st, n_steps / 2, clk, [&]() -> swf_status {
-    swf_status r = step(0);
-    return r == SWF_OK ? step(1) : r;
-  });
-  if (s != SWF_OK) return s;
-  if (n_steps % 2 && (s = step(0)) != SWF_OK) return s;
-  if (chain && (s = launch_eval_close<R>(ctx, open, F, st)) != SWF_OK) return s;
-  if (form == 2) {
-    ProfScope ps(ctx, "k_f2_final", st);
-    k_f2_final<<<n_inst, 288, 0, st>>>(p2.sspart, p2.nbs, p2.dpart, p2.nbx, (cpx<double>*)macc);
-  } else {
-    ProfScope ps(ctx, "k_mdot_final", st);
-    k_mdot_final<<<NP, 96, 0, st>>>((const cpx<double>*)ppart, nb, (cpx<double>*)macc);
   }
-  e = cudaMemcpyAsync(psi_out, py, state, cudaMemcpyDeviceToDevice, st);
-  if (e != cudaSuccess) return cuda_status(e, "copy psi(t_in)");
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_status(e, "Breit-Wheeler march kernels");
-  return SWF_OK;
+
+  swf_status pair() {
+    const swf_status r = step(0);
+    return r == SWF_OK ? step(1) : r;
+  }
+  swf_status prepare_pairs() {
+    return n_steps > 1 ? pairs.prepare(ctx, st, clk, [&] { return pair(); }) : SWF_OK;
+  }
+  swf_status launch_pair() {
+    return pairs.launch(ctx, clk, [&] { return pair(); });
+  }
+
+  // The odd step, the open evaluation's end, the integrals and the state.
+  swf_status finish(void* psi_out, double2* macc) {
+    swf_status s = pairs.finish();
+    if (s != SWF_OK) return s;
+    if (n_steps % 2 && (s = step(0)) != SWF_OK) return s;
+    if (chain && (s = launch_eval_close<R>(ctx, open, F, st)) != SWF_OK) return s;
+    if (form == 2) {
+      ProfScope ps(ctx, "k_f2_final", st);
+      k_f2_final<<<n_inst, 288, 0, st>>>(p2.sspart, p2.nbs, p2.dpart, p2.nbx, (cpx<double>*)macc);
+    } else if (form == 1) {
+      ProfScope ps(ctx, "k_mdot_final", st);
+      k_mdot_final<<<NP, 96, 0, st>>>((const cpx<double>*)ppart, nb, (cpx<double>*)macc);
+    }
+    cudaError_t e = cudaMemcpyAsync(psi_out, py, state, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return cuda_status(e, "copy psi(t_in)");
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e, "march kernels");
+    return SWF_OK;
+  }
+
+  // A march that runs alone: everything in order.
+  swf_status run(void* psi_out, double2* macc) {
+    swf_status s = first();
+    if (s == SWF_OK) s = prepare_pairs();
+    for (int p = 0; p < n_steps / 2 && s == SWF_OK; ++p) s = launch_pair();
+    if (s != SWF_OK) {
+      pairs.finish();
+      return s;
+    }
+    return finish(psi_out, macc);
+  }
+};
+
+template <typename R>
+static swf_status march_impl(swf_ctx* ctx, const GridDesc& g, double t_in, double t_out, int n_steps, int F,
+                             const FieldDesc* fd_host, void* psi_out, cudaStream_t st) {
+  MarchPlan<R> P;
+  const swf_status s = P.setup(ctx, "march", g, t_in, t_out, n_steps, F, fd_host, 0, nullptr, nullptr, 1, st);
+  return s == SWF_OK ? P.run(psi_out, nullptr) : s;
+}
+
+template <typename R>
+static swf_status march_bw_impl(swf_ctx* ctx, const GridDesc& g, double t_in, double t_out, int n_steps, int n_inst,
+                                const FieldDesc* fd_host, const double* photon_host, void* psi_out, double2* macc,
+                                cudaStream_t st, int form, const double* wave_k_host, int n_ph) {
+  MarchPlan<R> P;
+  const swf_status s =
+      P.setup(ctx, "march", g, t_in, t_out, n_steps, 2 * n_inst, fd_host, form, photon_host, wave_k_host, n_ph, st);
+  return s == SWF_OK ? P.run(psi_out, macc) : s;
 }
 
 swf_status march_bw(swf_ctx* ctx, const GridDesc& g, double t_in, double t_out, int n_steps, int n_inst,
@@ -2926,6 +2791,7 @@ static swf_status march_bw_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double
     for (int q = 0; q < 6; ++q) {
       B.kin[q] = (const cpx<R>*)pk[q + 1];
       B.coef[q] = 0.0;
+      B.coef_r[q] = (R)0;
     }
     B.write_y = 0;
     B.ystage = nullptr;
@@ -2974,6 +2840,7 @@ static swf_status march_bw_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double
       A.write_y = (i == 6);
       A.kout = (cpx<R>*)pk[i];
       A.c = DP_C[i];
+      set_next_node<R>(&A, 0, i);
       const bool weighted = i >= 2 && i <= 5;  // b_2 = b_7 = 0
       A.ystage = weighted ? (cpx<R>*)pys : nullptr;
       swf_status r = !chain ? launch_eval<R>(ctx, A, F, st)
@@ -3040,428 +2907,62 @@ swf_status march_bw_adaptive(swf_ctx* ctx, const GridDesc& g, double t_in, doubl
 }
 
 // ---------------------------------------------------------------- multi-grid march (batching of uneven grids)
-// Groups of fields on different grids that share one time grid (t_out, t_in, steps) are marched by
-// one launch per pass for all groups: persistent blocks (as many as fit the SMs at once) take work
-// items -- one item is one block of one group's pass -- from a device counter, the largest grids'
-// items first, and run the single-group kernels' per-block code on them.  A group's lines are
-// therefore transformed with exactly the arithmetic of marching that group alone (bitwise the same
-// result); the launch only decides which SM does which block, and the whole multi-grid step pair
-// is one CUDA graph.  The per-group arguments of every evaluation of the step pair sit in device
-// tables, uploaded once before the graph is captured (the slots rotate with period two).
+// Groups of fields on different grids that share one time grid (t_out, t_in, steps) march side by
+// side: each group is a MarchPlan with a workspace and a stream of its own, its step pair one CUDA
+// graph, and the graphs of all groups are replayed in turn, so that small grids fill the SMs together.
+// A group's kernels and shapes are those of marching it alone: bitwise the same result.
 
 constexpr int kMaxMultiGroups = 8;
-constexpr int kMultiCounters = 128;  // work counters of one step pair (one per grouped launch)
 
-struct MultiPlan {
-  int items;                       // work items of the launch
-  int first[kMaxMultiGroups + 1];  // first item of queue position q (largest grids first)
-  int gid[kMaxMultiGroups];        // table index of the group at queue position q
-  int gx[kMaxMultiGroups];         // blocks per field of that group in this pass
-  int shape[kMaxMultiGroups];      // rows per block (x passes) or log2 of the tile width (y, z passes)
-  int ld[kMaxMultiGroups];         // padded line stride
-};
-
-// Breit-Wheeler integrand arguments of one group (one photon per instance).
-template <typename R>
-struct MdotArgs {
-  const cpx<R>* ys;
-  const cpx<R>* gcplx;
-  const cpx<R>* kph;
-  const double* photon;
-  const cpx<double>* ptab;
-  cpx<double>* acc;
-  GridDesc g;
-  int tab_stride;
-  int nb;  // blocks per instance (the split of the single-group march)
-};
-
-// Persistent loop over the work items of a grouped launch: body(args, bx, by, shape, ld) with the
-// item's group arguments copied into shared memory.
-template <typename Args, typename Body>
-__device__ __forceinline__ void multi_loop(const Args* __restrict__ tab, const MultiPlan& P, int* counter,
-                                           Body&& body) {
-  __shared__ __align__(16) Args sA;
-  __shared__ MultiPlan sP;
-  __shared__ int s_item;
-  if (threadIdx.x == 0) sP = P;
-  int cur = -1;
-  for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
-    __syncthreads();
-    const int item = s_item;
-    if (item >= sP.items) break;
-    int q = 0;
-    while (q + 1 < kMaxMultiGroups && item >= sP.first[q + 1]) ++q;
-    if (q != cur) {
-      const int* src = reinterpret_cast<const int*>(tab + sP.gid[q]);
-      int* dst = reinterpret_cast<int*>(&sA);
-      for (int i = threadIdx.x; i < (int)(sizeof(Args) / sizeof(int)); i += blockDim.x) dst[i] = __ldg(src + i);
-      __syncthreads();
-      cur = q;
-    }
-    const int local = item - sP.first[q];
-    body(sA, local % sP.gx[q], local / sP.gx[q], sP.shape[q], sP.ld[q]);
-    __syncthreads();  // shared memory and s_item are reused by the next item
+// Streams of the groups (kept with the context) and their fork and join events.
+static swf_status multi_streams(swf_ctx* ctx, int n) {
+  while ((int)ctx->multi_st.size() < n) {
+    cudaStream_t s = nullptr;
+    cudaEvent_t ev = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess && (e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess)
+      cudaStreamDestroy(s);
+    if (e != cudaSuccess) return cuda_status(e, "multi-grid streams");
+    ctx->multi_st.push_back(s);
+    ctx->multi_ev.push_back(ev);
   }
-}
-
-// The per-group arguments come from shared memory instead of the constant bank, which costs the
-// kernels registers; the bounds keep them at the occupancy of the single-group kernels (a few
-// bytes of spills in complex64, about a hundred in complex128).
-template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_first_multi(const StageArgs<R>* __restrict__ tab, MultiPlan P, int only_x,
-                                                     int* counter) {
-  multi_loop(tab, P, counter, [&](const StageArgs<R>& A, int bx, int f, int rows, int ld) {
-    first_body<R>(A, bx, f, rows, ld, only_x);
-  });
-}
-
-template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_mid_multi(const StageArgs<R>* __restrict__ tab, MultiPlan P, int axis,
-                                                   int do_fwd, int do_h0, int do_inv, int* counter) {
-  multi_loop(tab, P, counter, [&](const StageArgs<R>& A, int bx, int f, int lgtx, int ld) {
-    mid_body<R>(A, bx, f, axis, lgtx, ld, do_fwd, do_h0, do_inv);
-  });
-}
-
-template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_last_multi(const StageArgs<R>* __restrict__ tab, MultiPlan P, int* counter) {
-  multi_loop(tab, P, counter, [&](const StageArgs<R>& A, int bx, int f, int rows, int ld) {
-    last_body<R>(A, bx, f, rows, ld);
-  });
-}
-
-template <typename R>
-__global__ void __launch_bounds__(256) k_mdot_multi(const MdotArgs<R>* __restrict__ tab, MultiPlan P,
-                                                    const MarchClock* clk, int ls, int stage, int* counter) {
-  multi_loop(tab, P, counter, [&](const MdotArgs<R>& M, int bx, int by, int, int) {
-    mdot_body<R, 1>(M.ys, M.gcplx, M.kph, M.photon, M.g, M.ptab, clk, ls, stage, M.tab_stride, 1, M.acc, bx, by,
-                    M.nb);
-  });
-}
-
-template <typename R>
-static swf_status set_multi_attrs() {
-  static std::atomic<bool> done[64];
-  const int dv = dev_slot();
-  if (done[dv].load(std::memory_order_acquire)) return SWF_OK;
-  cudaError_t e;
-  e = cudaFuncSetAttribute(k_first_multi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemTune);
-  if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_first_multi)");
-  e = cudaFuncSetAttribute(k_mid_multi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemTune);
-  if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_mid_multi)");
-  e = cudaFuncSetAttribute(k_last_multi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemTune);
-  if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_last_multi)");
-  done[dv].store(true, std::memory_order_release);
   return SWF_OK;
-}
-
-// Blocks of a persistent grouped launch: as many as can be resident at once (at most one per item).
-template <typename K>
-static int persistent_blocks(K kernel, size_t smem, int items, int threads = kThreads) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess || per_sm < 1) {
-    cudaGetLastError();
-    per_sm = 1;
-  }
-  return std::max(1, std::min(items, per_sm * sm_count()));
-}
-
-// Queue positions of the groups: largest grids first (their items take longest).
-static std::vector<int> multi_order(const std::vector<MultiGroup>& G) {
-  std::vector<int> ord(G.size());
-  for (size_t i = 0; i < G.size(); ++i) ord[i] = (int)i;
-  std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return G[a].g.N > G[b].g.N; });
-  return ord;
-}
-
-static MultiPlan make_plan(const std::vector<int>& ord, const std::vector<int>& gx, const std::vector<int>& per,
-                           const std::vector<int>& shape, const std::vector<int>& ld) {
-  MultiPlan P;
-  std::memset(&P, 0, sizeof(P));
-  int acc = 0;
-  for (int q = 0; q < kMaxMultiGroups; ++q) {
-    P.first[q] = acc;
-    if (q < (int)ord.size()) {
-      const int gi = ord[q];
-      P.gid[q] = gi;
-      P.gx[q] = gx[gi];
-      P.shape[q] = shape[gi];
-      P.ld[q] = ld[gi];
-      acc += gx[gi] * per[gi];
-    }
-  }
-  P.first[kMaxMultiGroups] = acc;
-  P.items = acc;
-  return P;
 }
 
 template <typename R>
 static swf_status march_multi_impl(swf_ctx* ctx, const std::vector<MultiGroup>& G, double t_in, double t_out,
                                    int n_steps, int bw, cudaStream_t st) {
   const int ng = (int)G.size();
-  constexpr int esz = (int)sizeof(cpx<R>);
-  swf_status s = set_multi_attrs<R>();
+  swf_status s = multi_streams(ctx, ng + 1);
   if (s != SWF_OK) return s;
-  const int ny0 = G[0].g.n[1], nz0 = G[0].g.n[2];
-  const bool only_x = (ny0 == 1 && nz0 == 1);
-  std::vector<StageArgs<R>> base(ng);
-  std::vector<void*> pk(7 * (size_t)ng), pys(ng, nullptr), ppart(ng, nullptr);
-  std::vector<MdotArgs<R>> mdot(ng);
-  std::vector<int> nb(ng, 1);
-  const double h = (t_in - t_out) / n_steps;
-  cudaError_t e;
+  std::vector<MarchPlan<R>> P(ng);
+  // tables and tuned shapes on st, one group after another (the tuner times its launches alone)
+  for (int gi = 0; gi < ng && s == SWF_OK; ++gi)
+    s = P[gi].setup(ctx, "mg" + std::to_string(gi), G[gi].g, t_in, t_out, n_steps, G[gi].F, G[gi].fd, bw ? 1 : 0,
+                    G[gi].photon, nullptr, 1, st);
+  if (s != SWF_OK) return s;
+  cudaError_t e = cudaEventRecord(ctx->multi_ev[ng], st);
+  for (int gi = 0; gi < ng && e == cudaSuccess; ++gi) {
+    P[gi].st = ctx->multi_st[gi];
+    e = cudaStreamWaitEvent(P[gi].st, ctx->multi_ev[ng], 0);
+  }
+  if (e != cudaSuccess) return cuda_status(e, "fork the multi-grid streams");
+  for (int gi = 0; gi < ng && s == SWF_OK; ++gi) s = P[gi].first();
+  for (int gi = 0; gi < ng && s == SWF_OK; ++gi) s = P[gi].prepare_pairs();
+  for (int p = 0; p < n_steps / 2 && s == SWF_OK; ++p)
+    for (int gi = 0; gi < ng && s == SWF_OK; ++gi) s = P[gi].launch_pair();
   for (int gi = 0; gi < ng; ++gi) {
-    const MultiGroup& M = G[gi];
-    const GridDesc& g = M.g;
-    const int F = M.F;
-    const std::string tag = "mg" + std::to_string(gi);
-    if ((s = prepare_args<R>(ctx, g, F, M.fd, &base[gi], tag.c_str(), st)) != SWF_OK) return s;
-    const size_t state = (size_t)F * 4 * g.N * esz;
-    void *py = nullptr, *pT = nullptr;
-    if ((s = ws_get(ctx, tag + ".y", state, &py)) != SWF_OK) return s;
-    if ((s = ws_get(ctx, tag + ".T", state, &pT)) != SWF_OK) return s;
-    for (int i = 0; i < 7; ++i)
-      if ((s = ws_get(ctx, tag + ".k" + std::to_string(i), state, &pk[7 * gi + i])) != SWF_OK) return s;
-    if ((e = cudaMemsetAsync(py, 0, state, st)) != cudaSuccess) return cuda_status(e, "memset state");
-    base[gi].y = (cpx<R>*)py;
-    base[gi].T = (cpx<R>*)pT;
-    if ((s = state_low_part<R>(ctx, tag + ".ylo", state, &base[gi], st)) != SWF_OK) return s;
-    if (bw) {
-      const int n_inst = F / 2;
-      const int nt = g.n[0] + g.n[1] + g.n[2];
-      void *pph = nullptr, *pkph = nullptr, *ptab = nullptr;
-      if ((s = ws_get(ctx, tag + ".ystage", state, &pys[gi])) != SWF_OK) return s;
-      if ((s = ws_get(ctx, tag + ".photon", sizeof(double) * 6 * n_inst, &pph)) != SWF_OK) return s;
-      if ((s = ws_get(ctx, tag + ".kph", sizeof(cpx<R>) * n_inst * nt, &pkph)) != SWF_OK) return s;
-      // the same split of the integrand sums as the single-group march of this group
-      nb[gi] = std::max(1, std::min((g.N + 1023) / 1024, (4 * sm_count() + n_inst - 1) / n_inst));
-      if ((s = ws_get(ctx, tag + ".ptab", sizeof(cpx<double>) * 3 * 7 * (size_t)n_steps * n_inst, &ptab)) != SWF_OK)
-        return s;
-      if ((s = ws_get(ctx, tag + ".mpart", sizeof(cpx<double>) * 3 * (size_t)nb[gi] * n_inst, &ppart[gi])) != SWF_OK)
-        return s;
-      if ((e = cudaMemcpyAsync(pph, M.photon, sizeof(double) * 6 * n_inst, cudaMemcpyHostToDevice, st)) != cudaSuccess)
-        return cuda_status(e, "upload photon table");
-      {
-        ProfScope ps(ctx, "k_photon_tables", st);
-        k_photon_tables<R><<<(n_inst * nt + 127) / 128, 128, 0, st>>>((const double*)pph, g, n_inst, (cpx<R>*)pkph);
-      }
-      {
-        const long total = (long)n_inst * n_steps * 7;
-        ProfScope ps(ctx, "k_bw_phase_table", st);
-        k_bw_phase_table<<<(int)std::min((total + 127) / 128, 4096L), 128, 0, st>>>(
-            base[gi].fd, (const double*)pph, n_inst, 1, n_steps, t_out, h, g.dx[0] * g.dx[1] * g.dx[2], 1,
-            (cpx<double>*)ptab);
-      }
-      if ((e = cudaMemsetAsync(ppart[gi], 0, sizeof(cpx<double>) * 3 * (size_t)nb[gi] * n_inst, st)) != cudaSuccess)
-        return cuda_status(e, "memset M accumulators");
-      mdot[gi] = MdotArgs<R>{(const cpx<R>*)pys[gi], base[gi].gcplx, (const cpx<R>*)pkph, (const double*)pph,
-                             (const cpx<double>*)ptab, (cpx<double>*)ppart[gi], g, 7 * n_steps, nb[gi]};
-    }
-    {  // launch shapes of this group by timing (as for a single-group march)
-      StageArgs<R> B = base[gi];
-      B.nterm = 6;
-      for (int q = 0; q < 6; ++q) {
-        B.kin[q] = (const cpx<R>*)pk[7 * gi + q + 1];
-        B.coef[q] = 0.0;
-      }
-      B.write_y = 0;
-      B.ystage = nullptr;
-      B.kout = (cpx<R>*)pk[7 * gi];
-      B.t = t_out;
-      if ((s = autotune_eval<R>(ctx, B, F, st)) != SWF_OK) return s;
-    }
+    if (s == SWF_OK) s = P[gi].finish(G[gi].psi_out, (double2*)G[gi].macc);
+    else P[gi].pairs.finish();
   }
-  // Per-pass plans.  The lead group (the largest grid, first in the queue) keeps its tuned shape
-  // and thread count; it fixes the launch's shared memory per block, and every other group takes
-  // the largest shape that fits that budget (more rows, or wider tiles, for smaller grids), so that
-  // its blocks do not reserve shared memory they leave unused.
-  const std::vector<int> ord = multi_order(G);
-  const int lead = ord[0];
-  std::vector<int> fper(ng), xg(ng), xrows(ng), xld(ng);
-  int xthr = kThreads;
-  size_t xsmem = 0;
-  {
-    const GridDesc& g = G[lead].g;
-    const int nrows = g.n[1] * g.n[2];
-    const int xv = tune_lookup(ctx, tune_key('x', esz, g.n[0], nrows, 0, G[lead].F),
-                               4 * x_rows<R>(g.n[0], nrows, G[lead].F));
-    xthr = (xv & 3) ? kThreads / 2 : kThreads;
-    xsmem = (size_t)2 * 4 * std::max(1, xv >> 2) * padded_len(g.n[0]) * esz;
+  for (int gi = 0; gi < ng; ++gi) {  // st continues after every group (also after an error)
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->multi_ev[gi], P[gi].st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ctx->multi_ev[gi], 0);
   }
-  for (int gi = 0; gi < ng; ++gi) {
-    const GridDesc& g = G[gi].g;
-    fper[gi] = G[gi].F;
-    const int nrows = g.n[1] * g.n[2];
-    xld[gi] = padded_len(g.n[0]);
-    const size_t line = (size_t)2 * 4 * xld[gi] * esz;
-    xrows[gi] = (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>(xsmem / line, 64), nrows));
-    xg[gi] = (nrows + xrows[gi] - 1) / xrows[gi];
-    xsmem = std::max(xsmem, (size_t)xrows[gi] * line);
-  }
-  const MultiPlan px = make_plan(ord, xg, fper, xrows, xld);
-  struct MidPass { int axis, fwd, h0, inv; MultiPlan plan; size_t smem; int blocks, threads; };
-  std::vector<MidPass> mids;
-  if (!only_x) {
-    std::vector<std::array<int, 4>> combos;
-    if (ny0 > 1 && nz0 > 1) combos = {{1, 1, 0, 0}, {2, 1, 1, 1}, {1, 0, 0, 1}};
-    else combos = {{ny0 > 1 ? 1 : 2, 1, 1, 1}};
-    for (const auto& cb : combos) {
-      const int axis = cb[0];
-      auto tuned = [&](int gi) {
-        const GridDesc& g = G[gi].g;
-        const int other = axis == 1 ? g.n[2] : g.n[1];
-        const int lg_h = mid_shape<R>(g.n[axis], g.n[0], (long)other * G[gi].F).lgtx;
-        return tune_lookup(ctx, tune_key('m', esz, axis * 8 + cb[1] * 4 + cb[2] * 2 + cb[3], g.n[axis], g.n[0],
-                                         (long)other * G[gi].F), 4 * lg_h);
-      };
-      const int mv_lead = tuned(lead);
-      const size_t budget = mid_shape_lg<R>(G[lead].g.n[axis], mv_lead >> 2).smem;
-      std::vector<int> mg(ng), lg(ng), ld(ng);
-      size_t sm = 0;
-      for (int gi = 0; gi < ng; ++gi) {
-        const GridDesc& g = G[gi].g;
-        const int other = axis == 1 ? g.n[2] : g.n[1];
-        int l = gi == lead ? (mv_lead >> 2) : mid_max_lg<R>(g.n[axis], g.n[0], budget);
-        const MidShape ms = mid_shape_lg<R>(g.n[axis], l);
-        lg[gi] = ms.lgtx;
-        ld[gi] = ms.ld;
-        mg[gi] = ((g.n[0] + (1 << ms.lgtx) - 1) >> ms.lgtx) * other;
-        sm = std::max(sm, ms.smem);
-      }
-      MidPass mp{axis, cb[1], cb[2], cb[3], make_plan(ord, mg, fper, lg, ld), sm, 0,
-                 (mv_lead & 3) ? kThreads / 2 : kThreads};
-      mp.blocks = persistent_blocks(k_mid_multi<R>, sm, mp.plan.items, mp.threads);
-      mids.push_back(mp);
-    }
-  }
-  const int xfb = persistent_blocks(k_first_multi<R>, xsmem, px.items, xthr);
-  const int xlb = persistent_blocks(k_last_multi<R>, xsmem, px.items, xthr);
-  MultiPlan pd;
-  int dblocks = 0;
-  if (bw) {
-    std::vector<int> ones(ng, 1), zero(ng, 0), ninst(ng);
-    for (int gi = 0; gi < ng; ++gi) ninst[gi] = G[gi].F / 2;
-    pd = make_plan(ord, nb, ninst, zero, zero);
-    dblocks = persistent_blocks(k_mdot_multi<R>, 0, pd.items);
-  }
-  // argument tables of every evaluation of a step pair: entry 0 the first evaluation k_1 = f(t_out, 0),
-  // then (ls, stage) for ls = 0, 1 and stages 1..6, with the slot rotation of the single-group march
-  const int n_ev = 1 + 12;
-  std::vector<StageArgs<R>> tab((size_t)n_ev * ng);
-  std::vector<std::array<int, 7>> slot(ng);
-  for (int gi = 0; gi < ng; ++gi) {
-    for (int i = 0; i < 7; ++i) slot[gi][i] = i;
-    StageArgs<R> A = base[gi];
-    A.nterm = 0;
-    A.write_y = 0;
-    A.kout = (cpx<R>*)pk[7 * gi + slot[gi][0]];
-    A.ls = 0;
-    A.c = 0.0;
-    A.ystage = nullptr;
-    A.t = t_out;
-    tab[gi] = A;
-  }
-  void* pclk = nullptr;
-  if ((s = ws_get(ctx, "mg.clock", sizeof(MarchClock), &pclk)) != SWF_OK) return s;
-  MarchClock* clk = (MarchClock*)pclk;
-  for (int ls = 0; ls < 2; ++ls) {
-    for (int i = 1; i < 7; ++i) {
-      for (int gi = 0; gi < ng; ++gi) {
-        StageArgs<R> A = base[gi];
-        int nt = 0;
-        for (int j = 0; j < i; ++j) {
-          if (DP_A[i][j] == 0.0) continue;
-          A.kin[nt] = (const cpx<R>*)pk[7 * gi + slot[gi][j]];
-          A.coef[nt] = h * DP_A[i][j];
-          ++nt;
-        }
-        A.nterm = nt;
-        A.write_y = (i == 6);
-        A.kout = (cpx<R>*)pk[7 * gi + slot[gi][i]];
-        A.ls = ls;
-        A.c = DP_C[i];
-        A.clk = clk;
-        A.ystage = (bw && i >= 2) ? (cpx<R>*)pys[gi] : nullptr;
-        tab[(size_t)(1 + 6 * ls + (i - 1)) * ng + gi] = A;
-      }
-    }
-    for (int gi = 0; gi < ng; ++gi) std::swap(slot[gi][0], slot[gi][6]);
-  }
-  void *ptabs = nullptr, *pmd = nullptr, *pcnt = nullptr;
-  if ((s = ws_get(ctx, "mg.tables", sizeof(StageArgs<R>) * tab.size(), &ptabs)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "mg.counters", sizeof(int) * kMultiCounters, &pcnt)) != SWF_OK) return s;
-  if ((e = cudaMemcpyAsync(ptabs, tab.data(), sizeof(StageArgs<R>) * tab.size(), cudaMemcpyHostToDevice, st)) !=
-      cudaSuccess)
-    return cuda_status(e, "upload multi-grid tables");
-  if (bw) {
-    if ((s = ws_get(ctx, "mg.mdot", sizeof(MdotArgs<R>) * ng, &pmd)) != SWF_OK) return s;
-    if ((e = cudaMemcpyAsync(pmd, mdot.data(), sizeof(MdotArgs<R>) * ng, cudaMemcpyHostToDevice, st)) != cudaSuccess)
-      return cuda_status(e, "upload multi-grid integrand table");
-  }
-  const StageArgs<R>* dtab = (const StageArgs<R>*)ptabs;
-  int* cnt = (int*)pcnt;
-  int ci = 0;  // next counter of the recorded sequence
-  auto eval = [&](int ev) {
-    const StageArgs<R>* t = dtab + (size_t)ev * ng;
-    {
-      ProfScope ps(ctx, "k_first_multi", st);
-      k_first_multi<R><<<xfb, xthr, xsmem, st>>>(t, px, only_x ? 1 : 0, cnt + ci++);
-    }
-    if (only_x) return;
-    for (const MidPass& mp : mids) {
-      ProfScope ps(ctx, "k_mid_multi", st);
-      k_mid_multi<R><<<mp.blocks, mp.threads, mp.smem, st>>>(t, mp.plan, mp.axis, mp.fwd, mp.h0, mp.inv, cnt + ci++);
-    }
-    ProfScope ps(ctx, "k_last_multi", st);
-    k_last_multi<R><<<xlb, xthr, xsmem, st>>>(t, px, cnt + ci++);
-  };
-  auto step = [&](int ls) {
-    for (int i = 1; i < 7; ++i) {
-      eval(1 + 6 * ls + (i - 1));
-      if (bw && i >= 2) {
-        ProfScope ps(ctx, "k_mdot_multi", st);
-        k_mdot_multi<R><<<dblocks, kThreads, 0, st>>>((const MdotArgs<R>*)pmd, pd, clk, ls, i, cnt + ci++);
-      }
-    }
-  };
-  // work counters used per step pair: every stage's passes, and the integrand at stages 2..6
-  const int per_eval = only_x ? 1 : 2 + (int)mids.size();
-  const int per_pair = 2 * (6 * per_eval + (bw ? 5 : 0));
-  if (per_pair > kMultiCounters) {
-    set_error("multi-grid march: too many launches per step pair");
-    return SWF_EUNSUPPORTED;
-  }
-  k_clock_set<<<1, 1, 0, st>>>(clk, t_out, h);
-  if ((e = cudaMemsetAsync(cnt, 0, sizeof(int) * kMultiCounters, st)) != cudaSuccess) return cuda_status(e, "reset work queues");
-  ci = 0;
-  eval(0);  // k_1 = f(t_out, 0) (the integrand of Eq. 17 vanishes at psi_s(t_out) = 0)
-  auto pair = [&]() -> swf_status {
-    cudaError_t r = cudaMemsetAsync(cnt, 0, sizeof(int) * kMultiCounters, st);
-    if (r != cudaSuccess) return cuda_status(r, "reset work queues");
-    ci = 0;
-    step(0);
-    step(1);
-    return SWF_OK;
-  };
-  if ((s = run_step_pairs(ctx, st, n_steps / 2, clk, pair)) != SWF_OK) return s;
-  if (n_steps % 2) {
-    if ((e = cudaMemsetAsync(cnt, 0, sizeof(int) * kMultiCounters, st)) != cudaSuccess) return cuda_status(e, "reset work queues");
-    ci = 0;
-    step(0);
-  }
-  for (int gi = 0; gi < ng; ++gi) {
-    const size_t state = (size_t)G[gi].F * 4 * G[gi].g.N * esz;
-    if (bw) {
-      ProfScope ps(ctx, "k_mdot_final", st);
-      k_mdot_final<<<G[gi].F / 2, 96, 0, st>>>((const cpx<double>*)ppart[gi], nb[gi], (cpx<double>*)G[gi].macc);
-    }
-    if ((e = cudaMemcpyAsync(G[gi].psi_out, base[gi].y, state, cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
-      return cuda_status(e, "copy psi(t_in)");
-  }
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e, "multi-grid march kernels");
-  // the host tables above are the sources of asynchronous uploads
-  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_status(e, "multi-grid march");
+  if (s != SWF_OK) return s;
+  // the host tables of the set-up are the sources of asynchronous uploads
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return cuda_status(e, "multi-grid march");
   ctx->multi_marches += 1;
   return SWF_OK;
 }
@@ -3482,8 +2983,11 @@ swf_status march_multi(swf_ctx* ctx, const std::vector<MultiGroup>& groups, doub
       return SWF_EINVAL;
     }
   }
-  if (prec == SWF_C64) return march_multi_impl<float>(ctx, groups, t_in, t_out, n_steps, bw, st);
-  return march_multi_impl<double>(ctx, groups, t_in, t_out, n_steps, bw, st);
+  ctx->in_multi = true;  // its kernels are timed under names of their own
+  const swf_status s = prec == SWF_C64 ? march_multi_impl<float>(ctx, groups, t_in, t_out, n_steps, bw, st)
+                                       : march_multi_impl<double>(ctx, groups, t_in, t_out, n_steps, bw, st);
+  ctx->in_multi = false;
+  return s;
 }
 
 // Plain marches of several groups (the spin reuse of march_fields within each group).
