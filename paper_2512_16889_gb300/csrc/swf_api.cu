@@ -1,5 +1,6 @@
 // C ABI of the SWF solver: context, validation, workspace and the orchestration of
 // march -> projections -> per-instance results (Sec. II Eqs. 6-9, Sec. IV).
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -233,43 +234,79 @@ struct InstDev {
   double Ku[3];  // trivial-axis momentum of the electron wave
 };
 
-// One block per instance: C, A, B, D and both lines of Eq. 8 (B and D as sums over the grid
-// modes with the energy projectors, sum_s' u u^+ = P_+ and sum_s' v v^+ = P_-).
-__global__ void __launch_bounds__(256) k_finalize(const InstDev* id, GridDesc g, double t_in,
-                                                  const cpx<double>* specU, const cpx<double>* specV,
-                                                  const cpx<double>* uq, const cpx<double>* vp,
-                                                  const double* normU, const double* normV,
-                                                  swf_result* res) {
+// B and D of the full pair number as sums over the grid modes with the energy projectors (sum_s' u u^+
+// = P_+, sum_s' v v^+ = P_-), U^+ P_+- V = (U^+V +- U^+ H0 V / E)/2: block (b, f) leaves its part of
+// instance f's two sums in part[f][b].  A block per instance took 0.58 ms for one 128 x 128 instance
+// (FP64 on one SM), of a 24 ms solve; spread over the SMs it no longer shows.
+__global__ void __launch_bounds__(256) k_pair_modes(const InstDev* id, GridDesc g, const cpx<double>* __restrict__ specU,
+                                                    const cpx<double>* __restrict__ specV, cpx<double>* part) {
   __shared__ cpx<double> red[8][2];
+  const int f = blockIdx.y;
+  const InstDev& I = id[f];
+  const cpx<double>* u = specU + (size_t)f * 4 * g.N;
+  const cpx<double>* v = specV + (size_t)f * 4 * g.N;
+  double dk[3];
+  for (int a = 0; a < 3; ++a) dk[a] = g.n[a] > 1 ? 6.283185307179586476925286766559 / g.L[a] : 0.0;
+  cpx<double> accB = mk<double>(0, 0), accD = mk<double>(0, 0);
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < g.N; j += gridDim.x * blockDim.x) {
+    const int iy0 = j / g.n[0];
+    const int jj[3] = {j - iy0 * g.n[0], iy0 % g.n[1], iy0 / g.n[1]};
+    double k[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      k[a] = g.n[a] > 1 ? (jj[a] < (g.n[a] + 1) / 2 ? jj[a] : jj[a] - g.n[a]) * dk[a] : I.Ku[a];
+    const double kx = k[0], ky = k[1], kz = k[2];
+    const double ie = rsqrt(1.0 + kx * kx + ky * ky + kz * kz);
+    cpx<double> uv[4], a[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      uv[c] = u[(size_t)c * g.N + j];
+      a[c] = v[(size_t)c * g.N + j];
+    }
+    // hv = H0(kappa) a
+    const cpx<double> hv[4] = {a[0] + kz * a[2] + kx * a[3] + ky * mul_mi(a[3]),
+                               a[1] + kx * a[2] + ky * mul_i(a[2]) - kz * a[3],
+                               kz * a[0] + kx * a[1] + ky * mul_mi(a[1]) - a[2],
+                               kx * a[0] + ky * mul_i(a[0]) - kz * a[1] - a[3]};
+    cpx<double> s = mk<double>(0, 0), t = mk<double>(0, 0);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      s = s + cdot(uv[c], a[c]);
+      t = t + cdot(uv[c], hv[c]);
+    }
+    accB = accB + 0.5 * (s + ie * t);
+    accD = accD + 0.5 * (s - ie * t);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    accB.x += __shfl_down_sync(0xffffffffu, accB.x, off);
+    accB.y += __shfl_down_sync(0xffffffffu, accB.y, off);
+    accD.x += __shfl_down_sync(0xffffffffu, accD.x, off);
+    accD.y += __shfl_down_sync(0xffffffffu, accD.y, off);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5][0] = accB;
+    red[threadIdx.x >> 5][1] = accD;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    cpx<double> s = mk<double>(0, 0);
+    for (int w = 0; w < 8; ++w) s = s + red[w][threadIdx.x];
+    part[((size_t)f * gridDim.x + blockIdx.x) * 2 + threadIdx.x] = s;
+  }
+}
+
+// One warp per instance: B and D from their parts (in a fixed order), C, A and both lines of Eq. 8.
+__global__ void __launch_bounds__(32) k_finalize(const InstDev* id, GridDesc g, double t_in, const cpx<double>* part,
+                                                 int nb, const cpx<double>* uq, const cpx<double>* vp,
+                                                 const double* normU, const double* normV, swf_result* res) {
   const int f = blockIdx.x;
   const InstDev& I = id[f];
   cpx<double> accB = mk<double>(0, 0), accD = mk<double>(0, 0);
   if (I.full) {
-    const cpx<double>* u = specU + (size_t)f * 4 * g.N;
-    const cpx<double>* v = specV + (size_t)f * 4 * g.N;
-    for (int j = threadIdx.x; j < g.N; j += blockDim.x) {
-      const int ix = j % g.n[0];
-      const int iy = (j / g.n[0]) % g.n[1];
-      const int iz = j / (g.n[0] * g.n[1]);
-      const double kx = g.n[0] > 1 ? mode_kappa(ix, g.n[0], g.L[0]) : I.Ku[0];
-      const double ky = g.n[1] > 1 ? mode_kappa(iy, g.n[1], g.L[1]) : I.Ku[1];
-      const double kz = g.n[2] > 1 ? mode_kappa(iz, g.n[2], g.L[2]) : I.Ku[2];
-      const double E = sqrt(1.0 + kx * kx + ky * ky + kz * kz);
-      cpx<double> uv[4], vv[4], hv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) { uv[a] = u[(size_t)a * g.N + j]; vv[a] = v[(size_t)a * g.N + j]; }
-      // hv = H0(kappa) vv
-      const cpx<double> a0 = vv[0], a1 = vv[1], a2 = vv[2], a3 = vv[3];
-      hv[0] = a0 + kz * a2 + kx * a3 + ky * mul_mi(a3);
-      hv[1] = a1 + kx * a2 + ky * mul_i(a2) - kz * a3;
-      hv[2] = kz * a0 + kx * a1 + ky * mul_mi(a1) - a2;
-      hv[3] = kx * a0 + ky * mul_i(a0) - kz * a1 - a3;
-      cpx<double> uv_v = mk<double>(0, 0), uv_hv = mk<double>(0, 0);
-#pragma unroll
-      for (int a = 0; a < 4; ++a) { uv_v = uv_v + cdot(uv[a], vv[a]); uv_hv = uv_hv + cdot(uv[a], hv[a]); }
-      // U^+ P_+- V = (U^+V +- U^+ H0 V / E)/2
-      accB = accB + 0.5 * (uv_v + (1.0 / E) * uv_hv);
-      accD = accD + 0.5 * (uv_v - (1.0 / E) * uv_hv);
+    for (int b = threadIdx.x; b < nb; b += 32) {
+      accB = accB + part[((size_t)f * nb + b) * 2];
+      accD = accD + part[((size_t)f * nb + b) * 2 + 1];
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -278,18 +315,15 @@ __global__ void __launch_bounds__(256) k_finalize(const InstDev* id, GridDesc g,
       accD.x += __shfl_down_sync(0xffffffffu, accD.x, off);
       accD.y += __shfl_down_sync(0xffffffffu, accD.y, off);
     }
-    if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = accB; red[threadIdx.x >> 5][1] = accD; }
   }
-  __syncthreads();
   if (threadIdx.x != 0) return;
   double vol = 1.0;
   for (int a = 0; a < 3; ++a)
     if (g.n[a] > 1) vol *= g.L[a];
   cpx<double> B = mk<double>(0, 0), D = mk<double>(0, 0);
   if (I.full) {
-    for (int w = 0; w < 8; ++w) { B = B + red[w][0]; D = D + red[w][1]; }
-    B = (1.0 / vol) * B;
-    D = (1.0 / vol) * D;
+    B = (1.0 / vol) * accB;
+    D = (1.0 / vol) * accD;
   }
   // C = (U_scat | V_back(r, q)) = exp(i q0 t_in) conj(U~(-q)) . v_r(q)
   double sp[8];
@@ -517,10 +551,18 @@ static swf_status solve_schwinger(swf_ctx* ctx, int n_inst, const swf_instance* 
     }
     cudaError_t e = cudaMemcpyAsync(pid, idv.data(), sizeof(InstDev) * F, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_status(e, "upload instance table");
+    void* part = nullptr;
+    const int nb = std::max(1, std::min(1024, (g.N + 1023) / 1024));
+    if (full) {
+      if ((s = ws_get(ctx, "solve.mode_part", sizeof(cpx<double>) * 2 * (size_t)nb * F, &part)) != SWF_OK) return s;
+      ProfScope pm(ctx, "k_pair_modes", st);
+      k_pair_modes<<<dim3(nb, F), 256, 0, st>>>((const InstDev*)pid, g, (const cpx<double>*)specU,
+                                                (const cpx<double>*)specV, (cpx<double>*)part);
+    }
     ProfScope ps(ctx, "finalize", st);
-    k_finalize<<<F, 256, 0, st>>>((const InstDev*)pid, g, i0.grid.t_in, (const cpx<double>*)specU,
-                                  (const cpx<double>*)specV, (const cpx<double>*)uq, (const cpx<double>*)vp,
-                                  (const double*)normU, (const double*)normV, results_dev);
+    k_finalize<<<F, 32, 0, st>>>((const InstDev*)pid, g, i0.grid.t_in, (const cpx<double>*)part, nb,
+                                 (const cpx<double>*)uq, (const cpx<double>*)vp, (const double*)normU,
+                                 (const double*)normV, results_dev);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_status(e, "finalize kernel");
     // the host-side tables above must outlive the asynchronous uploads
@@ -755,8 +797,8 @@ static swf_status bw_photon_scan(swf_ctx* ctx, const swf_instance& in, int n, co
                     (double2*)macc, st, 1, nullptr, n)) != SWF_OK)
     return s;
   if ((s = transform_fields(ctx, g, 2, prec, psi, (double2*)spec, st)) != SWF_OK) return s;
-  for (int j = 0; j < n; ++j)
-    if ((s = transform_at(ctx, g, 2, prec, psi, kat.data() + 6 * j, (double2*)tat + 8 * j, st)) != SWF_OK) return s;
+  // U~(k_j - q) and V~(p - k_j) of every photon in one launch
+  if ((s = transform_at(ctx, g, 2 * n, prec, psi, kat.data(), (double2*)tat, st, 2)) != SWF_OK) return s;
   if ((s = field_norms(ctx, g, 2, prec, psi, (double*)norms, st)) != SWF_OK) return s;
   if ((s = bw_finalize(ctx, g, n, bw.data(), in.grid.t_in, (const double2*)spec, (const double2*)tat,
                        (const double2*)macc, (const double*)norms, (swf_result*)res, st)) != SWF_OK)

@@ -2,6 +2,8 @@
 // with the energy projectors of Eq. 23, added to the finite-time terms integrated during the march
 // (Eqs. 17, 34-35); or the three terms of the partial-integration form (Eqs. 30-33) from the
 // accumulators of that march.
+#include <algorithm>
+
 #include "swf_internal.h"
 
 namespace swf {
@@ -49,65 +51,84 @@ struct BwInst {
   double Ku[3], Kv[3];
 };
 
-// One block per amplitude i (an instance, or one photon of a photon scan).  With c = bi[i].src:
-// U~ = spec[2c], V~ = spec[2c+1] (continuum-normalised transforms at t_in); tat[2i] = U~(k - q)
-// and tat[2i+1] = V~(p - k) by direct sums; macc = M(t_in) of the appended integral; norms[2c],
-// norms[2c+1] = ||U_scat||^2, ||V_scat||^2.
-__global__ void __launch_bounds__(256) k_bw_finalize(const BwInst* bi, GridDesc g, double t_in,
-                                                     const cpx<double>* spec, const cpx<double>* tat,
-                                                     const cpx<double>* macc, const double* norms,
-                                                     swf_result* res) {
+// (P_+ v, P_- v) of both waves of a mode pair: o = P_+(kappa) v, with E(kappa) for the caller.
+__device__ __forceinline__ double split_d(const double* k, const cpx<double>* v, cpx<double>* o) {
+  cpx<double> hv[4];
+  h0_d(k, v, hv);
+  const double e2 = 1.0 + k[0] * k[0] + k[1] * k[1] + k[2] * k[2];
+  const double ie = rsqrt(e2);
+  const double hh = 0.5 * ie;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) o[a] = mk<double>(0.5 * v[a].x + hh * hv[a].x, 0.5 * v[a].y + hh * hv[a].y);
+  return e2 * ie;
+}
+
+__device__ __forceinline__ cpx<double> form_d(const cpx<double>* x, const cpx<double>* y) {  // x^+ y
+  cpx<double> d = cdot(x[0], y[0]);
+#pragma unroll
+  for (int a = 1; a < 4; ++a)
+    d = mk<double>(d.x + x[a].x * y[a].x + x[a].y * y[a].y, d.y + x[a].x * y[a].y - x[a].y * y[a].x);
+  return d;
+}
+
+// The (scat, scat) past term's sum over U modes kappa with V at kappa - k (periodic), both energy signs
+// each: block (b, i) leaves its part of amplitude i's sum in part[i][b].  FP64 operations bound it
+// (about 280 per mode: the two splits, four products, four reciprocals), so the modes of one amplitude
+// are spread over many blocks: 32 pairs on 192^2 to 384^2 take under 2 ms, 43 ms
+// with a block per amplitude; 64 photons on one 192^2 pair 1.3 ms instead of 4.5 ms.
+// The split depends on the grid alone: a photon of a scan sums as a solve of that photon alone.
+__global__ void __launch_bounds__(256) k_bw_modes(const BwInst* bi, GridDesc g, const cpx<double>* __restrict__ spec,
+                                                  cpx<double>* part) {
   __shared__ cpx<double> red[8];
-  const int inst = blockIdx.x;
+  const int inst = blockIdx.y;
   const BwInst& I = bi[inst];
   const double k0 = sqrt(I.k[0] * I.k[0] + I.k[1] * I.k[1] + I.k[2] * I.k[2]);
+  const double eps[3] = {I.eps[0], I.eps[1], I.eps[2]};
+  double dk[3];  // mode spacing (trivial axes: 0, the fixed momentum is added)
+  for (int a = 0; a < 3; ++a) dk[a] = g.n[a] > 1 ? 6.283185307179586476925286766559 / g.L[a] : 0.0;
   const cpx<double>* su = spec + (size_t)(2 * I.src) * 4 * g.N;
   const cpx<double>* sv = spec + (size_t)(2 * I.src + 1) * 4 * g.N;
-  // scat, scat: sum over U modes kappa, V mode kappa - k (periodic), both energy signs each
   cpx<double> acc = mk<double>(0, 0);
-  for (int j = threadIdx.x; j < g.N; j += blockDim.x) {
-    const int ix = j % g.n[0];
-    const int iy = (j / g.n[0]) % g.n[1];
-    const int iz = j / (g.n[0] * g.n[1]);
-    const int id[3] = {ix, iy, iz};
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < g.N; j += gridDim.x * blockDim.x) {
+    const int iy0 = j / g.n[0];
+    const int id[3] = {j - iy0 * g.n[0], iy0 % g.n[1], iy0 / g.n[1]};
     double ku[3], kv[3];
-    int jv[3];
+    int jv[3], odd = 0;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-      jv[a] = ((id[a] - I.shift[a]) % g.n[a] + g.n[a]) % g.n[a];
-      ku[a] = g.n[a] > 1 ? mode_kappa(id[a], g.n[a], g.L[a]) : I.Ku[a];
-      kv[a] = g.n[a] > 1 ? mode_kappa(jv[a], g.n[a], g.L[a]) : I.Kv[a];
+      const int n = g.n[a];
+      jv[a] = (id[a] - I.shift[a]) % n;
+      if (jv[a] < 0) jv[a] += n;
+      const int fu = id[a] < (n + 1) / 2 ? id[a] : id[a] - n;
+      const int fv = jv[a] < (n + 1) / 2 ? jv[a] : jv[a] - n;
+      ku[a] = n > 1 ? fu * dk[a] : I.Ku[a];
+      kv[a] = n > 1 ? fv * dk[a] : I.Kv[a];
+      // the grid sum of the pair's plane waves, N e^{i(kappa_v + k - kappa_u).x0}: -1 for a V mode
+      // that wrapped around an odd axis length (an odd number of times), 1 otherwise
+      if (n > 1 && (n & 1)) odd ^= ((fu - fv - I.shift[a]) / n) & 1;
     }
     const int j2 = (jv[2] * g.n[1] + jv[1]) * g.n[0] + jv[0];
-    // the grid sum of the pair's plane waves, N e^{i(kappa_v + k - kappa_u).x0}: -1 for a V mode
-    // that wrapped around an odd axis length (an odd number of times), 1 otherwise
-    int odd = 0;
-    for (int a = 0; a < 3; ++a) {
-      if (g.n[a] > 1 && (g.n[a] & 1)) {
-        const long fu = id[a] < (g.n[a] + 1) / 2 ? id[a] : id[a] - g.n[a];
-        const long fv = jv[a] < (g.n[a] + 1) / 2 ? jv[a] : jv[a] - g.n[a];
-        odd ^= (int)(((fu - fv - I.shift[a]) / g.n[a]) & 1);
-      }
-    }
-    const double wrap = odd ? -1.0 : 1.0;
-    cpx<double> u[4], v[4];
+    cpx<double> u[4], v[4], up[4], vp[4], av[4], avp[4];
+#pragma unroll
     for (int a = 0; a < 4; ++a) {
       u[a] = su[(size_t)a * g.N + j];
       v[a] = sv[(size_t)a * g.N + j2];
     }
-    const double Eu = sqrt(1.0 + ku[0] * ku[0] + ku[1] * ku[1] + ku[2] * ku[2]);
-    const double Ev = sqrt(1.0 + kv[0] * kv[0] + kv[1] * kv[1] + kv[2] * kv[2]);
-    for (int sg = -1; sg <= 1; sg += 2) {
-      cpx<double> pu[4];
-      proj_d(ku, sg, u, pu);
-      for (int sgp = -1; sgp <= 1; sgp += 2) {
-        cpx<double> pv[4], apv[4];
-        proj_d(kv, sgp, v, pv);
-        alpha_eps_d(I.eps, pv, apv);
-        cpx<double> d = mk<double>(0, 0);
-        for (int a = 0; a < 4; ++a) d = d + cdot(pu[a], apv[a]);
-        acc = acc + div_i(wrap * d, sg * Eu - sgp * Ev - k0);
-      }
+    const double Eu = split_d(ku, u, up), Ev = split_d(kv, v, vp);
+    alpha_eps_d(eps, v, av);
+    alpha_eps_d(eps, vp, avp);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      u[a] = u[a] - up[a];     // P_- u
+      av[a] = av[a] - avp[a];  // (alpha.eps) P_- v
     }
+    // sum over signs of (P u)^+ (alpha.eps) (P v) / Omega, Omega = sigma E_u - sigma' E_v - k0
+    const double sum = Eu + Ev, dif = Eu - Ev;
+    const double w0 = 1.0 / (dif - k0), w1 = 1.0 / (sum - k0), w2 = -1.0 / (sum + k0), w3 = -1.0 / (dif + k0);
+    const cpx<double> d0 = form_d(up, avp), d1 = form_d(up, av), d2 = form_d(u, avp), d3 = form_d(u, av);
+    const cpx<double> t = mk<double>(w0 * d0.x + w1 * d1.x + w2 * d2.x + w3 * d3.x,
+                                     w0 * d0.y + w1 * d1.y + w2 * d2.y + w3 * d3.y);
+    acc = odd ? acc - t : acc + t;
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -119,6 +140,27 @@ __global__ void __launch_bounds__(256) k_bw_finalize(const BwInst* bi, GridDesc 
   if (threadIdx.x != 0) return;
   cpx<double> ss = mk<double>(0, 0);
   for (int w = 0; w < 8; ++w) ss = ss + red[w];
+  part[(size_t)inst * gridDim.x + blockIdx.x] = div_i(ss, 1.0);
+}
+
+// One warp per amplitude i (an instance, or one photon of a photon scan): the mode sum's parts (in a
+// fixed order), the other past terms and the totals.  With c = bi[i].src: tat[2i] = U~(k - q) and
+// tat[2i+1] = V~(p - k) by direct sums; macc = M(t_in) of the appended integral; norms[2c],
+// norms[2c+1] = ||U_scat||^2, ||V_scat||^2.
+__global__ void __launch_bounds__(32) k_bw_finalize(const BwInst* bi, GridDesc g, double t_in,
+                                                    const cpx<double>* part, int nb, const cpx<double>* tat,
+                                                    const cpx<double>* macc, const double* norms, swf_result* res) {
+  const int inst = blockIdx.x;
+  const BwInst& I = bi[inst];
+  const double k0 = sqrt(I.k[0] * I.k[0] + I.k[1] * I.k[1] + I.k[2] * I.k[2]);
+  cpx<double> ss = mk<double>(0, 0);
+  for (int b = threadIdx.x; b < nb; b += 32) ss = ss + part[(size_t)inst * nb + b];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    ss.x += __shfl_down_sync(0xffffffffu, ss.x, off);
+    ss.y += __shfl_down_sync(0xffffffffu, ss.y, off);
+  }
+  if (threadIdx.x != 0) return;
   double vol = 1.0;
   for (int a = 0; a < 3; ++a)
     if (g.n[a] > 1) vol *= g.L[a];
@@ -183,10 +225,18 @@ swf_status bw_finalize(swf_ctx* ctx, const GridDesc& g, int n_inst, const void* 
   if (s != SWF_OK) return s;
   cudaError_t e = cudaMemcpyAsync(pb, bw_host, sizeof(BwInst) * n_inst, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_status(e, "upload Breit-Wheeler table");
+  // four modes per thread, at most 1024 blocks per amplitude
+  const int nb = std::max(1, std::min(1024, (g.N + 1023) / 1024));
+  void* pp;
+  if ((s = ws_get(ctx, "bw.mode_part", sizeof(cpx<double>) * (size_t)nb * n_inst, &pp)) != SWF_OK) return s;
+  {
+    ProfScope ps(ctx, "k_bw_modes", st);
+    k_bw_modes<<<dim3(nb, n_inst), 256, 0, st>>>((const BwInst*)pb, g, (const cpx<double>*)spec, (cpx<double>*)pp);
+  }
   {
     ProfScope ps(ctx, "k_bw_finalize", st);
-    k_bw_finalize<<<n_inst, 256, 0, st>>>((const BwInst*)pb, g, t_in, (const cpx<double>*)spec,
-                                          (const cpx<double>*)tat, (const cpx<double>*)macc, norms, results);
+    k_bw_finalize<<<n_inst, 32, 0, st>>>((const BwInst*)pb, g, t_in, (const cpx<double>*)pp, nb,
+                                         (const cpx<double>*)tat, (const cpx<double>*)macc, norms, results);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e, "Breit-Wheeler finalize");
@@ -283,16 +333,19 @@ swf_status bw_finalize_partial(swf_ctx* ctx, const GridDesc& g, int n_inst, cons
 }
 
 // Photon wave packet sampled on grid momenta (Sec. IV, closing paragraphs): by linearity in the
-// photon wave function its amplitude is sum_j w_j M(k_j, eps_j).  One thread adds the n amplitudes
-// (per term and in total) in order.
-__global__ void k_bw_packet(const swf_result* res, int n, const double* w, cpx<double>* out) {
-  if (threadIdx.x != 0) return;
-  cpx<double> acc[4] = {mk<double>(0, 0), mk<double>(0, 0), mk<double>(0, 0), mk<double>(0, 0)};
-  for (int j = 0; j < n; ++j) {
-    const cpx<double> wj = mk<double>(w[2 * j], w[2 * j + 1]);
-    for (int c = 0; c < 4; ++c) acc[c] = acc[c] + wj * mk<double>(res[j].amp[2 * c], res[j].amp[2 * c + 1]);
+// photon wave function its amplitude is sum_j w_j M(k_j, eps_j).  Warp c adds the n amplitudes of term
+// c (the three terms and M): lane l takes j = l, l + 32, .., then a fixed tree.
+__global__ void __launch_bounds__(128) k_bw_packet(const swf_result* res, int n, const double* w, cpx<double>* out) {
+  const int c = threadIdx.x >> 5;
+  cpx<double> acc = mk<double>(0, 0);
+  for (int j = threadIdx.x & 31; j < n; j += 32)
+    acc = acc + mk<double>(w[2 * j], w[2 * j + 1]) * mk<double>(res[j].amp[2 * c], res[j].amp[2 * c + 1]);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    acc.x += __shfl_down_sync(0xffffffffu, acc.x, off);
+    acc.y += __shfl_down_sync(0xffffffffu, acc.y, off);
   }
-  for (int c = 0; c < 4; ++c) out[c] = acc[c];
+  if ((threadIdx.x & 31) == 0) out[c] = acc;
 }
 
 swf_status bw_packet(swf_ctx* ctx, int n, const swf_result* results, const double* weights_host, double2* out,
@@ -304,7 +357,7 @@ swf_status bw_packet(swf_ctx* ctx, int n, const swf_result* results, const doubl
   if (e != cudaSuccess) return cuda_status(e, "upload packet weights");
   {
     ProfScope ps(ctx, "k_bw_packet", st);
-    k_bw_packet<<<1, 32, 0, st>>>(results, n, (const double*)pw, (cpx<double>*)out);
+    k_bw_packet<<<1, 128, 0, st>>>(results, n, (const double*)pw, (cpx<double>*)out);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e, "photon packet sum");

@@ -259,10 +259,10 @@ swf_status transform_fields(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precis
 swf_status c_spectrum(swf_ctx* ctx, const GridDesc& g, int n_f, const FieldDesc* fd_host,
                       double t_in, const double2* spec, double2* c_out, double* prob,
                       cudaStream_t st);
-// Direct FP64 transform of each field at one wave vector per field: out [F][4] double2.
-swf_status transform_at(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precision prec,
-                        const void* psi, const double* kappa_host /* [F][3] */, double2* out,
-                        cudaStream_t st);
+// Direct FP64 transforms, n wave vectors: entry e is field e % n_fields (0: n_fields = n, one entry per
+// field) at kappa e: out [n][4] double2.  The split of a sum depends on n_fields, not on n.
+swf_status transform_at(swf_ctx* ctx, const GridDesc& g, int n, swf_precision prec, const void* psi,
+                        const double* kappa_host /* [n][3] */, double2* out, cudaStream_t st, int n_fields = 0);
 // ||psi_f||^2 (grid inner product) per field: out [F].
 swf_status field_norms(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precision prec,
                        const void* psi, double* out, cudaStream_t st);

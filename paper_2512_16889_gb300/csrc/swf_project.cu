@@ -121,9 +121,10 @@ __device__ __forceinline__ cpx<double> ld_d(const void* p, size_t i) {
   return cvt<double>(reinterpret_cast<const cpx<Rin>*>(p)[i]);
 }
 
-// One block per field: dx^d sum_x psi_a(x) exp(-i kappa.x) for a = 0..3 (deterministic order).
+// Entry f (field f % n_fields at kappa f): blocks' parts of sum_x psi_a(x) exp(-i kappa.x) for a = 0..3
+// (deterministic order).
 template <typename Rin>
-__global__ void __launch_bounds__(kT) k_transform_at(const void* psi, GridDesc g, const double* kappa,
+__global__ void __launch_bounds__(kT) k_transform_at(const void* psi, GridDesc g, int n_fields, const double* kappa,
                                                      cpx<double>* part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<double>* ph = reinterpret_cast<cpx<double>*>(smem_raw);  // nx + ny + nz phases
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(kT) k_transform_at(const void* psi, GridDesc g
   cpx<double> acc[4];
 #pragma unroll
   for (int a = 0; a < 4; ++a) acc[a] = mk<double>(0, 0);
-  const size_t fo = (size_t)f * 4 * g.N;
+  const size_t fo = (size_t)(f % n_fields) * 4 * g.N;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < g.N; j += gridDim.x * blockDim.x) {
     const int ix = j % g.n[0];
     const int iy = (j / g.n[0]) % g.n[1];
@@ -300,22 +301,23 @@ swf_status c_spectrum(swf_ctx* ctx, const GridDesc& g, int n_f, const FieldDesc*
 }
 
 swf_status transform_at(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precision prec, const void* psi,
-                        const double* kappa_host, double2* out, cudaStream_t st) {
+                        const double* kappa_host, double2* out, cudaStream_t st, int n_fields) {
+  if (n_fields < 1) n_fields = n_f;
   void* pk = nullptr;
   swf_status s = ws_get(ctx, "proj.kappa", sizeof(double) * 3 * n_f, &pk);
   if (s != SWF_OK) return s;
   cudaError_t e = cudaMemcpyAsync(pk, kappa_host, sizeof(double) * 3 * n_f, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_status(e, "upload wave vectors");
   const size_t sm = (size_t)(g.n[0] + g.n[1] + g.n[2]) * sizeof(cpx<double>);
-  const int nb = reduction_blocks(g.N, n_f);
+  const int nb = reduction_blocks(g.N, n_fields);
   void* part = nullptr;
   if ((s = ws_get(ctx, "proj.part", sizeof(cpx<double>) * 4 * (size_t)nb * n_f, &part)) != SWF_OK) return s;
   {
     ProfScope ps(ctx, "k_transform_at", st);
     if (prec == SWF_C64)
-      k_transform_at<float><<<dim3(nb, n_f), kT, sm, st>>>(psi, g, (const double*)pk, (cpx<double>*)part);
+      k_transform_at<float><<<dim3(nb, n_f), kT, sm, st>>>(psi, g, n_fields, (const double*)pk, (cpx<double>*)part);
     else
-      k_transform_at<double><<<dim3(nb, n_f), kT, sm, st>>>(psi, g, (const double*)pk, (cpx<double>*)part);
+      k_transform_at<double><<<dim3(nb, n_f), kT, sm, st>>>(psi, g, n_fields, (const double*)pk, (cpx<double>*)part);
   }
   {
     ProfScope ps(ctx, "k_sum_parts", st);
