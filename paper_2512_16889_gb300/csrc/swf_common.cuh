@@ -1,5 +1,5 @@
-// Shared device helpers of the SWF march: complex arithmetic, small DFT butterflies and a
-// shared-memory Stockham pass for the pseudo-spectral derivative (Sec. II.A, Eq. 10).
+// Shared device helpers of the SWF march: complex arithmetic, small DFT butterflies and
+// the radix plan of an axis.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -111,68 +111,14 @@ template <typename R> struct Dft<R, 5> {
   }
 };
 
-// ------------------------------------------------------------------ Stockham pass in smem
-// One radix-RAD pass of a self-sorting (Stockham) FFT over `nlines` lines of length n stored
-// at buf + line*ld.  p is the product of the radices already applied (1 on the first pass).
-// Butterfly b (line l, index i < n/RAD) reads l[i + q n/RAD], q < RAD, multiplies by the
-// twiddles exp(-+ 2 pi i q k/(p RAD)) with k = i mod p, applies the RAD-point DFT and writes
-// l[(i - k) RAD + k + q p].  After all passes the line holds its DFT in natural order.
-// tw[m] = exp(-2 pi i m/n) for m < n (rounded once from FP64).  All reads of the pass finish
-// (barrier) before any write, so the pass works in place.  SLOTS*blockDim must cover the
-// pass's butterflies.
 // Unsigned division by d via a multiply-high with M = ceil(2^32 / d) (the round-up variant of
 // Granlund & Montgomery, 1994): floor(x M / 2^32) = floor(x / d) whenever x (M d - 2^32) < 2^32,
-// which holds for every x < 2^32 / d; the butterfly indices here stay below 2^16 and d <= 512.
+// which holds for every x < 2^32 / d (d <= 512 here: x < 2^23).
 struct FastDiv {
   unsigned d, mag;
   __device__ __forceinline__ explicit FastDiv(unsigned d_) : d(d_), mag(d_ > 1 ? 0xFFFFFFFFu / d_ + 1u : 0u) {}
   __device__ __forceinline__ unsigned div(unsigned x) const { return d > 1 ? __umulhi(x, mag) : x; }
 };
-
-template <typename R, int RAD, int SLOTS>
-__device__ __forceinline__ void stockham_pass(cpx<R>* buf, int ld, int nlines, int n, int p,
-                                              bool inv, const cpx<R>* __restrict__ tw) {
-  const int m = n / RAD;
-  const int nb = nlines * m;
-  const int twstep = n / (p * RAD);
-  const FastDiv fm((unsigned)m), fp((unsigned)p);
-  cpx<R> v[SLOTS][RAD];
-#pragma unroll
-  for (int s = 0; s < SLOTS; ++s) {
-    const int b = threadIdx.x + s * blockDim.x;
-    if (b < nb) {
-      const int line = (int)fm.div((unsigned)b);
-      const int i = b - line * m;
-      const int k = i - p * (int)fp.div((unsigned)i);
-      const cpx<R>* src = buf + line * ld;
-#pragma unroll
-      for (int q = 0; q < RAD; ++q) v[s][q] = src[i + q * m];
-      if (k != 0) {
-#pragma unroll
-        for (int q = 1; q < RAD; ++q) {
-          cpx<R> w = tw[q * k * twstep];
-          if (inv) w.y = -w.y;
-          v[s][q] = v[s][q] * w;
-        }
-      }
-      Dft<R, RAD>::run(v[s], inv);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int s = 0; s < SLOTS; ++s) {
-    const int b = threadIdx.x + s * blockDim.x;
-    if (b < nb) {
-      const int line = (int)fm.div((unsigned)b);
-      const int i = b - line * m;
-      const int k = i - p * (int)fp.div((unsigned)i);
-      cpx<R>* dst = buf + line * ld + (i - k) * RAD + k;
-#pragma unroll
-      for (int q = 0; q < RAD; ++q) dst[q * p] = v[s][q];
-    }
-  }
-  __syncthreads();
-}
 
 // Radix plan of one axis: radices applied in order (product = n), at most 12 passes.
 struct RadixPlan {
@@ -180,21 +126,5 @@ struct RadixPlan {
   int npass;
   int rad[12];
 };
-
-// Full in-place FFT of `nlines` lines (forward when !inv).  MAXE bounds the elements a
-// thread holds per pass: blockDim * MAXE >= nlines * n + blockDim * 5 must hold.
-template <typename R, int MAXE>
-__device__ __forceinline__ void fft_lines(cpx<R>* buf, int ld, int nlines, const RadixPlan& pl,
-                                          bool inv, const cpx<R>* __restrict__ tw) {
-  int p = 1;
-  for (int ps = 0; ps < pl.npass; ++ps) {
-    const int r = pl.rad[ps];
-    if (r == 4) stockham_pass<R, 4, MAXE / 4>(buf, ld, nlines, pl.n, p, inv, tw);
-    else if (r == 2) stockham_pass<R, 2, MAXE / 2>(buf, ld, nlines, pl.n, p, inv, tw);
-    else if (r == 3) stockham_pass<R, 3, MAXE / 3>(buf, ld, nlines, pl.n, p, inv, tw);
-    else stockham_pass<R, 5, MAXE / 5>(buf, ld, nlines, pl.n, p, inv, tw);
-    p *= r;
-  }
-}
 
 }  // namespace swf

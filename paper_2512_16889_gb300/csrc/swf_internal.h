@@ -252,9 +252,9 @@ swf_status rhs_eval_scratch(const GridDesc& g, const FieldDesc& fd, swf_precisio
 
 // ---- projections (swf_project.cu)
 // psi [F][4][N] (march precision) -> FP64 transform on every grid mode, with the continuum
-// normalisation dx^d and the grid-origin phase: spec [F][4][N] double2.
+// normalisation dx^d and the grid-origin phase (raw: without them): spec [F][4][N] double2.
 swf_status transform_fields(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precision prec,
-                            const void* psi, double2* spec, cudaStream_t st);
+                            const void* psi, double2* spec, cudaStream_t st, bool raw = false);
 // C-spectrum from electron-wave transforms: c_out [F][2][N] double2, prob [F][2][N].
 swf_status c_spectrum(swf_ctx* ctx, const GridDesc& g, int n_f, const FieldDesc* fd_host,
                       double t_in, const double2* spec, double2* c_out, double* prob,

@@ -1,117 +1,139 @@
 // Projections at t_in (Sec. II, Eqs. 8-9) in FP64: grid transforms of the scattered waves,
 // the C-spectrum (U_scat(m) | V_back(r, q)) over every grid positron, direct transforms at
 // off-grid wave vectors, and grid norms.
+#include <atomic>
 #include <cstring>
 
-#include "swf_internal.h"
+#include "swf_pass.cuh"
 
 namespace swf {
 
 namespace {
 
 constexpr int kT = 256;
-constexpr int kMaxE = 20;  // FP64 elements a thread holds per FFT pass
 
+// One axis of the forward transform of every component plane (F*4 planes of N points): lines along
+// `axis` from `in` to `out` (in place when they are the same), nl of them per block (consecutive rows
+// on the x axis, consecutive x columns otherwise), tpl threads per line.  scale: the last axis
+// multiplies by it and, with sign, by the phase exp(-i kappa.x0) of a grid that starts at x0 = -L/2,
+// which is (-1)^(j'x + j'y + j'z) exactly.  FP64 operations bound it (25 per point: radix-4 passes and
+// their twiddles, a floor of 170 us per axis for 16 fields of 256^2; measured 231 us, 333 us with every
+// pass in shared memory); the conversion of a complex64 input (28 us as a pass of its own) and the
+// scale and sign (436 us with a sine and cosine per mode) ride along.
 template <typename Rin>
-__global__ void k_to_double(const cpx<Rin>* __restrict__ in, cpx<double>* __restrict__ out, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = cvt<double>(in[i]);
-}
-
-// Forward FFT along `axis` of every component plane (planes = F*4, each of N points).
-__global__ void __launch_bounds__(kT) k_fft_axis(cpx<double>* data, GridDesc g, int axis, RadixPlan pl,
-                                                 const cpx<double>* __restrict__ tw, int lines) {
+__global__ void __launch_bounds__(kPassThreads, 1)
+k_fft_axis(const cpx<Rin>* in, cpx<double>* out, GridDesc g, int axis, const __grid_constant__ RadixPlan pl,
+           const cpx<double>* __restrict__ tw, int nl, int ld, int tpl, double scale, int sign) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<double>* buf = reinterpret_cast<cpx<double>*>(smem_raw);
-  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2], na = pl.n;
   const size_t plane = (size_t)blockIdx.y * g.N;
-  const int na = g.n[axis];
+  int l, b0, o = 0;    // line within the block, first butterfly, index on the other axis
+  size_t base, stride;
+  bool ok;
   if (axis == 0) {
-    const int nrows = ny * nz;
-    const int row0 = blockIdx.x * lines;
-    for (int e = threadIdx.x; e < lines * nx; e += blockDim.x) {
-      const int j = e / nx, x = e - j * nx;
-      buf[j * nx + x] = (row0 + j < nrows) ? data[plane + (size_t)(row0 + j) * nx + x] : mk<double>(0, 0);
-    }
-    __syncthreads();
-    fft_lines<double, kMaxE>(buf, nx, lines, pl, false, tw);
-    for (int e = threadIdx.x; e < lines * nx; e += blockDim.x) {
-      const int j = e / nx, x = e - j * nx;
-      if (row0 + j < nrows) data[plane + (size_t)(row0 + j) * nx + x] = buf[j * nx + x];
-    }
-    return;
+    l = threadIdx.x / tpl;
+    b0 = threadIdx.x - l * tpl;
+    o = blockIdx.x * nl + l;  // row
+    ok = l < nl && o < ny * nz;
+    base = plane + (size_t)o * nx;
+    stride = 1;
+  } else {
+    const int ntx = (nx + nl - 1) / nl, xt = blockIdx.x % ntx;
+    o = blockIdx.x / ntx;  // z (axis 1) or y (axis 2)
+    b0 = threadIdx.x / nl;
+    l = threadIdx.x - b0 * nl;
+    ok = b0 < tpl && xt * nl + l < nx;
+    base = plane + (axis == 1 ? (size_t)o * nx * ny : (size_t)o * nx) + xt * nl + l;
+    stride = axis == 1 ? (size_t)nx : (size_t)nx * ny;
   }
-  const int TX = lines;
-  const int ntx = (nx + TX - 1) / TX;
-  const int xt = blockIdx.x % ntx;
-  const int o = blockIdx.x / ntx;
-  const size_t base = axis == 1 ? (size_t)o * nx * ny : (size_t)o * nx;
-  const size_t stride = axis == 1 ? (size_t)nx : (size_t)nx * ny;
-  for (int e = threadIdx.x; e < TX * na; e += blockDim.x) {
-    const int m = e / TX, t = e - m * TX;
-    const int x = xt * TX + t;
-    buf[t * na + m] = x < nx ? data[plane + base + m * stride + x] : mk<double>(0, 0);
-  }
+  cpx<double>* a = reinterpret_cast<cpx<double>*>(smem_raw);
+  cpx<double>* b2 = a + nl * ld;
+  if (ok)
+    with_radix(end_radix(pl, true), [&](auto rc) {
+      constexpr int R0 = decltype(rc)::value;
+      const int nb = na / R0;
+      for (int b = b0; b < nb; b += tpl) {
+        cpx<double> v[R0];
+#pragma unroll
+        for (int q = 0; q < R0; ++q) v[q] = cvt<double>(in[base + (size_t)(b + q * nb) * stride]);
+        first_butterfly<double, R0>(v, b, false, a + l * ld);
+      }
+    });
   __syncthreads();
-  fft_lines<double, kMaxE>(buf, na, TX, pl, false, tw);
-  for (int e = threadIdx.x; e < TX * na; e += blockDim.x) {
-    const int m = e / TX, t = e - m * TX;
-    const int x = xt * TX + t;
-    if (x < nx) data[plane + base + m * stride + x] = buf[t * na + m];
+  const cpx<double>* cur = middle_passes<double>(a, b2, ld, nl, pl, false, tw);
+  if (!ok) return;
+  int par = 0;  // parity of the other axes' mode numbers j'
+  if (sign) {
+    auto parity = [&](int j, int n) { return n > 1 ? (j < (n + 1) / 2 ? j : j - n) & 1 : 0; };
+    if (axis == 0) par = 0;  // x is the last axis only where it is the only one
+    else if (axis == 1) par = parity((int)((base - plane) % nx), nx) ^ parity(o, nz);
+    else par = parity((int)((base - plane) % nx), nx) ^ parity(o, ny);
   }
-}
-
-// Continuum normalisation dx^d and the phase exp(-i kappa.x0) of a grid starting at x0.
-__global__ void k_mode_scale(cpx<double>* data, GridDesc g, size_t total) {
-  const double cell = g.dx[0] * g.dx[1] * g.dx[2];
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int j = (int)(i % g.N);
-    const int ix = j % g.n[0];
-    const int iy = (j / g.n[0]) % g.n[1];
-    const int iz = j / (g.n[0] * g.n[1]);
-    const double ph = -(mode_kappa(ix, g.n[0], g.L[0]) * g.x0[0] + mode_kappa(iy, g.n[1], g.L[1]) * g.x0[1] +
-                        mode_kappa(iz, g.n[2], g.L[2]) * g.x0[2]);
-    double sn, cs;
-    sincos(ph, &sn, &cs);
-    data[i] = cell * (data[i] * mk<double>(cs, sn));
-  }
+  with_radix(end_radix(pl, false), [&](auto rc) {
+    constexpr int RL = decltype(rc)::value;
+    const int nm = na / RL;
+    for (int b = b0; b < nm; b += tpl) {
+      cpx<double> m[RL];
+      last_butterfly<double, RL>(cur + l * ld, b, na, pl.npass < 2, false, tw, m);
+#pragma unroll
+      for (int q = 0; q < RL; ++q) {
+        const int j = b + q * nm;
+        double sc = scale;
+        if (sign && (((j < (na + 1) / 2 ? j : j - na) ^ par) & 1)) sc = -scale;
+        out[base + (size_t)j * stride] = sc * m[q];
+      }
+    }
+  });
 }
 
 // C(m, (r, q)) = exp(i q0 t_in) sum_a conj(U~_a(-q)) v_{r,a}(q); the positron at mode j has
-// q = -kappa_j (trivial axes: kappa = K of the electron wave).
-__global__ void k_c_spectrum(const cpx<double>* __restrict__ spec, const FieldDesc* fd, GridDesc g, int F,
-                             double t_in, cpx<double>* c_out, double* prob) {
-  const size_t total = (size_t)F * g.N;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int f = (int)(i / g.N);
-    const int j = (int)(i - (size_t)f * g.N);
-    const int ix = j % g.n[0];
-    const int iy = (j / g.n[0]) % g.n[1];
-    const int iz = j / (g.n[0] * g.n[1]);
-    const FieldDesc& F0 = fd[f];
-    double q[3];
-    q[0] = -(g.n[0] > 1 ? mode_kappa(ix, g.n[0], g.L[0]) : F0.K[0]);
-    q[1] = -(g.n[1] > 1 ? mode_kappa(iy, g.n[1], g.L[1]) : F0.K[1]);
-    q[2] = -(g.n[2] > 1 ? mode_kappa(iz, g.n[2], g.L[2]) : F0.K[2]);
-    const double q0 = energy3(q);
-    double sn, cs;
-    sincos(q0 * t_in, &sn, &cs);
-    const cpx<double> ph = mk<double>(cs, sn);
+// q = -kappa_j (trivial axes: kappa = K of the electron wave).  A thread holds the two spinors of one
+// mode, phase included, for fc fields (they depend on the mode and K alone; a field with another K has
+// its own): the square roots and the sine and cosine in FP64 are about four times a field's products
+// (16 fields of 256^2: 309 -> 149 us).
+__global__ void __launch_bounds__(kT) k_c_spectrum(const cpx<double>* __restrict__ spec, const FieldDesc* fd, GridDesc g,
+                                                   int F, int fc, double t_in, cpx<double>* c_out, double* prob) {
+  const int f0 = blockIdx.y * fc, f1 = min(F, f0 + fc);
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= g.N) return;
+  const int row = j / g.n[0];
+  const int id[3] = {j - row * g.n[0], row % g.n[1], row / g.n[1]};
+  double kap[3], v[2][8];
+  for (int a = 0; a < 3; ++a) kap[a] = mode_kappa(id[a], g.n[a], g.L[a]);
+  for (int f = f0; f < f1; ++f) {
+    const double* K = fd[f].K;
+    const bool same = f > f0 && K[0] == fd[f - 1].K[0] && K[1] == fd[f - 1].K[1] && K[2] == fd[f - 1].K[2];
+    if (!same) {
+      double q[3];
+      for (int a = 0; a < 3; ++a) q[a] = -(g.n[a] > 1 ? kap[a] : K[a]);
+      double sn = 0.0, cs = 1.0;
+      if (c_out) sincos(energy3(q) * t_in, &sn, &cs);  // |C|^2 does not see it
+#pragma unroll
+      for (int ir = 0; ir < 2; ++ir) {
+        double w[8];
+        spinor_uv(q, ir == 0 ? 1 : -1, true, w);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          v[ir][2 * a] = cs * w[2 * a] - sn * w[2 * a + 1];
+          v[ir][2 * a + 1] = cs * w[2 * a + 1] + sn * w[2 * a];
+        }
+      }
+    }
     const cpx<double>* u = spec + (size_t)f * 4 * g.N + j;
     cpx<double> uc[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) uc[a] = u[(size_t)a * g.N];
 #pragma unroll
     for (int ir = 0; ir < 2; ++ir) {
-      double v[8];
-      spinor_uv(q, ir == 0 ? 1 : -1, true, v);
       cpx<double> acc = mk<double>(0, 0);
 #pragma unroll
-      for (int a = 0; a < 4; ++a) acc = acc + cdot(uc[a], mk<double>(v[2 * a], v[2 * a + 1]));
-      acc = ph * acc;
-      const size_t o = ((size_t)f * 2 + ir) * g.N + j;
-      if (c_out) c_out[o] = acc;
-      if (prob) prob[o] = acc.x * acc.x + acc.y * acc.y;
+      for (int a = 0; a < 4; ++a) {
+        acc.x += uc[a].x * v[ir][2 * a] + uc[a].y * v[ir][2 * a + 1];
+        acc.y += uc[a].x * v[ir][2 * a + 1] - uc[a].y * v[ir][2 * a];
+      }
+      const size_t e = ((size_t)f * 2 + ir) * g.N + j;
+      if (c_out) c_out[e] = acc;
+      if (prob) prob[e] = acc.x * acc.x + acc.y * acc.y;
     }
   }
 }
@@ -220,63 +242,59 @@ __global__ void __launch_bounds__(kT) k_norms(const void* psi, GridDesc g, doubl
   }
 }
 
-bool smem_ready[64] = {false};
+constexpr size_t kFftSmem = 200 * 1024;
 
 swf_status ensure_smem() {
+  static std::atomic<bool> ready[64];
   const int dv = dev_slot();
-  if (smem_ready[dv]) return SWF_OK;
-  cudaError_t e = cudaFuncSetAttribute(k_fft_axis, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kT * (kMaxE - 4) * (int)sizeof(cpx<double>));
+  if (ready[dv].load(std::memory_order_acquire)) return SWF_OK;
+  cudaError_t e = cudaFuncSetAttribute(k_fft_axis<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFftSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_fft_axis<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFftSmem);
   if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_fft_axis)");
-  smem_ready[dv] = true;
+  ready[dv].store(true, std::memory_order_release);
   return SWF_OK;
 }
 
 }  // namespace
 
 swf_status transform_fields(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precision prec, const void* psi,
-                            double2* spec, cudaStream_t st) {
+                            double2* spec, cudaStream_t st, bool raw) {
   swf_status s = ensure_smem();
   if (s != SWF_OK) return s;
-  const size_t total = (size_t)n_f * 4 * g.N;
   cpx<double>* d = reinterpret_cast<cpx<double>*>(spec);
-  const int nb = (int)((total + kT - 1) / kT < 65536 ? (total + kT - 1) / kT : 65536);
-  {
-    ProfScope ps(ctx, "k_to_double", st);
-    if (prec == SWF_C64) k_to_double<float><<<nb, kT, 0, st>>>((const cpx<float>*)psi, d, total);
-    else k_to_double<double><<<nb, kT, 0, st>>>((const cpx<double>*)psi, d, total);
-  }
-  const int cap = kT * (kMaxE - 4);
-  for (int axis = 0; axis < 3; ++axis) {
-    const int na = g.n[axis];
-    if (na <= 1) continue;
+  int axes[3], nax = 0;
+  for (int a = 0; a < 3; ++a)
+    if (g.n[a] > 1) axes[nax++] = a;
+  if (nax == 0) axes[nax++] = 0;  // a single point: the conversion alone
+  for (int k = 0; k < nax; ++k) {
+    const int axis = axes[k], na = g.n[axis];
     RadixPlan pl;
-    if (!make_radix_plan(na, &pl)) {
+    if (!make_pass_plan(na, &pl)) {
       set_error("grid size must factor into 2, 3 and 5");
       return SWF_EINVAL;
     }
     const void* tw = nullptr;
     if ((s = twiddles(ctx, na, 1, &tw)) != SWF_OK) return s;
-    int lines = cap / na;
-    if (axis == 0) {
-      const int nrows = g.n[1] * g.n[2];
-      if (lines > nrows) lines = nrows;
-      dim3 grid((nrows + lines - 1) / lines, n_f * 4);
-      ProfScope ps(ctx, "k_fft_axis", st);
-      k_fft_axis<<<grid, kT, (size_t)lines * na * sizeof(cpx<double>), st>>>(d, g, 0, pl, (const cpx<double>*)tw, lines);
-    } else {
-      if (lines > 16) lines = 16;
-      if (lines > g.n[0]) lines = g.n[0];
-      const int ntx = (g.n[0] + lines - 1) / lines;
-      const int other = axis == 1 ? g.n[2] : g.n[1];
-      dim3 grid(ntx * other, n_f * 4);
-      ProfScope ps(ctx, "k_fft_axis", st);
-      k_fft_axis<<<grid, kT, (size_t)lines * na * sizeof(cpx<double>), st>>>(d, g, axis, pl, (const cpx<double>*)tw, lines);
-    }
-  }
-  {
-    ProfScope ps(ctx, "k_mode_scale", st);
-    k_mode_scale<<<nb, kT, 0, st>>>(d, g, total);
+    // lines per block: about 256 threads; eight neighbouring x columns (128 bytes) at most
+    const int tpl = pass_threads(pl, 1);
+    const int nrows = axis == 0 ? g.n[1] * g.n[2] : g.n[0];
+    const int ld = padded_len<double>(na) | 1;
+    int nl = std::max(1, std::min(std::min(axis == 0 ? 64 : 8, kT / tpl), nrows));
+    while (nl > 1 && (size_t)2 * nl * ld * 16 > kFftSmem) --nl;
+    const int blocks = axis == 0 ? (nrows + nl - 1) / nl : (nrows + nl - 1) / nl * (axis == 1 ? g.n[2] : g.n[1]);
+    const dim3 grid(blocks, n_f * 4);
+    const size_t smem = (size_t)2 * nl * ld * 16;
+    const bool last = k + 1 == nax;
+    const double scale = last && !raw ? g.dx[0] * g.dx[1] * g.dx[2] : 1.0;
+    const int sign = last && !raw ? 1 : 0;
+    ProfScope ps(ctx, "k_fft_axis", st);
+    if (k == 0 && prec == SWF_C64)
+      k_fft_axis<float><<<grid, nl * tpl, smem, st>>>((const cpx<float>*)psi, d, g, axis, pl, (const cpx<double>*)tw, nl,
+                                                      ld, tpl, scale, sign);
+    else
+      k_fft_axis<double><<<grid, nl * tpl, smem, st>>>(k == 0 ? (const cpx<double>*)psi : d, d, g, axis, pl,
+                                                       (const cpx<double>*)tw, nl, ld, tpl, scale, sign);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e, "transform kernels");
@@ -290,11 +308,13 @@ swf_status c_spectrum(swf_ctx* ctx, const GridDesc& g, int n_f, const FieldDesc*
   if (s != SWF_OK) return s;
   cudaError_t e = cudaMemcpyAsync(pfd, fd_host, sizeof(FieldDesc) * n_f, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_status(e, "upload field descriptors");
-  const size_t total = (size_t)n_f * g.N;
-  const int nb = (int)((total + kT - 1) / kT < 65536 ? (total + kT - 1) / kT : 65536);
+  // fields per thread: as many as leave about two blocks per SM
+  const int nb = (g.N + kT - 1) / kT;
+  const int chunks = std::max(1, std::min(n_f, 304 / nb));
+  const int fc = (n_f + chunks - 1) / chunks;
   ProfScope ps(ctx, "k_c_spectrum", st);
-  k_c_spectrum<<<nb, kT, 0, st>>>((const cpx<double>*)spec, (const FieldDesc*)pfd, g, n_f, t_in,
-                                  (cpx<double>*)c_out, prob);
+  k_c_spectrum<<<dim3(nb, (n_f + fc - 1) / fc), kT, 0, st>>>((const cpx<double>*)spec, (const FieldDesc*)pfd, g, n_f, fc,
+                                                             t_in, (cpx<double>*)c_out, prob);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e, "c-spectrum kernel");
   return SWF_OK;
