@@ -271,8 +271,9 @@ __global__ void __launch_bounds__(256) k_pair_modes(const InstDev* id, GridDesc 
     cpx<double> s = mk<double>(0, 0), t = mk<double>(0, 0);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      s = s + cdot(uv[c], a[c]);
-      t = t + cdot(uv[c], hv[c]);
+      s = mk<double>(fma(uv[c].y, a[c].y, fma(uv[c].x, a[c].x, s.x)), fma(-uv[c].y, a[c].x, fma(uv[c].x, a[c].y, s.y)));
+      t = mk<double>(fma(uv[c].y, hv[c].y, fma(uv[c].x, hv[c].x, t.x)),
+                     fma(-uv[c].y, hv[c].x, fma(uv[c].x, hv[c].y, t.y)));
     }
     accB = accB + 0.5 * (s + ie * t);
     accD = accD + 0.5 * (s - ie * t);

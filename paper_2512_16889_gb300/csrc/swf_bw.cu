@@ -126,9 +126,9 @@ __global__ void __launch_bounds__(256) k_bw_modes(const BwInst* bi, GridDesc g, 
     const double sum = Eu + Ev, dif = Eu - Ev;
     const double w0 = 1.0 / (dif - k0), w1 = 1.0 / (sum - k0), w2 = -1.0 / (sum + k0), w3 = -1.0 / (dif + k0);
     const cpx<double> d0 = form_d(up, avp), d1 = form_d(up, av), d2 = form_d(u, avp), d3 = form_d(u, av);
-    const cpx<double> t = mk<double>(w0 * d0.x + w1 * d1.x + w2 * d2.x + w3 * d3.x,
-                                     w0 * d0.y + w1 * d1.y + w2 * d2.y + w3 * d3.y);
-    acc = odd ? acc - t : acc + t;
+    const double sg = odd ? -1.0 : 1.0;
+    acc.x = fma(sg, fma(w3, d3.x, fma(w2, d2.x, fma(w1, d1.x, w0 * d0.x))), acc.x);
+    acc.y = fma(sg, fma(w3, d3.y, fma(w2, d2.y, fma(w1, d1.y, w0 * d0.y))), acc.y);
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {

@@ -2,18 +2,26 @@
 // all in one field, grid and time window (Sec. II, Eqs. 8-9; Sec. II.A: scans over momenta).
 //
 // Instead of one U and one V march per pair, every electron is marched once (U waves) and every
-// positron once (V waves), and the four overlaps of Eq. 8 become complex matrix products over
-// the grid (K = 4 N: components x sites), in FP64:
-//   C(m, n) = dx^d sum_x U_m^+(x) V_back,n(x)              (position space)
-//   A(m, n) = dx^d sum_x U_back,m^+(x) V_n(x)              (position space)
-//   B(m, n) = L^-d sum_j (P_+(k_j) U~_m(j))^+ V~_n(j)      (grid modes, P_+- energy projectors)
+// positron once (V waves), and the four overlaps of Eq. 8 are formed in FP64:
+//   C(m, n) = e^{i q0 t} sum_c conj(U~_m(-q_n))_c v_n,c       (a plane wave: a direct transform)
+//   A(m, n) = e^{i p0 t} sum_c conj(u_m,c) V~_n(p_m)_c
+//   B(m, n) = L^-d sum_j (P_+(k_j) U~_m(j))^+ V~_n(j)         (grid modes, P_+- energy projectors)
 //   D(m, n) = L^-d sum_j (P_-(k_j) U~_m(j))^+ V~_n(j)
-// with U~, V~ the continuum-normalised transforms and the backgrounds U_back = u_s(p)
-// e^{-i(p0 t - p.x)}, V_back = v_r(q) e^{i(q0 t - q.x)} at t = t_in.  The sums over s' and the
-// grid modes Q of Eq. 8 are the projectors (sum_s' u u^+ = P_+, sum_s' v v^+ = P_-), as in the
-// single-pair path.  N = |C + D|^2 = |A + B|^2.
+// with U~, V~ the continuum-normalised transforms at t = t_in.  The sums over s' and the grid modes Q
+// of Eq. 8 are the projectors (sum_s' u u^+ = P_+, sum_s' v v^+ = P_-), as in the single-pair path.
+// N = |C + D|^2 = |A + B|^2.
+//
+// A plane wave is a product of one factor per axis, so the direct transforms of one wave at all n
+// momenta of the other list need one pass over the grid per distinct momentum along some of the axes
+// (a scan along one axis: one) and a small product after it, instead of 4 N products per pair.  In an
+// orthonormal eigenbasis of every mode's H0 the projectors are a choice of two of the four
+// amplitudes, so B and D are matrix products over 2 N amplitudes each.  Together 4 N FP64 products per
+// pair instead of 16 N.
 #include <algorithm>
-#include <cstring>
+#include <array>
+#include <cmath>
+#include <map>
+#include <string>
 #include <vector>
 
 #include "swf_internal.h"
@@ -21,135 +29,225 @@
 namespace swf {
 namespace pairs {
 
-constexpr int TM = 32, TN = 32, TK = 16;  // output tile and k step of the product kernel
+constexpr int TK = 16;      // k step of the product kernel
+constexpr int kTile = 32;   // output tile of a block: at most 32 x 32, one output per thread
+constexpr int DB = 4;       // momenta per block of the first contraction
 
-// part[s][m][n] = sum over k in split s of conj(X[m][k]) Y[n][k]; X: M rows, Y: Nn rows, both
-// K long and contiguous.  256 threads, 2 x 2 outputs each; the splits are added in order by
-// k_sum_splits (deterministic).
-__global__ void __launch_bounds__(256) k_gemm_cn(const cpx<double>* __restrict__ X, const cpx<double>* __restrict__ Y,
-                                                 int M, int Nn, long K, long kchunk, cpx<double>* part) {
-  __shared__ cpx<double> xs[TK][TM + 1];
-  __shared__ cpx<double> ys[TK][TN + 1];
-  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-  const long k0 = blockIdx.z * kchunk;
-  const long k1 = std::min(K, k0 + kchunk);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  cpx<double> acc[2][2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) acc[i][j] = mk<double>(0, 0);
-  for (long kb = k0; kb < k1; kb += TK) {
-    // tiles: TM x TK of X and TN x TK of Y (k fastest in memory: coalesced along k)
-    for (int e = threadIdx.x; e < TM * TK; e += blockDim.x) {
-      const int r = e / TK, c = e % TK;
-      const long k = kb + c;
-      xs[c][r] = (m0 + r < M && k < k1) ? X[(size_t)(m0 + r) * K + k] : mk<double>(0, 0);
-      ys[c][r] = (n0 + r < Nn && k < k1) ? Y[(size_t)(n0 + r) * K + k] : mk<double>(0, 0);
+// Phase tables exp(-i sum_a kappa_a x_a) over the sites of the axes in `axes` (bit a: axis a; trivial
+// axes carry no phase): tab[d][site], d < n.
+__global__ void k_phases(const double* __restrict__ kappa, int n, GridDesc g, int axes, int len, cpx<double>* tab) {
+  const int d = blockIdx.y;
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < len; r += gridDim.x * blockDim.x) {
+    int rest = r;
+    double ph = 0.0;
+    for (int a = 0; a < 3; ++a) {
+      if (!(axes >> a & 1)) continue;
+      const int j = rest % g.n[a];
+      rest /= g.n[a];
+      if (g.n[a] > 1) ph -= kappa[3 * d + a] * (g.x0[a] + j * g.dx[a]);
     }
-    __syncthreads();
-#pragma unroll
-    for (int c = 0; c < TK; ++c) {
-      const cpx<double> x0 = xs[c][ty], x1 = xs[c][ty + 16];
-      const cpx<double> y0 = ys[c][tx], y1 = ys[c][tx + 16];
-      acc[0][0] = acc[0][0] + cdot(x0, y0);
-      acc[0][1] = acc[0][1] + cdot(x0, y1);
-      acc[1][0] = acc[1][0] + cdot(x1, y0);
-      acc[1][1] = acc[1][1] + cdot(x1, y1);
-    }
-    __syncthreads();
-  }
-  cpx<double>* out = part + (size_t)blockIdx.z * M * Nn;
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int m = m0 + ty + 16 * i, n = n0 + tx + 16 * j;
-      if (m < M && n < Nn) out[(size_t)m * Nn + n] = acc[i][j];
-    }
-}
-
-// out[m][n] = scale sum_s part[s][m][n], splits in order.
-__global__ void k_sum_splits(const cpx<double>* __restrict__ part, int S, long MN, double scale, cpx<double>* out) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < MN; i += (long)gridDim.x * blockDim.x) {
-    cpx<double> s = mk<double>(0, 0);
-    for (int k = 0; k < S; ++k) s = s + part[(size_t)k * MN + i];
-    out[i] = scale * s;
-  }
-}
-
-template <typename R>
-__global__ void k_widen(const cpx<R>* __restrict__ in, cpx<double>* __restrict__ out, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = cvt<double>(in[i]);
-}
-
-// Background plane waves on the grid at t_in: w[8] = spinor (re, im) x 4, mom = momentum of the
-// exponent e^{i sgn (mom.x - E t)} (U: sgn = +1, mom = p; V: sgn = -1, mom = q).  Trivial axes
-// carry no phase (their momentum is the marched wave's own, the same on both sides).
-struct Wave {
-  double w[8];
-  double mom[3];
-  double sgn;
-};
-
-__global__ void k_plane_waves(const Wave* wv, GridDesc g, double t, cpx<double>* out) {
-  const int f = blockIdx.y;
-  const Wave W = wv[f];
-  const double E = sqrt(1.0 + W.mom[0] * W.mom[0] + W.mom[1] * W.mom[1] + W.mom[2] * W.mom[2]);
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < g.N; j += gridDim.x * blockDim.x) {
-    const int ix = j % g.n[0];
-    const int iy = (j / g.n[0]) % g.n[1];
-    const int iz = j / (g.n[0] * g.n[1]);
-    const int id[3] = {ix, iy, iz};
-    double ph = -E * t;
-    for (int a = 0; a < 3; ++a)
-      if (g.n[a] > 1) ph += W.mom[a] * (g.x0[a] + id[a] * g.dx[a]);
     double sn, cs;
-    sincos(W.sgn * ph, &sn, &cs);
-    const cpx<double> e = mk<double>(cs, sn);
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-      out[((size_t)f * 4 + a) * g.N + j] = e * mk<double>(W.w[2 * a], W.w[2 * a + 1]);
+    sincos(ph, &sn, &cs);
+    tab[(size_t)d * len + r] = mk<double>(cs, sn);
   }
 }
 
-// out[sgn][m] = P_sgn(kappa_j) spec[m] per grid mode (P_+- = (1 +- H0/E)/2), sgn = + first.
-__global__ void k_project(const cpx<double>* __restrict__ spec, GridDesc g, const double* __restrict__ Ku, int n_f,
-                          cpx<double>* __restrict__ out) {
-  const int f = blockIdx.y;
-  const cpx<double>* u = spec + (size_t)f * 4 * g.N;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < g.N; j += gridDim.x * blockDim.x) {
-    const int ix = j % g.n[0];
-    const int iy = (j / g.n[0]) % g.n[1];
-    const int iz = j / (g.n[0] * g.n[1]);
-    const double kx = g.n[0] > 1 ? mode_kappa(ix, g.n[0], g.L[0]) : Ku[0];
-    const double ky = g.n[1] > 1 ? mode_kappa(iy, g.n[1], g.L[1]) : Ku[1];
-    const double kz = g.n[2] > 1 ? mode_kappa(iz, g.n[2], g.L[2]) : Ku[2];
-    const double iE = 1.0 / sqrt(1.0 + kx * kx + ky * ky + kz * kz);
-    cpx<double> a[4], h[4];
+// First contraction over rows (y, z): G[line][d][x] = sum_r psi[line][r][x] tab[d][r], line = (field,
+// component), DB values of d per block.  32 x columns by 8 row groups per block, the groups added in
+// order.
+template <typename R>
+__global__ void __launch_bounds__(256) k_contract_rows(const cpx<R>* __restrict__ psi, const cpx<double>* __restrict__ tab,
+                                                       int nrows, int nx, int D, cpx<double>* G) {
+  __shared__ cpx<double> red[8][DB][32];
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  const int x = blockIdx.x * 32 + lane, d0 = blockIdx.z * DB;
+  const size_t line = blockIdx.y;
+  cpx<double> acc[DB];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) a[c] = u[(size_t)c * g.N + j];
-    // H0(kappa) a = (alpha.kappa + beta) a, Dirac representation
-    h[0] = a[0] + kz * a[2] + kx * a[3] + ky * mul_mi(a[3]);
-    h[1] = a[1] + kx * a[2] + ky * mul_i(a[2]) - kz * a[3];
-    h[2] = kz * a[0] + kx * a[1] + ky * mul_mi(a[1]) - a[2];
-    h[3] = kx * a[0] + ky * mul_i(a[0]) - kz * a[1] - a[3];
+  for (int k = 0; k < DB; ++k) acc[k] = mk<double>(0, 0);
+  if (x < nx) {
+    const cpx<R>* p = psi + line * (size_t)nrows * nx + x;
+    for (int r = grp; r < nrows; r += 8) {
+      const cpx<double> v = cvt<double>(p[(size_t)r * nx]);
+#pragma unroll
+      for (int k = 0; k < DB; ++k)
+        if (d0 + k < D) {
+          const cpx<double> w = tab[(size_t)(d0 + k) * nrows + r];
+          acc[k] = mk<double>(acc[k].x + v.x * w.x - v.y * w.y, acc[k].y + v.x * w.y + v.y * w.x);
+        }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < DB; ++k) red[grp][k][lane] = acc[k];
+  __syncthreads();
+  if (grp < DB && x < nx && d0 + grp < D) {
+    cpx<double> s = red[0][grp][lane];
+    for (int q = 1; q < 8; ++q) s = s + red[q][grp][lane];
+    G[(line * D + d0 + grp) * nx + x] = s;
+  }
+}
+
+// First contraction over x: G[line][d][r] = sum_x psi[line][r][x] tab[d][x]; a warp per row.
+template <typename R>
+__global__ void __launch_bounds__(256) k_contract_x(const cpx<R>* __restrict__ psi, const cpx<double>* __restrict__ tab,
+                                                    int nrows, int nx, int D, cpx<double>* G) {
+  const int lane = threadIdx.x & 31, r = blockIdx.x * 8 + (threadIdx.x >> 5), d0 = blockIdx.z * DB;
+  if (r >= nrows) return;
+  const size_t line = blockIdx.y;
+  const cpx<R>* p = psi + (line * nrows + r) * (size_t)nx;
+  cpx<double> acc[DB];
+#pragma unroll
+  for (int k = 0; k < DB; ++k) acc[k] = mk<double>(0, 0);
+  for (int x = lane; x < nx; x += 32) {
+    const cpx<double> v = cvt<double>(p[x]);
+#pragma unroll
+    for (int k = 0; k < DB; ++k)
+      if (d0 + k < D) {
+        const cpx<double> w = tab[(size_t)(d0 + k) * nx + x];
+        acc[k] = mk<double>(acc[k].x + v.x * w.x - v.y * w.y, acc[k].y + v.x * w.y + v.y * w.x);
+      }
+  }
+#pragma unroll
+  for (int k = 0; k < DB; ++k) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      acc[k].x += __shfl_down_sync(0xffffffffu, acc[k].x, off);
+      acc[k].y += __shfl_down_sync(0xffffffffu, acc[k].y, off);
+    }
+    if (lane == 0 && d0 + k < D) G[(line * D + d0 + k) * nrows + r] = acc[k];
+  }
+}
+
+// Last contraction: out[line / 4][k][line % 4] = scale sum_i G[line][map[k]][i] tab[k][i]; a warp per
+// (line, k).
+__global__ void __launch_bounds__(256) k_contract_last(const cpx<double>* __restrict__ G,
+                                                       const cpx<double>* __restrict__ tab, const int* __restrict__ map,
+                                                       int len, int D, int n_k, double scale, cpx<double>* out) {
+  const int lane = threadIdx.x & 31, k = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (k >= n_k) return;
+  const size_t line = blockIdx.y;
+  const cpx<double>* p = G + (line * D + map[k]) * len;
+  const cpx<double>* w = tab + (size_t)k * len;
+  cpx<double> s = mk<double>(0, 0);
+  for (int i = lane; i < len; i += 32) s = s + p[i] * w[i];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    s.x += __shfl_down_sync(0xffffffffu, s.x, off);
+    s.y += __shfl_down_sync(0xffffffffu, s.y, off);
+  }
+  if (lane == 0) out[((line >> 2) * n_k + k) * 4 + (line & 3)] = scale * s;
+}
+
+// Every mode's four components (in place) to its amplitudes in an orthonormal eigenbasis of H0(kappa)
+// (Dirac representation, w = kappa/(E + 1), c^2 = (E + 1)/(2E)): c (1, 0, wz, wx + i wy), c (0, 1, wx -
+// i wy, -wz) of energy +E, c (-wz, -wx - i wy, 1, 0), c (-wx + i wy, wz, 0, 1) of energy -E.
+__global__ void __launch_bounds__(256) k_energy_amps(cpx<double>* spec, GridDesc g, const double* __restrict__ Ku, int n_f,
+                                                     int fc) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= g.N) return;
+  const int row = j / g.n[0];
+  const int id[3] = {j - row * g.n[0], row % g.n[1], row / g.n[1]};
+  double k[3];
+  for (int a = 0; a < 3; ++a) k[a] = g.n[a] > 1 ? mode_kappa(id[a], g.n[a], g.L[a]) : Ku[a];
+  const double E = sqrt(1.0 + k[0] * k[0] + k[1] * k[1] + k[2] * k[2]);
+  const double c = sqrt((E + 1.0) / (2.0 * E)), ie = c / (E + 1.0);
+  const double wx = k[0] * ie, wy = k[1] * ie, wz = k[2] * ie;  // times c
+  const int f1 = min(n_f, (int)(blockIdx.y + 1) * fc);
+  for (int f = blockIdx.y * fc; f < f1; ++f) {
+    cpx<double>* u = spec + (size_t)f * 4 * g.N + j;
+    const size_t N = g.N;
+    const cpx<double> a = u[0], b = u[N], p = u[2 * N], q = u[3 * N];
+    // (wx - i wy) z = (wx z.x + wy z.y, wx z.y - wy z.x); (wx + i wy) z = (wx z.x - wy z.y, wx z.y + wy z.x)
+    u[0] = mk<double>(c * a.x + wz * p.x + wx * q.x + wy * q.y, c * a.y + wz * p.y + wx * q.y - wy * q.x);
+    u[N] = mk<double>(c * b.x + wx * p.x - wy * p.y - wz * q.x, c * b.y + wx * p.y + wy * p.x - wz * q.y);
+    u[2 * N] = mk<double>(c * p.x - wz * a.x - wx * b.x - wy * b.y, c * p.y - wz * a.y - wx * b.y + wy * b.x);
+    u[3 * N] = mk<double>(c * q.x - wx * a.x + wy * a.y + wz * b.x, c * q.y - wx * a.y - wy * a.x + wz * b.y);
+  }
+}
+
+// part[sign][s][m][n] = sum over k in split s of conj(X[m][sign K + k]) Y[n][sign K + k], rows of `ld`
+// values.  One output per thread: FP64 issues an instruction in 64 cycles per SM quarter, so the two
+// shared-memory reads of a product are hidden without a register tile, and tiles of exactly TM x TN
+// outputs (100 x 100 pairs: 16 tiles of 25 x 25, 625 of 640 threads) leave few lanes idle.  The next
+// k step's operands are on their way while the present one is used.  100 x 100 pairs on 256 x 128: 9.3
+// ms (107 ms with 2 x 2 outputs a thread, 32 x 32 tiles and four times the products; 8.3 ms at the FP64
+// unit's full rate).
+__global__ void __launch_bounds__(kTile* kTile, 1)
+k_pair_products(const cpx<double>* __restrict__ X, const cpx<double>* __restrict__ Y, int M, int Nn, long K, long ld,
+                long kchunk, int S, int TM, int TN, cpx<double>* part) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lx = TM | 1, ly = TN | 1;
+  cpx<double>* xs = reinterpret_cast<cpx<double>*>(smem_raw);  // [2][TK][lx], then [2][TK][ly]
+  cpx<double>* ys = xs + 2 * TK * lx;
+  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+  const int sign = blockIdx.z / S, sp = blockIdx.z - sign * S;
+  const long k0 = sp * kchunk, k1 = min(K, k0 + kchunk), off = sign * K;
+  const int m = threadIdx.x / TN, n = threadIdx.x - m * TN;
+  const bool live = m < TM;
+  const int total = (TM + TN) * TK;
+  // element e of a step: row e / TK of X's TM rows, then Y's TN rows; column e % TK
+  auto fetch = [&](long kb, int e) {
+    const int r = e / TK;
+    const long k = kb + e % TK;
+    if (k >= k1) return mk<double>(0, 0);
+    if (r < TM) return m0 + r < M ? X[(size_t)(m0 + r) * ld + off + k] : mk<double>(0, 0);
+    return n0 + r - TM < Nn ? Y[(size_t)(n0 + r - TM) * ld + off + k] : mk<double>(0, 0);
+  };
+  auto store = [&](int buf, int e, cpx<double> v) {
+    const int r = e / TK, c = e % TK;
+    if (r < TM) xs[(buf * TK + c) * lx + r] = v;
+    else ys[(buf * TK + c) * ly + r - TM] = v;
+  };
+  for (int e = threadIdx.x; e < total; e += blockDim.x) store(0, e, fetch(k0, e));
+  __syncthreads();
+  cpx<double> acc = mk<double>(0, 0);
+  int buf = 0;
+  for (long kb = k0; kb < k1; kb += TK, buf ^= 1) {
+    const bool more = kb + TK < k1;
+    const int e0 = threadIdx.x;
+    cpx<double> nxt = mk<double>(0, 0);
+    if (more && e0 < total) nxt = fetch(kb + TK, e0);
+    if (live) {
+      const cpx<double>* xp = xs + buf * TK * lx + m;
+      const cpx<double>* yp = ys + buf * TK * ly + n;
+#pragma unroll
+      for (int c = 0; c < TK; ++c) {
+        const cpx<double> x = xp[c * lx], y = yp[c * ly];
+        acc.x = fma(x.y, y.y, fma(x.x, y.x, acc.x));
+        acc.y = fma(-x.y, y.x, fma(x.x, y.y, acc.y));
+      }
+    }
+    if (more) {
+      if (e0 < total) store(buf ^ 1, e0, nxt);
+      for (int e = e0 + blockDim.x; e < total; e += blockDim.x) store(buf ^ 1, e, fetch(kb + TK, e));
+    }
+    __syncthreads();
+  }
+  if (live && m0 + m < M && n0 + n < Nn) part[((size_t)blockIdx.z * M + m0 + m) * Nn + n0 + n] = acc;
+}
+
+// results[m][n]: C and A from the direct transforms (TU[m][n][4] = U~_m(-q_n), TV[n][m][4] = V~_n(p_m))
+// and the backgrounds' spinors with their time phases, B and D from the products' parts (splits in
+// order, times sBD).
+__global__ void k_pair_results(const cpx<double>* __restrict__ TU, const cpx<double>* __restrict__ TV,
+                               const cpx<double>* __restrict__ wU, const cpx<double>* __restrict__ wV,
+                               const cpx<double>* __restrict__ part, int S, double sBD, const double* normU,
+                               const double* normV, int n_e, int n_p, swf_result* res) {
+  const long MN = (long)n_e * n_p;
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < MN; i += (long)gridDim.x * blockDim.x) {
+    const long m = i / n_p, n = i % n_p;
+    cpx<double> C = mk<double>(0, 0), A = mk<double>(0, 0), B = mk<double>(0, 0), D = mk<double>(0, 0);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      out[((size_t)f * 4 + c) * g.N + j] = 0.5 * (a[c] + iE * h[c]);
-      out[((size_t)(n_f + f) * 4 + c) * g.N + j] = 0.5 * (a[c] - iE * h[c]);
+      C = C + cdot(TU[4 * i + c], wV[4 * n + c]);
+      A = A + cdot(wU[4 * m + c], TV[4 * (n * n_e + m) + c]);
     }
-  }
-}
-
-// results[m][n] from the four overlap matrices (B and D stacked: rows m and n_e + m).
-__global__ void k_pair_results(const cpx<double>* __restrict__ Cm, const cpx<double>* __restrict__ Am,
-                               const cpx<double>* __restrict__ BDm, const double* normU, const double* normV, int n_e,
-                               int n_p, swf_result* res) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_e * n_p; i += gridDim.x * blockDim.x) {
-    const int m = i / n_p, n = i % n_p;
-    const cpx<double> C = Cm[i], A = Am[i], B = BDm[(size_t)m * n_p + n], D = BDm[(size_t)(n_e + m) * n_p + n];
+    for (int s = 0; s < S; ++s) {
+      B = B + part[s * MN + i];
+      D = D + part[(S + s) * MN + i];
+    }
+    B = sBD * B;
+    D = sBD * D;
     swf_result o;
     o.amp[0] = C.x; o.amp[1] = C.y;
     o.amp[2] = D.x; o.amp[3] = D.y;
@@ -171,33 +269,88 @@ int sms() {
   return n;
 }
 
-// out = scale X^+ Y (M x Nn) with split K, through the part buffer.
-swf_status gemm_cn(swf_ctx* ctx, const cpx<double>* X, const cpx<double>* Y, int M, int Nn, long K, double scale,
-                   cpx<double>* out, const char* tag, cudaStream_t st) {
-  const int tiles = ((Nn + TN - 1) / TN) * ((M + TM - 1) / TM);
-  long S = std::max(1L, (2L * sms() + tiles - 1) / tiles);
-  S = std::min(S, std::max(1L, K / 256));
-  S = std::min(S, 1024L);
-  long kchunk = (K + S - 1) / S;
-  kchunk = (kchunk + TK - 1) / TK * TK;
-  S = (K + kchunk - 1) / kchunk;
-  void* part = nullptr;
-  swf_status s = ws_get(ctx, "pairs.part", sizeof(cpx<double>) * (size_t)S * M * Nn, &part);
-  if (s != SWF_OK) return s;
+// out[f][k][4] = dx^d sum_x psi_f(x) exp(-i kappa_k.x) for every field f and wave vector k.  One of two
+// orders: rows (y, z) first and then x, or x first and then the rows; the first contraction runs once
+// per distinct momentum of its axes, over the whole grid, so the order with fewer of those is taken
+// (the second is smaller by the length it leaves).  Fields go in chunks that keep the intermediate
+// below 256 MB.
+swf_status transform_many(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precision prec, const void* psi,
+                          const std::vector<double>& kappa, const std::string& tag, cpx<double>* out, cudaStream_t st) {
+  const int n_k = (int)(kappa.size() / 3);
+  const int nx = g.n[0], nrows = g.n[1] * g.n[2];
+  // distinct momenta along the axes of `mask`, and every wave vector's index among them
+  auto distinct = [&](int mask, std::vector<double>& vals, std::vector<int>& map) {
+    std::map<std::array<double, 3>, int> seen;
+    map.resize(n_k);
+    for (int k = 0; k < n_k; ++k) {
+      std::array<double, 3> key = {0, 0, 0};
+      for (int a = 0; a < 3; ++a)
+        if ((mask >> a & 1) && g.n[a] > 1) key[a] = kappa[3 * k + a];
+      auto it = seen.find(key);
+      if (it == seen.end()) {
+        it = seen.emplace(key, (int)seen.size()).first;
+        vals.insert(vals.end(), key.begin(), key.end());
+      }
+      map[k] = it->second;
+    }
+    return (int)seen.size();
+  };
+  std::vector<double> vx, vr;
+  std::vector<int> mx, mr;
+  const int Dx = distinct(1, vx, mx), Dr = distinct(6, vr, mr);
+  const double cost_rows = 4.0 * g.N * Dr + 4.0 * nx * n_k, cost_x = 4.0 * g.N * Dx + 4.0 * nrows * n_k;
+  const bool rows_first = cost_rows <= cost_x;
+  const int D = rows_first ? Dr : Dx, len1 = rows_first ? nrows : nx, len2 = rows_first ? nx : nrows;
+  const std::vector<double>& v1 = rows_first ? vr : vx;
+  const std::vector<int>& m1 = rows_first ? mr : mx;
+  const size_t per = (size_t)4 * D * len2 * 16;
+  const int fc = (int)std::max<size_t>(1, std::min<size_t>(n_f, ((size_t)256 << 20) / per));
+  void *pk, *pv, *pm, *t1, *t2, *G;
+  swf_status s;
+  if ((s = ws_get(ctx, tag + ".kappa", sizeof(double) * kappa.size(), &pk)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, tag + ".distinct", sizeof(double) * v1.size(), &pv)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, tag + ".map", sizeof(int) * n_k, &pm)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, tag + ".phase1", (size_t)D * len1 * 16, &t1)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, tag + ".phase2", (size_t)n_k * len2 * 16, &t2)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, "pairs.G", per * fc, &G)) != SWF_OK) return s;
+  cudaError_t e = cudaMemcpyAsync(pk, kappa.data(), sizeof(double) * kappa.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(pv, v1.data(), sizeof(double) * v1.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(pm, m1.data(), sizeof(int) * n_k, cudaMemcpyHostToDevice, st);
+  if (e != cudaSuccess) return cuda_status(e, "upload pair momenta");
+  const int ax1 = rows_first ? 6 : 1, ax2 = 7 - ax1;
   {
-    ProfScope ps(ctx, "k_gemm_cn", st);
-    k_gemm_cn<<<dim3((Nn + TN - 1) / TN, (M + TM - 1) / TM, (unsigned)S), 256, 0, st>>>(X, Y, M, Nn, K, kchunk,
-                                                                                        (cpx<double>*)part);
+    ProfScope ps(ctx, "k_phases", st);
+    k_phases<<<dim3((len1 + 127) / 128, D), 128, 0, st>>>((const double*)pv, D, g, ax1, len1, (cpx<double>*)t1);
+    k_phases<<<dim3((len2 + 127) / 128, n_k), 128, 0, st>>>((const double*)pk, n_k, g, ax2, len2, (cpx<double>*)t2);
   }
-  {
-    ProfScope ps(ctx, "k_sum_splits", st);
-    const long MN = (long)M * Nn;
-    k_sum_splits<<<(int)std::min((MN + 255) / 256, 4096L), 256, 0, st>>>((const cpx<double>*)part, (int)S, MN, scale,
-                                                                          out);
+  const double cell = g.dx[0] * g.dx[1] * g.dx[2];
+  const size_t elem = prec == SWF_C64 ? 8 : 16;
+  for (int f0 = 0; f0 < n_f; f0 += fc) {
+    const int nf = std::min(fc, n_f - f0);
+    const void* src = (const unsigned char*)psi + (size_t)f0 * 4 * g.N * elem;
+    {
+      ProfScope ps(ctx, "k_contract", st);
+      const dim3 grid(rows_first ? (nx + 31) / 32 : (nrows + 7) / 8, 4 * nf, (D + DB - 1) / DB);
+      const cpx<double>* tab = (const cpx<double>*)t1;
+      if (rows_first && prec == SWF_C64)
+        k_contract_rows<float><<<grid, 256, 0, st>>>((const cpx<float>*)src, tab, nrows, nx, D, (cpx<double>*)G);
+      else if (rows_first)
+        k_contract_rows<double><<<grid, 256, 0, st>>>((const cpx<double>*)src, tab, nrows, nx, D, (cpx<double>*)G);
+      else if (prec == SWF_C64)
+        k_contract_x<float><<<grid, 256, 0, st>>>((const cpx<float>*)src, tab, nrows, nx, D, (cpx<double>*)G);
+      else
+        k_contract_x<double><<<grid, 256, 0, st>>>((const cpx<double>*)src, tab, nrows, nx, D, (cpx<double>*)G);
+    }
+    ProfScope ps(ctx, "k_contract_last", st);
+    k_contract_last<<<dim3((n_k + 7) / 8, 4 * nf), 256, 0, st>>>((const cpx<double>*)G, (const cpx<double>*)t2,
+                                                                 (const int*)pm, len2, D, n_k, cell,
+                                                                 out + (size_t)f0 * n_k * 4);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_status(e, tag);
-  return SWF_OK;
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_status(e, "pair transforms");
+  // the tables above are the sources of asynchronous uploads
+  e = cudaStreamSynchronize(st);
+  return e == cudaSuccess ? SWF_OK : cuda_status(e, "pair transforms");
 }
 
 bool same_grid(const swf_grid& a, const swf_grid& b) {
@@ -252,97 +405,117 @@ extern "C" swf_status swf_pair_matrix(swf_ctx* ctx, int n_e, const swf_instance*
   const GridDesc g = make_grid(i0.grid);
   const long K = 4L * g.N;
   const size_t elem = prec == SWF_C64 ? 8 : 16;
+  const double t_in = i0.grid.t_in;
+  // spinors with their background's time phase at t_in (e^{i p0 t} of conj(U_back), e^{i q0 t} of V_back),
+  // and the wave vectors of the direct transforms
   std::vector<FieldDesc> fdU(n_e), fdV(n_p);
-  std::vector<pairs::Wave> wu(n_e), wv(n_p);
+  std::vector<double> wU(8 * (size_t)n_e), wV(8 * (size_t)n_p), kU(3 * (size_t)n_p), kV(3 * (size_t)n_e);
+  auto wave = [&](const double* mom, int spin, bool positron, double* w) {
+    double sp[8];
+    spinor_uv(mom, spin, positron, sp);
+    const double ph = (positron ? 1.0 : -1.0) * energy3(mom) * t_in, cs = std::cos(ph), sn = std::sin(ph);
+    for (int c = 0; c < 4; ++c) {
+      w[2 * c] = cs * sp[2 * c] - sn * sp[2 * c + 1];
+      w[2 * c + 1] = cs * sp[2 * c + 1] + sn * sp[2 * c];
+    }
+  };
   for (int m = 0; m < n_e; ++m) {
     fdU[m] = make_field_desc(electrons[m], 0);
-    spinor_uv(electrons[m].p, electrons[m].s, false, wu[m].w);
-    for (int a = 0; a < 3; ++a) wu[m].mom[a] = electrons[m].p[a];
-    wu[m].sgn = 1.0;
+    wave(electrons[m].p, electrons[m].s, false, &wU[8 * (size_t)m]);
+    for (int a = 0; a < 3; ++a) kV[3 * (size_t)m + a] = electrons[m].p[a];
   }
   for (int n = 0; n < n_p; ++n) {
     fdV[n] = make_field_desc(positrons[n], 1);
-    spinor_uv(positrons[n].q, positrons[n].r, true, wv[n].w);
-    for (int a = 0; a < 3; ++a) wv[n].mom[a] = positrons[n].q[a];
-    wv[n].sgn = -1.0;
+    wave(positrons[n].q, positrons[n].r, true, &wV[8 * (size_t)n]);
+    for (int a = 0; a < 3; ++a) kU[3 * (size_t)n + a] = -positrons[n].q[a];
   }
-  void *psiU, *psiV, *specU, *specV, *xU, *xV, *wU, *wV, *proj, *normU, *normV, *Cm, *Am, *BDm, *pw, *pku, *pres;
+  void *psiU, *psiV, *specU, *specV, *TU, *TV, *pwU, *pwV, *normU, *normV, *pku, *pres;
   if ((s = ws_get(ctx, "pairs.psiU", (size_t)n_e * K * elem, &psiU)) != SWF_OK) return s;
   if ((s = ws_get(ctx, "pairs.psiV", (size_t)n_p * K * elem, &psiV)) != SWF_OK) return s;
   if ((s = ws_get(ctx, "pairs.specU", (size_t)n_e * K * 16, &specU)) != SWF_OK) return s;
   if ((s = ws_get(ctx, "pairs.specV", (size_t)n_p * K * 16, &specV)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "pairs.xU", (size_t)n_e * K * 16, &xU)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "pairs.xV", (size_t)n_p * K * 16, &xV)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "pairs.waveU", (size_t)n_e * K * 16, &wU)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "pairs.waveV", (size_t)n_p * K * 16, &wV)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "pairs.proj", (size_t)2 * n_e * K * 16, &proj)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, "pairs.TU", (size_t)n_e * n_p * 64, &TU)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, "pairs.TV", (size_t)n_e * n_p * 64, &TV)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, "pairs.wU", (size_t)n_e * 64, &pwU)) != SWF_OK) return s;
+  if ((s = ws_get(ctx, "pairs.wV", (size_t)n_p * 64, &pwV)) != SWF_OK) return s;
   if ((s = ws_get(ctx, "pairs.normU", (size_t)n_e * 8, &normU)) != SWF_OK) return s;
   if ((s = ws_get(ctx, "pairs.normV", (size_t)n_p * 8, &normV)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "pairs.C", (size_t)n_e * n_p * 16, &Cm)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "pairs.A", (size_t)n_e * n_p * 16, &Am)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "pairs.BD", (size_t)2 * n_e * n_p * 16, &BDm)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "pairs.waves", sizeof(pairs::Wave) * (size_t)(n_e + n_p), &pw)) != SWF_OK) return s;
   if ((s = ws_get(ctx, "pairs.Ku", 3 * sizeof(double), &pku)) != SWF_OK) return s;
   if ((s = ws_get(ctx, "pairs.results", sizeof(swf_result) * (size_t)n_e * n_p, &pres)) != SWF_OK) return s;
   // one march per electron (U waves) and per positron (V waves), then their FP64 transforms
-  const double t_in = i0.grid.t_in;
   const int adaptive = (i0.flags & SWF_ADAPTIVE) ? 1 : 0;
   if ((s = march_fields(ctx, g, t_in, i0.grid.t_out, i0.grid.n_steps, n_e, fdU.data(), prec, psiU, st, adaptive)) != SWF_OK)
     return s;
   if ((s = march_fields(ctx, g, t_in, i0.grid.t_out, i0.grid.n_steps, n_p, fdV.data(), prec, psiV, st, adaptive)) != SWF_OK)
     return s;
-  if ((s = transform_fields(ctx, g, n_e, prec, psiU, (double2*)specU, st)) != SWF_OK) return s;
-  if ((s = transform_fields(ctx, g, n_p, prec, psiV, (double2*)specV, st)) != SWF_OK) return s;
+  if ((s = transform_fields(ctx, g, n_e, prec, psiU, (double2*)specU, st, true)) != SWF_OK) return s;
+  if ((s = transform_fields(ctx, g, n_p, prec, psiV, (double2*)specV, st, true)) != SWF_OK) return s;
   if ((s = field_norms(ctx, g, n_e, prec, psiU, (double*)normU, st)) != SWF_OK) return s;
   if ((s = field_norms(ctx, g, n_p, prec, psiV, (double*)normV, st)) != SWF_OK) return s;
-  cudaError_t e = cudaMemcpyAsync(pw, wu.data(), sizeof(pairs::Wave) * n_e, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync((pairs::Wave*)pw + n_e, wv.data(), sizeof(pairs::Wave) * n_p, cudaMemcpyHostToDevice, st);
+  if ((s = pairs::transform_many(ctx, g, n_e, prec, psiU, kU, "pairs.U", (cpx<double>*)TU, st)) != SWF_OK) return s;
+  if ((s = pairs::transform_many(ctx, g, n_p, prec, psiV, kV, "pairs.V", (cpx<double>*)TV, st)) != SWF_OK) return s;
+  cudaError_t e = cudaMemcpyAsync(pwU, wU.data(), (size_t)n_e * 64, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(pwV, wV.data(), (size_t)n_p * 64, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(pku, fdU[0].K, 3 * sizeof(double), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_status(e, "upload pair tables");
-  const int gx = (int)std::min<long>((g.N + 255) / 256, 1024);
   {
-    ProfScope ps(ctx, "k_widen", st);
-    const size_t nu = (size_t)n_e * K, nv = (size_t)n_p * K;
-    const int bu = (int)std::min<size_t>((nu + 255) / 256, 8192), bv = (int)std::min<size_t>((nv + 255) / 256, 8192);
-    if (prec == SWF_C64) {
-      pairs::k_widen<float><<<bu, 256, 0, st>>>((const cpx<float>*)psiU, (cpx<double>*)xU, nu);
-      pairs::k_widen<float><<<bv, 256, 0, st>>>((const cpx<float>*)psiV, (cpx<double>*)xV, nv);
-    } else {
-      pairs::k_widen<double><<<bu, 256, 0, st>>>((const cpx<double>*)psiU, (cpx<double>*)xU, nu);
-      pairs::k_widen<double><<<bv, 256, 0, st>>>((const cpx<double>*)psiV, (cpx<double>*)xV, nv);
+    ProfScope ps(ctx, "k_energy_amps", st);
+    const int nb = (g.N + 255) / 256;
+    const int fc = std::max(1, 8 * nb / (4 * pairs::sms()));  // fields per thread: enough blocks to fill the SMs
+    for (int k = 0; k < 2; ++k) {
+      const int n = k ? n_p : n_e;
+      const int f = std::min(n, std::max(fc, (n + 65534) / 65535));
+      pairs::k_energy_amps<<<dim3(nb, (n + f - 1) / f), 256, 0, st>>>((cpx<double>*)(k ? specV : specU), g,
+                                                                       (const double*)pku, n, f);
     }
   }
-  {
-    ProfScope ps(ctx, "k_plane_waves", st);
-    pairs::k_plane_waves<<<dim3(gx, n_e), 256, 0, st>>>((const pairs::Wave*)pw, g, t_in, (cpx<double>*)wU);
-    pairs::k_plane_waves<<<dim3(gx, n_p), 256, 0, st>>>((const pairs::Wave*)pw + n_e, g, t_in, (cpx<double>*)wV);
+  // tiles as even as they come, k split so that the blocks fill the SMs
+  const int TM = (n_e + (n_e + pairs::kTile - 1) / pairs::kTile - 1) / ((n_e + pairs::kTile - 1) / pairs::kTile);
+  const int TN = (n_p + (n_p + pairs::kTile - 1) / pairs::kTile - 1) / ((n_p + pairs::kTile - 1) / pairs::kTile);
+  const int tx = (n_p + TN - 1) / TN, ty = (n_e + TM - 1) / TM;
+  const int thr = (TM * TN + 31) & ~31;
+  const size_t smem = (size_t)2 * pairs::TK * ((TM | 1) + (TN | 1)) * 16;
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pairs::k_pair_products, thr, smem) != cudaSuccess || per_sm < 1) {
+    cudaGetLastError();
+    per_sm = 1;
   }
+  const long Ks = 2L * g.N;
+  // the split whose blocks fill whole waves best (at least 256 values of k each; fewer splits on a tie)
+  const long slots = (long)per_sm * pairs::sms(), tiles = 2L * tx * ty;
+  long S = 1;
+  double best = 0.0;
+  for (long c = 1; c <= std::min(64L, std::max(1L, Ks / 256)); ++c) {
+    const double fill = (double)(tiles * c) / (double)((tiles * c + slots - 1) / slots * slots);
+    if (fill > best + 0.01) {
+      best = fill;
+      S = c;
+    }
+  }
+  const long kchunk = ((Ks + S - 1) / S + pairs::TK - 1) / pairs::TK * pairs::TK;
+  S = (Ks + kchunk - 1) / kchunk;
+  void* part = nullptr;
+  if ((s = ws_get(ctx, "pairs.part", (size_t)2 * S * n_e * n_p * 16, &part)) != SWF_OK) return s;
   {
-    ProfScope ps(ctx, "k_project", st);
-    pairs::k_project<<<dim3(gx, n_e), 256, 0, st>>>((const cpx<double>*)specU, g, (const double*)pku, n_e,
-                                                    (cpx<double>*)proj);
+    ProfScope ps(ctx, "k_pair_products", st);
+    pairs::k_pair_products<<<dim3(tx, ty, (unsigned)(2 * S)), thr, smem, st>>>(
+        (const cpx<double>*)specU, (const cpx<double>*)specV, n_e, n_p, Ks, K, kchunk, (int)S, TM, TN, (cpx<double>*)part);
   }
   double vol = 1.0;
   for (int a = 0; a < 3; ++a)
     if (g.n[a] > 1) vol *= g.L[a];
   const double cell = g.dx[0] * g.dx[1] * g.dx[2];
-  if ((s = pairs::gemm_cn(ctx, (const cpx<double>*)xU, (const cpx<double>*)wV, n_e, n_p, K, cell, (cpx<double>*)Cm,
-                          "pair overlaps C", st)) != SWF_OK)
-    return s;
-  if ((s = pairs::gemm_cn(ctx, (const cpx<double>*)wU, (const cpx<double>*)xV, n_e, n_p, K, cell, (cpx<double>*)Am,
-                          "pair overlaps A", st)) != SWF_OK)
-    return s;
-  if ((s = pairs::gemm_cn(ctx, (const cpx<double>*)proj, (const cpx<double>*)specV, 2 * n_e, n_p, K, 1.0 / vol,
-                          (cpx<double>*)BDm, "pair overlaps B, D", st)) != SWF_OK)
-    return s;
   {
     ProfScope ps(ctx, "k_pair_results", st);
-    pairs::k_pair_results<<<(n_e * n_p + 255) / 256, 256, 0, st>>>((const cpx<double>*)Cm, (const cpx<double>*)Am,
-                                                                   (const cpx<double>*)BDm, (const double*)normU,
-                                                                   (const double*)normV, n_e, n_p, (swf_result*)pres);
+    const long MN = (long)n_e * n_p;
+    pairs::k_pair_results<<<(unsigned)std::min((MN + 127) / 128, 65535L), 128, 0, st>>>(
+        (const cpx<double>*)TU, (const cpx<double>*)TV, (const cpx<double>*)pwU, (const cpx<double>*)pwV,
+        (const cpx<double>*)part, (int)S, cell * cell / vol, (const double*)normU, (const double*)normV, n_e, n_p,
+        (swf_result*)pres);
   }
-  e = cudaMemcpyAsync(results, pres, sizeof(swf_result) * (size_t)n_e * n_p, cudaMemcpyDeviceToHost, st);
+  e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(results, pres, sizeof(swf_result) * (size_t)n_e * n_p, cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return cuda_status(e, "download pair results");
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_status(e, "pair matrix");

@@ -90,7 +90,7 @@ k_fft_axis(const cpx<Rin>* in, cpx<double>* out, GridDesc g, int axis, const __g
 // q = -kappa_j (trivial axes: kappa = K of the electron wave).  A thread holds the two spinors of one
 // mode, phase included, for fc fields (they depend on the mode and K alone; a field with another K has
 // its own): the square roots and the sine and cosine in FP64 are about four times a field's products
-// (16 fields of 256^2: 309 -> 149 us).
+// (16 fields of 256^2: 309 -> 108 us).
 __global__ void __launch_bounds__(kT) k_c_spectrum(const cpx<double>* __restrict__ spec, const FieldDesc* fd, GridDesc g,
                                                    int F, int fc, double t_in, cpx<double>* c_out, double* prob) {
   const int f0 = blockIdx.y * fc, f1 = min(F, f0 + fc);
@@ -128,8 +128,8 @@ __global__ void __launch_bounds__(kT) k_c_spectrum(const cpx<double>* __restrict
       cpx<double> acc = mk<double>(0, 0);
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        acc.x += uc[a].x * v[ir][2 * a] + uc[a].y * v[ir][2 * a + 1];
-        acc.y += uc[a].x * v[ir][2 * a + 1] - uc[a].y * v[ir][2 * a];
+        acc.x = fma(uc[a].y, v[ir][2 * a + 1], fma(uc[a].x, v[ir][2 * a], acc.x));
+        acc.y = fma(-uc[a].y, v[ir][2 * a], fma(uc[a].x, v[ir][2 * a + 1], acc.y));
       }
       const size_t e = ((size_t)f * 2 + ir) * g.N + j;
       if (c_out) c_out[e] = acc;
