@@ -896,33 +896,39 @@ struct ErrWeights {
 };
 
 // part[f][b] = sum over block b's entries of field f of (|e| / (atol + rtol max(|y|, |y_new|)))^2,
-// e = h sum_i (b_i - b*_i) k_i, in FP64 (fixed order inside the block).
+// e = h sum_i (b_i - b*_i) k_i, in FP64 (fixed order inside the block).  FP64 operations bound it, so
+// one square root serves both norms (of the larger square), the sums are chains of fused
+// multiply-adds, and the blocks are small enough (four entries a thread) to load all SMs alike: six
+// fields of 240 x 135 took 137 us with two roots and 16 entries a thread.
+constexpr int kErrThreads = 256;
+static int error_blocks(size_t per_field) { return (int)std::min<size_t>((per_field + 4 * kErrThreads - 1) / (4 * kErrThreads), 4096); }
 template <typename R>
-__global__ void __launch_bounds__(256) k_step_error(const cpx<R>* __restrict__ y, const cpx<R>* __restrict__ ynew,
-                                                    const cpx<R>* k0, const cpx<R>* k1, const cpx<R>* k2,
-                                                    const cpx<R>* k3, const cpx<R>* k4, const cpx<R>* k5,
-                                                    const cpx<R>* k6, ErrWeights W, const StepControl* ctl,
-                                                    size_t per_field, double* part) {
-  __shared__ double red[8];
+__global__ void __launch_bounds__(kErrThreads) k_step_error(const cpx<R>* __restrict__ y, const cpx<R>* __restrict__ ynew,
+                                                            const cpx<R>* __restrict__ k0, const cpx<R>* __restrict__ k2,
+                                                            const cpx<R>* __restrict__ k3, const cpx<R>* __restrict__ k4,
+                                                            const cpx<R>* __restrict__ k5, const cpx<R>* __restrict__ k6,
+                                                            ErrWeights W, const StepControl* ctl, size_t per_field,
+                                                            double* part) {
+  __shared__ double red[kErrThreads / 32];
   if (ctl->done) return;
   const int f = blockIdx.y;
   const double h = ctl->h, rtol = ctl->rtol, atol = ctl->atol;
-  const cpx<R>* ks[7] = {k0, k1, k2, k3, k4, k5, k6};
+  const cpx<R>* ks[6] = {k0, k2, k3, k4, k5, k6};  // the second weight is zero
+  const double w[6] = {W.db[0], W.db[2], W.db[3], W.db[4], W.db[5], W.db[6]};
   double acc = 0.0;
   const size_t off = (size_t)f * per_field;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < per_field; i += (size_t)gridDim.x * blockDim.x) {
+  for (size_t i = blockIdx.x * (size_t)kErrThreads + threadIdx.x; i < per_field; i += (size_t)gridDim.x * kErrThreads) {
     double ex = 0.0, ey = 0.0;
 #pragma unroll
-    for (int j = 0; j < 7; ++j) {
-      if (W.db[j] == 0.0) continue;
+    for (int j = 0; j < 6; ++j) {
       const cpx<R> kv = ks[j][off + i];
-      ex += W.db[j] * (double)kv.x;
-      ey += W.db[j] * (double)kv.y;
+      ex = fma(w[j], (double)kv.x, ex);
+      ey = fma(w[j], (double)kv.y, ey);
     }
-    const cpx<R> a = y[off + i], b = ynew[off + i];
-    const double ya = sqrt((double)a.x * a.x + (double)a.y * a.y), yb = sqrt((double)b.x * b.x + (double)b.y * b.y);
-    const double sc = atol + rtol * fmax(ya, yb);
-    acc += h * h * (ex * ex + ey * ey) / (sc * sc);
+    const cpx<double> a = cvt<double>(y[off + i]), b = cvt<double>(ynew[off + i]);
+    const double m = fmax(fma(a.x, a.x, a.y * a.y), fma(b.x, b.x, b.y * b.y));
+    const double sc = fma(rtol, sqrt(m), atol);
+    acc += fma(ex, ex, ey * ey) / (sc * sc);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -930,24 +936,34 @@ __global__ void __launch_bounds__(256) k_step_error(const cpx<R>* __restrict__ y
   __syncthreads();
   if (threadIdx.x == 0) {
     double sum = 0.0;
-    for (int w = 0; w < 8; ++w) sum += red[w];
-    part[(size_t)f * gridDim.x + blockIdx.x] = sum;
+    for (int w8 = 0; w8 < kErrThreads / 32; ++w8) sum += red[w8];
+    part[(size_t)f * gridDim.x + blockIdx.x] = h * h * sum;
   }
 }
 
-// One thread: err = max over fields of the RMS scaled error; accept when err <= 1 (and finite);
-// next step h min(10, max(0.2, 0.9 err^(-1/5))), clamped so as not to pass t_in.
-__global__ void k_step_control(StepControl* ctl, const double* part, int nb, int F, double count) {
-  if (threadIdx.x != 0 || ctl->done) {
+// err = max over fields of the RMS scaled error (a warp per field in turn, lanes in a fixed order);
+// accept when err <= 1 (and finite); next step h min(10, max(0.2, 0.9 err^(-1/5))), clamped so as not
+// to pass t_in.  One block; one thread of it took 19 us to add 200 parts.
+__global__ void __launch_bounds__(256) k_step_control(StepControl* ctl, const double* __restrict__ part, int nb, int F,
+                                                      double count) {
+  __shared__ double s_err[8];
+  if (ctl->done) {
     if (threadIdx.x == 0) ctl->ok = 0;
     return;
   }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double err = 0.0;
-  for (int f = 0; f < F; ++f) {
+  for (int f = warp; f < F; f += 8) {
     double sum = 0.0;
-    for (int b = 0; b < nb; ++b) sum += part[(size_t)f * nb + b];
+    for (int b = lane; b < nb; b += 32) sum += part[(size_t)f * nb + b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     err = fmax(err, sqrt(sum / count));
   }
+  if (lane == 0) s_err[warp] = err;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 0; w < 8; ++w) err = fmax(err, s_err[w]);
   if (!(err == err) || isinf(err)) {  // non-finite: stop
     ctl->ok = 0;
     ctl->failed = 1;
@@ -1148,7 +1164,7 @@ static swf_status march_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double t_
     std::snprintf(nm, sizeof nm, "march.k%d", i);
     if ((s = ws_get(ctx, nm, state, &pk[i])) != SWF_OK) return s;
   }
-  const int nbe = (int)std::max<size_t>(1, std::min<size_t>((per_field + 4095) / 4096, 64));
+  const int nbe = error_blocks(per_field);
   if ((s = ws_get(ctx, "march.ctl", sizeof(StepControl), &pctl)) != SWF_OK) return s;
   if ((s = ws_get(ctx, "march.err_part", sizeof(double) * (size_t)nbe * F, &ppart)) != SWF_OK) return s;
   cudaError_t e = cudaMemsetAsync(py, 0, state, st);
@@ -1220,14 +1236,13 @@ static swf_status march_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double t_
     }
     {
       ProfScope ps(ctx, "k_step_error", st);
-      k_step_error<R><<<dim3(nbe, F), 256, 0, st>>>(
-          (const cpx<R>*)py, (const cpx<R>*)pyn, (const cpx<R>*)pk[0], (const cpx<R>*)pk[1], (const cpx<R>*)pk[2],
-          (const cpx<R>*)pk[3], (const cpx<R>*)pk[4], (const cpx<R>*)pk[5], (const cpx<R>*)pk[6], W, ctl, per_field,
-          (double*)ppart);
+      k_step_error<R><<<dim3(nbe, F), kErrThreads, 0, st>>>(
+          (const cpx<R>*)py, (const cpx<R>*)pyn, (const cpx<R>*)pk[0], (const cpx<R>*)pk[2], (const cpx<R>*)pk[3],
+          (const cpx<R>*)pk[4], (const cpx<R>*)pk[5], (const cpx<R>*)pk[6], W, ctl, per_field, (double*)ppart);
     }
     {
       ProfScope ps(ctx, "k_step_control", st);
-      k_step_control<<<1, 32, 0, st>>>(ctl, (const double*)ppart, nbe, F, (double)per_field);
+      k_step_control<<<1, 256, 0, st>>>(ctl, (const double*)ppart, nbe, F, (double)per_field);
     }
     {
       ProfScope ps(ctx, "k_step_accept", st);
@@ -2573,7 +2588,7 @@ static swf_status march_bw_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double
     std::snprintf(nm, sizeof nm, "march.k%d", i);
     if ((s = ws_get(ctx, nm, state, &pk[i])) != SWF_OK) return s;
   }
-  const int nbe = (int)std::max<size_t>(1, std::min<size_t>((per_field + 4095) / 4096, 64));
+  const int nbe = error_blocks(per_field);
   const int nb = std::max(1, std::min((g.N + 1023) / 1024, (4 * sm_count() + n_inst - 1) / n_inst));
   const size_t nacc = (size_t)3 * nb * n_inst;
   if ((s = ws_get(ctx, "march.ctl", sizeof(StepControl), &pctl)) != SWF_OK) return s;
@@ -2681,14 +2696,13 @@ static swf_status march_bw_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double
     }
     {
       ProfScope ps(ctx, "k_step_error", st);
-      k_step_error<R><<<dim3(nbe, F), 256, 0, st>>>(
-          (const cpx<R>*)py, (const cpx<R>*)pyn, (const cpx<R>*)pk[0], (const cpx<R>*)pk[1], (const cpx<R>*)pk[2],
-          (const cpx<R>*)pk[3], (const cpx<R>*)pk[4], (const cpx<R>*)pk[5], (const cpx<R>*)pk[6], W, ctl, per_field,
-          (double*)ppart);
+      k_step_error<R><<<dim3(nbe, F), kErrThreads, 0, st>>>(
+          (const cpx<R>*)py, (const cpx<R>*)pyn, (const cpx<R>*)pk[0], (const cpx<R>*)pk[2], (const cpx<R>*)pk[3],
+          (const cpx<R>*)pk[4], (const cpx<R>*)pk[5], (const cpx<R>*)pk[6], W, ctl, per_field, (double*)ppart);
     }
     {
       ProfScope ps(ctx, "k_step_control", st);
-      k_step_control<<<1, 32, 0, st>>>(ctl, (const double*)ppart, nbe, F, (double)per_field);
+      k_step_control<<<1, 256, 0, st>>>(ctl, (const double*)ppart, nbe, F, (double)per_field);
     }
     {
       ProfScope ps(ctx, "k_step_accept", st);
