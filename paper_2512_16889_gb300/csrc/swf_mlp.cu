@@ -5,10 +5,8 @@
 //   L = mean_b [ (y_b - mu_b)^2 exp(-l_b) + l_b ] / 2.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
-#include <map>
-#include <cstring>
-#include <string>
 #include <vector>
 
 #include "swf_internal.h"
@@ -25,24 +23,6 @@ __host__ __device__ constexpr int n_params() {
   for (int l = 0; l < NL; ++l) n += DIN[l] * DOUT[l] + DOUT[l];
   return n;
 }
-
-// ---------------------------------------------------------------- BF16 GEMM (FP32 accumulate)
-// C(m, n) = sum_k A(m, k) B(k, n); element (i, j) of a matrix X at X[i * sr + j * sc].
-struct Mat {
-  const __nv_bfloat16* p;
-  long sr, sc;
-};
-
-enum Epi { EPI_FWD_HIDDEN = 0, EPI_FWD_OUT = 1, EPI_DX = 2, EPI_DW = 3 };
-
-struct EpiArgs {
-  int mode;
-  const float* bias;          // FWD: [N]
-  float* z;                   // FWD: pre-activation out [M][N]; DW: gradient out [M][N]
-  __nv_bfloat16* act;         // FWD_HIDDEN: bf16 GELU(z) [M][N]; DX: bf16 dZ of the previous layer
-  float* dz32;                // DX: fp32 dZ of the previous layer [M][N]
-  const float* zprev;         // DX: pre-activation of the previous layer [M][N]
-};
 
 // The normal distribution function Phi(x) = (1 + erf(x / sqrt 2)) / 2 and the density phi(x),
 // with erf from Abramowitz and Stegun's formula 7.1.26 (Hastings' rational approximation):
@@ -78,157 +58,390 @@ __global__ void k_gelu_eval(const float* __restrict__ x, int n, float* __restric
   }
 }
 
-constexpr int TM = 64, TN = 64, TK = 16, SP = 24;  // tile, k step, padded smem row (bf16)
+// ---------------------------------------------------------------- training
+// One step is three launches: k_train_rows takes 16 rows of the batch through the network and back
+// (forward, dL/dz of every layer), k_train_dw forms the gradients and the loss, k_train_update applies
+// Adam.  Operands are BF16 on the tensor cores (mma.sync m16n8k16, FP32
+// accumulation in ascending k): a batch of 256 is 16 row blocks of 256 x 256 layers, far below what a
+// tcgen05 tile needs to fill (M = 128), and what bounds it is the chain of layers and the launches, not
+// the tensor rate.  A batch of 256 takes 33 us a step and one of 4096 101 us; as 25 kernels on 64 x 64
+// tiles, each waiting on two-byte loads of its operands, they took 480 and 3170 us.  Every sum runs in
+// the order it had there (ascending k and rows), so the results are the same bits.
+namespace tr {
 
-__device__ __forceinline__ uint32_t ld32(const __nv_bfloat16* p) { return *reinterpret_cast<const uint32_t*>(p); }
+constexpr int ROWS = 16;         // rows per block of k_train_rows: one m16 tile
+constexpr int THREADS = 512;     // 16 warps, warp w owns columns 16 w .. 16 w + 15 of every hidden layer
+constexpr int AST = 264;         // bf16 row stride of an operand tile (528 bytes: odd in 16-byte units)
+constexpr int TILE = 32;         // weight-gradient tile
+constexpr int CHUNK = 64;        // rows per stage of its ring
 
-__global__ void __launch_bounds__(128) k_gemm(Mat A, Mat B, int M, int N, int K, EpiArgs E) {
-  __shared__ __align__(16) __nv_bfloat16 As[TM][SP];   // [m][k]
-  __shared__ __align__(16) __nv_bfloat16 Bs[TN][SP];   // [n][k]
-  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-  const int g = lane >> 2, t4 = lane & 3;
-  float acc[2][4][4];
+// First weight of layer l in the parameter array, first bias after its weights.
+__host__ __device__ constexpr int nweights(int l) { return l == 0 ? 6 * 256 : l < 4 ? 256 * 256 : 2 * 256; }
+__host__ __device__ constexpr int woff(int l) { return l == 0 ? 0 : 7 * 256 + (l - 1) * 257 * 256; }
+__host__ __device__ constexpr int boff(int l) { return woff(l) + nweights(l); }
+
+// Weights of layers 1-3 in the order in which a lane of mma.m16n8k16 holds its B operand, for the
+// forward pass (column n, reduction k) and the backward pass (column k, reduction n): per column tile
+// of 8 and pair of k16 steps, 32 lanes of 8 bf16 (16 bytes).  col, red: column and reduction index.
+__host__ __device__ __forceinline__ int frag_index(int col, int red) {
+  const int nt = col >> 3, g = col & 7, ks = red >> 4, r = red & 15;
+  const int t = (r & 7) >> 1, j = (r & 1) + ((r >> 3) << 1);
+  return ((nt * 8 + (ks >> 1)) * 32 + g * 4 + t) * 8 + (ks & 1) * 4 + j;
+}
+
+__device__ __forceinline__ void mma(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm(uint32_t* r, const __nv_bfloat16* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
+}
+__device__ __forceinline__ void ldsm_t(uint32_t* r, const __nv_bfloat16* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// What the three kernels hand on, rows padded to ROWS with zero dL/dz.
+struct Bufs {
+  __nv_bfloat16* act[4];  // [rows][256]: outputs of hidden layers 0..3 (inputs of layers 1..4)
+  __nv_bfloat16* dz[4];   // [rows][256]: dL/dz of hidden layers 0..3
+  __nv_bfloat16* xin;     // [rows][8]: standardised inputs
+  __nv_bfloat16* dzo;     // [rows][2]: dL/dz of the output layer
+  float* dz32[4];         // the same before rounding (bias gradients)
+  float* dzo32;
+  float* zo;              // [rows][2]: the network's outputs
+};
+
+// B operands of one 256 x 256 layer for this warp's two column tiles: 16 loads of 16 bytes per lane,
+// issued before the barrier that the previous layer's results need.
+__device__ __forceinline__ void load_frags(uint4* b, const __nv_bfloat16* __restrict__ pack, int warp, int lane) {
+  const uint4* p = reinterpret_cast<const uint4*>(pack) + (size_t)(2 * warp) * 8 * 32 + lane;
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < 16; ++i) b[i] = __ldg(p + i * 32);
+}
+// acc (two column tiles) = A (16 rows in shared memory) times the loaded operands
+__device__ __forceinline__ void layer_mma(float acc[2][4], const __nv_bfloat16* sa, const uint4* b, int lane) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+  for (int j = 0; j < 2; ++j)
 #pragma unroll
-      for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.f;
-  const __nv_bfloat16 zero = __float2bfloat16(0.f);
-  for (int k0 = 0; k0 < K; k0 += TK) {
-    for (int e = threadIdx.x; e < TM * TK; e += blockDim.x) {
-      const int r = e / TK, c = e % TK;
-      const int m = m0 + r, k = k0 + c;
-      As[r][c] = (m < M && k < K) ? A.p[m * A.sr + k * A.sc] : zero;
-      const int n = n0 + r;
-      Bs[r][c] = (n < N && k < K) ? B.p[k * B.sr + n * B.sc] : zero;
+    for (int r = 0; r < 4; ++r) acc[j][r] = 0.f;
+  const __nv_bfloat16* p = sa + (lane & 15) * AST + (lane >> 4) * 8;
+#pragma unroll
+  for (int ks = 0; ks < 16; ++ks) {
+    uint32_t a[4];
+    ldsm(a, p + ks * 16);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const uint4 w = b[j * 8 + (ks >> 1)];
+      if (ks & 1) mma(acc[j], a, w.z, w.w);
+      else mma(acc[j], a, w.x, w.y);
     }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int ra = wm + 16 * i;
-      uint32_t a0 = ld32(&As[ra + g][2 * t4]), a1 = ld32(&As[ra + g + 8][2 * t4]);
-      uint32_t a2 = ld32(&As[ra + g][2 * t4 + 8]), a3 = ld32(&As[ra + g + 8][2 * t4 + 8]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int nb = wn + 8 * j;
-        uint32_t b0 = ld32(&Bs[nb + g][2 * t4]), b1 = ld32(&Bs[nb + g][2 * t4 + 8]);
-        asm volatile(
-            "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-            "{%0, %1, %2, %3};"
-            : "+f"(acc[i][j][0]), "+f"(acc[i][j][1]), "+f"(acc[i][j][2]), "+f"(acc[i][j][3])
-            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int m = m0 + wm + 16 * i + g + (r >> 1) * 8;
-        const int n = n0 + wn + 8 * j + 2 * t4 + (r & 1);
-        if (m >= M || n >= N) continue;
-        const float v = acc[i][j][r];
-        const long o = (long)m * N + n;
-        if (E.mode == EPI_FWD_HIDDEN) {
-          const float z = v + E.bias[n];
-          E.z[o] = z;
-          E.act[o] = __float2bfloat16(gelu(z));
-        } else if (E.mode == EPI_FWD_OUT) {
-          E.z[o] = v + E.bias[n];
-        } else if (E.mode == EPI_DX) {
-          const float d = v * gelu_grad(E.zprev[o]);
-          E.dz32[o] = d;
-          E.act[o] = __float2bfloat16(d);
-        } else {
-          E.z[o] = v;
-        }
-      }
-}
-
-// ---------------------------------------------------------------- small kernels
-__global__ void k_set_hyper(float* hyper, float lr, float c1, float c2) {
-  hyper[0] = lr;
-  hyper[1] = c1;
-  hyper[2] = c2;
-}
-
-// network input: standardised features, x' = (x - shift) * scale per feature
-__global__ void k_inputs(const float* x, const float* shift, const float* scale, __nv_bfloat16* y, long n) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const int f = (int)(i % 6);
-    y[i] = __float2bfloat16((x[i] - shift[f]) * scale[f]);
   }
 }
 
-// network output in the target's units: mu = mu'/ys + y0, log sigma^2 = l' - 2 ln ys
-__global__ void k_outputs(const float* z, float y0, float ys, float* out, int B) {
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x) {
-    out[2 * b] = z[2 * b] / ys + y0;
-    out[2 * b + 1] = z[2 * b + 1] - 2.0f * logf(ys);
+// 16 rows: forward, Gaussian NLL on the standardised target y' = (y - y0) ys (loss: mean over the batch),
+// backward.  Pre-activations stay in registers: the thread that holds columns 16 warp + 8 j + 2 t (+ 1)
+// of rows g, g + 8 in the forward pass holds the same elements of dL/dz in the backward pass.
+__global__ void __launch_bounds__(THREADS, 1)
+k_train_rows(const float* __restrict__ x, const float* __restrict__ y, int B, const __nv_bfloat16* __restrict__ wbf,
+             const __nv_bfloat16* __restrict__ fpack, const __nv_bfloat16* __restrict__ bpack,
+             const float* __restrict__ params, const float* __restrict__ shift, const float* __restrict__ scale, float y0,
+             float ys, Bufs W) {
+  __shared__ __align__(16) __nv_bfloat16 sA[2][ROWS * AST];
+  __shared__ uint32_t sDz[ROWS];   // (dmu, dl) of a row in bf16
+  __shared__ float sBias[4][256];
+  __shared__ uint32_t sX[ROWS][4];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int row0 = blockIdx.x * ROWS;
+  const int col = 16 * warp + 2 * t;  // first column of tile j: col + 8 j
+  uint4 b[16];
+  load_frags(b, fpack, warp, lane);
+  for (int i = tid; i < 4 * 256; i += THREADS) sBias[i >> 8][i & 255] = params[boff(i >> 8) + (i & 255)];
+  if (tid < ROWS * 4) {  // standardised inputs x' = (x - shift) scale, features 6 and 7 zero
+    const int r = tid >> 2, f = 2 * (tid & 3);
+    float v[2] = {0.f, 0.f};
+    if (row0 + r < B && f < 6)
+      for (int u = 0; u < 2; ++u) v[u] = (x[(size_t)(row0 + r) * 6 + f + u] - shift[f + u]) * scale[f + u];
+    const uint32_t w = pack2(v[0], v[1]);
+    sX[r][tid & 3] = w;
+    reinterpret_cast<uint32_t*>(W.xin)[(size_t)(row0 + r) * 4 + (tid & 3)] = w;
   }
-}
-
-__global__ void k_to_bf16(const float* x, __nv_bfloat16* y, long n) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    y[i] = __float2bfloat16(x[i]);
-}
-
-// Gaussian NLL of the two output heads on the standardised target y' = (y - y0) ys: loss (mean
-// over the batch) and dL/d(mu', l').
-__global__ void k_nll(const float* out, const float* y, float y0, float ys, int B, float* dz32, __nv_bfloat16* dz16,
-                      float* loss) {
-  __shared__ float red[256];
-  float acc = 0.f;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    const float mu = out[2 * b], l = out[2 * b + 1];
-    const float r = (y[b] - y0) * ys - mu, w = __expf(-l);
-    acc += 0.5f * (r * r * w + l);
-    const float dmu = -r * w / B, dl = 0.5f * (1.0f - r * r * w) / B;
-    dz32[2 * b] = dmu;
-    dz32[2 * b + 1] = dl;
-    dz16[2 * b] = __float2bfloat16(dmu);
-    dz16[2 * b + 1] = __float2bfloat16(dl);
-  }
-  red[threadIdx.x] = acc;
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+  float z[4][2][4];
+  // hidden layer l's outputs from its pre-activations: to the next operand tile and to memory
+  auto activate = [&](int l, int buf) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int c = col + 8 * j;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        z[l][j][2 * h] += sBias[l][c];
+        z[l][j][2 * h + 1] += sBias[l][c + 1];
+        const uint32_t w = pack2(gelu(z[l][j][2 * h]), gelu(z[l][j][2 * h + 1]));
+        *reinterpret_cast<uint32_t*>(&sA[buf][(g + 8 * h) * AST + c]) = w;
+        *reinterpret_cast<uint32_t*>(W.act[l] + (size_t)(row0 + g + 8 * h) * 256 + c) = w;
+      }
+    }
+  };
+  {  // layer 0: one k16 step, features beyond 6 are zero
+    uint32_t a[4] = {sX[g][t], sX[g + 8][t], 0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) z[0][j][r] = 0.f;
+      const int n = 16 * warp + 8 * j + g;
+      const uint32_t b0 = t < 3 ? *reinterpret_cast<const uint32_t*>(wbf + woff(0) + n * 6 + 2 * t) : 0u;
+      mma(z[0][j], a, b0, 0u);
+    }
+    activate(0, 0);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int l = 1; l < 4; ++l) {
+    layer_mma(z[l], sA[(l - 1) & 1], b, lane);
+    if (l < 3) load_frags(b, fpack + (size_t)l * 65536, warp, lane);
+    activate(l, l & 1);
     __syncthreads();
   }
-  if (threadIdx.x == 0 && loss) *loss = red[0] / B;
+  load_frags(b, bpack + (size_t)2 * 65536, warp, lane);  // layer 3's, for the backward pass
+  if (warp == 0) {  // output layer and loss
+    float o[4] = {0.f, 0.f, 0.f, 0.f};
+    const __nv_bfloat16* p = sA[1] + (lane & 15) * AST + (lane >> 4) * 8;
+    const uint32_t* w4 = reinterpret_cast<const uint32_t*>(wbf + woff(4) + g * 256);
+#pragma unroll
+    for (int ks = 0; ks < 16; ++ks) {
+      uint32_t a[4];
+      ldsm(a, p + ks * 16);
+      mma(o, a, g < 2 ? w4[ks * 8 + t] : 0u, g < 2 ? w4[ks * 8 + t + 4] : 0u);
+    }
+    if (t == 0) {
+      const float bm = params[boff(4)], bl = params[boff(4) + 1];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int b = row0 + g + 8 * h;
+        float dmu = 0.f, dl = 0.f;
+        if (b < B) {
+          const float mu = o[2 * h] + bm, l = o[2 * h + 1] + bl;
+          const float r = (y[b] - y0) * ys - mu, w = __expf(-l);
+          dmu = -r * w / B;
+          dl = 0.5f * (1.0f - r * r * w) / B;
+          reinterpret_cast<float2*>(W.zo)[b] = make_float2(mu, l);
+        }
+        reinterpret_cast<float2*>(W.dzo32)[b] = make_float2(dmu, dl);
+        const uint32_t d = pack2(dmu, dl);
+        sDz[g + 8 * h] = d;
+        reinterpret_cast<uint32_t*>(W.dzo)[b] = d;
+      }
+    }
+  }
+  __syncthreads();
+  // dL/dz of hidden layer l from dL/d(its output) in d: to the next operand tile and to memory
+  auto descend = [&](int l, float d[2][4], int buf) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int c = col + 8 * j;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float d0 = d[j][2 * h] * gelu_grad(z[l][j][2 * h]), d1 = d[j][2 * h + 1] * gelu_grad(z[l][j][2 * h + 1]);
+        const uint32_t w = pack2(d0, d1);
+        const size_t e = (size_t)(row0 + g + 8 * h) * 256 + c;
+        if (l > 0) *reinterpret_cast<uint32_t*>(&sA[buf][(g + 8 * h) * AST + c]) = w;
+        *reinterpret_cast<uint32_t*>(W.dz[l] + e) = w;
+        *reinterpret_cast<float2*>(W.dz32[l] + e) = make_float2(d0, d1);
+      }
+    }
+  };
+  float d[2][4];
+  {  // through the output layer: two reduction terms, one k16 step
+    uint32_t a[4] = {t == 0 ? sDz[g] : 0u, t == 0 ? sDz[g + 8] : 0u, 0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) d[j][r] = 0.f;
+      const int k = 16 * warp + 8 * j + g;
+      uint32_t b0 = 0u;
+      if (t == 0) {
+        const __nv_bfloat162 v = __halves2bfloat162(wbf[woff(4) + k], wbf[woff(4) + 256 + k]);
+        b0 = *reinterpret_cast<const uint32_t*>(&v);
+      }
+      mma(d[j], a, b0, 0u);
+    }
+    descend(3, d, 0);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int l = 3; l > 0; --l) {
+    layer_mma(d, sA[(3 - l) & 1], b, lane);
+    if (l > 1) load_frags(b, bpack + (size_t)(l - 2) * 65536, warp, lane);
+    descend(l - 1, d, (4 - l) & 1);
+    if (l > 1) __syncthreads();
+  }
 }
 
-// db(n) = sum_b dZ(b, n), one thread per output unit, fixed order
-__global__ void k_bias_grad(const float* dz, int B, int N, float* db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s += dz[(long)b * N + n];
-  db[n] = s;
+// Gradients.  Blocks 0 .. 207: weight gradients dW(n, k) = sum_b dZ(b, n) X(b, k), one 32 x 32 tile of
+// one layer each (64 tiles of layers 1-3, 8 of layers 0 and 4), accumulated over the whole batch in
+// ascending rows; both operands come row by row through a ring of kStages chunks in shared memory
+// (asynchronous copies) and are transposed by ldmatrix.  Blocks 208 .. 211: bias gradients of the hidden
+// layers, one column per thread, in ascending rows; block 212: the loss and the output layer's biases.
+constexpr int kTiles = 3 * 64 + 2 * 8;
+constexpr int kStages = 4;
+
+__device__ __forceinline__ void cp_async(void* dst, const void* src, int bytes, bool valid) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if (bytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
 }
 
-// Adam on the FP32 master parameters, then the BF16 copies of the weight matrices.  The step's
-// learning rate and bias corrections come from device memory (hyper = {lr, 1 - b1^t, 1 - b2^t}),
-// so that a captured training step can be replayed.
-__global__ void k_adam(float* p, const float* g, float* m, float* v, long n, const float* hyper, float b1, float b2,
-                       float eps) {
-  const float lr = hyper[0], c1 = hyper[1], c2 = hyper[2];
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const float gi = g[i];
+__global__ void __launch_bounds__(128) k_train_dw(const float* __restrict__ y, int B, int rows, float y0, float ys, Bufs W,
+                                                  float* __restrict__ grads, float* loss, float* loss_user) {
+  __shared__ __align__(16) __nv_bfloat16 sD[kStages][CHUNK][TILE + 8], sX[kStages][CHUNK][TILE + 8];
+  const int tid = threadIdx.x, blk = blockIdx.x;
+  if (blk >= kTiles + 8) {  // the loss: 128 threads as the 256 strided partial sums, then halves
+    __shared__ float red[256];
+    for (int h = 0; h < 2; ++h) {
+      float acc = 0.f;
+      for (int b = tid + 128 * h; b < B; b += 256) {
+        const float mu = W.zo[2 * b], l = W.zo[2 * b + 1];
+        const float r = (y[b] - y0) * ys - mu, w = __expf(-l);
+        acc += 0.5f * (r * r * w + l);
+      }
+      red[tid + 128 * h] = acc;
+    }
+    __syncthreads();
+    for (int q = 128; q > 0; q >>= 1) {
+      if (tid < q) red[tid] += red[tid + q];
+      __syncthreads();
+    }
+    if (tid == 0) {
+      *loss = red[0] / B;
+      if (loss_user) *loss_user = red[0] / B;
+    }
+    if (tid < 2) {
+      float s = 0.f;
+#pragma unroll 32
+      for (int b = 0; b < B; ++b) s += W.dzo32[2 * b + tid];
+      grads[boff(4) + tid] = s;
+    }
+    return;
+  }
+  if (blk >= kTiles) {
+    const int col = (blk - kTiles) * 128 + tid, l = col >> 8, n = col & 255;
+    const float* d = W.dz32[l] + n;
+    float s = 0.f;
+#pragma unroll 32
+    for (int b = 0; b < B; ++b) s += d[(size_t)b * 256];
+    grads[boff(l) + n] = s;
+    return;
+  }
+  // layer, tile origin (n0, k0)
+  const int l = blk < 192 ? 1 + blk / 64 : (blk < 200 ? 0 : 4);
+  const int n0 = blk < 192 ? (blk % 64 / 8) * TILE : (l == 0 ? (blk - 192) * TILE : 0);
+  const int k0 = blk < 192 ? (blk % 8) * TILE : (l == 0 ? 0 : (blk - 200) * TILE);
+  const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int wm = (warp >> 1) * 16, wn = (warp & 1) * 16;
+  for (int i = tid; i < kStages * CHUNK * (TILE + 8) / 2; i += 128) {  // the columns that layers 0 and 4 lack
+    reinterpret_cast<uint32_t*>(sD)[i] = 0u;
+    reinterpret_cast<uint32_t*>(sX)[i] = 0u;
+  }
+  __syncthreads();
+  const int nch = (rows + CHUNK - 1) / CHUNK;
+  auto fetch = [&](int ch) {
+    if (ch < nch) {
+      const int st = ch % kStages, b0 = ch * CHUNK;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int e = tid + 128 * i, r = e >> 2, c = (e & 3) * 8;
+        const bool in = b0 + r < rows;
+        const size_t row = in ? b0 + r : 0;
+        if (l < 4) cp_async(&sD[st][r][c], W.dz[l] + row * 256 + n0 + c, 16, in);
+        if (l > 0) cp_async(&sX[st][r][c], W.act[l - 1] + row * 256 + k0 + c, 16, in);
+      }
+      if (tid < CHUNK) {
+        const bool in = b0 + tid < rows;
+        const size_t row = in ? b0 + tid : 0;
+        if (l == 0) cp_async(&sX[st][tid][0], W.xin + row * 8, 16, in);
+        if (l == 4) cp_async(&sD[st][tid][0], W.dzo + row * 2, 4, in);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[2][4];
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[j][r] = 0.f;
+  for (int ch = 0; ch < kStages - 1; ++ch) fetch(ch);
+  for (int ch = 0; ch < nch; ++ch) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    __syncthreads();  // chunk ch has landed for all threads; chunk ch - 1's readers are done
+    fetch(ch + kStages - 1);
+    const int st = ch % kStages;
+#pragma unroll
+    for (int kk = 0; kk < CHUNK; kk += 16) {
+      uint32_t a[4], b[4];
+      // A, lanes 0-7, 8-15, 16-23, 24-31: rows k 0-7 at m, k 0-7 at m + 8, k 8-15 at m, k 8-15 at m + 8
+      ldsm_t(a, &sD[st][kk + (lane & 7) + ((lane >> 4) << 3)][wm + ((lane >> 3) & 1) * 8]);
+      // B: rows k 0-7 and k 8-15 at n, then both at n + 8
+      ldsm_t(b, &sX[st][kk + (lane & 7) + ((lane >> 3) & 1) * 8][wn + (lane >> 4) * 8]);
+      mma(acc[0], a, b[0], b[1]);
+      mma(acc[1], a, b[2], b[3]);
+    }
+  }
+  const int nk = l == 0 ? 6 : 256, nn = l == 4 ? 2 : 256;
+  float* out = grads + woff(l);
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int n = n0 + wm + g + 8 * (r >> 1), k = k0 + wn + 8 * j + 2 * t + (r & 1);
+      if (n < nn && k < nk) out[(size_t)n * nk + k] = acc[j][r];
+    }
+}
+
+// BF16 copy of parameter i and, for the weights of layers 1-3, its places in the operand images.
+__device__ __forceinline__ void store_bf16(int i, float v, __nv_bfloat16* wbf, __nv_bfloat16* fpack, __nv_bfloat16* bpack,
+                                           __nv_bfloat16* wpack);
+
+// Adam on the FP32 master parameters, then their BF16 copies.
+__global__ void __launch_bounds__(256)
+k_train_update(const float* __restrict__ grads, float lr, float c1, float c2, float b1, float b2, float eps, float* p,
+               float* m, float* v, __nv_bfloat16* wbf, __nv_bfloat16* fpack, __nv_bfloat16* bpack, __nv_bfloat16* wpack) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_params(); i += gridDim.x * blockDim.x) {
+    const float gi = grads[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float np = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = np;
+    store_bf16(i, np, wbf, fpack, bpack, wpack);
   }
 }
 
+// The BF16 copies of all parameters (after creation).
+__global__ void k_refresh(const float* p, __nv_bfloat16* wbf, __nv_bfloat16* fpack, __nv_bfloat16* bpack,
+                          __nv_bfloat16* wpack) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_params(); i += gridDim.x * blockDim.x)
+    store_bf16(i, p[i], wbf, fpack, bpack, wpack);
+}
+
+}  // namespace tr
 
 // ---------------------------------------------------------------- fused inference on tcgen05
 // One CTA (256 threads) per SM, persistent over tiles of 128 rows.  Layer 0 (K = 6) and the
@@ -513,18 +726,23 @@ k_mlp_forward(const float* __restrict__ x, int B, const __nv_bfloat16* __restric
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256u) : "memory");
 }
 
-// Operand image of the weights of layers 1-3 (W[n][k] as the B operand: row n, column k).
-__global__ void k_pack_weights(const __nv_bfloat16* __restrict__ wbf, __nv_bfloat16* __restrict__ wpack) {
-  const long per = 256L * 256;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < 3 * per; i += (long)gridDim.x * blockDim.x) {
-    const int l = (int)(i / per) + 1;
-    const int n = (int)((i % per) / 256), k = (int)(i % 256);
-    const long woffl = 6 * 256 + 256 + (long)(l - 1) * (256 * 256 + 256);
-    wpack[(l - 1) * per + op_offset(n, k) / 2] = wbf[woffl + (long)n * 256 + k];
-  }
-}
-
 }  // namespace tc
+
+namespace tr {
+__device__ __forceinline__ void store_bf16(int i, float v, __nv_bfloat16* wbf, __nv_bfloat16* fpack, __nv_bfloat16* bpack,
+                                           __nv_bfloat16* wpack) {
+  const __nv_bfloat16 h = __float2bfloat16(v);
+  wbf[i] = h;
+  const int per = 256 * 256 + 256, r = i - woff(1);
+  if (r < 0 || r >= 3 * per) return;
+  const int l = r / per, e = r - l * per;
+  if (e >= 65536) return;
+  const int n = e >> 8, k = e & 255;
+  fpack[(size_t)l * 65536 + frag_index(n, k)] = h;
+  bpack[(size_t)l * 65536 + frag_index(k, n)] = h;
+  wpack[(size_t)l * 65536 + tc::op_offset(n, k) / 2] = h;
+}
+}  // namespace tr
 }  // namespace mlp
 }  // namespace swf
 
@@ -540,34 +758,21 @@ struct swf_mlp {
   float* adam_m;
   float* adam_v;
   __nv_bfloat16* wbf;        // BF16 copy of all parameters (same layout)
-  __nv_bfloat16* act[NL];    // bf16 input of layer l: [B][DIN[l]]
-  float* z[NL];              // fp32 pre-activation of layer l: [B][DOUT[l]]
-  float* dz32[NL];           // fp32 dL/dz of layer l
-  __nv_bfloat16* dz16[NL];   // bf16 copy
+  __nv_bfloat16* fpack;      // layers 1-3 in the training kernels' operand order, forward and backward
+  __nv_bfloat16* bpack;
+  __nv_bfloat16* wpack;      // layers 1-3 in the tensor-core operand image (inference kernel)
+  tr::Bufs train;
   float* loss;
   float* in_shift;           // [6] feature standardisation
   float* in_scale;           // [6]
   float y0, ys;              // target standardisation
-  __nv_bfloat16* wpack;      // layers 1-3 in the tensor-core operand image (inference kernel)
   int* err;                  // set by the inference kernel when a wait timed out
   int nsm;
   cudaStream_t last_stream;
-  float* xs;                 // training batch staged for the captured step: [max_batch][6]
-  float* ysg;                // [max_batch]
-  float* hyper;              // {lr, 1 - b1^t, 1 - b2^t} of the current step
-  cudaStream_t cap_stream;   // stream the training step is captured on
-  std::map<int, cudaGraphExec_t> train_graphs;  // captured training step per batch size
   std::vector<void*> allocs;
 };
 
 namespace {
-long woff(int l) {
-  long o = 0;
-  for (int i = 0; i < l; ++i) o += (long)DIN[i] * DOUT[i] + DOUT[i];
-  return o;
-}
-long boff(int l) { return woff(l) + (long)DIN[l] * DOUT[l]; }
-
 swf_status mlp_alloc(swf_mlp* m, void** p, size_t bytes) {
   cudaError_t e = cudaMalloc(p, bytes);
   if (e != cudaSuccess) {
@@ -579,54 +784,21 @@ swf_status mlp_alloc(swf_mlp* m, void** p, size_t bytes) {
   return SWF_OK;
 }
 
-void gemm(const Mat& A, const Mat& B, int M, int N, int K, const EpiArgs& E, cudaStream_t st) {
-  dim3 grid((N + TN - 1) / TN, (M + TM - 1) / TM);
-  k_gemm<<<grid, 128, 0, st>>>(A, B, M, N, K, E);
-}
-
-void refresh_bf16(swf_mlp* m, cudaStream_t st) {
-  k_to_bf16<<<128, 256, 0, st>>>(m->params, m->wbf, n_params());
-  tc::k_pack_weights<<<192, 256, 0, st>>>(m->wbf, m->wpack);
-}
-
-// forward pass on x (fp32 [B][6]); leaves activations for the backward pass; output in z[NL-1]
-void forward(swf_mlp* m, const float* x, int B, cudaStream_t st) {
-  k_inputs<<<64, 256, 0, st>>>(x, m->in_shift, m->in_scale, m->act[0], (long)B * DIN[0]);
-  for (int l = 0; l < NL; ++l) {
-    const Mat A = {m->act[l], DIN[l], 1};
-    const Mat W = {m->wbf + woff(l), 1, DIN[l]};  // B(k, n) = W[n][k]
-    EpiArgs E = {};
-    E.mode = l < NL - 1 ? EPI_FWD_HIDDEN : EPI_FWD_OUT;
-    E.bias = m->params + boff(l);
-    E.z = m->z[l];
-    E.act = l < NL - 1 ? m->act[l + 1] : nullptr;
-    gemm(A, W, B, DOUT[l], DIN[l], E, st);
+// One pass over a batch: the gradients into grads and the loss, then (update) an Adam step.
+cudaError_t train_pass(swf_mlp* m, const float* x, const float* y, int B, bool update, float lr, float* grads, float* loss,
+                       cudaStream_t st) {
+  const int nblk = (B + tr::ROWS - 1) / tr::ROWS, rows = nblk * tr::ROWS;
+  tr::k_train_rows<<<nblk, tr::THREADS, 0, st>>>(x, y, B, m->wbf, m->fpack, m->bpack, m->params, m->in_shift, m->in_scale,
+                                                 m->y0, m->ys, m->train);
+  tr::k_train_dw<<<tr::kTiles + 8 + 1, 128, 0, st>>>(y, B, rows, m->y0, m->ys, m->train, grads, m->loss, loss);
+  if (update) {
+    m->step += 1;
+    const double b1 = 0.9, b2 = 0.999;
+    tr::k_train_update<<<(n_params() + 511) / 512, 256, 0, st>>>(
+        grads, lr, (float)(1.0 - std::pow(b1, (double)m->step)), (float)(1.0 - std::pow(b2, (double)m->step)), 0.9f, 0.999f,
+        1e-8f, m->params, m->adam_m, m->adam_v, m->wbf, m->fpack, m->bpack, m->wpack);
   }
-}
-
-// backward pass from dz of the output layer; fills m->grads
-void backward(swf_mlp* m, int B, cudaStream_t st) {
-  for (int l = NL - 1; l >= 0; --l) {
-    // dW(n, k) = sum_b dZ(b, n) X(b, k)
-    const Mat dZt = {m->dz16[l], 1, DOUT[l]};  // A(n, b) = dZ[b][n]
-    const Mat X = {m->act[l], DIN[l], 1};      // B(b, k) = X[b][k]
-    EpiArgs E = {};
-    E.mode = EPI_DW;
-    E.z = m->grads + woff(l);
-    gemm(dZt, X, DOUT[l], DIN[l], B, E, st);
-    k_bias_grad<<<(DOUT[l] + 127) / 128, 128, 0, st>>>(m->dz32[l], B, DOUT[l], m->grads + boff(l));
-    if (l > 0) {
-      // dX(b, k) = sum_n dZ(b, n) W(n, k), then times GELU'(z_{l-1})
-      const Mat dZ = {m->dz16[l], DOUT[l], 1};
-      const Mat W = {m->wbf + woff(l), DIN[l], 1};  // B(n, k) = W[n][k]
-      EpiArgs D = {};
-      D.mode = EPI_DX;
-      D.zprev = m->z[l - 1];
-      D.dz32 = m->dz32[l - 1];
-      D.act = m->dz16[l - 1];
-      gemm(dZ, W, B, DIN[l], DOUT[l], D, st);
-    }
-  }
+  return cudaGetLastError();
 }
 }  // namespace
 
@@ -648,7 +820,6 @@ swf_status swf_mlp_create(swf_mlp** out, int device, const float* init_params, i
   swf_status s;
   auto fail = [&](swf_status st) {
     for (void* p : m->allocs) cudaFree(p);
-    if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
     delete m;
     return st;
   };
@@ -662,26 +833,27 @@ swf_status swf_mlp_create(swf_mlp** out, int device, const float* init_params, i
   if ((s = mlp_alloc(m, (void**)&m->in_scale, 6 * 4)) != SWF_OK) return fail(s);
   if ((s = mlp_alloc(m, (void**)&m->wpack, (size_t)3 * 256 * 256 * 2)) != SWF_OK) return fail(s);
   if ((s = mlp_alloc(m, (void**)&m->err, sizeof(int))) != SWF_OK) return fail(s);
-  if ((s = mlp_alloc(m, (void**)&m->xs, (size_t)max_batch * DIN[0] * 4)) != SWF_OK) return fail(s);
-  if ((s = mlp_alloc(m, (void**)&m->ysg, (size_t)max_batch * 4)) != SWF_OK) return fail(s);
-  if ((s = mlp_alloc(m, (void**)&m->hyper, 4 * sizeof(float))) != SWF_OK) return fail(s);
-  m->cap_stream = nullptr;
+  if ((s = mlp_alloc(m, (void**)&m->fpack, (size_t)3 * 65536 * 2)) != SWF_OK) return fail(s);
+  if ((s = mlp_alloc(m, (void**)&m->bpack, (size_t)3 * 65536 * 2)) != SWF_OK) return fail(s);
   m->last_stream = 0;
   m->nsm = 0;
   e = cudaDeviceGetAttribute(&m->nsm, cudaDevAttrMultiProcessorCount, device);
   if (e != cudaSuccess || m->nsm < 1) return fail(cuda_status(e, "SM count"));
   e = cudaFuncSetAttribute(tc::k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::SMEM);
   if (e != cudaSuccess) return fail(cuda_status(e, "cudaFuncSetAttribute(k_mlp_forward)"));
-  e = cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking);
-  if (e != cudaSuccess) return fail(cuda_status(e, "capture stream"));
   m->y0 = norm[12];
   m->ys = norm[13];
-  for (int l = 0; l < NL; ++l) {
-    if ((s = mlp_alloc(m, (void**)&m->act[l], (size_t)max_batch * DIN[l] * 2)) != SWF_OK) return fail(s);
-    if ((s = mlp_alloc(m, (void**)&m->z[l], (size_t)max_batch * DOUT[l] * 4)) != SWF_OK) return fail(s);
-    if ((s = mlp_alloc(m, (void**)&m->dz32[l], (size_t)max_batch * DOUT[l] * 4)) != SWF_OK) return fail(s);
-    if ((s = mlp_alloc(m, (void**)&m->dz16[l], (size_t)max_batch * DOUT[l] * 2)) != SWF_OK) return fail(s);
+  const size_t nblk = ((size_t)max_batch + tr::ROWS - 1) / tr::ROWS, rows = nblk * tr::ROWS;
+  for (int l = 0; l < 4; ++l) {
+    if ((s = mlp_alloc(m, (void**)&m->train.act[l], rows * 512)) != SWF_OK) return fail(s);
+    if ((s = mlp_alloc(m, (void**)&m->train.dz[l], rows * 512)) != SWF_OK) return fail(s);
   }
+  if ((s = mlp_alloc(m, (void**)&m->train.xin, rows * 16)) != SWF_OK) return fail(s);
+  if ((s = mlp_alloc(m, (void**)&m->train.dzo, rows * 4)) != SWF_OK) return fail(s);
+  for (int l = 0; l < 4; ++l)
+    if ((s = mlp_alloc(m, (void**)&m->train.dz32[l], rows * 1024)) != SWF_OK) return fail(s);
+  if ((s = mlp_alloc(m, (void**)&m->train.dzo32, rows * 8)) != SWF_OK) return fail(s);
+  if ((s = mlp_alloc(m, (void**)&m->train.zo, rows * 8)) != SWF_OK) return fail(s);
   e = cudaMemcpy(m->params, init_params, np * 4, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return fail(cuda_status(e, "upload parameters"));
   e = cudaMemcpy(m->in_shift, norm, 6 * 4, cudaMemcpyHostToDevice);
@@ -691,7 +863,7 @@ swf_status swf_mlp_create(swf_mlp** out, int device, const float* init_params, i
   cudaMemset(m->adam_m, 0, np * 4);
   cudaMemset(m->adam_v, 0, np * 4);
   cudaMemset(m->err, 0, sizeof(int));
-  refresh_bf16(m, 0);
+  tr::k_refresh<<<256, 256>>>(m->params, m->wbf, m->fpack, m->bpack, m->wpack);
   e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return fail(cuda_status(e, "surrogate set-up"));
   *out = m;
@@ -702,8 +874,6 @@ swf_status swf_mlp_destroy(swf_mlp* m) {
   if (!m) return SWF_OK;
   cudaSetDevice(m->device);
   cudaDeviceSynchronize();
-  for (auto& kv : m->train_graphs) cudaGraphExecDestroy(kv.second);
-  if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
   for (void* p : m->allocs) cudaFree(p);
   delete m;
   return SWF_OK;
@@ -745,28 +915,9 @@ swf_status swf_mlp_gradients(swf_mlp* m, const float* x_dev, const float* y_dev,
     return SWF_EINVAL;
   }
   cudaSetDevice(m->device);
-  cudaStream_t st = (cudaStream_t)stream;
-  forward(m, x_dev, B, st);
-  k_nll<<<1, 256, 0, st>>>(m->z[NL - 1], y_dev, m->y0, m->ys, B, m->dz32[NL - 1], m->dz16[NL - 1],
-                           loss_dev ? loss_dev : m->loss);
-  backward(m, B, st);
-  if (grad_dev) {
-    cudaError_t e = cudaMemcpyAsync(grad_dev, m->grads, (size_t)n_params() * 4, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return cuda_status(e, "copy gradients");
-  }
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = train_pass(m, x_dev, y_dev, B, false, 0.f, grad_dev ? grad_dev : m->grads, loss_dev, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_status(e, "surrogate gradients");
   return SWF_OK;
-}
-
-// The kernels of one training step on the staged batch (forward, loss, backward, Adam, BF16
-// copies and operand image), B rows.
-static void record_train_step(swf_mlp* m, int B, cudaStream_t st) {
-  forward(m, m->xs, B, st);
-  k_nll<<<1, 256, 0, st>>>(m->z[NL - 1], m->ysg, m->y0, m->ys, B, m->dz32[NL - 1], m->dz16[NL - 1], m->loss);
-  backward(m, B, st);
-  k_adam<<<128, 256, 0, st>>>(m->params, m->grads, m->adam_m, m->adam_v, n_params(), m->hyper, 0.9f, 0.999f, 1e-8f);
-  refresh_bf16(m, st);
 }
 
 swf_status swf_mlp_train_step(swf_mlp* m, const float* x_dev, const float* y_dev, int B, float lr, float* loss_dev,
@@ -776,37 +927,7 @@ swf_status swf_mlp_train_step(swf_mlp* m, const float* x_dev, const float* y_dev
     return SWF_EINVAL;
   }
   cudaSetDevice(m->device);
-  cudaStream_t st = (cudaStream_t)stream;
-  // the step runs as one CUDA graph per batch size (about 25 kernels, captured once) on the
-  // staged batch; the batch, the learning rate and the bias corrections are set before it
-  cudaError_t e = cudaMemcpyAsync(m->xs, x_dev, (size_t)B * DIN[0] * 4, cudaMemcpyDeviceToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(m->ysg, y_dev, (size_t)B * 4, cudaMemcpyDeviceToDevice, st);
-  if (e != cudaSuccess) return cuda_status(e, "stage the training batch");
-  m->step += 1;
-  const double b1 = 0.9, b2 = 0.999;
-  k_set_hyper<<<1, 1, 0, st>>>(m->hyper, lr, (float)(1.0 - std::pow(b1, (double)m->step)),
-                               (float)(1.0 - std::pow(b2, (double)m->step)));
-  auto it = m->train_graphs.find(B);
-  if (it == m->train_graphs.end()) {
-    cudaGraphExec_t exec = nullptr;
-    e = cudaStreamBeginCapture(m->cap_stream, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-      record_train_step(m, B, m->cap_stream);
-      cudaGraph_t g = nullptr;
-      e = cudaStreamEndCapture(m->cap_stream, &g);
-      if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
-      if (g) cudaGraphDestroy(g);
-    }
-    if (e != cudaSuccess) return cuda_status(e, "capture the training step");
-    it = m->train_graphs.emplace(B, exec).first;
-  }
-  e = cudaGraphLaunch(it->second, st);
-  if (e != cudaSuccess) return cuda_status(e, "training step");
-  if (loss_dev) {
-    e = cudaMemcpyAsync(loss_dev, m->loss, 4, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return cuda_status(e, "copy loss");
-  }
-  e = cudaGetLastError();
+  const cudaError_t e = train_pass(m, x_dev, y_dev, B, true, lr, m->grads, loss_dev, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_status(e, "surrogate update");
   return SWF_OK;
 }
