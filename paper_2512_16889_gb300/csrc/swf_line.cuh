@@ -227,6 +227,8 @@ __global__ void __launch_bounds__(kXLineThreads, sizeof(R) == 4 ? 2 : 1)
 k_xline(const __grid_constant__ StageArgs<R> P, const __grid_constant__ StageArgs<R> A, int rows, int flags) {
   constexpr int TPL = line_threads(R1, R2);
   constexpr int S = R2 | 1, LS = xline_stride(R1, R2);
+  chain_wait();
+  chain_release();
   if (A.ctl && A.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ R s_ft[16];
@@ -311,6 +313,8 @@ template <typename R, int R1, int R2>
 __global__ void __launch_bounds__(line_max_threads((int)sizeof(cpx<R>)), sizeof(R) == 4 && R1 <= 16 && R2 <= 16 ? 2 : 1)
 k_line(const __grid_constant__ StageArgs<R> A, int axis, int lgtx, int flags) {
   constexpr int LS = line_stride(R1, R2);
+  chain_wait();
+  chain_release();
   if (A.ctl && A.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nx = A.g.n[0], ny = A.g.n[1], nz = A.g.n[2];

@@ -77,6 +77,14 @@ struct MarchClock {
   int pad;
 };
 
+// Programmatic dependent launch (the kernels of a march's steps, see launch_chained): the next kernel of
+// the chain is set up while this one runs.  chain_wait() returns when the kernels before this one have
+// ended and their results are visible: nothing of theirs is read or overwritten before it.
+// chain_release() lets the next kernel's blocks come in as this one's leave.  Without the launch
+// attribute both do nothing.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 template <typename R>
 __device__ __forceinline__ double node_time(const StageArgs<R>& A, int ls, double c) {
   if (A.ctl) return A.ctl->t + c * A.ctl->h;
