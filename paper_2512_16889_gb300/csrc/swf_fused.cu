@@ -1015,11 +1015,16 @@ __global__ void __launch_bounds__(v2::NT2, 2) k_fused2(Args A) {
 // paired through lane ^ 16) into the inverse y-FFT.  The arithmetic is that of `k_fused`, in the
 // same order; only the data movement differs.
 //
-// Both exchange buffers are 2 x 16 chunks of 16 x 16 values: chunk (c, a) of component c holds, in
+// Both exchange buffers are 16 x 2 chunks of 16 x 16 values: chunk (a, c) of component c holds, in
 // the row buffer X1, the 16 rows of this CTA at x in [16 a, 16 a + 16), and in the column buffer
-// X2, the 16 columns of this CTA at y in [16 a, 16 a + 16).  Chunk (c, s) of one CTA is exactly
-// chunk (c, rank) of CTA s after the transpose, so each transpose is 32 contiguous 2 KB copies per
-// CTA.  Inside a chunk, row b keeps its 16 values at positions d ^ b (an XOR swizzle written by the
+// X2, the 16 columns of this CTA at y in [16 a, 16 a + 16).  Chunk (s, c) of one CTA is exactly
+// chunk (rank, c) of CTA s after the transpose, so each transpose is 16 contiguous 4 KB copies per
+// CTA, one per warp.  Of the 26.4 thousand cycles of an evaluation (28.8 thousand when one warp issued
+// 32 copies of 2 KB) the two transposes take 5.4 and 5.8 thousand (about the cluster network's 13
+// bytes per cycle and SM), of which the local term and the stage combine hide 3.4 and 4.3; the row and
+// column FFTs take 12.3 and the end of an evaluation (k_i, next stage value) 2.9.  Moving y to L2 to
+// give the FFTs a third buffer, four block barriers fewer, made it slower (27.2: its loads share the
+// SM's port with the transposes).  Inside a chunk, row b keeps its 16 values at positions d ^ b (an XOR swizzle written by the
 // producer and kept by the copy), so that every FFT pass reads and writes without bank conflicts.
 //
 // Ordering.  Each CTA arms its receive barrier for a transpose before it arrives at the cluster
@@ -1053,9 +1058,10 @@ static_assert(OFF_X2 % 16 == 0 && OFF_X1 % 16 == 0, "bulk-copy alignment");
 static_assert(SMEM3 <= 227 * 1024, "shared memory");
 }  // namespace v3
 
-// position of value (c, a, b, d) in an exchange buffer: chunk (c, a), row b, column d ^ b
+// position of value (c, a, b, d) in an exchange buffer: chunk (a, c), row b, column d ^ b (the two
+// components of a chunk are neighbours: one copy per peer)
 __host__ __device__ __forceinline__ int q3(int c, int a, int b, int d) {
-  return ((((c << 4) + a) << 4) + b) * 16 + (d ^ b);
+  return ((((a << 1) + c) << 4) + b) * 16 + (d ^ b);
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -1181,13 +1187,14 @@ __device__ __forceinline__ void fft_cols3_h0(float2* X, const float2* twp, const
   for (int n2 = 0; n2 < 16; ++n2) a[n2] = X[q3(c, j, n2, col)];
   dft16<false>(a);
   const float kx = kxc[col];
+  const float sg = c ? -1.f : 1.f;
 #pragma unroll
   for (int k2 = 0; k2 < 16; ++k2) {
-    const float2 own = a[k2];
-    const float2 oth = make_float2(__shfl_xor_sync(0xffffffffu, own.x, 16), __shfl_xor_sync(0xffffffffu, own.y, 16));
-    float2 o0, o1;
-    h0_pair(c ? oth : own, c ? own : oth, kx, kyt[j + 16 * k2], inv_n, o0, o1);
-    a[k2] = c ? o1 : o0;
+    const float2 oth = make_float2(__shfl_xor_sync(0xffffffffu, a[k2].x, 16), __shfl_xor_sync(0xffffffffu, a[k2].y, 16));
+    const float ky = sg * kyt[j + 16 * k2];
+    const float2 h = make_float2(__fmaf_rn(ky, oth.y, __fmaf_rn(kx, oth.x, sg * a[k2].x)),
+                                 __fmaf_rn(-ky, oth.x, __fmaf_rn(kx, oth.y, sg * a[k2].y)));
+    a[k2] = scl(inv_n, rot<false>(h));
   }
   dft16<true>(a);
 #pragma unroll
@@ -1266,8 +1273,11 @@ __global__ void __launch_bounds__(NT, 1) k_fused3(Args A) {
   cl_arrive();                             // barriers initialised and armed
   uint32_t par_f = 0, par_b = 0;
   bool err = false;
-  // lane L of warp 0 copies chunk (L / 16, peer) to peer (rank + L) % 16
-  const int cc = lane >> 4, peer = (rank + (lane & 15)) & (CL - 1);
+  // one lane of warp w copies both components' chunk to peer (rank + w) % 16: a warp issues its bulk
+  // copies one after another, 50 cycles each, so 32 of them from the lanes of one warp held the
+  // transposes up by 1600 cycles
+  const int peer = (rank + warp) & (CL - 1);
+  const uint32_t push_to = (uint32_t)(2 * rank * CHK * 8), push_from = (uint32_t)(2 * peer * CHK * 8);
   // the sites this thread owns
   const int oc = own_c(), orow = own_row(), ojj = own_jj();
 
@@ -1354,9 +1364,8 @@ __global__ void __launch_bounds__(NT, 1) k_fused3(Args A) {
       fence_async_smem();
       __syncthreads();
       cl_wait();  // every CTA's X2 is free and its receive barrier armed
-      if (warp == 0 && !__any_sync(0xffffffffu, err) && !A.drop)
-        bulk_push(peer_addr(x2a + (uint32_t)((cc * CL + rank) * CHK * 8), peer),
-                  x1a + (uint32_t)((cc * CL + peer) * CHK * 8), CHK * 8, peer_addr(bar_f, peer));
+      if (!__any_sync(0xffffffffu, err) && !A.drop && lane == 0)
+        bulk_push(peer_addr(x2a + push_to, peer), x1a + push_from, 2 * CHK * 8, peer_addr(bar_f, peer));
 
       // ---- meanwhile: local term Z = -i V (Y + psi_b) of this stage, from the stash (Y, both
       // components through the partner lane) to the stash
@@ -1410,9 +1419,8 @@ __global__ void __launch_bounds__(NT, 1) k_fused3(Args A) {
       fence_async_smem();
       __syncthreads();
       cl_wait();  // every CTA's X1 is free and its receive barrier armed
-      if (warp == 0 && !__any_sync(0xffffffffu, err) && !A.drop)
-        bulk_push(peer_addr(x1a + (uint32_t)((cc * CL + rank) * CHK * 8), peer),
-                  x2a + (uint32_t)((cc * CL + peer) * CHK * 8), CHK * 8, peer_addr(bar_b, peer));
+      if (!__any_sync(0xffffffffu, err) && !A.drop && lane == 0)
+        bulk_push(peer_addr(x1a + push_to, peer), x2a + push_from, 2 * CHK * 8, peer_addr(bar_b, peer));
 
       // ---- meanwhile: the next stage combine without its newest term, P = y + h sum_{j < new} a_j k_j
       // (h sum b_j k_j without y before the last stage), in the order of k_fused
