@@ -9,7 +9,8 @@
 
 namespace swf {
 
-#define X(n, r1, r2) {n, r1, r2, k_xline<SWF_LINE_REAL, r1, r2>, k_line<SWF_LINE_REAL, r1, r2>},
+#define X(n, r1, r2) {n, r1, r2, k_xline<SWF_LINE_REAL, r1, r2>, k_line<SWF_LINE_REAL, r1, r2>, \
+                      k_f2_line<SWF_LINE_REAL, r1, r2>},
 #define LIST_(l) SWF_LINES_##l(X)
 #define LIST(l) LIST_(l)
 static const LineEntry<SWF_LINE_REAL> entries[] = {LIST(SWF_LINE_LIST)};

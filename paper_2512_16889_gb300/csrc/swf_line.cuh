@@ -36,13 +36,17 @@ enum : int { LN_FWD = 1, LN_H0 = 2, LN_INV = 4 };
 
 template <typename R> using XLineKernel = void (*)(StageArgs<R>, StageArgs<R>, int, int);
 template <typename R> using LineKernel = void (*)(StageArgs<R>, int, int, int);
+template <typename R>
+using F2LineKernel = void (*)(StageArgs<R>, const cpx<R>*, cpx<R>*, const cpx<R>*, const cpx<double>*, int, int,
+                              cpx<double>*, int);
 
-// One length n = r1 r2 and its two kernels.
+// One length n = r1 r2 and its kernels.
 template <typename R>
 struct LineEntry {
   int n, r1, r2;
   XLineKernel<R> x;
   LineKernel<R> line;
+  F2LineKernel<R> f2;
 };
 
 // Threads per line and shared-memory complex values per line of the two kernels.  x pass: rows of R2
@@ -92,11 +96,31 @@ __device__ __forceinline__ void close_sites(const StageArgs<R>& P, size_t gs, in
   }
 }
 
+// The local term Z = -i V (Y + psi_b): V has one non-zero component, so every component of Z comes from
+// one component of Y + psi_b.  Component c feeds component source_component (A_1, A_2: the mirrored one,
+// A_3: two away): -i V phi = rot a phi with rot = -i, times i (-i) for A_2's even (odd) components, times
+// -1 for A_3's odd ones; 0 without a field.
+__device__ __forceinline__ int source_component(int acomp, int c) {
+  return acomp == 1 || acomp == 2 ? 3 - c : acomp == 3 ? (c ^ 2) : c;
+}
+template <typename R>
+__device__ __forceinline__ cpx<R> source_rotation(int acomp, int c) {
+  return acomp < 0 ? mk<R>(0, 0)
+         : acomp == 2 ? ((c & 1) ? mk<R>(-1, 0) : mk<R>(1, 0))
+         : acomp == 3 && (c & 1) ? mk<R>(0, 1)
+                                 : mk<R>(0, -1);
+}
+// rot a (y + br e), rot = +-1 or +-i (or 0)
+template <typename R>
+__device__ __forceinline__ cpx<R> source_term(cpx<R> y, cpx<R> br, cpx<R> e, R a, cpx<R> rot) {
+  const cpx<R> phi = mk<R>(a * ((y.x + br.x * e.x) - br.y * e.y), a * ((y.y + br.x * e.y) + br.y * e.x));
+  return rot.x != (R)0 ? rot.x * phi : mk<R>(-rot.y * phi.y, rot.y * phi.x);
+}
+
 // The last of A's stage combine and the local term: v becomes the stage value Y, which is stored where
-// A asks for it, and Z = -i V (Y + psi_b) goes to the output slot until the evaluation is closed.  V
-// has one non-zero component, so every component of Z comes from one component of Y + psi_b: this
-// thread writes the component that its own feeds (A_1, A_2: the mirrored one, A_3: two away).
-// x = x0 + q stride are the sites' x indices, f, c, row the line, ftr and tf its time factors.
+// A asks for it, and Z goes to the output slot (of the component this thread's one feeds) until the
+// evaluation is closed.  x = x0 + q stride are the sites' x indices, f, c, row the line, ftr and tf its
+// time factors.
 template <typename R, int NV>
 __device__ __forceinline__ void open_sites(const StageArgs<R>& A, bool ff, size_t gs, int x0, int stride, int f, int c,
                                            int row, R ftr, cpx<R> tf, cpx<R>* v) {
@@ -131,20 +155,12 @@ __device__ __forceinline__ void open_sites(const StageArgs<R>& A, bool ff, size_
   const R ar = ftr * gx[nx + iy] * gx[nx + ny + iz];                       // A_mu = ar gx
   const cpx<R> br = ex[nt + c] * (tf * (ex[nx + iy] * ex[nx + ny + iz]));  // psi_b = br ex
   const int acomp = A.fd[f].acomp;
-  const int oc = acomp == 1 || acomp == 2 ? 3 - c : acomp == 3 ? (c ^ 2) : c;
-  // -i V phi = rot a phi with rot = -i, times i (-i) for A_2's even (odd) components, times -1 for
-  // A_3's odd ones
-  const cpx<R> rot = acomp < 0 ? mk<R>(0, 0)
-                     : acomp == 2 ? ((c & 1) ? mk<R>(-1, 0) : mk<R>(1, 0))
-                     : acomp == 3 && (c & 1) ? mk<R>(0, 1)
-                                             : mk<R>(0, -1);
+  const int oc = source_component(acomp, c);
+  const cpx<R> rot = source_rotation<R>(acomp, c);
   cpx<R>* zo = A.kout + ((size_t)f * 4 + oc) * N + (size_t)row * nx + x0;
 #pragma unroll
   for (int q = 0; q < NV; ++q) {
-    const cpx<R> e = ex[x0 + q * stride];
-    const R a = ar * gx[x0 + q * stride];
-    const cpx<R> phi = mk<R>(a * ((v[q].x + br.x * e.x) - br.y * e.y), a * ((v[q].y + br.x * e.y) + br.y * e.x));
-    zo[q * stride] = acomp == 2 ? rot.x * phi : mk<R>(-rot.y * phi.y, rot.y * phi.x);
+    zo[q * stride] = source_term<R>(v[q], br, ex[x0 + q * stride], ar * gx[x0 + q * stride], rot);
   }
 }
 
@@ -384,6 +400,107 @@ k_line(const __grid_constant__ StageArgs<R> A, int axis, int lgtx, int flags) {
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) A.T[base + (size_t)(g + k2 * R1) * stride] = m[k2];
   }
+}
+
+// The direct-transform sums of a block of wave f: red[component][row][thread] holds the threads' sums (in
+// the march precision; the caller has synchronised), a warp per component adds them in a fixed order, and
+// trow[w] (the stage's weight and time phase) times adds them to the block's own FP64 accumulators
+// dpart[f][block][4].
+template <typename R>
+__device__ __forceinline__ void direct_sums(const StageArgs<R>& A, const cpx<R>* red, int per, int f,
+                                            const cpx<double>* __restrict__ ptab, int tab_stride, int stage,
+                                            cpx<double>* dpart) {
+  const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+  const int step = min(32, (int)blockDim.x - (int)(threadIdx.x & ~31));  // threads of this warp
+  const unsigned full = step == 32 ? 0xffffffffu : (1u << step) - 1u;
+  for (int k = threadIdx.x >> 5; k < 4; k += nw) {
+    cpx<R> sacc = mk<R>(0, 0);
+    for (int e = lane; e < per; e += step) sacc = sacc + red[k * per + e];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const R x = __shfl_down_sync(full, sacc.x, off), y = __shfl_down_sync(full, sacc.y, off);
+      if (lane + off < step) sacc = mk<R>(sacc.x + x, sacc.y + y);
+    }
+    if (lane == 0) {
+      const long tab_row = (long)(A.clk->step + A.ls) * 7 + stage;
+      const cpx<double> wt = ptab[3 * (tab_row + (long)(f >> 1) * tab_stride) + (f & 1)];
+      cpx<double>& d = dpart[((size_t)f * gridDim.x + blockIdx.x) * 4 + k];
+      d = d + wt * cvt<double>(sacc);
+    }
+  }
+}
+
+// The x pass of the partial-integration integrand (see k_f2_x in swf_march.cu) on the register lines: Z =
+// -i V (Y + psi_b) of the stage value in ys, its forward x-FFT into Zspec and its direct transform.  Its
+// traffic is one read and one write of the waves; with the new mode sum it took four steps of 16 pairs on
+// 384^2 from 29.5 to 21.2 ms (33.7 ms with small-radix passes here).
+template <typename R, int R1, int R2>
+__global__ void __launch_bounds__(kXLineThreads, 2)
+k_f2_line(const __grid_constant__ StageArgs<R> A, const cpx<R>* __restrict__ ys, cpx<R>* __restrict__ Zspec,
+          const cpx<R>* __restrict__ dph, const cpx<double>* __restrict__ ptab, int tab_stride, int stage,
+          cpx<double>* dpart, int rows) {
+  constexpr int TPL = line_threads(R1, R2);
+  constexpr int S = R2 | 1, LS = xline_stride(R1, R2);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ R s_ft[16];
+  __shared__ cpx<R> s_tf;
+  cpx<R>* sm = reinterpret_cast<cpx<R>*>(smem_raw);
+  const int nx = R1 * R2, ny = A.g.n[1], nz = A.g.n[2], nt = nx + ny + nz;
+  const size_t N = A.g.N;
+  const int f = blockIdx.y, row0 = blockIdx.x * rows;
+  const int line = threadIdx.x / TPL, g = threadIdx.x - line * TPL;
+  const int c = line & 3, j = line >> 2, row = row0 + j;
+  const int mline = threadIdx.x / R1, gm = threadIdx.x - mline * R1;
+  const bool ok = row < A.nrows, site = ok && g < R2;
+  const bool mode = mline < 4 * rows && row0 + (mline >> 2) < A.nrows;
+  const cpx<R>* __restrict__ tw = A.ltw[0];
+  const int acomp = A.fd[f].acomp, oc = source_component(acomp, c);
+  const size_t gs = ((size_t)f * 4 + c) * N + (size_t)row * nx + g;
+  cpx<R> v[R1];
+  if (site) {
+#pragma unroll
+    for (int q = 0; q < R1; ++q) v[q] = ys[gs + q * R2];
+  }
+  row_factors(A, false, f, row0, rows, s_ft, &s_tf);
+  __syncthreads();
+  cpx<R> dsum = mk<R>(0, 0);
+  if (site) {
+    const R* __restrict__ gx = A.greal + (size_t)f * nt;
+    const cpx<R>* __restrict__ ex = A.gcplx + (size_t)f * (nt + 4);
+    const cpx<R>* __restrict__ dx = dph + (size_t)f * nt;
+    const int iy = row % ny, iz = row / ny;
+    const R ar = s_ft[j] * gx[nx + iy] * gx[nx + ny + iz];
+    const cpx<R> br = ex[nt + c] * (s_tf * (ex[nx + iy] * ex[nx + ny + iz]));
+    const cpx<R> rot = source_rotation<R>(acomp, c);
+#pragma unroll
+    for (int q = 0; q < R1; ++q) {
+      const int x = g + q * R2;
+      v[q] = source_term<R>(v[q], br, ex[x], ar * gx[x], rot);
+      const cpx<R> e = dx[x];
+      dsum = mk<R>(dsum.x + v[q].x * e.x - v[q].y * e.y, dsum.y + v[q].x * e.y + v[q].y * e.x);
+    }
+    dsum = dsum * (dx[nx + iy] * dx[nx + ny + iz]);
+    Dft<R, R1>::run(v, false);
+    cpx<R>* sl = sm + (4 * j + oc) * LS + g;
+    sl[0] = v[0];
+#pragma unroll
+    for (int k1 = 1; k1 < R1; ++k1) sl[k1 * S] = v[k1] * tw[k1 * R2 + g];
+  }
+  __syncthreads();
+  if (mode) {
+    const size_t gt = ((size_t)f * 4 + (mline & 3)) * N + (size_t)(row0 + (mline >> 2)) * nx + gm;
+    const cpx<R>* sl = sm + mline * LS + gm * S;
+    cpx<R> m[R2];
+#pragma unroll
+    for (int i = 0; i < R2; ++i) m[i] = sl[i];
+    Dft<R, R2>::run(m, false);
+#pragma unroll
+    for (int k2 = 0; k2 < R2; ++k2) Zspec[gt + k2 * R1] = m[k2];
+  }
+  __syncthreads();
+  sm[(oc * rows + j) * TPL + g] = dsum;
+  __syncthreads();
+  direct_sums(A, sm, rows * TPL, f, ptab, tab_stride, stage, dpart);
 }
 #endif
 

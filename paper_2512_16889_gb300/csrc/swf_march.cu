@@ -1695,16 +1695,14 @@ __device__ __forceinline__ cpx<R> warp_sum(cpx<R> v) {
   return v;
 }
 
-// (alpha . eps) v for a real polarisation eps (Dirac representation), every rounding fixed (the
-// integrand must give the same bits in every launch variant).
+// (alpha . e) v for a real vector e (Dirac representation).
 template <typename R>
 __device__ __forceinline__ void alpha_eps(const R* e, const cpx<R>* v, cpx<R>* o) {
-  // sigma.eps (u0, u1) = (ez u0 + ex u1 - i ey u1, ex u0 + i ey u0 - ez u1)
-  const R mz = -e[2];
-  o[0] = xadd(xadd(xscale(e[2], v[2]), xscale(e[0], v[3])), xscale(e[1], mul_mi(v[3])));
-  o[1] = xadd(xadd(xscale(e[0], v[2]), xscale(e[1], mul_i(v[2]))), xscale(mz, v[3]));
-  o[2] = xadd(xadd(xscale(e[2], v[0]), xscale(e[0], v[1])), xscale(e[1], mul_mi(v[1])));
-  o[3] = xadd(xadd(xscale(e[0], v[0]), xscale(e[1], mul_i(v[0]))), xscale(mz, v[1]));
+  // sigma.e (u0, u1) = (ez u0 + ex u1 - i ey u1, ex u0 + i ey u0 - ez u1)
+  o[0] = mk<R>(e[2] * v[2].x + e[0] * v[3].x + e[1] * v[3].y, e[2] * v[2].y + e[0] * v[3].y - e[1] * v[3].x);
+  o[1] = mk<R>(e[0] * v[2].x - e[1] * v[2].y - e[2] * v[3].x, e[0] * v[2].y + e[1] * v[2].x - e[2] * v[3].y);
+  o[2] = mk<R>(e[2] * v[0].x + e[0] * v[1].x + e[1] * v[1].y, e[2] * v[0].y + e[0] * v[1].y - e[1] * v[1].x);
+  o[3] = mk<R>(e[0] * v[0].x - e[1] * v[0].y - e[2] * v[1].x, e[0] * v[0].y + e[1] * v[0].x - e[2] * v[1].y);
 }
 
 // J_a = x^+ alpha_a y for a = x, y, z (Dirac representation), every rounding fixed: the integrand of a
@@ -1897,156 +1895,126 @@ __global__ void k_f2_omega_table(const F2Table* tabs, GridDesc g, int n_tab, R* 
   }
 }
 
-// x lines of `rows` grid rows of wave f = 2 inst + (0: U, 1: V) at a weighted stage:
-// Z = -i V (Y + psi_b) of the stage value Y (from ys; the local term of the right-hand side,
-// evaluated as in k_first) x-transformed into Zspec[f], and with do_y also Y into Yspec[f] (grids
-// without a y or z pass; otherwise the right-hand side's pass writes the transform of Y); and
-// the block's part of sum_x exp(-i kappa.x) Z(x) (the wave's direct transform), which
-// trow[w] (w_i and its time phase) times adds to the block's own FP64 accumulators
-// dpart[f][block][4] (no other block touches them: the sum is deterministic).
-template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_f2_x(StageArgs<R> A, const cpx<R>* __restrict__ ys, cpx<R>* __restrict__ Yspec,
-                                              cpx<R>* __restrict__ Zspec, int do_y, const cpx<R>* __restrict__ dph,
-                                              const cpx<double>* __restrict__ ptab, int tab_stride, int stage,
-                                              cpx<double>* dpart, int rows, int ld) {
+// x pass of wave f = 2 inst + (0: U, 1: V) at a weighted stage (the shape of k_xpass, for lengths and
+// precisions without line kernels; the others run k_f2_line): Z = -i V (Y + psi_b) of the stage value Y
+// (from ys; the local term of the right-hand side) x-transformed into Zspec[f], and with do_y also Y into
+// Yspec[f] (grids without a y or z pass; otherwise the right-hand side's pass writes the transform of Y);
+// and the block's part of sum_x exp(-i kappa.x) Z(x) (the wave's direct transform), which trow[w] (w_i
+// and its time phase) times adds to the block's own FP64 accumulators dpart[f][block][4] (no other block
+// touches them: the sum is deterministic).  A thread that holds sites of Y's component c works on the
+// component of Z that c feeds.  Rows per block are fixed, not tuned: they decide the order of the sum.
+// Bound by FP64 issue; the threads' four or fewer values fill every quarter of every SM.  Two instances
+// of 128^2 in FP64: 80 us, where whole lines of one thread group took 106 us.
+template <typename R, int R0>
+__global__ void __launch_bounds__(kPassThreads, 1)
+k_f2_x(const __grid_constant__ StageArgs<R> A, const cpx<R>* __restrict__ ys, cpx<R>* __restrict__ Yspec,
+       cpx<R>* __restrict__ Zspec, int do_y, const cpx<R>* __restrict__ dph, const cpx<double>* __restrict__ ptab,
+       int tab_stride, int stage, cpx<double>* dpart, int rows, int ld, int tpl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<R>* buf = reinterpret_cast<cpx<R>*>(smem_raw);
-  cpx<R>* buf2 = buf + 4 * rows * ld;
-  __shared__ R s_ft[64];  // field time factor per row, computed in FP64 and rounded once
+  __shared__ R s_ft[64];
   __shared__ cpx<R> s_tf;
-  __shared__ cpx<double> red[8][4];
-  const int f = blockIdx.y;
-  const int inst = f >> 1, w = f & 1;
-  const int row0 = blockIdx.x * rows;
-  const int nx = A.g.n[0], ny = A.g.n[1], nz = A.g.n[2];
-  const int N = A.g.N;
-  const size_t fo = (size_t)f * 4 * N;
-  const size_t cs = (size_t)N;
-  const FieldDesc* F = A.fd + f;
-  const double tst = stage_time(A);
-  for (int j = threadIdx.x; j < rows; j += blockDim.x) {
-    const int iy = (row0 + j) % ny;
-    const double yc = ny > 1 ? A.g.x0[1] + iy * A.g.dx[1] : 0.0;
-    s_ft[j] = (R)field_time_factor(*F, tst, yc);
-  }
-  if (threadIdx.x == 0) {
-    double sn, c;
-    sincos(F->tsign * F->e0 * tst, &sn, &c);
-    s_tf = mk<R>((R)c, (R)sn);
-  }
+  const RadixPlan& pl = A.plan[0];
+  const int nx = pl.n, ny = A.g.n[1], nz = A.g.n[2], nb = nx / R0, rl = end_radix(pl, false);
+  const size_t N = A.g.N;
+  const int f = blockIdx.y, row0 = blockIdx.x * rows;
+  const int line = threadIdx.x / tpl, g = threadIdx.x - line * tpl;
+  const int c = line & 3, jr = line >> 2, row = row0 + jr;
+  const bool ok = line < 4 * rows && row < A.nrows;
+  cpx<R>* a = reinterpret_cast<cpx<R>*>(smem_raw);
+  cpx<R>* b2 = a + 4 * rows * ld;
+  const cpx<R>* __restrict__ tw = A.tw[0];
+  const bool one = pl.npass < 2;
+  row_factors(A, false, f, row0, rows, s_ft, &s_tf);
   __syncthreads();
   const int nt = nx + ny + nz;
-  const R* gx = A.greal + (size_t)f * nt;
-  const R* gy = gx + nx;
-  const R* gz = gy + ny;
-  const cpx<R>* ex = A.gcplx + (size_t)f * (nt + 4);
-  const cpx<R>* ey = ex + nx;
-  const cpx<R>* ez = ey + ny;
-  const cpx<R>* wsp = ez + nz;
-  const cpx<R>* dx = dph + (size_t)f * nt;
-  const int acomp = F->acomp;
-  const int per = rows * nx;
-  cpx<R>* sy = Yspec + fo;
-  cpx<R>* sz = Zspec + fo;
-  cpx<R> dsum[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) dsum[c] = mk<R>(0, 0);
+  const R* __restrict__ gx = A.greal + (size_t)f * nt;
+  const cpx<R>* __restrict__ ex = A.gcplx + (size_t)f * (nt + 4);
+  const cpx<R>* __restrict__ dx = dph + (size_t)f * nt;
+  const int acomp = A.fd[f].acomp;
+  const int oc = source_component(acomp, c);
+  const cpx<R> rot = source_rotation<R>(acomp, c);
+  const size_t gl = ((size_t)f * 4 + c) * N + (size_t)row * nx;   // Y's line
+  const size_t go = ((size_t)f * 4 + oc) * N + (size_t)row * nx;  // the line of Z
+  const int iy = ok ? row % ny : 0, iz = ok ? row / ny : 0;
+  const R ar = ok ? s_ft[jr] * gx[nx + iy] * gx[nx + ny + iz] : (R)0;
+  const cpx<R> br = ex[nt + c] * (s_tf * (ex[nx + iy] * ex[nx + ny + iz]));
+  cpx<R> dsum = mk<R>(0, 0);
   for (int part = do_y ? 0 : 1; part < 2; ++part) {
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / nx;
-      const int x = e - j * nx;
-      const int row = row0 + j;
-      cpx<R> v[4];
-      if (row < A.nrows) {
-        const size_t gi = fo + (size_t)row * nx + x;
+    const int sl = part ? 4 * jr + oc : line;  // the exchange line of what this thread transforms
+    if (ok)
+      for (int b = g; b < nb; b += tpl) {
+        cpx<R> v[R0];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = ys[gi + c * cs];
-        if (part == 1) {
-          const int iy = row % ny, iz = row / ny;
-          const R a = s_ft[j] * gx[x] * gy[iy] * gz[iz];
-          const cpx<R> ph = s_tf * ex[x] * ey[iy] * ez[iz];
-          cpx<R> phi[4], vz[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) phi[c] = v[c] + wsp[c] * ph;
-          apply_v<R>(acomp, a, phi, vz);
-          const cpx<R> dp = dx[x] * dx[nx + iy] * dx[nx + ny + iz];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            v[c] = mul_mi(vz[c]);
-            dsum[c] = dsum[c] + v[c] * dp;
+        for (int q = 0; q < R0; ++q) {
+          const int x = b + q * nb;
+          v[q] = ys[gl + x];
+          if (part) {
+            v[q] = source_term<R>(v[q], br, ex[x], ar * gx[x], rot);
+            const cpx<R> e = dx[x];
+            dsum = mk<R>(dsum.x + v[q].x * e.x - v[q].y * e.y, dsum.y + v[q].x * e.y + v[q].y * e.x);
           }
         }
-      } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = mk<R>(0, 0);
+        first_butterfly<R, R0>(v, b, false, a + sl * ld);
       }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) buf[(c * rows + j) * ld + pad<R>(x)] = v[c];
-    }
     __syncthreads();
-    cpx<R>* res = fft_pp<R>(buf, buf2, ld, 4 * rows, A.plan[0], false, A.tw[0]);
-    cpx<R>* dst = part == 0 ? sy : sz;
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / nx;
-      const int x = e - j * nx;
-      const int row = row0 + j;
-      if (row < A.nrows) {
-        const size_t gi = (size_t)row * nx + x;
+    const cpx<R>* cur = middle_passes<R>(a, b2, ld, 4 * rows, pl, false, tw);
+    if (ok)
+      with_radix(rl, [&](auto rc) {
+        constexpr int RL = decltype(rc)::value;
+        const int nm = nx / RL;
+        cpx<R>* dst = part ? Zspec + go : Yspec + gl;
+        for (int b = g; b < nm; b += tpl) {
+          cpx<R> m[RL];
+          last_butterfly<R, RL>(cur + sl * ld, b, nx, one, false, tw, m);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) dst[gi + c * cs] = res[(c * rows + j) * ld + pad<R>(x)];
-      }
-    }
+          for (int q = 0; q < RL; ++q) dst[b + q * nm] = m[q];
+        }
+      });
     __syncthreads();
   }
-  // block sum of the direct transform (warp trees in the march precision, FP64 across warps)
-  cpx<R> ds[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) ds[c] = warp_sum<R>(dsum[c]);
-  if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-    for (int c = 0; c < 4; ++c) red[threadIdx.x >> 5][c] = cvt<double>(ds[c]);
-  }
+  // direct transform: the phases of the other axes, then the sum over the block's threads
+  cpx<R>* red = a;
+  if (line < 4 * rows) red[(oc * rows + jr) * tpl + g] = ok ? dsum * (dx[nx + iy] * dx[nx + ny + iz]) : mk<R>(0, 0);
   __syncthreads();
-  if (threadIdx.x < 4) {
-    const long tab_row = (long)(A.clk->step + A.ls) * 7 + stage;
-    const cpx<double> wt = ptab[3 * (tab_row + (long)inst * tab_stride) + w];
-    cpx<double> sacc = mk<double>(0, 0);
-    for (int wi = 0; wi < (int)(blockDim.x >> 5); ++wi) sacc = sacc + red[wi][threadIdx.x];
-    cpx<double>& a = dpart[((size_t)f * gridDim.x + blockIdx.x) * 4 + threadIdx.x];
-    a = a + wt * sacc;
-  }
+  direct_sums(A, red, rows * tpl, f, ptab, tab_stride, stage, dpart);
 }
 
-// o = P_+(kappa) x = (x + H0(kappa) x / E) / 2, the positive-energy part (evolves as e^{-iEt}).
+// o = P_+(kappa) x = (x + H0(kappa) x / E) / 2, the positive-energy part (evolves as e^{-iEt}); ke =
+// kappa / (2 E), hp, hm = (1 +- 1/E) / 2.
 template <typename R>
-__device__ __forceinline__ void proj_plus(const R* kk, R inv_e, const cpx<R>* x, cpx<R>* o) {
-  cpx<R> hx[4];
-  alpha_eps<R>(kk, x, hx);
-  const R hh = (R)0.5 * inv_e;
-  o[0] = (R)0.5 * x[0] + hh * (hx[0] + x[0]);
-  o[1] = (R)0.5 * x[1] + hh * (hx[1] + x[1]);
-  o[2] = (R)0.5 * x[2] + hh * (hx[2] - x[2]);
-  o[3] = (R)0.5 * x[3] + hh * (hx[3] - x[3]);
+__device__ __forceinline__ void proj_plus(const R* ke, R hp, R hm, const cpx<R>* x, cpx<R>* o) {
+  alpha_eps<R>(ke, x, o);
+  o[0] = o[0] + hp * x[0];
+  o[1] = o[1] + hp * x[1];
+  o[2] = o[2] + hm * x[2];
+  o[3] = o[3] + hm * x[3];
 }
+__device__ __forceinline__ float inv_root(float x) { return 1.0f / sqrtf(x); }
+__device__ __forceinline__ double inv_root(double x) { return rsqrt(x); }
 
-// sum_a conj(x_a) (alpha.eps y)_a
+// s += sum_a conj(x_a) (a y_a + b z_a)
 template <typename R>
-__device__ __forceinline__ cpx<R> form_ae(const cpx<R>* x, const cpx<R>* aey) {
-  cpx<R> d = cdot(x[0], aey[0]);
+__device__ __forceinline__ void form_add(cpx<R>& s, const cpx<R>* x, R a, const cpx<R>* y, R b, const cpx<R>* z) {
 #pragma unroll
-  for (int a = 1; a < 4; ++a) d = d + cdot(x[a], aey[a]);
-  return d;
+  for (int c = 0; c < 4; ++c) {
+    const cpx<R> w = mk<R>(a * y[c].x + b * z[c].x, a * y[c].y + b * z[c].y);
+    s.x = s.x + x[c].x * w.x + x[c].y * w.y;
+    s.y = s.y + x[c].x * w.y - x[c].y * w.x;
+  }
 }
 
 // The mode sum of the (scat, scat) integrand at one weighted stage, on the raw transforms Yspec, Zspec
 // of the waves (no cell factor, no origin phase):
 //   sum_j sum_{sigma,sigma'} 1/Omega [ (P_s Zu~)^+ (alpha.eps) P_s' Yv~ + (P_s Yu~)^+ (alpha.eps) P_s' Zv~ ]
 // with U quantities at mode j and V quantities at mode j - shift.  Block (b, inst) adds trow[2]
-// (w_i e^{-i k0 t}) times its part to its own accumulator sspart[inst][b].
+// (w_i e^{-i k0 t}) times its part to its own accumulator sspart[inst][b].  In FP64 the instruction count
+// is what bounds it: alpha.eps as additions of scaled components, both projections of a vector from one
+// H0 x, both signs of sigma' summed before the contraction.  Two instances of 128^2 in FP64: 70 us, where
+// a projection and a contraction for every sign took 113 us.
 // f2i per instance: shift[3], table index.
 template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_f2_ss(const cpx<R>* __restrict__ Yspec, const cpx<R>* __restrict__ Zspec,
-                                               GridDesc g, const FieldDesc* fd,
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_f2_ss(const cpx<R>* __restrict__ Yspec,
+                                               const cpx<R>* __restrict__ Zspec, GridDesc g, const FieldDesc* fd,
                                                const double* photon, const int* __restrict__ f2i,
                                                const R* __restrict__ omt, const cpx<double>* __restrict__ ptab,
                                                const MarchClock* clk, int ls, int stage, int tab_stride,
@@ -2085,44 +2053,47 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_f2_ss(const cpx
       kv[a] = n > 1 ? du[a] * (R)fv : (R)FV.K[a];
     }
     const int j2 = (jv[2] * g.n[1] + jv[1]) * g.n[0] + jv[0];
-    const R ieu = (R)1 / sqrt((R)1 + ku[0] * ku[0] + ku[1] * ku[1] + ku[2] * ku[2]);
-    const R iev = (R)1 / sqrt((R)1 + kv[0] * kv[0] + kv[1] * kv[1] + kv[2] * kv[2]);
-    cpx<R> y[4], z[4], ap[4], am[4], dap[4], dam[4];
+    const R ieu = inv_root((R)1 + ku[0] * ku[0] + ku[1] * ku[1] + ku[2] * ku[2]);
+    const R iev = inv_root((R)1 + kv[0] * kv[0] + kv[1] * kv[1] + kv[2] * kv[2]);
+    const R hu = (R)0.5 * ieu, hv = (R)0.5 * iev;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      y[c] = Yu[(size_t)c * N + j];
-      z[c] = Zu[(size_t)c * N + j];
+    for (int a = 0; a < 3; ++a) {
+      ku[a] *= hu;
+      kv[a] *= hv;
     }
-    proj_plus<R>(ku, ieu, y, ap);
-    proj_plus<R>(ku, ieu, z, dap);
+    // U side: the parts of Y and Z; V side: (alpha.eps) on the parts
+    cpx<R> ym[4], yp[4], zm[4], zp[4], t[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      am[c] = y[c] - ap[c];
-      dam[c] = z[c] - dap[c];
+      ym[c] = Yu[(size_t)c * N + j];
+      zm[c] = Zu[(size_t)c * N + j];
     }
+    proj_plus<R>(ku, (R)0.5 + hu, (R)0.5 - hu, ym, yp);
+    proj_plus<R>(ku, (R)0.5 + hu, (R)0.5 - hu, zm, zp);
+    cpx<R> y[4], z[4], ayp[4], aym[4], azp[4], azm[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
+      ym[c] = ym[c] - yp[c];
+      zm[c] = zm[c] - zp[c];
       y[c] = Yv[(size_t)c * N + j2];
       z[c] = Zv[(size_t)c * N + j2];
     }
-    cpx<R> bp[4], bm[4], dbp[4], dbm[4], t1[4], t2[4];
-    proj_plus<R>(kv, iev, y, t1);
-    proj_plus<R>(kv, iev, z, t2);
-    alpha_eps<R>(eps, t1, bp);
-    alpha_eps<R>(eps, t2, dbp);
+    proj_plus<R>(kv, (R)0.5 + hv, (R)0.5 - hv, y, t);
+    alpha_eps<R>(eps, t, ayp);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      t1[c] = y[c] - t1[c];
-      t2[c] = z[c] - t2[c];
-    }
-    alpha_eps<R>(eps, t1, bm);
-    alpha_eps<R>(eps, t2, dbm);
+    for (int c = 0; c < 4; ++c) t[c] = y[c] - t[c];
+    alpha_eps<R>(eps, t, aym);
+    proj_plus<R>(kv, (R)0.5 + hv, (R)0.5 - hv, z, t);
+    alpha_eps<R>(eps, t, azp);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) t[c] = z[c] - t[c];
+    alpha_eps<R>(eps, t, azm);
     const R* o = om + 4 * (size_t)j;
     const R opp = o[0], opm = o[1], omp = o[2], omm = o[3];
-    tacc = tacc + opp * (form_ae<R>(dap, bp) + form_ae<R>(ap, dbp));
-    tacc = tacc + opm * (form_ae<R>(dap, bm) + form_ae<R>(ap, dbm));
-    tacc = tacc + omp * (form_ae<R>(dam, bp) + form_ae<R>(am, dbp));
-    tacc = tacc + omm * (form_ae<R>(dam, bm) + form_ae<R>(am, dbm));
+    form_add<R>(tacc, zp, opp, ayp, opm, aym);
+    form_add<R>(tacc, yp, opp, azp, opm, azm);
+    form_add<R>(tacc, zm, omp, ayp, omm, aym);
+    form_add<R>(tacc, ym, omp, azp, omm, azm);
   }
   const cpx<R> s = warp_sum<R>(tacc);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = cvt<double>(s);
@@ -2170,36 +2141,52 @@ struct F2Plan {
   R* omt = nullptr;          // [tables][N][4]: rho / Omega
   cpx<double>* dpart = nullptr;   // [2 n_inst][nbx][4]
   cpx<double>* sspart = nullptr;  // [n_inst][nbs]
-  int n_inst = 0, nbx = 0, nbs = 0, rows = 0, ld = 0, xthr = 256;
+  int n_inst = 0, nbx = 0, nbs = 0, rows = 0, ld = 0, tpl = 0;  // (k_f2_x: rows per block, threads per line)
+  RadixPlan plan;
+  const LineEntry<R>* entry = nullptr;  // the x axis's line kernels, if it has some
   size_t smem_x = 0;
 };
+
+template <typename R, int... R0>
+static cudaError_t f2_attrs(std::integer_sequence<int, R0...>) {
+  cudaError_t e = cudaSuccess;
+  ((e = e != cudaSuccess ? e : cudaFuncSetAttribute(k_f2_x<R, R0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmemMax)), ...);
+  return e;
+}
 
 template <typename R>
 static swf_status f2_prepare(swf_ctx* ctx, const GridDesc& g, int n_inst, const FieldDesc* fd_host,
                              const double* photon_host, const double* wave_k_host,
                              F2Plan<R>* p, cudaStream_t st) {
-  static bool attr_done[64] = {false};
-  const int dv = dev_slot();
   cudaError_t e;
-  if (!attr_done[dv]) {
-    e = cudaFuncSetAttribute(k_f2_x<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmem);
-    if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_f2_x)");
-    attr_done[dv] = true;
+  {
+    static std::atomic<bool> done[64];
+    const int dv = dev_slot();
+    if (!done[dv].load(std::memory_order_acquire)) {
+      if ((e = f2_attrs<R>(std::integer_sequence<int, 1, 2, 3, 4, 5>())) != cudaSuccess)
+        return cuda_status(e, "cudaFuncSetAttribute(k_f2_x)");
+      done[dv].store(true, std::memory_order_release);
+    }
   }
   const int nx = g.n[0];
   const int nrows = g.n[1] * g.n[2];
   const int nt = g.n[0] + g.n[1] + g.n[2];
   p->n_inst = n_inst;
-  // a fixed shape (not the tuned one of the right-hand side's x passes): the block's rows and
-  // threads decide the order of the direct-transform sums, which must not depend on timing
-  p->rows = x_rows<R>(nx, nrows, 2 * n_inst);
-  p->xthr = kThreads;
-  if (p->rows < 1) {
-    set_error("partial-integration integrand: an x line does not fit shared memory");
-    return SWF_EUNSUPPORTED;
+  // a fixed shape (not the tuned one of the right-hand side's x passes): the block's rows decide the order
+  // of the direct-transform sums, which must not depend on timing.  About 128 threads: as many rows as
+  // that takes, at most 64.
+  p->entry = line_of<R>(g, 0);
+  if (p->entry) {
+    p->tpl = line_threads(p->entry->r1, p->entry->r2);
+    p->rows = std::max(1, std::min(128 / (4 * p->tpl), nrows));
+    p->smem_x = xline_smem<R>(p->entry, p->rows);  // (at least as many values as threads)
+  } else {
+    make_pass_plan(nx, &p->plan);
+    p->tpl = pass_threads(p->plan, 4);
+    p->ld = padded_len<R>(nx);
+    p->rows = std::max(1, std::min(std::min(128 / (4 * p->tpl), 64), nrows));
+    p->smem_x = (size_t)8 * p->rows * p->ld * sizeof(cpx<R>);
   }
-  p->ld = padded_len<R>(nx);
-  p->smem_x = (size_t)2 * 4 * p->rows * p->ld * sizeof(cpx<R>);
   p->nbx = (nrows + p->rows - 1) / p->rows;
   // one mode per thread where the grid allows (the gathers of the V modes are latency-bound)
   p->nbs = std::max(1, std::min((g.N + 255) / 256, (32 * sm_count() + n_inst - 1) / n_inst));
@@ -2289,11 +2276,25 @@ static swf_status f2_integrand(swf_ctx* ctx, const StageArgs<R>& A, const F2Plan
   StageArgs<R> B = A;
   B.ls = ls;
   B.c = DP_C[stage];
-  if (sizeof(R) == 4) make_march_plan(g.n[0], &B.plan[0]);  // a whole-line transform (lengths were checked)
+  B.plan[0] = p.plan;
   {
     ProfScope ps(ctx, "k_f2_x", st);
-    k_f2_x<R><<<dim3(p.nbx, 2 * G), p.xthr, p.smem_x, st>>>(B, ys, p.Yspec, p.Zspec, p.has_mid ? 0 : 1, p.dph,
-                                                             ptab, tab_stride, stage, p.dpart, p.rows, p.ld);
+    const dim3 grid(p.nbx, 2 * G);
+    if (p.entry) {
+      p.entry->f2<<<grid, 4 * p.rows * p.tpl, p.smem_x, st>>>(B, ys, p.Zspec, p.dph, ptab, tab_stride, stage, p.dpart,
+                                                              p.rows);
+    } else {
+      auto* kernel = k_f2_x<R, 1>;
+      switch (end_radix(p.plan, true)) {
+        case 4: kernel = k_f2_x<R, 4>; break;
+        case 2: kernel = k_f2_x<R, 2>; break;
+        case 3: kernel = k_f2_x<R, 3>; break;
+        case 5: kernel = k_f2_x<R, 5>; break;
+        default: break;
+      }
+      kernel<<<grid, 4 * p.rows * p.tpl, p.smem_x, st>>>(B, ys, p.Yspec, p.Zspec, p.has_mid ? 0 : 1, p.dph, ptab,
+                                                          tab_stride, stage, p.dpart, p.rows, p.ld, p.tpl);
+    }
   }
   StageArgs<R> C = A;
   C.T = p.Zspec;
