@@ -444,43 +444,66 @@ __global__ void k_refresh(const float* p, __nv_bfloat16* wbf, __nv_bfloat16* fpa
 }  // namespace tr
 
 // ---------------------------------------------------------------- fused inference on tcgen05
-// One CTA (256 threads) per SM, persistent over tiles of 128 rows.  Layer 0 (K = 6) and the
-// output layer (N = 2) run on the CUDA cores; the three 256 x 256 layers are single-CTA
-// tcgen05.mma (kind::f16, BF16 operands, M = 128, N = 256, K = 16 per instruction) from shared
-// memory into an FP32 accumulator of 256 tensor-memory columns.  Operands use the K-major
-// no-swizzle canonical layout: element (r, k) of a 256-wide operand at byte
+// One CTA per SM, persistent over tiles of 128 rows, two tiles in flight.  Layer 0 (K = 6) and the
+// output layer (N = 2) run on the CUDA cores; the three 256 x 256 layers are single-CTA tcgen05.mma
+// (kind::f16, BF16 operands, M = 128, N = 128, K = 16 per instruction) from shared memory into an FP32
+// accumulator of 256 tensor-memory columns per tile.  Operands use the K-major no-swizzle canonical
+// layout, 8 x 8 core matrices of 128 contiguous bytes: element (r, k) of an activation tile is at byte
 //     (r / 8) * 4096 + (k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2,
-// i.e. 8 x 8 core matrices of 128 contiguous bytes, K-adjacent core matrices 128 B apart (the
-// descriptor's leading byte offset) and 8-row groups 4096 B apart (its stride byte offset).
-// The weights of layers 1-3 are kept in global memory in exactly that image (packed after every
-// update) and brought in with one bulk asynchronous copy per layer, overlapping the previous
-// layer's epilogue.  The epilogue adds the bias, applies GELU and writes the BF16 activation
-// back into the operand buffer; after layer 3 it contracts with the output weights.
+// i.e. K-adjacent core matrices 128 B apart (the descriptor's leading byte offset) and 8-row groups
+// 4096 B apart (its stride byte offset); a layer's weights are cut into eight blocks of 128 rows and 64 k
+// (16 KB), 8-row groups 1024 B apart, and kept in global memory in that image (packed after every
+// update).
+//
+// What bounds it is the GELU: 1024 values a row, each about 12 multiply-adds (run as packed pairs), an
+// exponential and a reciprocal: 16 k issue slots a tile and scheduler.  The matrix products (6.2k cycles
+// a tile) and the weights' way from L2 (384 KB a tile) therefore have to hide behind it.  Two groups of
+// eight warps each own a tile and its operand buffer; while one waits for a layer the other applies the
+// activation.  A layer goes by halves of its columns: the products of the first column half with the
+// first half of K start while the second half of the layer before is still being activated, and its
+// activation starts while the second column half is being multiplied.  One thread issues all MMAs in a
+// fixed order (layer by layer, group by group), another keeps a ring of four weight blocks filled in
+// that order; both loops are unrolled over a layer's blocks, because the time that these two threads
+// take between blocks is what a layer waits for.
+// A million rows take 0.72 ms (0.41 ms of multiply-adds); with one tile in flight, whole layers and
+// scalar GELUs they took 1.18 ms, and one tile alone 30 us instead of 27.  The halves gave the last 0.07 ms,
+// unrolling those two threads' loops 0.03.
 namespace tc {
 
-constexpr int THREADS = 512;
+constexpr int GROUP = 256;                        // threads of a tile
+constexpr int THREADS = 2 * GROUP + 64;           // two groups, the weights' warp, the MMAs' warp
 constexpr int TILE = 128;
-constexpr uint32_t OP_BYTES_A = TILE * 256 * 2;   // 64 KB
-constexpr uint32_t OP_BYTES_W = 256 * 256 * 2;    // 128 KB
+constexpr int KB = 64;                            // k per weight block
+constexpr int NBLK = 2 * 256 / KB;                // weight blocks of a layer: column half, then k
+constexpr int RING = 4;                           // half a layer: a block's slot and parity follow from its place
+constexpr uint32_t A_BYTES = TILE * 256 * 2;      // 64 KB
+constexpr uint32_t W_BYTES = 128 * KB * 2;        // 16 KB
 constexpr uint32_t OFF_A = 0;
-constexpr uint32_t OFF_W = OFF_A + OP_BYTES_A;
-constexpr uint32_t OFF_W0 = OFF_W + OP_BYTES_W;   // float [256][6]
-constexpr uint32_t OFF_B = OFF_W0 + 256 * 6 * 4;  // float [4][256]: b0..b3
-constexpr uint32_t OFF_W4 = OFF_B + 4 * 256 * 4;  // float [2][256]
-constexpr uint32_t OFF_RED = OFF_W4 + 2 * 256 * 4;  // float [4][128][2]
-constexpr uint32_t OFF_MISC = OFF_RED + 4 * TILE * 2 * 4;
-constexpr uint32_t SMEM = OFF_MISC + 64;
+constexpr uint32_t OFF_W = OFF_A + 2 * A_BYTES;
+constexpr uint32_t OFF_W0 = OFF_W + RING * W_BYTES;   // float [128][16]: per column pair the weights
+                                                      // (w_c0, w_d0, w_c1, ...), then the biases
+constexpr uint32_t OFF_B = OFF_W0 + 128 * 16 * 4;     // float [3][256]: b1..b3
+constexpr uint32_t OFF_W4 = OFF_B + 3 * 256 * 4;      // float [256][2]
+constexpr uint32_t OFF_RED = OFF_W4 + 2 * 256 * 4;    // float [2][128][4]
+constexpr uint32_t OFF_X = OFF_RED + 2 * TILE * 4 * 4;  // float [2][128][6]: inputs
+constexpr uint32_t OFF_MISC = OFF_X + 2 * TILE * 6 * 4;
+constexpr uint32_t SMEM = OFF_MISC + 256;
 constexpr long long WAIT_CYCLES = 4000000000LL;   // about two seconds at the maximum clock
 
-// instruction descriptor: D FP32, A and B BF16, both K-major, N = 128 (one column half), M = 128
+// instruction descriptor: D FP32, A and B BF16, both K-major, N = 128, M = 128
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
-__host__ __device__ __forceinline__ uint32_t op_offset(int r, int k) {
+__device__ __forceinline__ uint32_t act_offset(int r, int k) {
   return (uint32_t)((r >> 3) * 4096 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
 }
+// element (n, k) of a layer's weights in its image, in bytes
+__host__ __device__ __forceinline__ uint32_t weight_offset(int n, int k) {
+  return (uint32_t)(((n >> 7) * (256 / KB) + k / KB) * (int)W_BYTES + ((n & 127) >> 3) * (KB / 8 * 128) +
+                    ((k % KB) >> 3) * 128 + (n & 7) * 16 + (k & 7) * 2);
+}
 
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(4096u >> 4) << 32) |
+__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t stride) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(stride >> 4) << 32) |
          (1ull << 46);
 }
 
@@ -489,75 +512,129 @@ __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cv
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 
-// Waits for the phase with the given parity to complete; false after WAIT_CYCLES.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  const long long t0 = clock64();
-  while (true) {
+// Waits for the phase with the given parity to complete; false after WAIT_CYCLES, or as soon as another
+// thread has given up (*abort, where given), which it then says itself.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
+  auto done = [&] {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(bar), "r"(parity)
         : "memory");
-    if (ok) return true;
-    if (clock64() - t0 > WAIT_CYCLES) return false;
+    return ok != 0;
+  };
+  if (done()) return true;
+  const long long t0 = clock64();
+  while (!done()) {
+    if ((abort && *abort) || clock64() - t0 > WAIT_CYCLES) {
+      if (abort) *abort = 1;
+      return false;
+    }
   }
+  return true;
 }
 
-__device__ __forceinline__ void load_weights(uint32_t dst, const void* src, uint32_t bar) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(OP_BYTES_W) : "memory");
-  for (uint32_t c = 0; c < OP_BYTES_W; c += 32768)
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst + c),
-                 "l"((const char*)src + c), "r"(32768u), "r"(bar)
-                 : "memory");
+__device__ __forceinline__ void load_block(uint32_t dst, const void* src, uint32_t bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(W_BYTES) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(W_BYTES), "r"(bar)
+               : "memory");
 }
 
-// D[:, 0:128) = A W_half^T over K = 256 (16 instructions); W_half = rows [128 h, 128 h + 128) of W
-__device__ __forceinline__ void mma_half(uint32_t tmem_d, uint32_t a_base, uint32_t w_base) {
-#pragma unroll
-  for (int kk = 0; kk < 16; ++kk) {
-    const uint64_t ad = smem_desc(a_base + kk * 256), bd = smem_desc(w_base + kk * 256);
-    const uint32_t acc = kk > 0 ? 1u : 0u;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
-            tmem_d),
-        "l"(ad), "l"(bd), "r"(IDESC), "r"(acc)
-        : "memory");
-  }
+// D (+)= A W^T over one k16 step
+__device__ __forceinline__ void mma_step(uint32_t tmem_d, uint64_t ad, uint64_t bd, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
+          tmem_d),
+      "l"(ad), "l"(bd), "r"(IDESC), "r"(acc)
+      : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
+// 16 columns of this warp's 32 rows; complete after tmem_wait on the same registers
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
-
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
+__device__ __forceinline__ void tmem_wait(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])::"memory");
 }
 
 __device__ __forceinline__ float round_bf16(float a) { return __bfloat162float(__float2bfloat16(a)); }
 
+// Two floats in one register pair: one instruction per operation on both, each rounded as alone.
+using pair = unsigned long long;
+__device__ __forceinline__ pair pack(float a, float b) {
+  pair r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack(pair p, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+}
+__device__ __forceinline__ pair both(float a) { return pack(a, a); }
+__device__ __forceinline__ pair fma2(pair a, pair b, pair c) {
+  pair r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ pair mul2(pair a, pair b) {
+  pair r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ pair add2(pair a, pair b) {
+  pair r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// gelu() of two values, the same operations and bits (below |x| = 13; beyond it a tail smaller than the
+// smallest normal number is zero): factors 1/2 are folded into constants, which is exact, and the select
+// between tail and 1 - tail is an addition, 0 + tail or 1 - tail.
+__device__ __forceinline__ pair gelu2(pair x) {
+  float x0, x1, y0, y1, t0, t1, e0, e1;
+  unpack(x, x0, x1);
+  unpack(fma2(both(0.3275911f), pack(fabsf(x0) * 0.70710678118654752f, fabsf(x1) * 0.70710678118654752f), both(1.0f)), y0, y1);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(y0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(y1));
+  const pair t = pack(t0, t1);
+  pair h = fma2(t, both(0.5f * 1.061405429f), both(0.5f * -1.453152027f));
+  h = fma2(t, h, both(0.5f * 1.421413741f));
+  h = fma2(t, h, both(0.5f * -0.284496736f));
+  h = fma2(t, h, both(0.5f * 0.254829592f));
+  // e^{-x^2 / 2}: log2(e) as a float, halved
+  unpack(mul2(mul2(x, x), both(-0.5f * 1.44269502f)), e0, e1);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(e0));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(e1));
+  unpack(mul2(mul2(t, h), pack(e0, e1)), t0, t1);  // the tail (1 - erf) / 2
+  return mul2(x, add2(pack(copysignf(t0, -x0), copysignf(t1, -x1)), pack(x0 >= 0.0f ? 1.0f : 0.0f, x1 >= 0.0f ? 1.0f : 0.0f)));
+}
+__device__ __forceinline__ uint32_t pack_bf16(pair p) {
+  float a, b;
+  unpack(p, a, b);
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
 // x [B][6] fp32 features; wpack: layers 1-3 in the operand image; wbf: all parameters in BF16
 // (W0 and W4 read from it); params: FP32 parameters (biases read from it).  Writes out [B][2]
 // = (mu, log sigma^2) in the target's units.  *err is set to 1 if a wait timed out.
-// 16 warps: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (its rows) and columns
-// [64 (w / 4), + 64).  Each layer's MMAs run as two column halves with their own commits, so
-// the warps of half 0 start their epilogue while half 1 is still multiplying; every warp holds
-// its BF16 results in registers until both halves are done (all of A feeds both halves).
+// Warp w of a group reads tensor-memory lanes 32 (w % 4) .. + 31 (its rows) and 64 columns of each half.
 __global__ void __launch_bounds__(THREADS, 1)
 k_mlp_forward(const float* __restrict__ x, int B, const __nv_bfloat16* __restrict__ wpack,
               const __nv_bfloat16* __restrict__ wbf, const float* __restrict__ params, const float* __restrict__ shift,
@@ -566,164 +643,251 @@ k_mlp_forward(const float* __restrict__ x, int B, const __nv_bfloat16* __restric
   float* sW0 = reinterpret_cast<float*>(sm + OFF_W0);
   float* sB = reinterpret_cast<float*>(sm + OFF_B);
   float* sW4 = reinterpret_cast<float*>(sm + OFF_W4);
-  float* sRed = reinterpret_cast<float*>(sm + OFF_RED);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + OFF_MISC);  // [0] weights, [1] MMA half 0, [2] MMA half 1
-  uint32_t* sTmem = reinterpret_cast<uint32_t*>(sm + OFF_MISC + 24);
-  int* sAbort = reinterpret_cast<int*>(sm + OFF_MISC + 28);
-  float* sB4 = reinterpret_cast<float*>(sm + OFF_MISC + 32);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const uint32_t a_base = saddr(sm + OFF_A), w_base = saddr(sm + OFF_W);
-  const uint32_t barW = saddr(&bars[0]), barM0 = saddr(&bars[1]), barM1 = saddr(&bars[2]);
-  const int ntiles = (B + TILE - 1) / TILE;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + OFF_MISC);
+  // per weight block: filled, free; per group: halves of the operand written (a), column halves
+  // multiplied (d), first half of the operand no longer needed (k), partial outputs written (r)
+  const uint32_t bar_full = saddr(bars), bar_free = saddr(bars + RING), bar_a = saddr(bars + 2 * RING);
+  const uint32_t bar_d = bar_a + 32, bar_k = bar_a + 64, bar_r = bar_a + 80, bar_end = bar_a + 96;
+  uint32_t* sTmem = reinterpret_cast<uint32_t*>(sm + OFF_MISC + 192);
+  volatile int* sAbort = reinterpret_cast<volatile int*>(sm + OFF_MISC + 196);
+  float* sB4 = reinterpret_cast<float*>(sm + OFF_MISC + 200);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ntiles = (B + TILE - 1) / TILE, step = 2 * gridDim.x;
+  // tiles of group g: blockIdx.x + g gridDim.x, then every step-th
+  const int n_own[2] = {(ntiles - (int)blockIdx.x + step - 1) / step,
+                        max(0, (ntiles - (int)blockIdx.x - (int)gridDim.x + step - 1) / step)};
 
-  // small parameters (BF16 weights as the GEMM path rounds them, FP32 biases)
-  constexpr long W0OFF = 0, B0OFF = 6 * 256;
-  for (int i = tid; i < 256 * 6; i += THREADS) sW0[i] = __bfloat162float(wbf[W0OFF + i]);
-  for (int l = 0; l < 4; ++l) {
-    const long bo = (l == 0) ? B0OFF : B0OFF + 256 + (long)(l - 1) * (256 * 256 + 256) + 256 * 256;
-    for (int i = tid; i < 256; i += THREADS) sB[l * 256 + i] = params[bo + i];
+  // a tile's inputs (zero beyond the batch) into its group's buffer
+  auto fetch_x = [&](int tile, int g) {
+    for (int e = tid & (GROUP - 1); e < TILE * 6; e += GROUP) {
+      const long i = (long)tile * (TILE * 6) + e;
+      const bool in = i < (long)B * 6;
+      tr::cp_async(sm + OFF_X + (g * TILE * 6 + e) * 4, x + (in ? i : 0), 4, in);
+    }
+  };
+  if (tid < 2 * GROUP) fetch_x(blockIdx.x + (tid / GROUP) * gridDim.x, tid / GROUP);
+  // small parameters (BF16 weights, FP32 biases)
+  for (int i = tid; i < 256 * 6; i += THREADS) {
+    const int c = i / 6, f = i - 6 * c;
+    sW0[(c >> 1) * 16 + 2 * f + (c & 1)] = __bfloat162float(wbf[tr::woff(0) + i]);
   }
-  const long w4off = B0OFF + 256 + 3L * (256 * 256 + 256);
-  for (int i = tid; i < 2 * 256; i += THREADS) sW4[i] = __bfloat162float(wbf[w4off + i]);
-  if (tid < 2) sB4[tid] = params[w4off + 2 * 256 + tid];
+  for (int c = tid; c < 256; c += THREADS) {
+    sW0[(c >> 1) * 16 + 12 + (c & 1)] = params[tr::boff(0) + c];
+    for (int l = 1; l < 4; ++l) sB[(l - 1) * 256 + c] = params[tr::boff(l) + c];
+    for (int u = 0; u < 2; ++u) sW4[2 * c + u] = __bfloat162float(wbf[tr::woff(4) + u * 256 + c]);
+  }
+  if (tid < 2) sB4[tid] = params[tr::boff(4) + tid];
   if (tid == 0) {
     *sAbort = 0;
-    mbar_init(barW, 1);
-    mbar_init(barM0, 1);
-    mbar_init(barM1, 1);
+    for (int i = 0; i < RING; ++i) {
+      mbar_init(bar_full + 8 * i, 1);
+      mbar_init(bar_free + 8 * i, 1);
+    }
+    for (int g = 0; g < 2; ++g) {
+      for (int h = 0; h < 2; ++h) {
+        mbar_init(bar_a + 16 * g + 8 * h, GROUP);
+        mbar_init(bar_d + 16 * g + 8 * h, 1);
+      }
+      mbar_init(bar_k + 8 * g, 1);
+      mbar_init(bar_r + 8 * g, GROUP / 2);
+    }
+    mbar_init(bar_end, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
     const uint32_t dst = saddr(sTmem);
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(256u) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *sTmem;
-  uint32_t phW = 0, phM = 0;
-  if (tid == 0 && blockIdx.x < ntiles) load_weights(w_base, wpack, barW);
 
-  const int q = warp & 3, cq = warp >> 2;    // TMEM lane quarter and column quarter of this warp
-  const int half = cq >> 1;                  // MMA column half whose commit this warp waits for
-  const int erow = 32 * q + (tid & 31);      // epilogue row
-  const uint32_t bar_mine = half ? barM1 : barM0;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const bool more = tile + (int)gridDim.x < ntiles;
-    // layer 0 on the CUDA cores: row r, columns [64 h, 64 h + 64)
-    {
-      const int r = tid & (TILE - 1), h = tid >> 7;
-      const long row = (long)tile * TILE + r;
-      float xin[6];
+  if (warp == 2 * GROUP / 32) {
+    if (lane == 0) {  // the weights: per tile and layer its blocks in ascending k
+      const uint32_t w_base = saddr(sm + OFF_W);
+      bool ok = true;
+      int used = 0;  // blocks fetched
+      for (int i = 0; ok && i < n_own[0]; ++i)  // the order of the MMAs: tile pair, layer, group, block
+        for (int l = 0; ok && l < 3; ++l)
+          for (int g = 0; ok && g < 2 && i < n_own[g]; ++g) {
+            const char* src = (const char*)wpack + (size_t)l * (NBLK * W_BYTES);
 #pragma unroll
-      for (int f = 0; f < 6; ++f) xin[f] = row < B ? round_bf16((x[row * 6 + f] - shift[f]) * scale[f]) : 0.f;
-      for (int c0 = 64 * h; c0 < 64 * h + 64; c0 += 8) {
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-          float z[2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const float* wr = sW0 + (c0 + j + u) * 6;
-            float acc = 0.f;
-#pragma unroll
-            for (int f = 0; f < 6; ++f) acc = fmaf(xin[f], wr[f], acc);
-            z[u] = gelu(acc + sB[c0 + j + u]);
-          }
-          w[j >> 1] = pack_bf16(z[0], z[1]);
-        }
-        *reinterpret_cast<uint4*>(sm + OFF_A + op_offset(r, c0)) = make_uint4(w[0], w[1], w[2], w[3]);
-      }
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    for (int l = 1; l <= 3; ++l) {
-      if (tid == 0) {
-        if (!mbar_wait(barW, phW)) {
-          *sAbort = 1;
-        } else {
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          mma_half(tmem, a_base, w_base);
-          mma_commit(barM0);
-          mma_half(tmem + 128, a_base, w_base + 65536);
-          mma_commit(barM1);
-        }
-      }
-      phW ^= 1;
-      __syncthreads();
-      if (*sAbort) break;
-      // warp-uniform outcome: tcgen05.ld below is a warp-wide instruction
-      bool ok = __all_sync(0xffffffffu, mbar_wait(bar_mine, phM));
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16);
-      const float* bias = sB + l * 256;
-      uint32_t packed[32];
-      float o0 = 0.f, o1 = 0.f;
-      if (ok) {
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-          const int c0 = 64 * cq + 16 * cc;
-          float v[16];
-          tmem_ld16(trow + c0, v);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] = gelu(v[i] + bias[c0 + i]);
-          if (l < 3) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) packed[8 * cc + i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float a = round_bf16(v[i]);
-              o0 = fmaf(a, sW4[c0 + i], o0);
-              o1 = fmaf(a, sW4[256 + c0 + i], o1);
+            for (int kb = 0; kb < NBLK; ++kb) {
+              const int s = kb % RING;
+              // the block before in this slot has been multiplied (nothing to wait for the first time)
+              ok = ok && mbar_wait(bar_free + 8 * s, (kb / RING + 1) & 1, sAbort);
+              if (ok) load_block(w_base + s * W_BYTES, src + kb * W_BYTES, bar_full + 8 * s), ++used;
             }
           }
-        }
-      }
-      // every MMA of the layer is done before the operand buffers are overwritten; the weight
-      // buffer is then free for the next layer's (or the next tile's first) weights
-      if (half == 0 && l < 3) ok = __all_sync(0xffffffffu, ok && mbar_wait(barM1, phM));
-      if (!ok) atomicExch(sAbort, 1);
-      phM ^= 1;
-      if (tid == 256 && ok && (l < 3 || more))
-        load_weights(w_base, wpack + (size_t)(l < 3 ? l : 0) * 256 * 256, barW);
-      if (ok && l < 3) {
-#pragma unroll
-        for (int cc = 0; cc < 8; ++cc) {
-          const int c0 = 64 * cq + 8 * cc;
-          *reinterpret_cast<uint4*>(sm + OFF_A + op_offset(erow, c0)) =
-              make_uint4(packed[4 * cc], packed[4 * cc + 1], packed[4 * cc + 2], packed[4 * cc + 3]);
-        }
-      }
-      if (l == 3) {
-        sRed[(cq * TILE + erow) * 2] = o0;
-        sRed[(cq * TILE + erow) * 2 + 1] = o1;
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();
-      if (*sAbort) break;
+      // given up: the last copy into each slot lands before the block ends
+      for (int s = 0; !ok && s < RING && s < used; ++s)
+        mbar_wait(bar_full + 8 * s, ((used - 1 - s) / RING) & 1, nullptr);
     }
-    if (*sAbort) break;
-    if (tid < TILE) {
-      const long row = (long)tile * TILE + tid;
-      if (row < B) {
-        float z0 = sB4[0], z1 = sB4[1];
+  } else if (warp == 2 * GROUP / 32 + 1) {
+    if (lane == 0) {
+      const uint64_t a_desc = smem_desc(saddr(sm + OFF_A), 4096), w_desc = smem_desc(saddr(sm + OFF_W), KB / 8 * 128);
+      bool ok = true;
+      for (int i = 0; ok && i < n_own[0]; ++i)
+        for (int l = 0; ok && l < 3; ++l)
+          for (int g = 0; ok && g < 2 && i < n_own[g]; ++g) {
+            const uint64_t ad = a_desc + g * (A_BYTES / 16);
+            const uint32_t parity = (3 * i + l) & 1;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          z0 += sRed[(c * TILE + tid) * 2];
-          z1 += sRed[(c * TILE + tid) * 2 + 1];
+            for (int b = 0; b < NBLK; ++b) {
+              const int s = b % RING, half = b / (NBLK / 2), kb = b % (NBLK / 2);
+              // the first half of the operand is written and its accumulators are read; then the others
+              if (b % (NBLK / 4) == 0 && b < NBLK / 2) {
+                ok = ok && mbar_wait(bar_a + 16 * g + 8 * (b > 0), parity, sAbort);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              }
+              ok = ok && mbar_wait(bar_full + 8 * s, (b / RING) & 1, sAbort);
+              if (ok) {
+#pragma unroll
+                for (int kk = 0; kk < KB / 16; ++kk)  // 16 k are two core matrices, 256 bytes
+                  mma_step(tmem + 256 * g + 128 * half, ad + kb * (KB / 8 * 128 / 16) + kk * 16,
+                           w_desc + s * (W_BYTES / 16) + kk * 16, kb + kk > 0);
+                mma_commit(bar_free + 8 * s);
+                if (b == NBLK / 2 - 1 || b == NBLK - 1) mma_commit(bar_d + 16 * g + 8 * half);
+                if (b == NBLK / 2 + NBLK / 4 - 1) mma_commit(bar_k + 8 * g);
+              }
+            }
+          }
+      mma_commit(bar_end);  // nothing of this thread is in flight when the tensor memory is given back
+      mbar_wait(bar_end, 0, nullptr);
+    }
+  } else {
+    const int g = warp >> 3, q = warp & 3, half = (warp >> 2) & 1;
+    const int row_l = 32 * q + lane, c_first = 64 * half;  // and c_first + 128: a column quarter of each half
+    unsigned char* sA = sm + OFF_A + g * A_BYTES;
+    const uint32_t trow = tmem + 256 * g + c_first + ((uint32_t)(32 * q) << 16);
+    float* sRed = reinterpret_cast<float*>(sm + OFF_RED) + (g * TILE + row_l) * 4;
+    const uint32_t my_a = bar_a + 16 * g, my_d = bar_d + 16 * g, my_k = bar_k + 8 * g, my_r = bar_r + 8 * g;
+    // layer 0: two rows a thread (a weight read from shared memory serves both), 32 columns of each half
+    const int r0 = tid & 63, c0_first = 32 * ((tid >> 6) & 3);
+    const float* sX = reinterpret_cast<const float*>(sm + OFF_X) + g * TILE * 6;
+    int tile = blockIdx.x + g * gridDim.x;
+    uint32_t ph = 0;  // layers done, for the parity
+    bool ok = true;
+    for (; ok && tile < ntiles; tile += step) {
+      {
+        pair xs[2][6];
+#pragma unroll
+        for (int f = 0; f < 6; ++f)
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            xs[u][f] = both(round_bf16((sX[(r0 + 64 * u) * 6 + f] - __ldg(shift + f)) * __ldg(scale + f)));
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll 1
+          for (int c0 = 128 * h + c0_first; c0 < 128 * h + c0_first + 32; c0 += 8) {
+            uint32_t w[2][4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const ulonglong2* wr = reinterpret_cast<const ulonglong2*>(sW0 + (c0 / 2 + j) * 16);
+              const ulonglong2 w01 = wr[0], w23 = wr[1], w45 = wr[2];
+              const pair bias = *reinterpret_cast<const pair*>(wr + 3);
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                pair acc = fma2(xs[u][0], w01.x, both(0.0f));
+                acc = fma2(xs[u][1], w01.y, acc);
+                acc = fma2(xs[u][2], w23.x, acc);
+                acc = fma2(xs[u][3], w23.y, acc);
+                acc = fma2(xs[u][4], w45.x, acc);
+                acc = fma2(xs[u][5], w45.y, acc);
+                w[u][j] = pack_bf16(gelu2(add2(acc, bias)));
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+              *reinterpret_cast<uint4*>(sA + act_offset(r0 + 64 * u, c0)) = make_uint4(w[u][0], w[u][1], w[u][2], w[u][3]);
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          mbar_arrive(my_a + 8 * h);
         }
-        out[row * 2] = z0 / ys + y0;
-        out[row * 2 + 1] = z1 - 2.0f * logf(ys);
+      }
+      pair o[2] = {0, 0};  // (mu, log sigma^2) of this thread's two column quarters
+      for (int l = 1; l <= 3; ++l, ++ph) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          // warp-uniform outcome: tcgen05.ld below is a warp-wide instruction
+          ok = ok && __all_sync(0xffffffffu, mbar_wait(my_d + 8 * h, ph & 1, sAbort));
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          if (l == 1 && h == 0) fetch_x(tile + step, g);  // everyone in the group is done with this tile's
+          const int ch = c_first + 128 * h;
+          const float* bias = sB + (l - 1) * 256 + ch;
+          uint32_t r[2][16];
+          tmem_ld16(trow + 128 * h, r[0]);
+#pragma unroll 1
+          for (int c0 = 0; c0 < 64; c0 += 32)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int c = c0 + 16 * u;
+              tmem_wait(r[u]);
+              if (c < 48) tmem_ld16(trow + 128 * h + c + 16, r[u ^ 1]);
+              pair v[8];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(bias + c + 4 * i);
+                v[2 * i] = gelu2(add2(pack(__uint_as_float(r[u][4 * i]), __uint_as_float(r[u][4 * i + 1])), b.x));
+                v[2 * i + 1] = gelu2(add2(pack(__uint_as_float(r[u][4 * i + 2]), __uint_as_float(r[u][4 * i + 3])), b.y));
+              }
+              if (l < 3) {
+                // the second column half's products with the first half of the operand are done
+                if (h == 0 && c == 0) ok = __all_sync(0xffffffffu, mbar_wait(my_k, ph & 1, sAbort));
+                if (ok) {
+#pragma unroll
+                  for (int i = 0; i < 2; ++i)
+                    *reinterpret_cast<uint4*>(sA + act_offset(row_l, ch + c + 8 * i)) =
+                        make_uint4(pack_bf16(v[4 * i]), pack_bf16(v[4 * i + 1]), pack_bf16(v[4 * i + 2]), pack_bf16(v[4 * i + 3]));
+                }
+              } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                  const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(sW4 + 2 * (ch + c + 2 * i));
+                  const uint32_t a = pack_bf16(v[i]);  // rounded; a BF16 number is the upper half of its float
+                  o[h] = fma2(both(__uint_as_float(a << 16)), w.x, o[h]);
+                  o[h] = fma2(both(__uint_as_float(a & 0xffff0000u)), w.y, o[h]);
+                }
+              }
+            }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          if (l < 3) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if (l == 2) asm volatile("cp.async.wait_all;" ::: "memory");  // the next inputs: seen by all at layer 3
+            mbar_arrive(my_a + 8 * h);
+          }
+        }
+        if (!ok) break;
+      }
+      if (!ok) break;
+      // the output: bias, then the four column quarters in order
+      float q0, q1, q2, q3;
+      unpack(o[0], q0, q1);
+      unpack(o[1], q2, q3);
+      if (half) {
+        *reinterpret_cast<float4*>(sRed) = make_float4(q0, q1, q2, q3);
+        mbar_arrive(my_r);
+      } else {
+        ok = __all_sync(0xffffffffu, mbar_wait(my_r, (ph / 3 + 1) & 1, sAbort));
+        const long row = (long)tile * TILE + row_l;
+        if (ok && row < B) {
+          const float4 p = *reinterpret_cast<const float4*>(sRed);
+          out[row * 2] = (sB4[0] + q0 + p.x + q2 + p.z) / ys + y0;
+          out[row * 2 + 1] = (sB4[1] + q1 + p.y + q3 + p.w) - 2.0f * logf(ys);
+        }
       }
     }
   }
-  if (*sAbort && tid == 0) atomicExch(err, 1);
+  __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256u) : "memory");
+  if (*sAbort && tid == 0) atomicExch(err, 1);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
 }  // namespace tc
@@ -740,7 +904,7 @@ __device__ __forceinline__ void store_bf16(int i, float v, __nv_bfloat16* wbf, _
   const int n = e >> 8, k = e & 255;
   fpack[(size_t)l * 65536 + frag_index(n, k)] = h;
   bpack[(size_t)l * 65536 + frag_index(k, n)] = h;
-  wpack[(size_t)l * 65536 + tc::op_offset(n, k) / 2] = h;
+  wpack[(size_t)l * 65536 + tc::weight_offset(n, k) / 2] = h;
 }
 }  // namespace tr
 }  // namespace mlp
