@@ -51,38 +51,89 @@ __global__ void k_clock_advance(MarchClock* c, int by) {
   c->step += by;
 }
 
-// Per-field tables, computed in FP64 and rounded once to the march precision.
+// What a call's passes read, computed in FP64 and rounded once to the march precision: the fields' factors
+// and background phases per axis, the mode momenta and, where the call knows its first evaluation's time
+// (ft), that evaluation's time factors.  A single field comes with the launch (one; stored at fd), which
+// saves an upload from pageable memory.  Chains of FP64 instructions bound it (an exponential, a sine), so
+// every kind of entry has its own blocks.  A right-hand side on 64 x 64 takes 38 us; with the momenta as
+// a second launch (6 us), an upload of the field and the time factors left to the x pass (which took 12
+// instead of 10 us) it took 45.
+constexpr int kTableThreads = 64;
 template <typename R>
-__global__ void k_tables(const FieldDesc* fd, GridDesc g, R* greal, cpx<R>* gcplx) {
-  const int f = blockIdx.y;
-  const int nt = g.n[0] + g.n[1] + g.n[2];
-  const FieldDesc& F = fd[f];
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nt + 4; i += gridDim.x * blockDim.x) {
-    if (i < nt) {
-      int axis = 0, j = i;
-      while (j >= g.n[axis]) { j -= g.n[axis]; ++axis; }
-      const double xc = g.n[axis] > 1 ? g.x0[axis] + j * g.dx[axis] : 0.0;
-      greal[(size_t)f * nt + i] = (R)axis_factor(F, axis, xc);
+struct TableArgs {
+  FieldDesc one;
+  FieldDesc* fd;
+  int single;
+  GridDesc g;
+  R* greal;
+  cpx<R>* gcplx;
+  R* kap;
+  double t;
+  R* ft;
+  cpx<R>* tf;
+  int nb, nfb;  // blocks per kind of entry, blocks of time factors (the phase has one more)
+};
+template <typename R>
+__global__ void __launch_bounds__(kTableThreads) k_tables(const __grid_constant__ TableArgs<R> T) {
+  chain_release();
+  const GridDesc& g = T.g;
+  const int f = blockIdx.y, nt = g.n[0] + g.n[1] + g.n[2];
+  const FieldDesc& F = T.single ? T.one : T.fd[f];
+  const int what = min((int)blockIdx.x / T.nb, 3), i = (blockIdx.x - what * T.nb) * kTableThreads + threadIdx.x;
+  if (what == 3) {
+    const int iy = i;
+    if ((int)blockIdx.x < 3 * T.nb + T.nfb) {
+      if (iy < (F.kind == SWF_FIELD_PULSE_GAUSS ? g.n[1] : 1))
+        T.ft[(size_t)f * g.n[1] + iy] = (R)field_time_factor(F, T.t, g.n[1] > 1 ? g.x0[1] + iy * g.dx[1] : 0.0);
+    } else if (threadIdx.x == 0) {
       double sn, cs;
-      sincos(F.pmom[axis] * xc, &sn, &cs);
-      gcplx[(size_t)f * (nt + 4) + i] = mk<R>((R)cs, (R)sn);
-    } else {
-      const int c = i - nt;
-      gcplx[(size_t)f * (nt + 4) + i] = mk<R>((R)F.w[2 * c], (R)F.w[2 * c + 1]);
+      sincos(F.tsign * F.e0 * T.t, &sn, &cs);
+      T.tf[f] = mk<R>((R)cs, (R)sn);
     }
+    return;
+  }
+  if (i >= nt) {
+    if (what == 1 && i < nt + 4)
+      T.gcplx[(size_t)f * (nt + 4) + i] = mk<R>((R)F.w[2 * (i - nt)], (R)F.w[2 * (i - nt) + 1]);
+    return;
+  }
+  int axis = 0, j = i;
+  while (j >= g.n[axis]) { j -= g.n[axis]; ++axis; }
+  const double xc = g.n[axis] > 1 ? g.x0[axis] + j * g.dx[axis] : 0.0;
+  if (what == 0) {
+    T.greal[(size_t)f * nt + i] = (R)axis_factor(F, axis, xc);
+    if (T.single && i == 0) *T.fd = T.one;
+  } else if (what == 1) {
+    double sn, cs;
+    sincos(F.pmom[axis] * xc, &sn, &cs);
+    T.gcplx[(size_t)f * (nt + 4) + i] = mk<R>((R)cs, (R)sn);
+  } else if (f == 0) {
+    T.kap[i] = g.n[axis] > 1 ? (R)mode_kappa(j, g.n[axis], g.L[axis]) : (R)0;
   }
 }
-
-// The mode momenta of every axis, kap[off_a + j] = (R) mode_kappa(j, n_a, L_a) (0 on trivial axes):
-// the values the H0 step used to compute per element in FP64.
+// The tables of F fields (descriptors in host memory: copied with the launch if there is one, else
+// uploaded to A's) into A's buffers; t: the first evaluation's time, if its factors are wanted.
 template <typename R>
-__global__ void k_kappa_table(GridDesc g, R* kap) {
-  const int nt = g.n[0] + g.n[1] + g.n[2];
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nt; i += gridDim.x * blockDim.x) {
-    int axis = 0, j = i;
-    while (j >= g.n[axis]) { j -= g.n[axis]; ++axis; }
-    kap[i] = g.n[axis] > 1 ? (R)mode_kappa(j, g.n[axis], g.L[axis]) : (R)0;
+static cudaError_t fill_tables(const StageArgs<R>& A, int F, const FieldDesc* fd_host, const double* t, cudaStream_t st) {
+  TableArgs<R> T;
+  T.one = fd_host[0];
+  T.fd = const_cast<FieldDesc*>(A.fd);
+  T.single = F == 1;
+  T.g = A.g;
+  T.greal = const_cast<R*>(A.greal);
+  T.gcplx = const_cast<cpx<R>*>(A.gcplx);
+  T.kap = const_cast<R*>(A.kap);
+  T.t = t ? *t : 0.0;
+  T.ft = t ? A.ft : nullptr;
+  T.tf = A.tf;
+  T.nb = (A.g.n[0] + A.g.n[1] + A.g.n[2] + 4 + kTableThreads - 1) / kTableThreads;
+  T.nfb = T.ft ? (A.g.n[1] + kTableThreads - 1) / kTableThreads : 0;
+  if (!T.single) {
+    const cudaError_t e = cudaMemcpyAsync(T.fd, fd_host, sizeof(FieldDesc) * F, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
   }
+  k_tables<R><<<dim3(3 * T.nb + (T.ft ? T.nfb + 1 : 0), F), kTableThreads, 0, st>>>(T);
+  return cudaSuccess;  // a launch error stays for the caller's cudaGetLastError
 }
 
 // ---------------------------------------------------------------- pass kernels
@@ -550,7 +601,7 @@ static int mid_rule(const StageArgs<R>& A, int axis, long tiles) {
 
 // Launches a kernel of a march's chain so that its blocks may be set up before the kernel in front of it
 // on the stream has ended (it waits for that itself: chain_wait).  It pays where the passes are short
-// and launched one by one: a right-hand side on 64 x 64 takes 46 us, 52 us without; steps replayed from
+// and launched one by one: a right-hand side on 64 x 64 took 46 us with it, 52 us without; steps replayed from
 // a graph gain nothing and lose nothing.
 template <typename... P, typename... Q>
 static void launch_chained(void (*kernel)(P...), dim3 grid, int thr, size_t smem, cudaStream_t st, Q... args) {
@@ -655,8 +706,8 @@ static void launch_mids(swf_ctx* ctx, const StageArgs<R>& A, int F, cudaStream_t
 
 // Launches one right-hand-side evaluation for F fields (ctx may be null: no profiling).
 template <typename R>
-static swf_status launch_eval(swf_ctx* ctx, const StageArgs<R>& A, int F, cudaStream_t st) {
-  swf_status s = launch_x<R>(ctx, A, A, false, true, false, F, st);
+static swf_status launch_eval(swf_ctx* ctx, const StageArgs<R>& A, int F, cudaStream_t st, bool factors = false) {
+  swf_status s = launch_x<R>(ctx, A, A, false, true, factors, F, st);
   if (s != SWF_OK || (A.g.n[1] == 1 && A.g.n[2] == 1)) return s;
   launch_mids<R>(ctx, A, F, st);
   return launch_x<R>(ctx, A, A, true, false, false, F, st);
@@ -781,7 +832,7 @@ static swf_status autotune_eval(swf_ctx* ctx, const StageArgs<R>& B, int F, cuda
 
 template <typename R>
 static swf_status prepare_args(swf_ctx* ctx, const GridDesc& g, int F, const FieldDesc* fd_host,
-                               StageArgs<R>* A, const char* tag, cudaStream_t st) {
+                               StageArgs<R>* A, const char* tag, cudaStream_t st, const double* t_first = nullptr) {
   swf_status s = set_smem_attrs<R>();
   if (s != SWF_OK) return s;
   std::memset(A, 0, sizeof(*A));
@@ -817,20 +868,14 @@ static swf_status prepare_args(swf_ctx* ctx, const GridDesc& g, int F, const Fie
   if ((s = ws_get(ctx, t + ".gcplx", sizeof(cpx<R>) * F * (nt + 4), &pgc)) != SWF_OK) return s;
   void* pkap = nullptr;
   if ((s = ws_get(ctx, t + ".kap", sizeof(R) * nt, &pkap)) != SWF_OK) return s;
-  cudaError_t e = cudaMemcpyAsync(pfd, fd_host, sizeof(FieldDesc) * F, cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return cuda_status(e, "upload field descriptors");
   A->fd = (const FieldDesc*)pfd;
   A->greal = (const R*)pgr;
   A->gcplx = (const cpx<R>*)pgc;
   A->kap = (const R*)pkap;
   A->inv_n = (R)(1.0 / (double)g.N);
-  dim3 tg((nt + 4 + 127) / 128, F);
-  {
-    ProfScope ps(ctx, "k_tables", st);
-    k_tables<R><<<tg, 128, 0, st>>>(A->fd, g, (R*)pgr, (cpx<R>*)pgc);
-  }
-  ProfScope pk(ctx, "k_kappa_table", st);
-  k_kappa_table<R><<<(nt + 127) / 128, 128, 0, st>>>(g, (R*)pkap);
+  ProfScope ps(ctx, "k_tables", st);
+  const cudaError_t e = fill_tables<R>(*A, F, fd_host, t_first, st);
+  if (e != cudaSuccess) return cuda_status(e, "upload field descriptors");
   return SWF_OK;
 }
 
@@ -1507,7 +1552,7 @@ template <typename R>
 static swf_status rhs_impl(swf_ctx* ctx, const GridDesc& g, const FieldDesc& fd, double t,
                            const void* psi, void* out, cudaStream_t st) {
   StageArgs<R> A;
-  swf_status s = prepare_args<R>(ctx, g, 1, &fd, &A, "rhs", st);
+  swf_status s = prepare_args<R>(ctx, g, 1, &fd, &A, "rhs", st, &t);
   if (s != SWF_OK) return s;
   void* pT = nullptr;
   if ((s = ws_get(ctx, "rhs.T", (size_t)4 * g.N * sizeof(cpx<R>), &pT)) != SWF_OK) return s;
@@ -1517,7 +1562,7 @@ static swf_status rhs_impl(swf_ctx* ctx, const GridDesc& g, const FieldDesc& fd,
   A.nterm = 0;
   A.write_y = 0;
   A.t = t;
-  if ((s = launch_eval<R>(ctx, A, 1, st)) != SWF_OK) return s;
+  if ((s = launch_eval<R>(ctx, A, 1, st, A.ft != nullptr)) != SWF_OK) return s;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e, "rhs kernels");
   return SWF_OK;
@@ -1545,10 +1590,6 @@ __global__ void k_twiddles_into(cpx<R>* tw, int n, int r2) {
 }
 
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
-
-// Stores a field descriptor passed by value (kernel parameters are copied at launch, so no host
-// memory is referenced once the launch returns).
-__global__ void k_store_field_desc(FieldDesc fd, FieldDesc* dst) { *dst = fd; }
 
 size_t rhs_scratch_bytes(const GridDesc& g, swf_precision prec) {
   const size_t e = prec == SWF_C64 ? 8 : 16, r = prec == SWF_C64 ? 4 : 8;
@@ -1593,14 +1634,12 @@ static swf_status rhs_scratch_impl(const GridDesc& g, const FieldDesc& fd, doubl
     (le ? A.ltw : A.tw)[a] = tw;
     if (le && (s = line_ready<R>(le)) != SWF_OK) return s;
   }
-  k_store_field_desc<<<1, 1, 0, st>>>(fd, dfd);
-  k_tables<R><<<dim3((nt + 4 + 127) / 128, 1), 128, 0, st>>>(dfd, g, greal, gcplx);
-  k_kappa_table<R><<<(nt + 127) / 128, 128, 0, st>>>(g, kap);
   A.kap = kap;
   A.inv_n = (R)(1.0 / (double)g.N);
   A.fd = dfd;
   A.greal = greal;
   A.gcplx = gcplx;
+  fill_tables<R>(A, 1, &fd, nullptr, st);
   A.y = const_cast<cpx<R>*>((const cpx<R>*)psi);
   A.T = T;
   A.kout = (cpx<R>*)out;
