@@ -450,6 +450,24 @@ static swf_status premarch_schwinger(swf_ctx* ctx, const swf_instance* inst,
   return SWF_OK;
 }
 
+// The U and V fields of a group with the full pair number go in one fixed-step march (2 F fields, the
+// same arithmetic field by field) where one of them alone leaves the GPU waiting for launches and
+// latencies: below kPairSites field points.  Measured, one after the other / together: one field of
+// 64 x 64 3.44 / 1.91 ms (complex64, 30 steps), 192 x 192 5.2 / 2.9, 128 x 128 in FP64 12.1 / 9.4, four of
+// those 28.7 / 23.7, 256 x 256 in FP64 31.4 / 30.2; above the line 0.96 (two of 64^3, out of L2) to 1.04
+// times as fast.  Together they need twice the stage buffers, so under a workspace limit they do only if
+// an earlier call has left them.
+constexpr double kPairSites = 256.0 * 1024;
+static bool ws_has(swf_ctx* ctx, const std::string& name, size_t bytes) {
+  const auto it = ctx->ws.bufs.find(name);
+  return it != ctx->ws.bufs.end() && it->second.second >= bytes;
+}
+static bool march_as_pair(swf_ctx* ctx, const GridDesc& g, int F, const FieldDesc* fdUV, swf_precision prec) {
+  const size_t bytes = (size_t)2 * F * 4 * g.N * (prec == SWF_C64 ? 8 : 16);
+  if ((double)F * g.N >= kPairSites || (ctx->ws.limit && !ws_has(ctx, "solve.psiU", bytes))) return false;
+  return !(ctx->use_fused && (fused_applicable(g, F, fdUV, prec) || fused_applicable(g, F, fdUV + F, prec)));
+}
+
 static swf_status solve_schwinger(swf_ctx* ctx, int n_inst, const swf_instance* inst, swf_precision prec,
                                   swf_result* results_dev, double* spectrum_dev, cudaStream_t st) {
   std::map<GroupKey, std::vector<int>> groups;
@@ -506,15 +524,26 @@ static swf_status solve_schwinger(swf_ctx* ctx, int n_inst, const swf_instance* 
     }
     const size_t state = (size_t)F * 4 * g.N;
     void *psiU, *specU, *uq, *normU, *pid;
-    if ((s = ws_get(ctx, "solve.psiU", state * elem, &psiU)) != SWF_OK) return s;
+    bool paired = false;
+    if (full && !kv.first.adaptive && pre == premarched.end()) {
+      std::vector<FieldDesc> fdUV(fdU);
+      fdUV.insert(fdUV.end(), fdV.begin(), fdV.end());
+      if (march_as_pair(ctx, g, F, fdUV.data(), prec)) {
+        if ((s = ws_get(ctx, "solve.psiU", 2 * state * elem, &psiU)) == SWF_OK)
+          s = march_fields(ctx, g, i0.grid.t_in, i0.grid.t_out, i0.grid.n_steps, 2 * F, fdUV.data(), prec, psiU, st, 0);
+        if (s != SWF_OK && s != SWF_ENOMEM) return s;  // without the memory: one after the other
+        paired = s == SWF_OK;
+      }
+    }
+    if (!paired && (s = ws_get(ctx, "solve.psiU", state * elem, &psiU)) != SWF_OK) return s;
     if ((s = ws_get(ctx, "solve.specU", state * 16, &specU)) != SWF_OK) return s;
     if ((s = ws_get(ctx, "solve.uq", (size_t)F * 64, &uq)) != SWF_OK) return s;
     if ((s = ws_get(ctx, "solve.normU", (size_t)F * 8, &normU)) != SWF_OK) return s;
     if ((s = ws_get(ctx, "solve.inst", sizeof(InstDev) * F, &pid)) != SWF_OK) return s;
     if (pre != premarched.end()) {
       psiU = pre->second;  // U fields, then (full) V fields
-    } else if ((s = march_fields(ctx, g, i0.grid.t_in, i0.grid.t_out, i0.grid.n_steps, F, fdU.data(), prec, psiU, st,
-                                 kv.first.adaptive)) != SWF_OK) {
+    } else if (!paired && (s = march_fields(ctx, g, i0.grid.t_in, i0.grid.t_out, i0.grid.n_steps, F, fdU.data(), prec,
+                                            psiU, st, kv.first.adaptive)) != SWF_OK) {
       return s;
     }
     if ((s = transform_at(ctx, g, F, prec, psiU, kq.data(), (double2*)uq, st)) != SWF_OK) return s;
@@ -540,12 +569,15 @@ static swf_status solve_schwinger(swf_ctx* ctx, int n_inst, const swf_instance* 
       if ((s = ws_get(ctx, "solve.normV", (size_t)F * 8, &normV)) != SWF_OK) return s;
       if (pre != premarched.end()) {
         psiV = (unsigned char*)pre->second + state * elem;
-      } else {
-        if ((s = ws_get(ctx, "solve.psiV", state * elem, &psiV)) != SWF_OK) return s;
-        if ((s = march_fields(ctx, g, i0.grid.t_in, i0.grid.t_out, i0.grid.n_steps, F, fdV.data(), prec, psiV, st,
-                              kv.first.adaptive)) != SWF_OK)
-          return s;
+      } else if (paired || ws_has(ctx, "solve.psiU", 2 * state * elem)) {
+        psiV = (unsigned char*)psiU + state * elem;
+      } else if ((s = ws_get(ctx, "solve.psiV", state * elem, &psiV)) != SWF_OK) {
+        return s;
       }
+      if (pre == premarched.end() && !paired &&
+          (s = march_fields(ctx, g, i0.grid.t_in, i0.grid.t_out, i0.grid.n_steps, F, fdV.data(), prec, psiV, st,
+                            kv.first.adaptive)) != SWF_OK)
+        return s;
       if ((s = transform_fields(ctx, g, F, prec, psiV, (double2*)specV, st)) != SWF_OK) return s;
       if ((s = transform_at(ctx, g, F, prec, psiV, kp.data(), (double2*)vp, st)) != SWF_OK) return s;
       if ((s = field_norms(ctx, g, F, prec, psiV, (double*)normV, st)) != SWF_OK) return s;
