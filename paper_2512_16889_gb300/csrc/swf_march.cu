@@ -1942,8 +1942,8 @@ __global__ void k_f2_omega_table(const F2Table* tabs, GridDesc g, int n_tab, R* 
 // and its time phase) times adds to the block's own FP64 accumulators dpart[f][block][4] (no other block
 // touches them: the sum is deterministic).  A thread that holds sites of Y's component c works on the
 // component of Z that c feeds.  Rows per block are fixed, not tuned: they decide the order of the sum.
-// Bound by FP64 issue; the threads' four or fewer values fill every quarter of every SM.  Two instances
-// of 128^2 in FP64: 80 us, where whole lines of one thread group took 106 us.
+// Bound by FP64 issue; the threads' four or fewer values fill every quarter of every SM.  Three pairs
+// on 160^2 in FP64: 80 us, where whole lines of one thread group took 106 us.
 template <typename R, int R0>
 __global__ void __launch_bounds__(kPassThreads, 1)
 k_f2_x(const __grid_constant__ StageArgs<R> A, const cpx<R>* __restrict__ ys, cpx<R>* __restrict__ Yspec,
@@ -2048,7 +2048,7 @@ __device__ __forceinline__ void form_add(cpx<R>& s, const cpx<R>* x, R a, const 
 // with U quantities at mode j and V quantities at mode j - shift.  Block (b, inst) adds trow[2]
 // (w_i e^{-i k0 t}) times its part to its own accumulator sspart[inst][b].  In FP64 the instruction count
 // is what bounds it: alpha.eps as additions of scaled components, both projections of a vector from one
-// H0 x, both signs of sigma' summed before the contraction.  Two instances of 128^2 in FP64: 70 us, where
+// H0 x, both signs of sigma' summed before the contraction.  Three pairs on 160^2 in FP64: 70 us, where
 // a projection and a contraction for every sign took 113 us.
 // f2i per instance: shift[3], table index.
 template <typename R>
