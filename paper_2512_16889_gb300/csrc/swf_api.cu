@@ -379,9 +379,10 @@ struct GroupKey {
 };
 
 // In the automatic mode a set of groups is marched together when all of them hold fewer fields x
-// grid points than this (per evaluation): above it every group fills the GPU by itself and one
-// launch sequence per group was as fast (Breit-Wheeler on the uneven grids, 300 steps: grouped
-// +5 % at 8 instances, 2 per grid size; level at 16; -3 % at 32).
+// grid points than this (per evaluation): above it every group fills the GPU by itself, and side by side
+// they need all their workspaces at once (Breit-Wheeler on the uneven grids, 300 steps, side by side
+// against one after another: 1.40e9 against 1.27e9 site-updates/s at 8 instances, 2 per grid size;
+// 1.41e9 against 1.40e9 at 16; 1.49e9 against 1.47e9 at 32).
 constexpr double kMultiAutoSites = 4.0 * 1024 * 1024;
 
 // Time grid and non-trivial axes: groups that agree on these can be marched together.

@@ -7,8 +7,7 @@
 // inverse runs the same steps backwards.  Whatever happens on the sites between an inverse and the
 // next forward transform (k_i, the stage combine, the local term) or on the modes between a forward
 // and an inverse (H0) happens in the registers of the thread that owns them.  An evaluation's line
-// therefore passes through shared memory twice (the Stockham passes of swf_march.cu: six times, with
-// a barrier each), and global memory is read into and written from the same registers: n/R2 = R1
+// therefore passes through shared memory twice (Stockham passes: six times, with a barrier each), and global memory is read into and written from the same registers: n/R2 = R1
 // independent loads per thread and array, R2 (or R1) neighbouring points per load instruction.
 //
 // What bounds them, and what they measured against the Stockham passes they replaced (complex64, per
@@ -29,7 +28,7 @@ enum : int {
   XL_LAST = 1,     // close evaluation P: inverse x-FFT, k = (that) + Z
   XL_FIRST = 2,    // open evaluation A: stage combine, local term, forward x-FFT
   XL_REGK = 4,     // the newest term of A's stage combine is P's output (still in registers)
-  XL_FACTORS = 8,  // A's time factors were computed by the y or z pass before this launch
+  XL_FACTORS = 8,  // A's time factors were computed by a launch before this one (y or z pass, k_tables)
 };
 // What a y or z pass does (the flags of k_line).
 enum : int { LN_FWD = 1, LN_H0 = 2, LN_INV = 4 };
