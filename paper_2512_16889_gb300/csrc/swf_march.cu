@@ -1899,8 +1899,8 @@ __global__ void k_f2_dtables(const double* wave_k, GridDesc g, int n_waves, cpx<
   }
 }
 
-// Parameters of one mode-sum table: the photon's mode shift per axis, the fixed momenta of U and V
-// along trivial axes, and k0.
+// Parameters of one mode-sum table: the photon's mode shift per axis (0 <= shift < n), the fixed momenta
+// of U and V along trivial axes, and k0.
 struct F2Table {
   int shift[3];
   int pad;
@@ -1921,7 +1921,7 @@ __global__ void k_f2_omega_table(const F2Table* tabs, GridDesc g, int n_tab, R* 
     const int id[3] = {j % g.n[0], (j / g.n[0]) % g.n[1], j / (g.n[0] * g.n[1])};
     double ku[3], kv[3];
     for (int a = 0; a < 3; ++a) {
-      const int jv = ((id[a] - T.shift[a]) % g.n[a] + g.n[a]) % g.n[a];
+      const int jv = id[a] - T.shift[a] + (id[a] < T.shift[a] ? g.n[a] : 0);
       ku[a] = kappa_of(id[a], g.n[a], g.L[a], T.Ku[a]);
       kv[a] = kappa_of(jv, g.n[a], g.L[a], T.Kv[a]);
     }
@@ -2083,9 +2083,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_f2_ss(const cpx
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const int n = g.n[a];
-      jv[a] = id[a] - shift[a];
+      jv[a] = id[a] - shift[a];  // 0 <= shift < n
       if (jv[a] < 0) jv[a] += n;
-      if (jv[a] >= n) jv[a] -= n;
       const int fu = id[a] < (n + 1) / 2 ? id[a] : id[a] - n;
       const int fv = jv[a] < (n + 1) / 2 ? jv[a] : jv[a] - n;
       ku[a] = n > 1 ? du[a] * (R)fu : (R)FU.K[a];
@@ -2238,7 +2237,10 @@ static swf_status f2_prepare(swf_ctx* ctx, const GridDesc& g, int n_inst, const 
     std::memset(&T, 0, sizeof T);
     const double* k = photon_host + 6 * i;
     for (int a = 0; a < 3; ++a) {
-      T.shift[a] = g.n[a] > 1 ? (int)std::lround(k[a] * g.L[a] / 6.283185307179586476925286766559) : 0;
+      // the modes are periodic and a photon's may lie any number of boxes out: 0 <= shift < n, so that the
+      // mode sum reaches its partner with one wrap
+      const long m = g.n[a] > 1 ? std::lround(k[a] * g.L[a] / 6.283185307179586476925286766559) : 0;
+      T.shift[a] = (int)((m % g.n[a] + g.n[a]) % g.n[a]);
       T.Ku[a] = fd_host[2 * i].K[a];
       T.Kv[a] = fd_host[2 * i + 1].K[a];
     }
