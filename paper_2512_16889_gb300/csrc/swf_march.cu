@@ -1012,6 +1012,10 @@ __global__ void __launch_bounds__(kErrThreads) k_step_error(const cpx<R>* __rest
   }
 }
 
+// The larger of two error norms; NaN if either is (fmax would drop it, and a field gone bad would pass as
+// one without error).
+__device__ __forceinline__ double worse_error(double a, double b) { return a >= b ? a : (a == a ? b : a); }
+
 // err = max over fields of the RMS scaled error (a warp per field in turn, lanes in a fixed order);
 // accept when err <= 1 (and finite); next step h min(10, max(0.2, 0.9 err^(-1/5))), clamped so as not
 // to pass t_in.  One block; one thread of it took 19 us to add 200 parts.
@@ -1029,12 +1033,12 @@ __global__ void __launch_bounds__(256) k_step_control(StepControl* ctl, const do
     for (int b = lane; b < nb; b += 32) sum += part[(size_t)f * nb + b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    err = fmax(err, sqrt(sum / count));
+    err = worse_error(err, sqrt(sum / count));
   }
   if (lane == 0) s_err[warp] = err;
   __syncthreads();
   if (threadIdx.x != 0) return;
-  for (int w = 0; w < 8; ++w) err = fmax(err, s_err[w]);
+  for (int w = 0; w < 8; ++w) err = worse_error(err, s_err[w]);
   if (!(err == err) || isinf(err)) {  // non-finite: stop
     ctl->ok = 0;
     ctl->failed = 1;
