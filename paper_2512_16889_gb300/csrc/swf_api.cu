@@ -51,6 +51,15 @@ swf_status ws_get(swf_ctx* ctx, const std::string& name, size_t bytes, void** pt
   return SWF_OK;
 }
 
+swf_status ws_chunk(swf_ctx* ctx, const std::string& name, size_t per, int unit, int n, int* chunk, void** ptr) {
+  const size_t most = std::min<size_t>(65535, ((size_t)64 << 20) / per);
+  for (int units = (int)std::min<size_t>(n / unit, std::max<size_t>(1, most / unit));; units = (units + 1) / 2) {
+    *chunk = units * unit;
+    const swf_status s = ws_get(ctx, name, per * *chunk, ptr);
+    if (s != SWF_ENOMEM || units == 1) return s;
+  }
+}
+
 // Twiddles of length n in double or single precision, rounded once from long double: natural order
 // exp(-2 pi i m/n), m < n (r2 = 0), or the table of the register line kernels, entry k1 r2 + i =
 // exp(-2 pi i i k1/n).

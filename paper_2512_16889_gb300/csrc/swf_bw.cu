@@ -225,18 +225,22 @@ swf_status bw_finalize(swf_ctx* ctx, const GridDesc& g, int n_inst, const void* 
   if (s != SWF_OK) return s;
   cudaError_t e = cudaMemcpyAsync(pb, bw_host, sizeof(BwInst) * n_inst, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_status(e, "upload Breit-Wheeler table");
-  // four modes per thread, at most 1024 blocks per amplitude
+  // four modes per thread, at most 1024 blocks per amplitude; the parts of a chunk of amplitudes take the
+  // place of the direct transforms' (one amplitude's are never the larger ones)
   const int nb = std::max(1, std::min(1024, (g.N + 1023) / 1024));
+  int chunk;
   void* pp;
-  if ((s = ws_get(ctx, "bw.mode_part", sizeof(cpx<double>) * (size_t)nb * n_inst, &pp)) != SWF_OK) return s;
-  {
-    ProfScope ps(ctx, "k_bw_modes", st);
-    k_bw_modes<<<dim3(nb, n_inst), 256, 0, st>>>((const BwInst*)pb, g, (const cpx<double>*)spec, (cpx<double>*)pp);
-  }
-  {
+  if ((s = ws_chunk(ctx, "proj.part", sizeof(cpx<double>) * (size_t)nb, 1, n_inst, &chunk, &pp)) != SWF_OK) return s;
+  for (int i0 = 0; i0 < n_inst; i0 += chunk) {
+    const int n = std::min(chunk, n_inst - i0);
+    const BwInst* bi = (const BwInst*)pb + i0;
+    {
+      ProfScope ps(ctx, "k_bw_modes", st);
+      k_bw_modes<<<dim3(nb, n), 256, 0, st>>>(bi, g, (const cpx<double>*)spec, (cpx<double>*)pp);
+    }
     ProfScope ps(ctx, "k_bw_finalize", st);
-    k_bw_finalize<<<n_inst, 32, 0, st>>>((const BwInst*)pb, g, t_in, (const cpx<double>*)pp, nb,
-                                         (const cpx<double>*)tat, (const cpx<double>*)macc, norms, results);
+    k_bw_finalize<<<n, 32, 0, st>>>(bi, g, t_in, (const cpx<double>*)pp, nb, (const cpx<double>*)tat + 8 * (size_t)i0,
+                                    (const cpx<double>*)macc + 3 * (size_t)i0, norms, results);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e, "Breit-Wheeler finalize");

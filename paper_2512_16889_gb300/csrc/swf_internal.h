@@ -168,6 +168,10 @@ swf_status cuda_status(cudaError_t e, const char* what);
 
 // Returns a device buffer of at least `bytes` under `name` (grows, never shrinks).
 swf_status ws_get(swf_ctx* ctx, const std::string& name, size_t bytes, void** ptr);
+// A device buffer under `name` for a sum over up to n entries of `per` bytes each, taken in chunks: *chunk
+// receives the entries it holds, a multiple of `unit` (which divides n).  At most 64 MB and one grid.y
+// (65535 entries); less, down to one unit, where the workspace limit or the device's memory has no more.
+swf_status ws_chunk(swf_ctx* ctx, const std::string& name, size_t per, int unit, int n, int* chunk, void** ptr);
 // Device table exp(-2 pi i m/n), m < n, in float2 (is_double = 0) or double2; with r2 > 0 in the order
 // of the register line kernels.
 swf_status twiddles(swf_ctx* ctx, int n, int is_double, const void** ptr, int r2 = 0);

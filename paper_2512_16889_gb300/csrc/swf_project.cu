@@ -323,26 +323,28 @@ swf_status c_spectrum(swf_ctx* ctx, const GridDesc& g, int n_f, const FieldDesc*
 swf_status transform_at(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precision prec, const void* psi,
                         const double* kappa_host, double2* out, cudaStream_t st, int n_fields) {
   if (n_fields < 1) n_fields = n_f;
-  void* pk = nullptr;
-  swf_status s = ws_get(ctx, "proj.kappa", sizeof(double) * 3 * n_f, &pk);
-  if (s != SWF_OK) return s;
-  cudaError_t e = cudaMemcpyAsync(pk, kappa_host, sizeof(double) * 3 * n_f, cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return cuda_status(e, "upload wave vectors");
   const size_t sm = (size_t)(g.n[0] + g.n[1] + g.n[2]) * sizeof(cpx<double>);
   const int nb = reduction_blocks(g.N, n_fields);
+  // the parts of a chunk of entries, then its wave vectors: a chunk is a multiple of the fields
+  const size_t parts = sizeof(cpx<double>) * 4 * (size_t)nb;
+  int chunk;
   void* part = nullptr;
-  if ((s = ws_get(ctx, "proj.part", sizeof(cpx<double>) * 4 * (size_t)nb * n_f, &part)) != SWF_OK) return s;
-  {
-    ProfScope ps(ctx, "k_transform_at", st);
-    if (prec == SWF_C64)
-      k_transform_at<float><<<dim3(nb, n_f), kT, sm, st>>>(psi, g, n_fields, (const double*)pk, (cpx<double>*)part);
-    else
-      k_transform_at<double><<<dim3(nb, n_f), kT, sm, st>>>(psi, g, n_fields, (const double*)pk, (cpx<double>*)part);
-  }
-  {
+  swf_status s = ws_chunk(ctx, "proj.part", parts + 3 * sizeof(double), n_fields, n_f, &chunk, &part);
+  if (s != SWF_OK) return s;
+  double* pk = reinterpret_cast<double*>((unsigned char*)part + parts * chunk);
+  cudaError_t e;
+  for (int e0 = 0; e0 < n_f; e0 += chunk) {
+    const int n = std::min(chunk, n_f - e0);
+    e = cudaMemcpyAsync(pk, kappa_host + 3 * (size_t)e0, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return cuda_status(e, "upload wave vectors");
+    {
+      ProfScope ps(ctx, "k_transform_at", st);
+      if (prec == SWF_C64) k_transform_at<float><<<dim3(nb, n), kT, sm, st>>>(psi, g, n_fields, pk, (cpx<double>*)part);
+      else k_transform_at<double><<<dim3(nb, n), kT, sm, st>>>(psi, g, n_fields, pk, (cpx<double>*)part);
+    }
     ProfScope ps(ctx, "k_sum_parts", st);
-    k_sum_parts<cpx<double>><<<n_f, 32, 0, st>>>((const cpx<double>*)part, nb, 4, g.dx[0] * g.dx[1] * g.dx[2],
-                                                 (cpx<double>*)out);
+    k_sum_parts<cpx<double>><<<n, 32, 0, st>>>((const cpx<double>*)part, nb, 4, g.dx[0] * g.dx[1] * g.dx[2],
+                                               (cpx<double>*)out + 4 * (size_t)e0);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e, "direct transform kernel");
