@@ -51,6 +51,19 @@ swf_status ws_get(swf_ctx* ctx, const std::string& name, size_t bytes, void** pt
   return SWF_OK;
 }
 
+bool ws_has(swf_ctx* ctx, const std::string& name, size_t bytes) {
+  const auto it = ctx->ws.bufs.find(name);
+  return it != ctx->ws.bufs.end() && it->second.second >= bytes;
+}
+
+void ws_drop(swf_ctx* ctx, const std::string& name) {
+  const auto it = ctx->ws.bufs.find(name);
+  if (it == ctx->ws.bufs.end()) return;
+  cudaFree(it->second.first);
+  ctx->ws.total -= it->second.second;
+  ctx->ws.bufs.erase(it);
+}
+
 swf_status ws_chunk(swf_ctx* ctx, const std::string& name, size_t per, int unit, int n, int* chunk, void** ptr) {
   const size_t most = std::min<size_t>(65535, ((size_t)64 << 20) / per);
   for (int units = (int)std::min<size_t>(n / unit, std::max<size_t>(1, most / unit));; units = (units + 1) / 2) {
@@ -466,15 +479,12 @@ static swf_status premarch_schwinger(swf_ctx* ctx, const swf_instance* inst,
 // 64 x 64 3.44 / 1.91 ms (complex64, 30 steps), 192 x 192 5.2 / 2.9, 128 x 128 in FP64 12.1 / 9.4, four of
 // those 28.7 / 23.7, 256 x 256 in FP64 31.4 / 30.2; above the line 0.96 (two of 64^3, out of L2) to 1.04
 // times as fast.  Together they need twice the stage buffers, so under a workspace limit they do only if
-// an earlier call has left them.
+// earlier calls have left all of them.
 constexpr double kPairSites = 256.0 * 1024;
-static bool ws_has(swf_ctx* ctx, const std::string& name, size_t bytes) {
-  const auto it = ctx->ws.bufs.find(name);
-  return it != ctx->ws.bufs.end() && it->second.second >= bytes;
-}
 static bool march_as_pair(swf_ctx* ctx, const GridDesc& g, int F, const FieldDesc* fdUV, swf_precision prec) {
   const size_t bytes = (size_t)2 * F * 4 * g.N * (prec == SWF_C64 ? 8 : 16);
-  if ((double)F * g.N >= kPairSites || (ctx->ws.limit && !ws_has(ctx, "solve.psiU", bytes))) return false;
+  if ((double)F * g.N >= kPairSites) return false;
+  if (ctx->ws.limit && !(ws_has(ctx, "solve.psiU", bytes) && march_held(ctx, g, 2 * F, prec))) return false;
   return !(ctx->use_fused && (fused_applicable(g, F, fdUV, prec) || fused_applicable(g, F, fdUV + F, prec)));
 }
 
@@ -541,8 +551,12 @@ static swf_status solve_schwinger(swf_ctx* ctx, int n_inst, const swf_instance* 
       if (march_as_pair(ctx, g, F, fdUV.data(), prec)) {
         if ((s = ws_get(ctx, "solve.psiU", 2 * state * elem, &psiU)) == SWF_OK)
           s = march_fields(ctx, g, i0.grid.t_in, i0.grid.t_out, i0.grid.n_steps, 2 * F, fdUV.data(), prec, psiU, st, 0);
-        if (s != SWF_OK && s != SWF_ENOMEM) return s;  // without the memory: one after the other
+        if (s != SWF_OK && s != SWF_ENOMEM) return s;
         paired = s == SWF_OK;
+        if (!paired) {  // without the memory: one after the other, from buffers of that size
+          march_release(ctx, g);
+          ws_drop(ctx, "solve.psiU");
+        }
       }
     }
     if (!paired && (s = ws_get(ctx, "solve.psiU", state * elem, &psiU)) != SWF_OK) return s;

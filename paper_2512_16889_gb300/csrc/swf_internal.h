@@ -168,6 +168,9 @@ swf_status cuda_status(cudaError_t e, const char* what);
 
 // Returns a device buffer of at least `bytes` under `name` (grows, never shrinks).
 swf_status ws_get(swf_ctx* ctx, const std::string& name, size_t bytes, void** ptr);
+// Whether a buffer of at least `bytes` is held under `name`; gives one back (waits for the device).
+bool ws_has(swf_ctx* ctx, const std::string& name, size_t bytes);
+void ws_drop(swf_ctx* ctx, const std::string& name);
 // A device buffer under `name` for a sum over up to n entries of `per` bytes each, taken in chunks: *chunk
 // receives the entries it holds, a multiple of `unit` (which divides n).  At most 64 MB and one grid.y
 // (65535 entries); less, down to one unit, where the workspace limit or the device's memory has no more.
@@ -182,6 +185,10 @@ swf_status twiddles(swf_ctx* ctx, int n, int is_double, const void** ptr, int r2
 swf_status march_fields(swf_ctx* ctx, const GridDesc& g, double t_in, double t_out, int n_steps,
                         int n_f, const FieldDesc* fd_host, swf_precision prec, void* psi_out,
                         cudaStream_t st, int adaptive = 0);
+// Whether the context holds every buffer of such a fixed-step march on the pass kernels; gives those of
+// any such march on a grid back.
+bool march_held(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precision prec);
+void march_release(swf_ctx* ctx, const GridDesc& g);
 // Step-size-controlled march (first step h0, at most max_attempts attempts; tolerances from ctx)
 swf_status march_adaptive(swf_ctx* ctx, const GridDesc& g, double t_in, double t_out, double h0, int max_attempts,
                           int n_f, const FieldDesc* fd_host, swf_precision prec, void* psi_out, cudaStream_t st);

@@ -1408,30 +1408,45 @@ static int dedupe_fields(const GridDesc& g, int n_f, const FieldDesc* fd, std::v
   return (int)uniq.size();
 }
 
-// Sizes the pass-kernel march's workspace for F fields (the buffers prepare_args and march_impl
-// take) without touching the device: growing a workspace buffer frees the old one, which waits
-// for the whole device, so march_split does it before the fused kernel starts.
+// The buffers that prepare_args and march_impl take for F fields.
+template <typename R>
+static std::vector<std::pair<std::string, size_t>> march_buffers(const GridDesc& g, int F) {
+  const size_t nt = g.n[0] + g.n[1] + g.n[2];
+  const size_t state = (size_t)F * 4 * g.N * sizeof(cpx<R>);
+  std::vector<std::pair<std::string, size_t>> b = {
+      {"march.fd", sizeof(FieldDesc) * F}, {"march.greal", sizeof(R) * F * nt}, {"march.gcplx", sizeof(cpx<R>) * F * (nt + 4)},
+      {"march.y", state}, {"march.T", state}};
+  if (sizeof(R) == 4) b.push_back({"march.ylo", state});
+  for (int i = 0; i < 7; ++i) b.push_back({"march.k" + std::to_string(i), state});
+  b.push_back({"march.clock", sizeof(MarchClock)});
+  b.push_back({"march.kap", sizeof(R) * nt});
+  if (g.n[1] > 1 || g.n[2] > 1) {
+    b.push_back({"march.ft", sizeof(R) * F * g.n[1]});
+    b.push_back({"march.tf", sizeof(cpx<R>) * F});
+  }
+  return b;
+}
+
+bool march_held(swf_ctx* ctx, const GridDesc& g, int n_f, swf_precision prec) {
+  for (const auto& b : prec == SWF_C64 ? march_buffers<float>(g, n_f) : march_buffers<double>(g, n_f))
+    if (!ws_has(ctx, b.first, b.second)) return false;
+  return true;
+}
+
+void march_release(swf_ctx* ctx, const GridDesc& g) {
+  for (const auto& b : march_buffers<float>(g, 1)) ws_drop(ctx, b.first);  // single precision has them all
+  ws_drop(ctx, "march.unique");
+}
+
+// Sizes the pass-kernel march's workspace for F fields without touching the device: growing a
+// workspace buffer frees the old one, which waits for the whole device, so march_split does it before
+// the fused kernel starts.
 template <typename R>
 static swf_status reserve_march(swf_ctx* ctx, const GridDesc& g, int F) {
-  const int nt = g.n[0] + g.n[1] + g.n[2];
-  const size_t state = (size_t)F * 4 * g.N * sizeof(cpx<R>);
   void* p = nullptr;
   swf_status s;
-  if ((s = ws_get(ctx, "march.fd", sizeof(FieldDesc) * F, &p)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "march.greal", sizeof(R) * F * nt, &p)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "march.gcplx", sizeof(cpx<R>) * F * (nt + 4), &p)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "march.y", state, &p)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "march.T", state, &p)) != SWF_OK) return s;
-  if (sizeof(R) == 4 && (s = ws_get(ctx, "march.ylo", state, &p)) != SWF_OK) return s;
-  for (int i = 0; i < 7; ++i) {
-    char nm[32];
-    std::snprintf(nm, sizeof nm, "march.k%d", i);
-    if ((s = ws_get(ctx, nm, state, &p)) != SWF_OK) return s;
-  }
-  if ((s = ws_get(ctx, "march.clock", sizeof(MarchClock), &p)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "march.kap", sizeof(R) * nt, &p)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "march.ft", sizeof(R) * F * g.n[1], &p)) != SWF_OK) return s;
-  if ((s = ws_get(ctx, "march.tf", sizeof(cpx<R>) * F, &p)) != SWF_OK) return s;
+  for (const auto& b : march_buffers<R>(g, F))
+    if ((s = ws_get(ctx, b.first, b.second, &p)) != SWF_OK) return s;
   for (int a = 0; a < 3; ++a) {
     const void* tw = nullptr;
     if ((s = twiddles(ctx, g.n[a], Prec<R>::is_double, &tw)) != SWF_OK) return s;
