@@ -401,31 +401,47 @@ k_line(const __grid_constant__ StageArgs<R> A, int axis, int lgtx, int flags) {
   }
 }
 
+// s + e += b + be, e the rounding errors of s (Knuth's two-sum); double: s alone.
+__device__ __forceinline__ void add_exact(float& s, float& e, float b, float be) {
+  const float t = __fadd_rn(s, b), bp = __fsub_rn(t, s);
+  e = __fadd_rn(e, __fadd_rn(be, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(b, bp))));
+  s = t;
+}
+__device__ __forceinline__ void add_exact(double& s, double&, double b, double) { s += b; }
+
 // The direct-transform sums of a block of wave f: red[component][row][thread] holds the threads' sums (in
-// the march precision; the caller has synchronised), a warp per component adds them in a fixed order, and
-// trow[w] (the stage's weight and time phase) times adds them to the block's own FP64 accumulators
-// dpart[f][block][4].
+// the march precision; the caller has synchronised), eight lanes of the first warp per component (one in
+// a block of less than a warp) add them in a fixed order, and trow[w] (the stage's weight and time phase)
+// times adds them to the block's own FP64 accumulators dpart[f][block][4].  Single-precision sums carry
+// their rounding errors, which makes the block's as good as one in FP64: additions in FP64 itself hold an
+// SM quarter for 64 cycles each (16 pairs on 384^2, 21 launches of k_f2_line: 4.0 ms with them and a warp
+// per component, 3.25 ms so; 3.4 ms with rounded sums by a warp per component).
 template <typename R>
 __device__ __forceinline__ void direct_sums(const StageArgs<R>& A, const cpx<R>* red, int per, int f,
                                             const cpx<double>* __restrict__ ptab, int tab_stride, int stage,
                                             cpx<double>* dpart) {
-  const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-  const int step = min(32, (int)blockDim.x - (int)(threadIdx.x & ~31));  // threads of this warp
-  const unsigned full = step == 32 ? 0xffffffffu : (1u << step) - 1u;
-  for (int k = threadIdx.x >> 5; k < 4; k += nw) {
-    cpx<R> sacc = mk<R>(0, 0);
-    for (int e = lane; e < per; e += step) sacc = sacc + red[k * per + e];
+  const int g = blockDim.x >= 32 ? 8 : 1;
+  if (threadIdx.x >= 4 * g) return;
+  const int k = threadIdx.x / g, l = threadIdx.x - k * g;
+  cpx<R> s = mk<R>(0, 0), err = mk<R>(0, 0);
+  for (int e = l; e < per; e += g) {
+    const cpx<R> v = red[k * per + e];
+    add_exact(s.x, err.x, v.x, 0);
+    add_exact(s.y, err.y, v.y, 0);
+  }
+  if (g > 1) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const R x = __shfl_down_sync(full, sacc.x, off), y = __shfl_down_sync(full, sacc.y, off);
-      if (lane + off < step) sacc = mk<R>(sacc.x + x, sacc.y + y);
+    for (int off = 4; off > 0; off >>= 1) {
+      const cpx<R> v = shfl_xor(s, off), ve = shfl_xor(err, off);
+      add_exact(s.x, err.x, v.x, ve.x);
+      add_exact(s.y, err.y, v.y, ve.y);
     }
-    if (lane == 0) {
-      const long tab_row = (long)(A.clk->step + A.ls) * 7 + stage;
-      const cpx<double> wt = ptab[3 * (tab_row + (long)(f >> 1) * tab_stride) + (f & 1)];
-      cpx<double>& d = dpart[((size_t)f * gridDim.x + blockIdx.x) * 4 + k];
-      d = d + wt * cvt<double>(sacc);
-    }
+  }
+  if (l == 0) {
+    const long tab_row = (long)(A.clk->step + A.ls) * 7 + stage;
+    const cpx<double> wt = ptab[3 * (tab_row + (long)(f >> 1) * tab_stride) + (f & 1)];
+    cpx<double>& d = dpart[((size_t)f * gridDim.x + blockIdx.x) * 4 + k];
+    d = d + wt * mk<double>((double)s.x + (double)err.x, (double)s.y + (double)err.y);
   }
 }
 
