@@ -463,10 +463,6 @@ static swf_status premarch_schwinger(swf_ctx* ctx, const swf_instance* inst,
         premarched[k] = out;
       }
       s = march_fields_multi(ctx, mg, kv.first.t_in, kv.first.t_out, kv.first.n_steps, prec, st);
-      if (s == SWF_EUNSUPPORTED) {  // not a form the grouped launch takes: these groups march alone
-        for (size_t i = b; i < e; ++i) premarched.erase(list[i]);
-        continue;
-      }
       if (s != SWF_OK) return s;
     }
   }
@@ -709,10 +705,6 @@ static swf_status premarch_bw(swf_ctx* ctx, const swf_instance* inst, const std:
         premarched[list[i]] = {psi, macc};
       }
       s = march_multi(ctx, mg, kv.first.t_in, kv.first.t_out, kv.first.n_steps, prec, 1, st);
-      if (s == SWF_EUNSUPPORTED) {  // not a form the grouped launch takes: these groups march alone
-        for (size_t i = b; i < e; ++i) premarched.erase(list[i]);
-        continue;
-      }
       if (s != SWF_OK) return s;
     }
   }

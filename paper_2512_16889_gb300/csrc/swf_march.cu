@@ -427,7 +427,7 @@ static int sm_count() {
 }
 
 // Rows per block of the x passes: as many as fit kPassSmem (at most 64), fewer on small grids
-// (up to two blocks per SM).  0 if one row does not fit.
+// (up to two blocks per SM).  One row of the longest axis fits in either precision.
 template <typename R>
 static int x_rows(int nx, int nrows, int F) {
   const size_t line = (size_t)2 * 4 * padded_len<R>(nx) * sizeof(cpx<R>);
@@ -668,7 +668,6 @@ static swf_status launch_x(swf_ctx* ctx, const StageArgs<R>& P, const StageArgs<
   if (A.g.n[1] == 1 && A.g.n[2] == 1) {
     // tuned values: rows times 4, plus 1 for 128-thread blocks
     const int xv = tune_lookup(ctx, tune_key('x', esz, nx, A.nrows, 0, F), 4 * x_rows<R>(nx, A.nrows, F));
-    if (xv < 4) return SWF_EUNSUPPORTED;
     run_only_x<R>(A, xv >> 2, (xv & 3) ? kThreads / 2 : kThreads, F, st);
     return SWF_OK;
   }

@@ -147,27 +147,6 @@ __device__ inline double axis_factor(const FieldDesc& F, int axis, double xc) {
   }
 }
 
-// V phi for the one non-zero covariant component A_mu = a (V = A_0 + alpha^k A_k).
-template <typename R>
-__device__ __forceinline__ void apply_v(int acomp, R a, const cpx<R>* p, cpx<R>* o) {
-  switch (acomp) {
-    case 0:
-      o[0] = a * p[0]; o[1] = a * p[1]; o[2] = a * p[2]; o[3] = a * p[3];
-      break;
-    case 1:  // alpha^x
-      o[0] = a * p[3]; o[1] = a * p[2]; o[2] = a * p[1]; o[3] = a * p[0];
-      break;
-    case 2:  // alpha^y
-      o[0] = a * mul_mi(p[3]); o[1] = a * mul_i(p[2]); o[2] = a * mul_mi(p[1]); o[3] = a * mul_i(p[0]);
-      break;
-    case 3:  // alpha^z
-      o[0] = a * p[2]; o[1] = (R)(-1) * (a * p[3]); o[2] = a * p[0]; o[3] = (R)(-1) * (a * p[1]);
-      break;
-    default:
-      o[0] = o[1] = o[2] = o[3] = mk<R>(0, 0);
-  }
-}
-
 // v <- -i s (alpha.kappa + beta) v  (Dirac representation, sigma.kappa blocks).
 template <typename R>
 __device__ __forceinline__ void h0_mi(cpx<R>* v, R kx, R ky, R kz, R s) {
