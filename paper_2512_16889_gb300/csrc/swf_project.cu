@@ -207,8 +207,8 @@ __global__ void k_sum_parts(const T* __restrict__ part, int nb, int width, doubl
   }
 }
 
-// Blocks per field of a grid reduction: about four waves of the GPU, at least 8 elements a thread.
-int reduction_blocks(size_t elems, int n_f) {
+// Streaming multiprocessors of the device.
+int sms() {
   static int nsm = 0;
   if (nsm == 0) {
     int dev = 0;
@@ -216,8 +216,13 @@ int reduction_blocks(size_t elems, int n_f) {
                                                   cudaSuccess || nsm <= 0)
       nsm = 152;
   }
+  return nsm;
+}
+
+// Blocks per field of a grid reduction: about four waves of the GPU, at least 8 elements a thread.
+int reduction_blocks(size_t elems, int n_f) {
   const size_t by_size = (elems + 8 * kT - 1) / (8 * kT);
-  const size_t by_gpu = (4 * (size_t)nsm + n_f - 1) / n_f;
+  const size_t by_gpu = (4 * (size_t)sms() + n_f - 1) / n_f;
   size_t nb = by_size < by_gpu ? by_size : by_gpu;
   return nb < 1 ? 1 : (int)nb;
 }
@@ -310,7 +315,7 @@ swf_status c_spectrum(swf_ctx* ctx, const GridDesc& g, int n_f, const FieldDesc*
   if (e != cudaSuccess) return cuda_status(e, "upload field descriptors");
   // fields per thread: as many as leave about two blocks per SM
   const int nb = (g.N + kT - 1) / kT;
-  const int chunks = std::max(1, std::min(n_f, 304 / nb));
+  const int chunks = std::max(1, std::min(n_f, 2 * sms() / nb));
   const int fc = (n_f + chunks - 1) / chunks;
   ProfScope ps(ctx, "k_c_spectrum", st);
   k_c_spectrum<<<dim3(nb, (n_f + fc - 1) / fc), kT, 0, st>>>((const cpx<double>*)spec, (const FieldDesc*)pfd, g, n_f, fc,
