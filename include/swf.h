@@ -157,8 +157,9 @@ swf_status solve_swf_dev(swf_ctx* ctx, int n_inst, const swf_instance* inst, swf
  * momenta (Sec. II.A).  All instances must share field, grid and time window (EINVAL
  * otherwise); along trivial axes (n = 1) every p must be equal and every q = -p.  Only p, s of
  * the electrons and q, r of the positrons are read.  Marches each electron's U wave and each
- * positron's V wave once (n_e + n_p marches rather than 2 n_e n_p) and forms C, A, B and D as
- * complex FP64 matrix products over the grid (components x sites).
+ * positron's V wave once (n_e + n_p marches rather than 2 n_e n_p) and forms the overlaps in complex
+ * FP64: C and A as separable transforms of the marched waves at the other list's momenta, B and D as
+ * matrix products over the grid modes in the eigenbasis of their energies.
  * results: host array of n_e * n_p swf_result, row-major [m][n], with the layout of a
  * SWF_WANT_FULL_N instance: amp = {C, D, A, B}, prob = {|C + D|^2, |A + B|^2},
  * diag = {||psi_U,m||^2, ||psi_V,n||^2}.  Synchronous; uses the context's stream and workspace. */
@@ -205,7 +206,10 @@ swf_status swf_spectrum_dev(swf_ctx* ctx, int n_inst, const swf_instance* inst,
 
 /* Kernel timing hook (tracing).  When enabled, the context records a CUDA event pair on the
  * launching stream around every kernel it launches and accumulates the elapsed time per kernel
- * family.  swf_profile_read synchronises the context's events and returns up to max_entries
+ * family.  A family is what a launch does, not a kernel's name: k_first opens an evaluation (x pass),
+ * k_last closes one, k_last_first closes one and opens the next, k_mid is a y or z pass, whichever
+ * kernel the length and the precision take for them; launches of a multi-grid march have "_multi"
+ * appended.  swf_profile_read synchronises the context's events and returns up to max_entries
  * families: names (max_entries * 32 chars, NUL-terminated), total milliseconds and launch counts;
  * it then clears the accumulators.  *total_launches (optional) receives every kernel launched by
  * the context since the previous read, timed or not. */

@@ -7,12 +7,14 @@
 // inverse runs the same steps backwards.  Whatever happens on the sites between an inverse and the
 // next forward transform (k_i, the stage combine, the local term) or on the modes between a forward
 // and an inverse (H0) happens in the registers of the thread that owns them.  An evaluation's line
-// therefore passes through shared memory twice (Stockham passes: six times, with a barrier each), and global memory is read into and written from the same registers: n/R2 = R1
-// independent loads per thread and array, R2 (or R1) neighbouring points per load instruction.
+// therefore passes through shared memory twice (Stockham passes: six times, with a barrier each), and
+// global memory is read into and written from the same registers: n/R2 = R1 independent loads per thread
+// and array, R2 (or R1) neighbouring points per load instruction.
 //
 // What bounds them, and what they measured against the Stockham passes they replaced (complex64, per
-// launch): on 256^3 the x pass streams at 78 % of DRAM's peak (1276 -> 816 us) and the y and z passes
-// at 4.7 TB/s (489 -> 227 us); 16 fields of 256^2 beside the fused kernel, on 40 SMs: x pass 302 ->
+// launch): on 256^3 the x pass moves 8.8 arrays on average, 53 in the six launches of a step, at 5.8 TB/s,
+// 0.86 of the measured copy rate (1276 -> 816 us), and the y and z passes two each at 4.7 TB/s (489 ->
+// 227 us); 16 fields of 256^2 beside the fused kernel, on 40 SMs: x pass 302 ->
 // 177 us, y pass 147 -> 69 us (before: six barriers and six trips through shared memory per line, 20 %
 // of the issue slots used).  The x pass takes 128 registers (the older stage terms are summed before
 // the exchange, so that their loads overlap those of T); the y and z passes 64 where R1, R2 <= 16, for

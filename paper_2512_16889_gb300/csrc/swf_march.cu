@@ -745,7 +745,7 @@ static void set_next_node(StageArgs<R>* A, int ls, int i) {
 }
 
 // Times the candidate launch shapes of one evaluation's pass kernels (rows per block or tile
-// width, and 256- or 128-thread blocks) and records the fastest in ctx->tune (once per shape key).  B must be harmless to run repeatedly: it may write only
+// width; with x as the only axis also 256- or 128-thread blocks) and records the fastest in ctx->tune (once per shape key).  B must be harmless to run repeatedly: it may write only
 // T and its output slot, and read y and its input slots (the march calls this before its first
 // evaluation, when those hold nothing yet).  The shape decides only which lines a block
 // transforms, never the arithmetic of a line, so results do not depend on the choice.
@@ -1281,7 +1281,7 @@ static swf_status march_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double t_
   A.ynew = (cpx<R>*)pyn;
   ErrWeights W;
   for (int j = 0; j < 7; ++j) W.db[j] = DP_DB[j];
-  // the evaluations of an attempt chain through k_last_first; the attempt's last one is closed
+  // an attempt's evaluations chain (one x pass closes one and opens the next); the attempt's last one is closed
   // before the error estimate reads k_7
   const bool chain = !(g.n[1] == 1 && g.n[2] == 1);
   auto attempt = [&]() -> swf_status {
@@ -1461,11 +1461,13 @@ static swf_status reserve_march(swf_ctx* ctx, const GridDesc& g, int F) {
 // concurrently on those SMs, shortens the march when they finish within the fused kernel's
 // time.  With R = ceil(2 n_f / ncl) rounds of sectors per cluster, removing r rounds leaves
 // n_1 = floor((R - r) ncl / 2) fields to the clusters and n_2 = n_f - n_1 to the pass kernels,
-// which take about alpha n_2 rounds' time on the free SMs.  alpha was measured with 40 free SMs
-// on (2+1)D 256^2 complex64 marches: with the pushed-transpose kernel and the chained x passes,
-// 16 fields took 2.75 s on the free SMs while the fused launch took 32 rounds in 2.78 s
-// (alpha = 2.0); rounds of the pulled-transpose kernel are 1.46 times longer (alpha = 1.37).
-// alpha scales with 40 / (free SMs).  The largest r with alpha n_2 <= R - r is taken.
+// which take about alpha n_2 rounds' time on the free SMs.  alpha = 2.0 was measured with 40 free SMs
+// on (2+1)D 256^2 complex64 marches of 1000 steps with small-radix passes in shared memory: 16 fields took
+// 2.75 s on the free SMs while the fused launch took 32 rounds in 2.78 s; rounds of the pulled-transpose
+// kernel are 1.46 times longer (alpha = 1.37).  With the register lines 16 fields take 1.45 s beside 32
+// rounds in 2.46 s (alpha = 1.2), so the line lies on the safe side: the free SMs are done first.  Moving
+// it has not been measured.  alpha scales with 40 / (free SMs).  The largest r with alpha n_2 <= R - r is
+// taken.
 int fused_split_count(int n_f, int ncl, int n_sm, int variant) {
   const int free_sm = n_sm - kFusedClusterCtas * ncl;
   if (ncl < 1 || free_sm < 16 || n_f < 16) return 0;
@@ -2747,7 +2749,7 @@ static swf_status march_bw_adaptive_impl(swf_ctx* ctx, const GridDesc& g, double
                                                    (const double*)pph, g, (const cpx<double>*)prow, clk, 0, stage,
                                                    7, 1, (cpx<double>*)ptry);
   };
-  // the evaluations of an attempt chain through k_last_first (the integrand reads only the stage
+  // an attempt's evaluations chain through their x passes (the integrand reads only the stage
   // values); the attempt's last one is closed before the error estimate reads k_7
   const bool chain = !(g.n[1] == 1 && g.n[2] == 1);
   auto attempt = [&]() -> swf_status {
