@@ -118,13 +118,9 @@ __device__ __forceinline__ cpx<R> source_term(cpx<R> y, cpx<R> br, cpx<R> e, R a
   return rot.x != (R)0 ? rot.x * phi : mk<R>(-rot.y * phi.y, rot.y * phi.x);
 }
 
-// The last of A's stage combine and the local term: v becomes the stage value Y, which is stored where
-// A asks for it, and Z goes to the output slot (of the component this thread's one feeds) until the
-// evaluation is closed.  x = x0 + q stride are the sites' x indices, f, c, row the line, ftr and tf its
-// time factors.
+// The stage combine's end: v becomes the stage value Y, which is stored where A asks for it.
 template <typename R, int NV>
-__device__ __forceinline__ void open_sites(const StageArgs<R>& A, bool ff, size_t gs, int x0, int stride, int f, int c,
-                                           int row, R ftr, cpx<R> tf, cpx<R>* v) {
+__device__ __forceinline__ void finish_sites(const StageArgs<R>& A, bool ff, size_t gs, int stride, cpx<R>* v) {
   if (ff) {
     // the new state: (y, ylo) += the step's increment in float-float, so that the single-precision
     // rounding of y does not accumulate over steps
@@ -148,6 +144,15 @@ __device__ __forceinline__ void open_sites(const StageArgs<R>& A, bool ff, size_
 #pragma unroll
     for (int q = 0; q < NV; ++q) A.ystage[gs + q * stride] = v[q];
   }
+}
+
+// The same, then the local term: Z goes to the output slot (of the component this thread's one feeds)
+// until the evaluation is closed.  x = x0 + q stride are the sites' x indices, f, c, row the line, ftr and
+// tf its time factors.
+template <typename R, int NV>
+__device__ __forceinline__ void open_sites(const StageArgs<R>& A, bool ff, size_t gs, int x0, int stride, int f, int c,
+                                           int row, R ftr, cpx<R> tf, cpx<R>* v) {
+  finish_sites<R, NV>(A, ff, gs, stride, v);
   const int nx = A.g.n[0], ny = A.g.n[1], nz = A.g.n[2], nt = nx + ny + nz;
   const size_t N = A.g.N;
   const R* __restrict__ gx = A.greal + (size_t)f * nt;

@@ -137,58 +137,65 @@ static cudaError_t fill_tables(const StageArgs<R>& A, int F, const FieldDesc* fd
 }
 
 // ---------------------------------------------------------------- pass kernels
-// Shared memory of a whole-line transform (two line buffers, the FFT works out of place) by the fixed
-// rule, so that three blocks of 256 threads fit an SM; and the most that any pass may take.
-static const size_t kPassSmem = 72 * 1024;
-static const size_t kPassSmemMax = 200 * 1024;
+static const size_t kPassSmemMax = 200 * 1024;  // the most shared memory that a pass may take
 
-// Grids with x as the only non-trivial axis: `rows` rows (4 components each) per block, the whole
-// right-hand side in one launch.  Block (bx, f): rows bx*rows .. of field f.
+// Grids with x as the only non-trivial axis: the whole right-hand side of field blockIdx.y in one launch
+// and block.  A thread takes all four components of its sites, so that their loads are in flight together,
+// and what the sites share of the background is formed once: an evaluation of one field of 512 points
+// takes 15 us in complex64 and 65 in complex128, 18 and 77 with a component a thread (and, in complex128,
+// small radices for every length).
 template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_first(StageArgs<R> A, int rows, int ld) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_first(StageArgs<R> A, int ld) {
   if (A.ctl && A.ctl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* buf = reinterpret_cast<cpx<R>*>(smem_raw);
-  cpx<R>* buf2 = buf + 4 * rows * ld;
-  __shared__ R s_ft[64];
+  cpx<R>* buf2 = buf + 4 * ld;
+  __shared__ R s_ft;
   __shared__ cpx<R> s_tf;
-  const int f = blockIdx.y, row0 = blockIdx.x * rows;
-  const int nx = A.g.n[0];
-  const size_t N = A.g.N;
-  row_factors(A, false, f, row0, rows, s_ft, &s_tf);
+  const int f = blockIdx.y, nx = A.g.n[0];
+  const size_t N = A.g.N, fo = (size_t)f * 4 * N;
+  row_factors(A, false, f, 0, 1, &s_ft, &s_tf);
   __syncthreads();
   const bool ff = sizeof(R) == 4 && A.ylo && A.write_y;
-  for (int e = threadIdx.x; e < 4 * rows * nx; e += blockDim.x) {
-    const int l = e / nx, x = e - l * nx;  // line l: row l / 4, component l % 4
-    const int row = row0 + (l >> 2), c = l & 3;
-    cpx<R> v = mk<R>(0, 0);
-    if (row < A.nrows) {
-      const size_t gi = ((size_t)f * 4 + c) * N + (size_t)row * nx + x;
-      combine_sites<R, 1>(A, A.nterm, ff, gi, 0, &v);
-      open_sites<R, 1>(A, ff, gi, x, 0, f, c, row, s_ft[l >> 2], s_tf, &v);
+  const FieldDesc* F = A.fd + f;
+  const int acomp = F->acomp, nt = nx + 2;
+  const R* __restrict__ gx = A.greal + (size_t)f * nt;
+  const cpx<R>* __restrict__ ex = A.gcplx + (size_t)f * (nt + 4);
+  const R ar = s_ft * gx[nx] * gx[nx + 1];
+  cpx<R> br[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) br[c] = ex[nt + c] * (s_tf * (ex[nx] * ex[nx + 1]));
+  for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+    const cpx<R> e = ex[x];
+    const R a = ar * gx[x];
+    cpx<R> v[4];
+    combine_sites<R, 4>(A, A.nterm, ff, fo + x, A.g.N, v);
+    finish_sites<R, 4>(A, ff, fo + x, A.g.N, v);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      A.kout[fo + source_component(acomp, c) * N + x] = source_term<R>(v[c], br[c], e, a, source_rotation<R>(acomp, c));
+      buf[c * ld + pad<R>(x)] = v[c];
     }
-    buf[l * ld + pad<R>(x)] = v;
   }
   __syncthreads();
-  cpx<R>* res = fft_pp<R>(buf, buf2, ld, 4 * rows, A.plan[0], false, A.tw[0]);
-  const FieldDesc* F = A.fd + f;
+  cpx<R>* res = fft_pp<R>(buf, buf2, ld, 4, A.plan[0], false, A.tw[0]);
   const R kx0 = (R)F->K[0], ky = (R)F->K[1], kz = (R)F->K[2];
-  for (int e = threadIdx.x; e < rows * nx; e += blockDim.x) {
-    const int j = e / nx, x = e - j * nx;
-    cpx<R>* l = res + 4 * j * ld + pad<R>(x);
+  for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+    cpx<R>* l = res + pad<R>(x);
     cpx<R> v[4] = {l[0], l[ld], l[2 * ld], l[3 * ld]};
     h0_mi<R>(v, nx > 1 ? A.kap[x] : kx0, ky, kz, A.inv_n);
 #pragma unroll
     for (int c = 0; c < 4; ++c) l[c * ld] = v[c];
   }
   __syncthreads();
-  res = fft_pp<R>(res, res == buf ? buf2 : buf, ld, 4 * rows, A.plan[0], true, A.tw[0]);
-  for (int e = threadIdx.x; e < 4 * rows * nx; e += blockDim.x) {
-    const int l = e / nx, x = e - l * nx;
-    const int row = row0 + (l >> 2);
-    if (row >= A.nrows) continue;
-    const size_t gi = ((size_t)f * 4 + (l & 3)) * N + (size_t)row * nx + x;
-    A.kout[gi] = A.kout[gi] + res[l * ld + pad<R>(x)];
+  res = fft_pp<R>(res, res == buf ? buf2 : buf, ld, 4, A.plan[0], true, A.tw[0]);
+  for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+    cpx<R>* k = A.kout + fo + x;
+    cpx<R> v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = k[c * N];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) k[c * N] = v[c] + res[c * ld + pad<R>(x)];
   }
 }
 
@@ -405,12 +412,17 @@ static bool make_march_plan(int n, RadixPlan* pl) {
   return m == 1;
 }
 
-// The plan of an axis: whole-line transforms where x is the only axis in complex64, small-radix
-// passes otherwise.
+// The plan of an axis: small radices, and where x is the only axis the composite radices of whole-line
+// transforms in complex64 and, in complex128, for lines long enough that their few butterflies still give
+// every quarter of the SM a warp (one field of 512 points 13.0 against 13.6 ms for 40 steps, of 384 10.5
+// against 11.0; of 256 points 9.1 against 7.3 ms with small radices, and of lengths without a factor 16
+// the small ones are the faster ones as well).  The plan depends on the length alone: a field has the same
+// bits among any number of others.
 template <typename R>
 static bool make_line_plan(const GridDesc& g, int axis, RadixPlan* pl) {
-  const bool only_x = g.n[1] == 1 && g.n[2] == 1;
-  return sizeof(R) == 4 && only_x ? make_march_plan(g.n[axis], pl) : make_pass_plan(g.n[axis], pl);
+  const int n = g.n[axis];
+  const bool whole = g.n[1] == 1 && g.n[2] == 1 && (sizeof(R) == 4 || (n >= 384 && n % 16 == 0));
+  return whole ? make_march_plan(n, pl) : make_pass_plan(n, pl);
 }
 
 // Streaming multiprocessors of the current device (cached per device).
@@ -424,18 +436,6 @@ static int sm_count() {
     cache[dev] = n;
   }
   return cache[dev];
-}
-
-// Rows per block of the x passes: as many as fit kPassSmem (at most 64), fewer on small grids
-// (up to two blocks per SM).  One row of the longest axis fits in either precision.
-template <typename R>
-static int x_rows(int nx, int nrows, int F) {
-  const size_t line = (size_t)2 * 4 * padded_len<R>(nx) * sizeof(cpx<R>);
-  int rows = (int)(kPassSmem / line);
-  if (rows > 64) rows = 64;
-  if (rows > nrows) rows = nrows;
-  while (rows > 1 && (long)F * ((nrows + rows - 1) / rows) < 2L * sm_count()) rows = (rows + 1) / 2;
-  return rows;
 }
 
 // Keys of the tuned shapes: pass kind, element size and the sizes that decide the launch.
@@ -649,11 +649,11 @@ static void run_mid(const StageArgs<R>& A, int axis, int lg, int flags, bool fac
   else launch_chained(k_mid<R>, grid, S.thr, S.smem, st, A, axis, lg, S.ld, S.tpl, flags);
 }
 
-// Grids with x as the only axis: `rows` rows per block of k_first, `thr` threads.
+// Grids with x as the only axis: k_first with `thr` threads a block.
 template <typename R>
-static void run_only_x(const StageArgs<R>& A, int rows, int thr, int F, cudaStream_t st) {
+static void run_only_x(const StageArgs<R>& A, int thr, int F, cudaStream_t st) {
   const int ld = padded_len<R>(A.g.n[0]);
-  k_first<R><<<dim3((A.nrows + rows - 1) / rows, F), thr, (size_t)8 * rows * ld * sizeof(cpx<R>), st>>>(A, rows, ld);
+  k_first<R><<<dim3(1, F), thr, (size_t)8 * ld * sizeof(cpx<R>), st>>>(A, ld);
 }
 
 // One x pass: closes evaluation P (close) and/or opens evaluation A (open) on the same rows; factors:
@@ -666,9 +666,7 @@ static swf_status launch_x(swf_ctx* ctx, const StageArgs<R>& P, const StageArgs<
   const int nx = A.g.n[0];
   ProfScope ps(ctx, close ? (open ? "k_last_first" : "k_last") : "k_first", st);
   if (A.g.n[1] == 1 && A.g.n[2] == 1) {
-    // tuned values: rows times 4, plus 1 for 128-thread blocks
-    const int xv = tune_lookup(ctx, tune_key('x', esz, nx, A.nrows, 0, F), 4 * x_rows<R>(nx, A.nrows, F));
-    run_only_x<R>(A, xv >> 2, (xv & 3) ? kThreads / 2 : kThreads, F, st);
+    run_only_x<R>(A, tune_lookup(ctx, tune_key('x', esz, nx, A.nrows, 0, F), kThreads), F, st);
     return SWF_OK;
   }
   const int rows = tune_lookup(ctx, tune_key('X', esz, nx, A.nrows, 0, F), x_rule<R>(A, F));
@@ -781,15 +779,12 @@ static swf_status autotune_eval(swf_ctx* ctx, const StageArgs<R>& B, int F, cuda
   if (only_x) {
     const std::string key = tune_key('x', esz, nx, B.nrows, 0, F);
     if (!ctx->tune.best.count(key)) {
-      int rmax = (int)(kPassSmemMax / ((size_t)8 * padded_len<R>(nx) * esz));
-      rmax = std::min(std::min(rmax, 64), B.nrows);
-      int best = 4 * x_rows<R>(nx, B.nrows, F);
+      int best = kThreads;
       float tbest = 3.4e38f;
-      for (int rows = 1; rows <= rmax && status == SWF_OK; rows *= 2)
-        for (int half = 0; half < 2 && status == SWF_OK; ++half) {
-          const float t = timed([&] { run_only_x<R>(B, rows, half ? kThreads / 2 : kThreads, F, st); });
-          if (t < tbest) { tbest = t; best = 4 * rows + half; }
-        }
+      for (int thr = kThreads; thr >= kThreads / 2 && status == SWF_OK; thr /= 2) {
+        const float t = timed([&] { run_only_x<R>(B, thr, F, st); });
+        if (t < tbest) { tbest = t; best = thr; }
+      }
       if (status == SWF_OK) ctx->tune.best[key] = best;
     }
   } else {
