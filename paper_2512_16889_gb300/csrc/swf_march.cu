@@ -599,12 +599,25 @@ static int mid_rule(const StageArgs<R>& A, int axis, long tiles) {
   return lg;
 }
 
-// Launches a kernel of a march's chain so that its blocks may be set up before the kernel in front of it
-// on the stream has ended (it waits for that itself: chain_wait).  It pays where the passes are short
-// and launched one by one: a right-hand side on 64 x 64 took 46 us with it, 52 us without; steps replayed from
-// a graph gain nothing and lose nothing.
+// Whether a pass's blocks may be set up before the pass in front of it has ended.  It pays where the passes
+// are short and launched one by one (a right-hand side on 64 x 64 took 46 us with it, 52 us without), and
+// in complex64 also in the steps replayed from a graph (one field of 64 x 64 2.17 against 2.37 ms for 40
+// steps).  Replayed complex128 passes are launched plainly: blocks set up early go to the SMs that happen
+// to be free, and where a pass has a block or two per SM, FP64 issue then lies on some SMs twice and on
+// others not at all (four fields of 243 x 45: 25.7 ms, 21.2 launched plainly; of 405 x 30 23.3 and 18.7; two of
+// 128 x 128 13.0 and 11.3).  The smallest grids lose 2 to 6 % by it (one field of 64 x 64 6.12 and 6.40 ms).
+template <typename R>
+static bool may_chain(cudaStream_t st) {
+  if (sizeof(R) == 4) return true;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+}
+
+// Launches a kernel of a march's chain, with `chained` so that its blocks may be set up before the kernel
+// in front of it on the stream has ended (it waits for that itself: chain_wait).
 template <typename... P, typename... Q>
-static void launch_chained(void (*kernel)(P...), dim3 grid, int thr, size_t smem, cudaStream_t st, Q... args) {
+static void launch_chained(bool chained, void (*kernel)(P...), dim3 grid, int thr, size_t smem, cudaStream_t st,
+                           Q... args) {
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -614,7 +627,7 @@ static void launch_chained(void (*kernel)(P...), dim3 grid, int thr, size_t smem
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = chained ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, P(args)...);  // an error stays for the caller's cudaGetLastError
 }
 
@@ -624,7 +637,7 @@ static void run_x(const StageArgs<R>& P, const StageArgs<R>& A, int rows, int fl
   const PassShape S = x_shape<R>(A, rows);
   const dim3 grid((A.nrows + rows - 1) / rows, F);
   if (A.ltw[0]) {
-    launch_chained(line_entry<R>(A.g.n[0])->x, grid, S.thr, S.smem, st, P, A, rows, flags);
+    launch_chained(may_chain<R>(st), line_entry<R>(A.g.n[0])->x, grid, S.thr, S.smem, st, P, A, rows, flags);
     return;
   }
   auto* kernel = k_xpass<R, 1>;
@@ -635,7 +648,7 @@ static void run_x(const StageArgs<R>& P, const StageArgs<R>& A, int rows, int fl
     case 5: kernel = k_xpass<R, 5>; break;
     default: break;
   }
-  launch_chained(kernel, grid, S.thr, S.smem, st, P, A, rows, S.ld, S.tpl, flags);
+  launch_chained(may_chain<R>(st), kernel, grid, S.thr, S.smem, st, P, A, rows, S.ld, S.tpl, flags);
 }
 
 // Launches the y or z pass, 2^lg columns per block; factors: with the blocks that compute the coming
@@ -645,8 +658,9 @@ static void run_mid(const StageArgs<R>& A, int axis, int lg, int flags, bool fac
   const PassShape S = mid_shape<R>(A, axis, lg);
   const int tiles = ((A.g.n[0] + (1 << lg) - 1) >> lg) * (axis == 1 ? A.g.n[2] : A.g.n[1]);
   const dim3 grid(tiles + (factors ? 1 : 0), F);
-  if (A.ltw[axis]) launch_chained(line_entry<R>(A.g.n[axis])->line, grid, S.thr, S.smem, st, A, axis, lg, flags);
-  else launch_chained(k_mid<R>, grid, S.thr, S.smem, st, A, axis, lg, S.ld, S.tpl, flags);
+  const bool chained = may_chain<R>(st);
+  if (A.ltw[axis]) launch_chained(chained, line_entry<R>(A.g.n[axis])->line, grid, S.thr, S.smem, st, A, axis, lg, flags);
+  else launch_chained(chained, k_mid<R>, grid, S.thr, S.smem, st, A, axis, lg, S.ld, S.tpl, flags);
 }
 
 // Grids with x as the only axis: k_first with `thr` threads a block.
@@ -2529,7 +2543,7 @@ struct MarchPlan {
       }
       ProfScope ps(ctx, "k_mdot", st);
       auto* kernel = nph_blk == 1 ? k_mdot<R, 1> : nph_blk == 4 ? k_mdot<R, 4> : k_mdot<R, sizeof(R) == 4 ? 8 : 4>;
-      launch_chained(kernel, dim3(nb, n_inst * nchunk), 256, 0, st, (const cpx<R>*)pys, A.gcplx, (const cpx<R>*)pkph,
+      launch_chained(may_chain<R>(st), kernel, dim3(nb, n_inst * nchunk), 256, 0, st, (const cpx<R>*)pys, A.gcplx, (const cpx<R>*)pkph,
                      (const double*)pph, g, (const cpx<double>*)ptab, clk, ls, i, 7 * n_steps, n_ph, (cpx<double>*)ppart);
     }
     std::swap(slot[0], slot[6]);
