@@ -65,7 +65,10 @@ void ws_drop(swf_ctx* ctx, const std::string& name) {
 }
 
 swf_status ws_chunk(swf_ctx* ctx, const std::string& name, size_t per, int unit, int n, int* chunk, void** ptr) {
-  const size_t most = std::min<size_t>(65535, ((size_t)64 << 20) / per);
+  const auto held = ctx->ws.bufs.find(name);
+  const size_t room = !ctx->ws.limit ? (size_t)64 << 20
+                                     : std::max<size_t>((size_t)256 << 10, held == ctx->ws.bufs.end() ? 0 : held->second.second);
+  const size_t most = std::min<size_t>(65535, room / per);
   for (int units = (int)std::min<size_t>(n / unit, std::max<size_t>(1, most / unit));; units = (units + 1) / 2) {
     *chunk = units * unit;
     const swf_status s = ws_get(ctx, name, per * *chunk, ptr);
@@ -846,9 +849,11 @@ static swf_status bw_photon_scan(swf_ctx* ctx, const swf_instance& in, int n, co
                     (double2*)macc, st, 1, nullptr, n)) != SWF_OK)
     return s;
   if ((s = transform_fields(ctx, g, 2, prec, psi, (double2*)spec, st)) != SWF_OK) return s;
-  // U~(k_j - q) and V~(p - k_j) of every photon in one launch
-  if ((s = transform_at(ctx, g, 2 * n, prec, psi, kat.data(), (double2*)tat, st, 2)) != SWF_OK) return s;
+  // U~(k_j - q) and V~(p - k_j) of the photons, as many in a launch as there is room for beside the buffers
+  // that are needed after them
   if ((s = field_norms(ctx, g, 2, prec, psi, (double*)norms, st)) != SWF_OK) return s;
+  if ((s = bw_reserve(ctx, n, packet_out != nullptr)) != SWF_OK) return s;
+  if ((s = transform_at(ctx, g, 2 * n, prec, psi, kat.data(), (double2*)tat, st, 2)) != SWF_OK) return s;
   if ((s = bw_finalize(ctx, g, n, bw.data(), in.grid.t_in, (const double2*)spec, (const double2*)tat,
                        (const double2*)macc, (const double*)norms, (swf_result*)res, st)) != SWF_OK)
     return s;

@@ -368,6 +368,12 @@ swf_status bw_packet(swf_ctx* ctx, int n, const swf_result* results, const doubl
   return SWF_OK;
 }
 
+swf_status bw_reserve(swf_ctx* ctx, int n, bool packet) {
+  void* p;
+  const swf_status s = ws_get(ctx, "bw.inst", sizeof(BwInst) * n, &p);
+  return s == SWF_OK && packet ? ws_get(ctx, "bw.packet_w", sizeof(double) * 2 * (size_t)n, &p) : s;
+}
+
 size_t bw_inst_size() { return sizeof(BwInst); }
 
 void bw_fill_inst(void* dst, const swf_instance& in, int out, const FieldDesc& fu, const FieldDesc& fv,

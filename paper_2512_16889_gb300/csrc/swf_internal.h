@@ -172,8 +172,9 @@ swf_status ws_get(swf_ctx* ctx, const std::string& name, size_t bytes, void** pt
 bool ws_has(swf_ctx* ctx, const std::string& name, size_t bytes);
 void ws_drop(swf_ctx* ctx, const std::string& name);
 // A device buffer under `name` for a sum over up to n entries of `per` bytes each, taken in chunks: *chunk
-// receives the entries it holds, a multiple of `unit` (which divides n).  At most 64 MB and one grid.y
-// (65535 entries); less, down to one unit, where the workspace limit or the device's memory has no more.
+// receives the entries it holds, a multiple of `unit` (which divides n).  At most 64 MB, or under a
+// workspace limit (the room is other buffers' as well) what is held and at least 256 KB, and one grid.y
+// (65535 entries); less, down to one unit, where the limit or the device's memory has no more.
 swf_status ws_chunk(swf_ctx* ctx, const std::string& name, size_t per, int unit, int n, int* chunk, void** ptr);
 // Device table exp(-2 pi i m/n), m < n, in float2 (is_double = 0) or double2; with r2 > 0 in the order
 // of the register line kernels.
@@ -218,6 +219,8 @@ void bw_fill_inst(void* dst, const swf_instance& in, int out, const FieldDesc& f
 swf_status bw_finalize(swf_ctx* ctx, const GridDesc& g, int n_inst, const void* bw_host, double t_in,
                        const double2* spec, const double2* tat, const double2* macc, const double* norms,
                        swf_result* results, cudaStream_t st);
+// The tables that bw_finalize and (packet) bw_packet take for n amplitudes.
+swf_status bw_reserve(swf_ctx* ctx, int n, bool packet);
 // sum_j w_j amp_j of n results (4 complex: the three terms and M); weights_host [n] complex.
 swf_status bw_packet(swf_ctx* ctx, int n, const swf_result* results, const double* weights_host, double2* out,
                      cudaStream_t st);

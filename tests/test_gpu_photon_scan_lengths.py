@@ -51,16 +51,23 @@ def test_scan_beyond_one_launch(prec, count):
     ctx.close()
 
 
-def test_scan_under_a_workspace_limit():
-    """2000 photons on 320 x 320 need 114 MB without scratch that grows with the photons (its sums' parts
-    would take 16 MB more): the same bits under a limit just above."""
+# the buffers of such a scan without scratch that grows with the photons (its sums' parts would take 16 MB
+# more), and 8 KB for tables per row and field
+@pytest.mark.parametrize("prec,need", [("c64", 114_003_000), ("c128", 189_813_000)])
+def test_scan_under_a_workspace_limit(prec, need):
+    """2000 photons and their packet on 320 x 320 with room for no more than their own buffers: the same
+    bits, and again from the buffers that a scan without a limit has left."""
     from paper_2512_16889_gb300 import build, swf
     build.build()
-    inst, k, eps, _ = _scan(swf, (320, 320), 16 * np.pi, 2000)
+    p = swf.C64 if prec == "c64" else swf.C128
+    inst, k, eps, w = _scan(swf, (320, 320), 16 * np.pi, 2000)
     free, tight = swf.Context(0), swf.Context(0)
-    tight.set_workspace_limit(115_000_000)
-    a, _ = free.bw_photons(inst, k, eps, swf.C64)
-    b, _ = tight.bw_photons(inst, k, eps, swf.C64)
-    assert np.array_equal(a, b, equal_nan=True)  # a wrapped mode pair on the energy shell divides by zero
+    tight.set_workspace_limit(need + 8192)
+    a, pa = free.bw_photons(inst, k, eps, p, weights=w)
+    b, pb = tight.bw_photons(inst, k, eps, p, weights=w)
+    free.set_workspace_limit(1)
+    c, pc = free.bw_photons(inst, k, eps, p, weights=w)
+    for x, y in ((a, b), (pa, pb), (a, c), (pa, pc)):
+        assert np.array_equal(x, y, equal_nan=True)  # a wrapped mode pair on the energy shell divides by zero
     free.close()
     tight.close()
