@@ -538,11 +538,15 @@ static swf_status line_ready(const LineEntry<R>* e) {
 }
 
 // Launch shape of an x pass (v rows per block) or of a y or z pass (2^v columns per block) of either
-// kind, and the largest v that fits a block.
+// kind.  A small-radix y or z tile of more lines than have a thread per butterfly gives its threads several
+// butterflies each: with a thread per butterfly, lines of 243 points and more came one column at a time (8
+// bytes of every 32), and one field of 486 x 486 took 37 us a y pass in complex64 (29 in tiles of more
+// columns), of 512 x 512 189 us in complex128 (174).  The fixed rule keeps to a thread per butterfly, which
+// spreads small grids further; the timed shapes include both.
 struct PassShape {
   int thr = 0, ld = 0, tpl = 0;
   size_t smem = 0;
-  bool fits = false;
+  bool fits = false, shared = false;  // shared: a thread does several butterflies where one line has more threads
 };
 template <typename R>
 static PassShape x_shape(const StageArgs<R>& A, int rows) {
@@ -572,7 +576,8 @@ static PassShape mid_shape(const StageArgs<R>& A, int axis, int lg) {
     S.fits = lg <= line_max_lg<R>(e, nx);
   } else {
     S.ld = padded_len<R>(A.g.n[axis]) | 1;  // neighbouring threads hold neighbouring lines
-    S.tpl = pass_threads(A.plan[axis], 4);
+    S.tpl = pass_threads(A.plan[axis], 4 << lg);
+    S.shared = S.tpl < pass_threads(A.plan[axis], 4);
     S.thr = ((4 << lg) * S.tpl + 31) & ~31;  // whole warps: the shuffles of H0 name all 32 lanes
     S.smem = ((size_t)8 << lg) * S.ld * sizeof(cpx<R>);
     S.fits = lg <= 3 && (lg == 0 || (1 << lg) <= nx) && S.thr <= kPassThreads && S.smem <= kPassSmemMax;
@@ -594,7 +599,10 @@ template <typename R>
 static int mid_rule(const StageArgs<R>& A, int axis, long tiles) {
   const int nx = A.g.n[0], min_lg = sizeof(cpx<R>) == 8 ? 2 : 1;
   int lg = 3;
-  while (lg > 0 && !mid_shape<R>(A, axis, lg).fits) --lg;
+  for (; lg > 0; --lg) {
+    const PassShape S = mid_shape<R>(A, axis, lg);
+    if (S.fits && !S.shared) break;
+  }
   while (lg > min_lg && tiles * ((nx + (1 << lg) - 1) >> lg) < 2L * sm_count()) --lg;
   return lg;
 }
